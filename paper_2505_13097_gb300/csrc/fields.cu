@@ -198,7 +198,7 @@ __global__ void front_kernel(const Problem* dprob, int parity, int wall, double*
             const int i = c + lane;
             const double th = i < n ? theta_at(i) : 0.0;
             if (i < n) {
-                const double ph = 0.5 + 0.5 * tanh(th * pb.inv_delta);
+                const double ph = phi_of(th, pb.inv_delta);
                 sum += hot ? ph : 1.0 - ph;
             }
             if (fz < 0.0) {

@@ -63,7 +63,6 @@ __device__ __forceinline__ void ff_add(ff& a, float b)
     a.hi = s;
     a.lo = __fadd_rn(a.lo, e);
 }
-__device__ __forceinline__ double ff_to_double(const ff& a) { return (double)a.hi + (double)a.lo; }
 
 // Approximate float of a double from its high word only (sign, exponent and
 // 20 mantissa bits; relative error < 2^-20), using the integer pipe.  Values
@@ -77,6 +76,30 @@ __device__ __forceinline__ float approx_float(double d)
     return e <= 896 ? 0.0f : (e >= 1151 ? __int_as_float(0x7fc00000) : r);
 }
 
+// The same truncated to all 23 mantissa bits (relative error < 2^-23).
+__device__ __forceinline__ float trunc_float(double d)
+{
+    const unsigned hi = (unsigned)__double2hiint(d);
+    const int e = (int)((hi >> 20) & 0x7ff);
+    const unsigned bits = (hi & 0x80000000u) |
+                          (__funnelshift_l((unsigned)__double2loint(d), (hi & 0x7fffffffu) - (896u << 20), 3) & 0x7fffffffu);
+    return e <= 896 ? 0.0f : (e >= 1151 ? __int_as_float(0x7fc00000) : __uint_as_float(bits));
+}
+
+// A float as a double with integer operations (a conversion instruction runs
+// on the FP64 pipe, an SM's narrowest: 64 cycles of a quarter's issue slots).
+// Exact; subnormal floats give 0.
+__device__ __forceinline__ double widen(float f)
+{
+    const unsigned b = __float_as_uint(f);
+    const unsigned e = (b >> 23) & 0xffu;
+    if (e == 0xffu) return (double)f;   // infinity, NaN
+    const unsigned hi = e == 0u ? 0u : (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20));
+    return __hiloint2double((int)hi, e == 0u ? 0 : (int)(b << 29));
+}
+
+__device__ __forceinline__ double ff_to_double(const ff& a) { return widen(a.hi) + widen(a.lo); }
+
 // ---------------------------------------------------------------- liquid fraction
 // EEBM (Algorithm 2): temperature of an enthalpy, Theta(H) = H below 0, 0 on
 // the melting plateau [0, 1/Ste], H - 1/Ste above it.
@@ -89,8 +112,89 @@ __device__ __forceinline__ float eebm_theta(float H, float inv_ste)
     return H < 0.0f ? H : (H > inv_ste ? H - inv_ste : 0.0f);
 }
 
-// phi(x) = (1 + tanh(x/delta))/2 (Sec. 4.1) and phi' = (1 - t)(1 + t)/(2 delta).
-__device__ __forceinline__ double phi_of(double x, double inv_delta) { return 0.5 + 0.5 * tanh(x * inv_delta); }
+// 2^(j/64), rounded to nearest
+static __device__ const double kExp2[64] = {
+    0x1.p+0, 0x1.02c9a3e778061p+0, 0x1.059b0d3158574p+0, 0x1.0874518759bc8p+0,
+    0x1.0b5586cf9890fp+0, 0x1.0e3ec32d3d1a2p+0, 0x1.11301d0125b51p+0, 0x1.1429aaea92de0p+0,
+    0x1.172b83c7d517bp+0, 0x1.1a35beb6fcb75p+0, 0x1.1d4873168b9aap+0, 0x1.2063b88628cd6p+0,
+    0x1.2387a6e756238p+0, 0x1.26b4565e27cddp+0, 0x1.29e9df51fdee1p+0, 0x1.2d285a6e4030bp+0,
+    0x1.306fe0a31b715p+0, 0x1.33c08b26416ffp+0, 0x1.371a7373aa9cbp+0, 0x1.3a7db34e59ff7p+0,
+    0x1.3dea64c123422p+0, 0x1.4160a21f72e2ap+0, 0x1.44e086061892dp+0, 0x1.486a2b5c13cd0p+0,
+    0x1.4bfdad5362a27p+0, 0x1.4f9b2769d2ca7p+0, 0x1.5342b569d4f82p+0, 0x1.56f4736b527dap+0,
+    0x1.5ab07dd485429p+0, 0x1.5e76f15ad2148p+0, 0x1.6247eb03a5585p+0, 0x1.6623882552225p+0,
+    0x1.6a09e667f3bcdp+0, 0x1.6dfb23c651a2fp+0, 0x1.71f75e8ec5f74p+0, 0x1.75feb564267c9p+0,
+    0x1.7a11473eb0187p+0, 0x1.7e2f336cf4e62p+0, 0x1.82589994cce13p+0, 0x1.868d99b4492edp+0,
+    0x1.8ace5422aa0dbp+0, 0x1.8f1ae99157736p+0, 0x1.93737b0cdc5e5p+0, 0x1.97d829fde4e50p+0,
+    0x1.9c49182a3f090p+0, 0x1.a0c667b5de565p+0, 0x1.a5503b23e255dp+0, 0x1.a9e6b5579fdbfp+0,
+    0x1.ae89f995ad3adp+0, 0x1.b33a2b84f15fbp+0, 0x1.b7f76f2fb5e47p+0, 0x1.bcc1e904bc1d2p+0,
+    0x1.c199bdd85529cp+0, 0x1.c67f12e57d14bp+0, 0x1.cb720dcef9069p+0, 0x1.d072d4a07897cp+0,
+    0x1.d5818dcfba487p+0, 0x1.da9e603db3285p+0, 0x1.dfc97337b9b5fp+0, 0x1.e502ee78b3ff6p+0,
+    0x1.ea4afa2a490dap+0, 0x1.efa1bee615a27p+0, 0x1.f50765b6e4540p+0, 0x1.fa7c1819e90d8p+0,
+};
+
+// exp(-w) for w in [0, 39) by table-driven reduction (P. T. P. Tang, "Table-driven
+// implementation of the exponential function in IEEE floating-point arithmetic",
+// ACM TOMS 15, 1989): N = rint(-64 w / ln 2), r = -w - N ln2/64 with ln2/64 in two
+// parts, e^r from its Taylor polynomial (|r| <= 0.0055: the remainder is below
+// 4e-17), times 2^((N mod 64)/64) from the table and 2^(N div 64) added to the
+// exponent.  Ten FP64 instructions, no branch.
+__device__ __forceinline__ double exp_neg(double w)
+{
+    const double t = fma(w, -0x1.71547652b82fep+6, 0x1.8p+52);   // the integer N in the low word
+    const int n = __double2loint(t);
+    const double nd = t - 0x1.8p+52;
+    double r = fma(nd, -0x1.62e42fefa2000p-7, -w);
+    r = fma(nd, -0x1.9ef35793c7673p-47, r);
+    double p = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+    p = fma(p, r, 1.0 / 6.0);
+    p = fma(p, r, 0.5);
+    p = fma(r * r, p, r);
+    const double T = __ldg(&kExp2[n & 63]);
+    const double e = fma(T, p, T);
+    return __hiloint2double(__double2hiint(e) + ((n >> 6) << 20), __double2loint(e));
+}
+
+// 1/d for d in [1, 2]: an FP32 reciprocal (relative error e < 2^-21) and one
+// third-order step, r0 (1 + e + e^2), remainder e^3 < 2^-63.
+__device__ __forceinline__ double rcp_1_2(double d)
+{
+    const double r0 = widen(__frcp_rn(trunc_float(d)));
+    double e = fma(-d, r0, 1.0);
+    e = fma(e, e, e);
+    return fma(r0, e, r0);
+}
+
+// The liquid fraction phi(x) = (1 + tanh(x/delta))/2 (Sec. 4.1) as the logistic
+// function it is, 1/(1 + exp(-2x/delta)): with E = exp(-2|x|/delta) and
+// r = 1/(1 + E), phi = r for x >= 0 and E r below, and phi' = 2 E r^2 / delta.
+// One exponential and one reciprocal, without a branch between ranges (a warp
+// whose lanes straddle the ranges of a library tanh runs both): 17 FP64
+// instructions.  |x| >= 19.5 delta: E = 0, where tanh rounds to +-1.
+struct Phi {
+    double E, r;   // NaN for a NaN x
+    bool neg;
+    __device__ __forceinline__ double value() const { return neg ? E * r : r; }
+    __device__ __forceinline__ double s() const { return E * r * r; }   // phi (1 - phi) = phi' delta / 2
+};
+
+__device__ __forceinline__ Phi phi_parts(double x, double two_inv_delta)
+{
+    const double z = x * two_inv_delta;
+    const int h = __double2hiint(z) & 0x7fffffff;
+    Phi p;
+    p.neg = __double2hiint(z) < 0;
+    if (h >= 0x40438000) {   // |z| >= 39, infinite or NaN
+        const bool nan = h > 0x7ff00000 || (h == 0x7ff00000 && __double2loint(z) != 0);
+        p.E = nan ? z : 0.0;
+        p.r = nan ? z : 1.0;
+    } else {
+        p.E = exp_neg(__hiloint2double(h, __double2loint(z)));
+        p.r = rcp_1_2(1.0 + p.E);
+    }
+    return p;
+}
+
+__device__ __forceinline__ double phi_of(double x, double inv_delta) { return phi_parts(x, inv_delta + inv_delta).value(); }
 
 // Local Newton solve of Eq. (14): the root of
 //   F(x) = (x - m0) + (phi(x) - phi(theta))/Ste,   F' = 1 + phi'(x)/Ste >= 1,
@@ -107,16 +211,17 @@ struct NewtonOut {
     bool ok;
 };
 
-__device__ __forceinline__ NewtonOut newton_solve(double m0, double theta, double phi_theta, double inv_ste,
-                                                  double inv_delta, double tol, int maxit)
+// Not inlined: the mixed-precision solve below falls back to it, which is rare.
+static __device__ __noinline__ NewtonOut newton_solve(double m0, double theta, double phi_theta, double inv_ste,
+                                                      double inv_delta, double tol, int maxit)
 {
     double lo = m0 + (phi_theta - 1.0) * inv_ste, hi = m0 + phi_theta * inv_ste;
     double x = theta;
     double step_old = hi - lo, step = step_old;
     NewtonOut r;
     for (int k = 0; k < maxit; ++k) {
-        double t = tanh(x * inv_delta);
-        double ph = 0.5 + 0.5 * t;
+        const Phi p = phi_parts(x, 2.0 * inv_delta);
+        const double ph = p.value();
         double F = (x - m0) + (ph - phi_theta) * inv_ste;
         if (F == 0.0) {
             r.root = x; r.phi_root = ph; r.iters = k; r.ok = true;
@@ -124,7 +229,7 @@ __device__ __forceinline__ NewtonOut newton_solve(double m0, double theta, doubl
         }
         if (F < 0.0) lo = fmax(lo, x);
         else hi = fmin(hi, x);
-        double dph = 0.5 * (1.0 - t) * (1.0 + t) * inv_delta;
+        double dph = 2.0 * p.s() * inv_delta;
         double xn = x - F / (1.0 + dph * inv_ste);
         double sc = tol * fmax(1.0, fabs(x));
         if (fabs(xn - x) <= sc) {
@@ -151,92 +256,115 @@ __device__ __forceinline__ NewtonOut newton_solve(double m0, double theta, doubl
 }
 
 // Mixed-precision form of the same solve (same root, same stopping rule).
-//  1. FP32 Newton (tanhf) locates the root to FP32 accuracy, x0 (it stops at
-//     FP32 precision or once its updates stop halving).
-//  2. FP64 step from x0: one FP64 tanh gives t = tanh(x0/delta), F, F', F''
-//     and F''' (F^(k) = phi^(k)/Ste, phi2 = -t(1-t^2)/delta^2,
-//     phi3 = (1-t^2)(3t^2-1)/delta^3), the Newton update dn = -F/F' (1/F' from
-//     an FP32 reciprocal and one FP64 Newton step: relative error ~1e-14) and
-//     Halley's update d = dn / (1 + dn F''/(2F')).  Halley's error e is about
-//     |F''^2/(4F'^2) - F'''/(6F')| |dn|^3, and theta' = m0 + (phi(theta) -
+//  1. FP32 Newton for the step u = x - theta.  The equation is
+//     u - (m0 - theta) + (phi(theta + u) - phi(theta))/Ste = 0 with the
+//     difference of phi from expm1 (no cancellation: with b = 2u/delta and
+//     m = expm1(-b), phi(theta + u) - phi(theta) = -E m r r1, r1 = 1/(1 + E(1 + m)),
+//     for theta >= 0; theta < 0 is its mirror image), so u is good to a few
+//     FP32 ulps of itself.  It stops when an update is below 1e-3 delta: the
+//     next error is then of the order of 1e-6 delta.
+//  2. FP64 step from x0 = theta + u: phi(x0) gives F, F' and the Newton update
+//     dn = -F/F' (1/F' from an FP32 reciprocal and one FP64 Newton step:
+//     relative error ~1e-14).  The second and third derivatives enter as
+//     corrections of relative size 1e-4 at most and are formed in FP32: Halley's
+//     update d = dn / (1 + dn F_2/(2F')).  Halley's error e is about
+//     |F_2^2/(4F'^2) - F_3/(6F')| |dn|^3, and theta' = m0 + (phi(theta) -
 //     phi(root))/Ste inherits it as (F' - 1) e; when F' e is below
 //     0.1 tol max(1,|x|) and |d| <= 3e-5 delta, x0 + d is accepted and
 //     phi(x0 + d) comes from the cubic Taylor expansion (the quartic remainder
-//     is below (d/delta)^4 / 12 < 1e-19).  From the FP32 start (|dn| ~ 1e-8)
-//     one FP64 evaluation suffices; a plain Newton step would leave F' e ~
-//     |F''| dn^2 / 2, above the tolerance in the middle of the band, and need a
-//     second one.  Otherwise the FP64 iteration goes on.  Iterations of both
-//     precisions count against maxit.
+//     is below (d/delta)^4 / 12 < 1e-19).  Otherwise the FP64 iteration goes on.
+//     Iterations of both precisions count against maxit.
 //  3. Anything unexpected (no FP32 convergence, an FP64 update larger than
 //     1e-3 delta) falls back to newton_solve from theta.
-// The FP32 and derived constants come converted in the Problem: on this GPU
-// every FP64 instruction, conversions included, shares the narrow FP64 pipe.
-__device__ __forceinline__ NewtonOut newton_mixed(double m0, double theta, double phi_theta, const Problem& pb)
+// A solve is bound by the FP64 pipe, one warp instruction per 64 cycles of an SM
+// quarter: about 65 FP64 instructions per node with the evaluation of phi(theta)
+// (236 with the library's tanh, conversion instructions and FP64 corrections;
+// counted per warp on the front band of a 1021 x 777 melting lattice).
+__device__ __forceinline__ NewtonOut newton_mixed(double m0, double theta, const Phi& pt, const Problem& pb)
 {
-    const double inv_ste = pb.inv_ste, inv_delta = pb.inv_delta, tol = pb.tol;
+    const double inv_ste = pb.inv_ste, tol = pb.tol;
     const int maxit = pb.maxit;
-    const float mf = (float)m0, pf = (float)phi_theta, isf = pb.inv_ste_f, idf = pb.inv_delta_f;
-    float lo = mf + (pf - 1.0f) * isf, hi = mf + pf * isf;
-    float x = (float)theta;
-    const float xfloor = pb.delta_f;
+    const double phi_theta = pt.value();
+    const float isf = pb.inv_ste_f, idf2 = 2.0f * pb.inv_delta_f;
+    const float thf = fabsf(trunc_float(theta));
+    const float dm0 = trunc_float(m0 - theta);
+    const float dm = pt.neg ? -dm0 : dm0;            // mirrored to theta >= 0
+    const float E = trunc_float(pt.E), r0 = trunc_float(pt.r);
+    float lo = dm + (r0 - 1.0f) * isf, hi = dm + r0 * isf;
+    float u = 0.0f;
+    const float small = 1e-3f * pb.delta_f;
     float step_prev = hi - lo;
     int k = 0;
-    // FP32 stage: plain Newton inside the bracket; it stops at FP32 precision or
-    // when the update no longer halves (the FP32 rounding floor of F is reached).
-    // Only an iterate that leaves the bracket is replaced by the midpoint.
     for (; k < 16; ++k) {
-        const float t = tanhf(x * idf);
-        const float F = (x - mf) + (0.5f * t + 0.5f - pf) * isf;
-        if (F == 0.0f) break;
-        if (F < 0.0f) lo = fmaxf(lo, x);
-        else hi = fminf(hi, x);
-        const float dph = 0.5f * (1.0f - t) * (1.0f + t) * idf;
-        float xn = x - F / (1.0f + dph * isf);
-        if (!(xn >= lo && xn <= hi)) {
-            xn = 0.5f * (lo + hi);
+        const float b = idf2 * u;
+        float D, dph;   // phi(theta + u) - phi(theta), phi'(theta + u) delta / 2
+        if (fabsf(b) <= 20.0f) {
+            const float m = expm1f(-b);
+            const float E1 = fmaf(E, m, E);
+            const float r1 = __fdividef(1.0f, 1.0f + E1);
+            D = -E * m * r0 * r1;
+            dph = E1 * r1 * r1;
         } else {
-            const float st = fabsf(xn - x);
-            if (st <= 1e-7f * fmaxf(fabsf(x), xfloor) || (k >= 2 && st >= 0.5f * step_prev)) {
-                x = xn;
+            const float r1 = 1.0f / (1.0f + expf(-fmaf(idf2, thf, b)));
+            D = r1 - r0;
+            dph = r1 * (1.0f - r1);
+        }
+        const float F = (u - dm) + D * isf;
+        if (F == 0.0f) break;
+        if (F < 0.0f) lo = fmaxf(lo, u);
+        else hi = fminf(hi, u);
+        float un = u - F / (1.0f + dph * idf2 * isf);
+        if (!(un >= lo && un <= hi)) {
+            un = 0.5f * (lo + hi);
+        } else {
+            const float st = fabsf(un - u);
+            if (st <= small || (k >= 2 && st >= 0.5f * step_prev)) {
+                u = un;
                 ++k;
                 break;
             }
             step_prev = st;
         }
-        x = xn;
+        u = un;
     }
-    const bool conv32 = isfinite(x);
-    const double delta = pb.delta;
+    const bool conv32 = isfinite(u);
     if (conv32) {
-        double xd = (double)x;
+        double xd = theta + widen(pt.neg ? -u : u);
+        const float df = pb.delta_f, tolf = trunc_float(tol);
         for (int j = 0; j < 3; ++j) {
-            const double t = tanh(xd * inv_delta);
-            const double s = (1.0 - t) * (1.0 + t);
-            const double ph = 0.5 + 0.5 * t;
-            const double F = (xd - m0) + (ph - phi_theta) * inv_ste;
-            const double dph = 0.5 * s * inv_delta;
-            const double Fp = 1.0 + dph * inv_ste;
-            const double r0 = (double)(1.0f / (float)Fp);
-            const double rinv = fma(r0, fma(-Fp, r0, 1.0), r0);
+            const Phi p = phi_parts(xd, pb.two_inv_delta);
+            const double ph = p.value();
+            const double s = p.s();
+            const double F = fma(ph - phi_theta, inv_ste, xd - m0);
+            const double Fp = fma(s, pb.two_inv_delta_ste, 1.0);
+            const double g0 = widen(__frcp_rn(trunc_float(Fp)));
+            const double rinv = fma(g0, fma(-Fp, g0, 1.0), g0);
             const double dn = -F * rinv;   // Newton update
-            const double adn = fabs(dn);
-            if (adn > 1e-3 * delta) break;   // FP32 start not close enough: full FP64 solve
-            const double p2 = -t * s * pb.inv_delta2;                   // second derivative of phi
-            const double p3 = s * (3.0 * t * t - 1.0) * pb.inv_delta3;  // third derivative of phi
-            // Halley update d = dn / (1 + dn F''/(2F')), 1/(1 + eps) to second order (accepted only
+            const float dnf = trunc_float(dn), adn = fabsf(dnf);
+            if (!(adn <= 1e-3f * df)) break;   // FP32 start not close enough (or NaN): full FP64 solve
+            // derivatives of phi in units of delta: phi' = 2s/delta, phi_2 = -2 t phi'/delta,
+            // phi_3 = 2 phi' (3 t^2 - 1)/delta^2, t = tanh(x/delta) = +-(1 - E) r
+            const float sf = trunc_float(s), rf = trunc_float(p.r), Ef = trunc_float(p.E);
+            const float t = p.neg ? -(1.0f - Ef) * rf : (1.0f - Ef) * rf;
+            const float p1 = idf2 * sf;
+            const float p2 = -idf2 * t * p1;
+            const float p3 = 0.5f * idf2 * idf2 * (3.0f * t * t - 1.0f) * p1;
+            const float rif = trunc_float(rinv);
+            // Halley update d = dn / (1 + dn F_2/(2F')), 1/(1 + eps) to second order (accepted only
             // for |eps| <= 1e-4: the neglected eps^3 |dn| is below 1e-12 |dn|)
-            const double eps = 0.5 * dn * p2 * inv_ste * rinv;
-            const double d = dn * (1.0 - eps + eps * eps);
-            const double ad = fabs(d);
+            const float eps = 0.5f * dnf * p2 * isf * rif;
+            const double d = fma(dn, widen(eps * eps - eps), dn);
+            const float daf = trunc_float(d), ad = fabsf(daf);
             const double x1 = xd + d;
-            const double sc = tol * fmax(1.0, fabs(xd));
+            const float sc = tolf * fmaxf(1.0f, fabsf(trunc_float(xd)));
             // theta' = m0 + (phi(theta) - phi(x))/Ste carries a root error e as (F' - 1) e;
-            // after the Halley step F' e ~ |F''^2/(4F') - F'''/6| |dn|^3
-            const double g = (0.25 * p2 * p2 * inv_ste * rinv + fabs(p3) * (1.0 / 6.0)) * inv_ste;
-            if (ad <= sc || (ad <= 3e-5 * delta && fabs(eps) <= 1e-4 && g * adn * adn * adn <= 0.1 * sc)) {
+            // after the Halley step F' e ~ |F_2^2/(4F') - F_3/6| |dn|^3
+            const float g = (0.25f * p2 * p2 * isf * rif + fabsf(p3) * (1.0f / 6.0f)) * isf;
+            if (ad <= sc || (ad <= 3e-5f * df && fabsf(eps) <= 1e-4f && g * adn * adn * adn <= 0.1f * sc)) {
                 NewtonOut r;
                 r.root = x1;
-                r.phi_root = ph + d * (dph + d * (0.5 * p2 + d * p3 * (1.0 / 6.0)));
+                const double c1 = fma(s, pb.two_inv_delta, widen(daf * (0.5f * p2 + daf * p3 * (1.0f / 6.0f))));
+                r.phi_root = fma(d, c1, ph);
                 r.iters = k + j + 1;
                 r.ok = r.iters <= maxit;
                 return r;
@@ -244,7 +372,7 @@ __device__ __forceinline__ NewtonOut newton_mixed(double m0, double theta, doubl
             xd = x1;
         }
     }
-    NewtonOut r = newton_solve(m0, theta, phi_theta, inv_ste, inv_delta, tol, maxit);
+    NewtonOut r = newton_solve(m0, theta, phi_theta, inv_ste, pb.inv_delta, tol, maxit);
     r.iters += k;
     r.ok = r.ok && r.iters <= maxit;
     return r;
@@ -298,14 +426,30 @@ struct Fx {
     unsigned long long lo;
 };
 
+// With integer operations only (an FP64 conversion costs 64 cycles of an SM
+// quarter): v = m 2^(e - 1075), scaled by 2^60.  Bits below 2^-60 are dropped;
+// values of 2^66 and more, infinities and NaN give 0 (the solves report them).
 __device__ __forceinline__ Fx to_fixed(double v)
 {
-    Fx f;
-    const double s = v * 0.0625;   // v * 2^60 / 2^64
-    const double h = floor(s);
-    const double r = s - h;        // in [0, 1), exact
-    f.hi = (long long)h;
-    f.lo = __double2ull_rz(r * 18446744073709551616.0);
+    Fx f{0, 0ull};
+    const unsigned hw = (unsigned)__double2hiint(v);
+    const int e = (int)((hw >> 20) & 0x7ff);
+    const unsigned long long m = ((unsigned long long)((hw & 0xfffffu) | 0x100000u) << 32) | (unsigned)__double2loint(v);
+    const int sh = e - 1015;   // m * 2^(e - 1075 + 60)
+    unsigned long long lo = 0, hi = 0;
+    if (sh >= 0) {
+        if (sh >= 74) return f;
+        lo = sh < 64 ? m << sh : 0ull;
+        hi = sh == 0 ? 0ull : (sh < 64 ? m >> (64 - sh) : m << (sh - 64));
+    } else if (sh > -64 && e != 0) {
+        lo = m >> (-sh);
+    }
+    if (hw >> 31) {   // two's complement of the 128-bit value
+        lo = ~lo + 1ull;
+        hi = ~hi + (lo == 0ull ? 1ull : 0ull);
+    }
+    f.lo = lo;
+    f.hi = (long long)hi;
     return f;
 }
 

@@ -71,13 +71,13 @@ struct Problem {
     int nx, ny, pitch;
     int q;                   // 3 (D1Q3), 5 (D2Q5) or 9 (D2Q9)
     long long plane;         // elements per plane
-    double omega;            // 1/tau
+    double omega, omc;       // 1/tau, 1 - 1/tau
     double ste, inv_ste, delta, inv_delta;
     double tol;
     double sat;              // saturation threshold K*delta of the exact-source shortcut
     // constants of the mixed-precision Newton solve, converted on the host so
     // that a solve spends no FP64 instruction on them
-    double inv_delta2, inv_delta3;
+    double two_inv_delta, two_inv_delta_ste;   // 2/delta, 2/(delta Ste)
     float inv_ste_f, inv_delta_f, delta_f;
     float omega_f, omc_f, sat_f;   // (float) omega, (float)(1 - omega), (float) sat
     int maxit;

@@ -202,13 +202,14 @@ static void fill_problem(Problem& pb, int q, int nx, int ny, int pitch, double t
     // streams of a step do not fall on the same memory partitions
     pb.plane = (long long)(ny + 2) * pitch + LBM_PLANE_PAD;
     pb.omega = 1.0 / tau;
+    pb.omc = 1.0 - pb.omega;
     pb.ste = ste;
     pb.inv_ste = 1.0 / ste;
     pb.delta = delta;
     pb.inv_delta = 1.0 / delta;
     pb.tol = tol;
-    pb.inv_delta2 = pb.inv_delta * pb.inv_delta;
-    pb.inv_delta3 = pb.inv_delta2 * pb.inv_delta;
+    pb.two_inv_delta = 2.0 * pb.inv_delta;
+    pb.two_inv_delta_ste = pb.two_inv_delta * pb.inv_ste;
     pb.inv_ste_f = (float)pb.inv_ste;
     pb.inv_delta_f = (float)pb.inv_delta;
     pb.delta_f = (float)delta;
@@ -629,6 +630,7 @@ extern "C" lbm_status lbm_stefan_set_ste(lbm_stefan* h, double ste)
     h->hp.ste = ste;
     h->hp.inv_ste = 1.0 / ste;
     h->hp.inv_ste_f = (float)h->hp.inv_ste;
+    h->hp.two_inv_delta_ste = h->hp.two_inv_delta * h->hp.inv_ste;
     h->hp.sat = saturation_threshold(h->precision, h->hp.delta, ste);
     h->hp.sat_f = (float)h->hp.sat;
     h->graph.reset();

@@ -218,20 +218,21 @@ __device__ __forceinline__ NewtonResult newton_job_apply(const NewtonJob& jb, co
             ff_add(t, __ldg(sv + i * pb.plane));
             ff_add(mm, qv[i]);
         }
-        sh = (double)state_shift(pb, parity);
+        sh = widen(state_shift(pb, parity));
         m0 = ff_to_double(mm) + sh;
         th = ff_to_double(t) + sh;
     } else {
         m0 = jb.m0;
         th = jb.theta;
     }
-    const double pth = phi_of(th, pb.inv_delta);
-    const NewtonOut nr = newton_mixed(m0, th, pth, pb);
+    const Phi pt = phi_parts(th, pb.two_inv_delta);
+    const double pth = pt.value();
+    const NewtonOut nr = newton_mixed(m0, th, pt, pb);
     if (!nr.ok || !isfinite(nr.root)) atomicCAS(&stats[r.sidx].error, 0, 3);
     const double tn = m0 + (pth - nr.phi_root) * pb.inv_ste;
     // c = theta' - (1-omega) m0; stored values less w_i s: c - omega s
-    const P c = (P)((tn - sh) - (1.0 - pb.omega) * (m0 - sh));
-    const P omc = (P)(1.0 - pb.omega);
+    const P c = (P)((tn - sh) - pb.omc * (m0 - sh));
+    const P omc = sizeof(P) == 4 ? (P)pb.omc_f : (P)pb.omc;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         const P wi = lat_wp<P>(Q, i);
@@ -244,12 +245,39 @@ __device__ __forceinline__ NewtonResult newton_job_apply(const NewtonJob& jb, co
     return r;
 }
 
-// The warp's results, grouped by problem: the lowest lane of each group sums
-// its group's energy terms exactly and adds them, the node count, the
-// iteration sum and the largest iteration count once.
+// The warp's results, grouped by problem: the lowest lane of each group adds
+// its group's energy terms (summed exactly), node count, iteration sum and
+// largest iteration count once.  A warp whose jobs are of one problem (a single
+// problem always) sums by a tree, about 60 instructions; the loop over the 32
+// lanes, some 1,100, is left to warps that straddle problems.
 __device__ __forceinline__ void newton_group_add(const NewtonResult& r, DevStats* stats)
 {
     const int lane = threadIdx.x & 31;
+    const unsigned have = __ballot_sync(kFull, r.sidx >= 0);
+    if (have == 0u) return;
+    const int first = __ffs(have) - 1;
+    const int sidx = __shfl_sync(kFull, r.sidx, first);
+    if (__all_sync(kFull, r.sidx < 0 || r.sidx == sidx)) {
+        Fx sum = r.e;   // zero on idle lanes
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            Fx v;
+            v.hi = __shfl_xor_sync(kFull, sum.hi, o);
+            v.lo = __shfl_xor_sync(kFull, sum.lo, o);
+            fx_add(sum, v);
+        }
+        const int its = __reduce_add_sync(kFull, r.it);
+        const int mx = __reduce_max_sync(kFull, r.it);
+        if (lane == first) {
+            DevStats* st = &stats[sidx];
+            StepStripe* c = my_stripe(st);
+            acc_add_fx(&c->energy, sum);
+            atomicAdd(&c->newton, (unsigned long long)__popc(have));
+            atomicAdd(&c->iters, (unsigned long long)its);
+            atomicMax(&st->cur_maxit, mx);
+        }
+        return;
+    }
     const unsigned grp = __match_any_sync(kFull, r.sidx);
     const int leader = __ffs(grp) - 1;
     Fx sum{0, 0ull};

@@ -76,8 +76,9 @@ __device__ __forceinline__ NodeOut d1q3_node(const Problem& pb, int x, const P (
             tn = m0;
             phn = m0 > 0.0 ? 1.0 : 0.0;
         } else {
-            const double pth = phi_of(th, pb.inv_delta);
-            NewtonOut nr = newton_mixed(m0, th, pth, pb);
+            const Phi pt = phi_parts(th, pb.two_inv_delta);
+            const double pth = pt.value();
+            NewtonOut nr = newton_mixed(m0, th, pt, pb);
             r.fail = !nr.ok || !isfinite(nr.root);
             tn = m0 + (pth - nr.phi_root) * pb.inv_ste;
             phn = nr.phi_root;
