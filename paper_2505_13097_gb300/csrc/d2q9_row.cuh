@@ -190,12 +190,13 @@ __device__ __forceinline__ void row_update(const Problem& pb, int y, int x0, int
     P c[N];          // per node: theta' - (1-omega) m0, rounded to P
     double thn[REC ? N : 1];
     bool newton_k[N];
-    typename M0T<P>::T m0[N];
+    double m0[N];       // FP64 form
+    bool sat_k[N];
     bool any_wall = false;
     bool dir_k[N];
     int wall_k[N];
 #pragma unroll
-    for (int k = 0; k < N; ++k) { dir_k[k] = false; wall_k[k] = -1; }
+    for (int k = 0; k < N; ++k) { dir_k[k] = sat_k[k] = false; wall_k[k] = -1; }
     if constexpr (EDGE) {
 #pragma unroll
         for (int k = 0; k < N; ++k) {
@@ -219,7 +220,7 @@ __device__ __forceinline__ void row_update(const Problem& pb, int y, int x0, int
                     ff_add(ts.flux_f, fl.hi);
                     ts.flux_f.lo += fl.lo;
                 } else {
-                    ts.flux += wall_closure_d(qq, uu, x, y, pb, wall_k[k]);
+                    fx_add(ts.flux, to_fixed(wall_closure_d(qq, uu, x, y, pb, wall_k[k])));
                 }
                 dir_k[k] = wall_k[k] >= 0;
 #pragma unroll
@@ -245,10 +246,11 @@ __device__ __forceinline__ void row_update(const Problem& pb, int y, int x0, int
 #pragma unroll
             for (int i = 8; i >= 0; --i) mf += qf[i][k];
         } else {
-            m0_init(m0[k]);
+            double qk[9];
 #pragma unroll
-            for (int i = 8; i >= 0; --i) m0_add(m0[k], qf[i][k]);
-            mf = m0_f(m0[k]);
+            for (int i = 0; i < 9; ++i) qk[i] = qf[i][k];
+            m0[k] = sum_q<9>(qk);
+            mf = approx_float(m0[k]);
         }
         const float mt = sizeof(P) == 4 ? mf + sh : mf;   // M0(q)
         const float marg = 1e-5f * (1.0f + fabsf(tf));
@@ -266,8 +268,7 @@ __device__ __forceinline__ void row_update(const Problem& pb, int y, int x0, int
             const int wk = wall_k[k];
             ts.dir_count[wk] += 1;
             if constexpr (sizeof(P) == 4) {
-                ff mm;
-                m0_init(mm);
+                ff mm{0.f, 0.f};
 #pragma unroll
                 for (int i = 8; i >= 0; --i) ff_add(mm, qf[i][k]);
                 const float oc = (float)omc;
@@ -275,7 +276,7 @@ __device__ __forceinline__ void row_update(const Problem& pb, int y, int x0, int
                 c[k] = (P)(((pb.wall_th_hi[wk] - sh) - oc * mm.hi) + (pb.wall_th_lo[wk] - oc * mm.lo));
                 acc.add_ff(ff{pb.wall_th_hi[wk], pb.wall_th_lo[wk]});
             } else {
-                c[k] = (P)(pb.wall_theta[wk] - omc_d * m0_d(m0[k]));
+                c[k] = (P)(pb.wall_theta[wk] - omc_d * m0[k]);
                 acc.add_d(pb.wall_theta[wk]);
             }
             if constexpr (REC) thn[k] = pb.wall_theta[wk];
@@ -288,10 +289,10 @@ __device__ __forceinline__ void row_update(const Problem& pb, int y, int x0, int
                 ts.shifted += 1;
                 if constexpr (REC) thn[k] = (double)mf + (double)sh;
             } else {
-                const double md = m0_d(m0[k]);
-                c[k] = (P)(pb.omega * md);
-                acc.add_d(md);
-                if constexpr (REC) thn[k] = md;
+                c[k] = m0[k];   // omega is in the weight below
+                sat_k[k] = true;
+                acc.add_d(m0[k]);
+                if constexpr (REC) thn[k] = m0[k];
             }
             ts.liquid += sat_liq ? 1 : 0;
         }
@@ -324,11 +325,8 @@ __device__ __forceinline__ void row_update(const Problem& pb, int y, int x0, int
                 jb.m0 = jb.theta = 0.0;
             } else {
                 const P u[9] = {u0[k], u1[k], u2[k], u3[k], u4[k], u5[k], u6[k], u7[k], u8[k]};
-                double th = 0.0;
-#pragma unroll
-                for (int i = 8; i >= 0; --i) th += u[i];
-                jb.m0 = m0_d(m0[k]);
-                jb.theta = th;
+                jb.m0 = m0[k];
+                jb.theta = sum_q<9>(u);
             }
             sink.put(slot, jb);
             ++slot;
@@ -342,9 +340,16 @@ __device__ __forceinline__ void row_update(const Problem& pb, int y, int x0, int
     P wc[3][N];
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-        wc[0][k] = wP[0] * c[k];
-        wc[1][k] = wP[1] * c[k];
-        wc[2][k] = wP[2] * c[k];
+        if constexpr (sizeof(P) == 4) {
+            wc[0][k] = wP[0] * c[k];
+            wc[1][k] = wP[1] * c[k];
+            wc[2][k] = wP[2] * c[k];
+        } else {
+            // one multiplication: 4/9 and 1/36 are 4 and 1/4 times 1/9, and so are their roundings
+            wc[1][k] = (sat_k[k] ? pb.omega * wP[1] : wP[1]) * c[k];
+            wc[0][k] = scale2(wc[1][k], 2);
+            wc[2][k] = scale2(wc[1][k], -2);
+        }
     }
     if (row_newton) {
 #pragma unroll
@@ -410,7 +415,7 @@ __device__ __forceinline__ void row_update_eebm(const Problem& pb, int y, int x0
                         ff_add(ts.flux_f, fl.hi);
                         ts.flux_f.lo += fl.lo;
                     } else {
-                        ts.flux += wall_closure_d(qq, uu, x, y, pb, wall);
+                        fx_add(ts.flux, to_fixed(wall_closure_d(qq, uu, x, y, pb, wall)));
                     }
 #pragma unroll
                     for (int i = 0; i < 9; ++i) qf[i][k] = qq[i];
@@ -426,21 +431,29 @@ __device__ __forceinline__ void row_update_eebm(const Problem& pb, int y, int x0
     for (int k = 0; k < N; ++k) {
         const bool valid = !EDGE || x0 + k < nx;
         P Hs = 0;   // H less the shift (FP32 form)
+        if constexpr (sizeof(P) == 4) {
 #pragma unroll
-        for (int i = 8; i >= 0; --i) Hs += qf[i][k];
+            for (int i = 8; i >= 0; --i) Hs += qf[i][k];
+        } else {
+            P qk[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) qk[i] = qf[i][k];
+            Hs = sum_q<9>(qk);
+        }
         if (!valid) {
             Hs = 0;
 #pragma unroll
             for (int i = 0; i < 9; ++i) qf[i][k] = (P)0;
         }
-        hs += Hs;
+        if constexpr (sizeof(P) == 4) hs += Hs;
+        else acc.add_d(Hs);
         if constexpr (sizeof(P) == 4) {
             const float H = Hs + sh;
             const float th = eebm_theta(H, inv_ste);
             if constexpr (REC) thn[k] = (double)th;
             ts.shifted += valid ? 1 : 0;
             // stored values less w_i sh: omega (H - (1-w_0) theta - w_0 sh) and omega w_i (theta - sh)
-            qf[0][k] = fma(omc, qf[0][k], om * (H - ((P)1 - wP[0]) * th - wP[0] * sh));
+            qf[0][k] = fma(omc, qf[0][k], om * eebm_rest(H, th, wP[0], (P)sh));
             const float tr = th - sh;
 #pragma unroll
             for (int i = 1; i < 9; ++i) qf[i][k] = fma(omc, qf[i][k], om * (i <= 4 ? wP[1] : wP[2]) * tr);
@@ -448,13 +461,12 @@ __device__ __forceinline__ void row_update_eebm(const Problem& pb, int y, int x0
             const P H = Hs;
             const P th = eebm_theta(H, inv_ste);
             if constexpr (REC) thn[k] = (double)th;
-            qf[0][k] = fma(omc, qf[0][k], om * (H - ((P)1 - wP[0]) * th));
+            qf[0][k] = fma(omc, qf[0][k], om * eebm_rest(H, th, wP[0], (P)0));
 #pragma unroll
             for (int i = 1; i < 9; ++i) qf[i][k] = fma(omc, qf[i][k], om * (i <= 4 ? wP[1] : wP[2]) * th);
         }
     }
     if constexpr (sizeof(P) == 4) acc.add_ff(ff{hs, 0.f});
-    else acc.add_d(hs);
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         P o[N];

@@ -112,6 +112,17 @@ __device__ __forceinline__ float eebm_theta(float H, float inv_ste)
     return H < 0.0f ? H : (H > inv_ste ? H - inv_ste : 0.0f);
 }
 
+// H - (1 - w0) theta - w0 sh, the rest population's EEBM equilibrium less w0 sh.
+// The fused operations are spelled out, so that every kernel rounds alike.
+__device__ __forceinline__ float eebm_rest(float H, float theta, float w0, float sh)
+{
+    return __fmaf_rn(-w0, sh, __fmaf_rn(w0 - 1.0f, theta, H));
+}
+__device__ __forceinline__ double eebm_rest(double H, double theta, double w0, double sh)
+{
+    return fma(-w0, sh, fma(w0 - 1.0, theta, H));
+}
+
 // 2^(j/64), rounded to nearest
 static __device__ const double kExp2[64] = {
     0x1.p+0, 0x1.02c9a3e778061p+0, 0x1.059b0d3158574p+0, 0x1.0874518759bc8p+0,
@@ -291,15 +302,26 @@ __device__ __forceinline__ NewtonOut newton_mixed(double m0, double theta, const
     const float dm = pt.neg ? -dm0 : dm0;            // mirrored to theta >= 0
     const float E = trunc_float(pt.E), r0 = trunc_float(pt.r);
     float lo = dm + (r0 - 1.0f) * isf, hi = dm + r0 * isf;
-    float u = 0.0f;
-    const float small = 1e-3f * pb.delta_f;
-    float step_prev = hi - lo;
-    int k = 0;
-    for (; k < 16; ++k) {
-        const float b = idf2 * u;
+    const float small = 1e-3f * pb.delta_f, di = idf2 * isf;
+    // the first iterate from x = theta (F = -dm there) needs no exponential
+    float u = __fdividef(dm, fmaf(E * r0 * r0, di, 1.0f));
+    if (dm > 0.0f) lo = fmaxf(lo, 0.0f);
+    else hi = fminf(hi, 0.0f);
+    if (!(u >= lo && u <= hi)) u = 0.5f * (lo + hi);
+    float step_prev = fabsf(u);
+    int k = 1;
+    for (; k < 16 && step_prev > small; ++k) {
+        const float b = idf2 * u, ab = fabsf(b);
         float D, dph;   // phi(theta + u) - phi(theta), phi'(theta + u) delta / 2
-        if (fabsf(b) <= 20.0f) {
-            const float m = expm1f(-b);
+        if (ab <= 20.0f) {
+            // expm1(-b): its Taylor series to b^7, or the difference where that loses little
+            float m = fmaf(-b, 1.0f / 5040.0f, 1.0f / 720.0f);
+            m = fmaf(m, -b, 1.0f / 120.0f);
+            m = fmaf(m, -b, 1.0f / 24.0f);
+            m = fmaf(m, -b, 1.0f / 6.0f);
+            m = fmaf(m, -b, 0.5f);
+            m = fmaf(m * b, b, -b);
+            if (ab > 0.5f) m = expf(-b) - 1.0f;
             const float E1 = fmaf(E, m, E);
             const float r1 = __fdividef(1.0f, 1.0f + E1);
             D = -E * m * r0 * r1;
@@ -313,12 +335,12 @@ __device__ __forceinline__ NewtonOut newton_mixed(double m0, double theta, const
         if (F == 0.0f) break;
         if (F < 0.0f) lo = fmaxf(lo, u);
         else hi = fminf(hi, u);
-        float un = u - F / (1.0f + dph * idf2 * isf);
+        float un = u - __fdividef(F, fmaf(dph, di, 1.0f));
         if (!(un >= lo && un <= hi)) {
             un = 0.5f * (lo + hi);
         } else {
             const float st = fabsf(un - u);
-            if (st <= small || (k >= 2 && st >= 0.5f * step_prev)) {
+            if (k >= 2 && st >= 0.5f * step_prev) {
                 u = un;
                 ++k;
                 break;
@@ -376,6 +398,64 @@ __device__ __forceinline__ NewtonOut newton_mixed(double m0, double theta, const
     r.iters += k;
     r.ok = r.ok && r.iters <= maxit;
     return r;
+}
+
+// ---------------------------------------------------------------- exact sums
+// sum of Q doubles, to within 2^-6 ulp of the largest per term, rounded once:
+// the mantissas are aligned to the largest exponent with six guard bits (59
+// bits; nine of them stay below 2^63) and added as integers, 15 integer
+// instructions per term against 64 cycles of FP64 pipe per addition.  Terms
+// down to 2^-6 of the largest lose no bit.  Sums of tiny (2^-953), huge (2^1007)
+// or non-finite terms go through FP64 additions.
+__device__ __forceinline__ unsigned long long shr64(unsigned long long v, unsigned s)
+{
+    unsigned long long r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));   // 0 for s >= 64
+    return r;
+}
+
+template <int Q>
+__device__ __forceinline__ double sum_q(const double (&q)[Q])
+{
+    unsigned emax = 0;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) emax = max(emax, (unsigned)__double2hiint(q[i]) & 0x7ff00000u);
+    emax >>= 20;
+    if (emax < 70u || emax >= 2030u) {
+        double s = 0.0;
+#pragma unroll
+        for (int i = Q - 1; i >= 0; --i) s += q[i];
+        return s;
+    }
+    long long S = 0;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const unsigned h = (unsigned)__double2hiint(q[i]), l = (unsigned)__double2loint(q[i]);
+        const unsigned sh = emax - ((h >> 20) & 0x7ffu);
+        // the mantissa, shifted left by six (a zero's implicit bit is shifted out: sh >= 70)
+        const unsigned mh = __funnelshift_l(l, (h & 0xfffffu) | 0x100000u, 6);
+        const unsigned long long m = shr64(((unsigned long long)mh << 32) | (l << 6), sh);
+        const long long sg = (long long)(int)h >> 63;
+        S += ((long long)m ^ sg) - sg;
+    }
+    const bool neg = S < 0;
+    const unsigned long long a = neg ? 0ull - (unsigned long long)S : (unsigned long long)S;
+    if (a == 0ull) return 0.0;
+    const int lz = __clzll((long long)a);
+    const unsigned long long nrm = a << lz;
+    // round to nearest even at bit 11; a carry runs into the exponent
+    const unsigned low = (unsigned)nrm & 0x7ffu, lsb = ((unsigned)nrm >> 11) & 1u;
+    unsigned long long b = (nrm >> 11) + (low + lsb > 0x400u ? 1ull : 0ull);
+    b += (unsigned long long)((int)emax - lz + 5 - 1) << 52;   // the implicit bit adds 1
+    return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ull : 0ull)));
+}
+
+// v 2^k for a finite v that stays normal (else by multiplication)
+__device__ __forceinline__ double scale2(double v, int k)
+{
+    const int h = __double2hiint(v), e = (h >> 20) & 0x7ff;
+    if (e < 8 || e > 2040) return k > 0 ? v * (double)(1 << k) : v / (double)(1 << -k);
+    return __hiloint2double(h + (k << 20), __double2loint(v));
 }
 
 // ---------------------------------------------------------------- lane shifts
@@ -458,6 +538,18 @@ __device__ __forceinline__ void fx_add(Fx& a, const Fx& b)
     const unsigned long long lo = a.lo + b.lo;
     a.hi += b.hi + (lo < a.lo ? 1 : 0);
     a.lo = lo;
+}
+
+__device__ __forceinline__ Fx fx_tree(Fx v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        Fx w;
+        w.hi = __shfl_xor_sync(kFull, v.hi, o);
+        w.lo = __shfl_xor_sync(kFull, v.lo, o);
+        fx_add(v, w);
+    }
+    return v;
 }
 
 __device__ __forceinline__ void acc_add_fx(Acc128* a, const Fx& v)

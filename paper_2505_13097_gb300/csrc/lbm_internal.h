@@ -147,6 +147,22 @@ struct TmaMaps {
                                          // above its first row); -1: off
 };
 
+// The barrier of a resident launch (step_resident.cu).  All zero between launches.
+constexpr int kResidentRing = 32;   // sets of sums in flight to the statistics block
+struct ResidentBar {
+    unsigned int count, pad0[31];          // arrivals of the computing blocks since the launch
+    unsigned int abort, done, pad1[30];    // a wait ran out; blocks that have left
+    unsigned int read[kResidentRing];      // per set: times the statistics block has read it
+};
+// How a resident launch covers a lattice; blocks == 0: it does not.
+struct ResidentPlan {
+    int blocks = 0, threads = 0;   // blocks: the computing ones and one for the statistics
+    int strips = 0, th = 1, tiles = 0;   // first pass: column strips, rows of a tile, tiles
+    int nseg = 0, items = 0;       // second pass: 32-column segments of a row, items
+    int rot = 0;                   // rotation of the blocks' places from wave to wave
+    size_t slots = 0;              // slots of the steps' sums
+};
+
 // Per-launch arguments of the Newton job kernel (runs after every D2Q9 step).
 struct JobArgs {
     const Problem* probs;
@@ -217,6 +233,13 @@ int d2q9_tma_blocks_per_sm();
 // side: the launch beside the flat stencil kernel (kJobSideThreads per block), else 256
 cudaError_t launch_newton_jobs(int precision, int q, const JobArgs& a, cudaStream_t s, int grid = 0, int prio = 0,
                                bool side = false);
+
+// D2Q9 / D2Q5 steps in one cooperative launch (step_resident.cu); hp carries the
+// wall constants that launch_wall_constants sets
+ResidentPlan resident_plan(int precision, int q, int nx, int ny);
+size_t resident_slot_bytes();
+cudaError_t launch_resident(int precision, const ResidentPlan& plan, const Problem& hp, int parity, int nsteps, double* rec,
+                            DevStats* stats, void* slots, ResidentBar* bar, long long wait_ns, cudaStream_t s);
 
 // D2Q5 launchers (step_d2q5.cu): one tile per warp over a.nslots tiles
 cudaError_t launch_d2q5_step(int precision, const StepArgs& a, cudaStream_t s);

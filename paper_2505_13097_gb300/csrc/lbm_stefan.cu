@@ -93,6 +93,9 @@ struct lbm_stefan {
     cudaStream_t side = nullptr;       // split FP32 D2Q9 step: stream of the left half's Newton solves
     cudaEvent_t ev_fork = nullptr, ev_half = nullptr, ev_join = nullptr;
     cudaEvent_t ev_walls = nullptr;   // split step: the wall kernels are done (list A's wall part is final)
+    lbm::ResidentPlan res;             // D2Q9 / D2Q5: the resident step (blocks 0: the step's separate kernels)
+    void* dslots = nullptr;            // its per-warp sums
+    lbm::ResidentBar* dbar = nullptr;  // its barrier
     GraphCache graph;
     // captured adjoint segments (lbm_stefan_adjoint_segment): recompute + reverse
     // steps for one (length, trajectory, adjoint buffers) combination each
@@ -235,6 +238,8 @@ static lbm_status upload_problem(lbm_stefan* h)
 {
     CUDA_TRY(cudaMemcpyAsync(h->dprob, &h->hp, sizeof(Problem), cudaMemcpyHostToDevice, h->stream));
     CUDA_TRY(lbm::launch_wall_constants(h->dprob, 1, h->stream));
+    // the wall constants, for the kernels that take the problem by value
+    CUDA_TRY(cudaMemcpyAsync(&h->hp, h->dprob, sizeof(Problem), cudaMemcpyDeviceToHost, h->stream));
     CUDA_TRY(cudaStreamSynchronize(h->stream));
     return LBM_OK;
 }
@@ -444,6 +449,49 @@ static cudaError_t launch_one(lbm_stefan* h, int parity, double* rec)
     return lbm::launch_d1q3_step(h->precision, a, h->hp, h->stream);
 }
 
+// Bound of a wait at the resident step's barrier, and the most steps of one launch.
+constexpr long long kResidentWaitNs = 5000000000LL;
+constexpr int kResidentSteps = 8192;
+
+// nsteps steps by resident launches from state[parity] on; theta' planes to
+// rec, if given.  cudaErrorCooperativeLaunchTooLarge (nothing ran): the grid
+// does not fit, take the separate kernels.
+static cudaError_t run_resident(lbm_stefan* h, int nsteps, int parity, double* rec)
+{
+    const long long plane = (long long)h->hp.ny * h->hp.pitch;
+    while (nsteps > 0) {
+        const int n = std::min(nsteps, kResidentSteps);
+        const cudaError_t e = lbm::launch_resident(h->precision, h->res, h->hp, parity, n, rec, h->dstats, h->dslots, h->dbar,
+                                                   kResidentWaitNs, h->stream);
+        if (e != cudaSuccess) return e;
+        parity ^= n & 1;
+        nsteps -= n;
+        if (rec) rec += n * plane;
+    }
+    return cudaSuccess;
+}
+
+#ifndef LBM_RESIDENT
+#define LBM_RESIDENT 1
+#endif
+// The largest lattice that steps in resident launches (measured us per step, separate
+// kernels / resident).  FP32 D2Q9 IREBM: 235 / 231 at 4096^2, 850 / 871 at 8192^2; EEBM,
+// which has no Newton work to hide: 69 / 60 at 2048^2, 202 / 215 at 4096^2.  FP64 and
+// D2Q5 gain at every size (D2Q9 FP64 966 / 658 and D2Q5 FP32 183 / 128 at 4096^2): the
+// bound is that of the 32-bit indices, 2^31 elements of a state.
+static long long resident_max_nodes(int lattice, int precision, int method)
+{
+    if (!LBM_RESIDENT) return 0;
+    if (lattice == LBM_D2Q9 && precision == LBM_FP32) return method == LBM_EEBM ? 1ll << 23 : 1ll << 25;
+    return 1ll << 31;
+}
+
+static bool resident_on(const lbm_stefan* h)
+{
+    return h->res.blocks > 0 && h->withhold_load < 0 && h->hp.method != LBM_ILFBM &&
+           (long long)h->hp.nx * h->hp.ny <= resident_max_nodes(h->p.lattice, h->precision, h->hp.method);
+}
+
 static lbm_status check_stats_error(lbm_stefan* h, DevStats* out)
 {
     DevStats st;
@@ -590,6 +638,16 @@ extern "C" lbm_status lbm_stefan_create(const lbm_stefan_params* p, void* cuda_s
     // the list of deferred Newton nodes (D2Q9, D2Q5): one job per node at most
     // (split FP32 step: two lists, the first with room for the wall kernel's
     // and the left half's nodes)
+    if (e == cudaSuccess && q != 3 && q * h->hp.plane < 1ll << 31 &&
+        (long long)p->nx * p->ny <= resident_max_nodes(p->lattice, p->precision, LBM_IREBM)) {
+        const lbm::ResidentPlan plan = lbm::resident_plan(p->precision, q, p->nx, p->ny);
+        if (plan.blocks > 0) {
+            e = cudaMalloc(&h->dslots, plan.slots * lbm::resident_slot_bytes());
+            if (e == cudaSuccess) e = cudaMalloc(&h->dbar, sizeof(lbm::ResidentBar));
+            if (e == cudaSuccess) e = cudaMemset(h->dbar, 0, sizeof(lbm::ResidentBar));
+            h->res = plan;
+        }
+    }
     const size_t njobs = h->side ? split_cap_a(h->hp) + (size_t)(h->hp.pitch / lbm::kTmaW - h->hp.pitch / lbm::kTmaW / 2) *
                                                             lbm::kTmaW * p->ny
                                  : (size_t)p->nx * p->ny;
@@ -754,6 +812,16 @@ extern "C" lbm_status lbm_stefan_step(lbm_stefan* h, int nsteps)
         h->parity ^= nsteps & 1;
         return LBM_OK;
     }
+    if (resident_on(h)) {
+        const cudaError_t e = run_resident(h, nsteps, h->parity, nullptr);
+        if (e == cudaSuccess) {
+            h->parity ^= nsteps & 1;
+            return LBM_OK;
+        }
+        if (e != cudaErrorCooperativeLaunchTooLarge) CUDA_TRY(e);
+        (void)cudaGetLastError();
+        h->res.blocks = 0;
+    }
     int left = nsteps;
     if (h->parity == 1) {
         CUDA_TRY(launch_one(h, 1, nullptr));
@@ -855,6 +923,16 @@ extern "C" lbm_status lbm_stefan_step_record(lbm_stefan* h, int nsteps, double* 
         CUDA_TRY(lbm::launch_d1q3_fused(h->precision, a, h->hp, nsteps, h->parity, traj, h->stream));
         h->parity ^= nsteps & 1;
         return LBM_OK;
+    }
+    if (resident_on(h) && nsteps > 0) {
+        const cudaError_t e = run_resident(h, nsteps, h->parity, traj);
+        if (e == cudaSuccess) {
+            h->parity ^= nsteps & 1;
+            return LBM_OK;
+        }
+        if (e != cudaErrorCooperativeLaunchTooLarge) CUDA_TRY(e);
+        (void)cudaGetLastError();
+        h->res.blocks = 0;
     }
     for (int k = 0; k < nsteps; ++k) {
         CUDA_TRY(launch_one(h, h->parity, traj + k * plane));
@@ -1079,9 +1157,13 @@ static cudaError_t segment_launches(lbm_stefan* h, int nsteps, double* traj, voi
     cudaError_t e = lbm::launch_fields(h->precision, h->dprob, h->hp, parity0, nullptr, nullptr, nullptr, traj,
                                        h->stream);
     int par = parity0;
-    for (int k = 0; k < nsteps && e == cudaSuccess; ++k) {
-        e = launch_one(h, par, traj + (k + 1) * plane);
-        par ^= 1;
+    if (resident_on(h) && e == cudaSuccess) {
+        e = run_resident(h, nsteps, par, traj + plane);
+    } else {
+        for (int k = 0; k < nsteps && e == cudaSuccess; ++k) {
+            e = launch_one(h, par, traj + (k + 1) * plane);
+            par ^= 1;
+        }
     }
     void* buf[2] = {a, b};
     int cur = 0;
@@ -1168,6 +1250,8 @@ extern "C" void lbm_stefan_destroy(lbm_stefan* h)
     if (h->ev_join) cudaEventDestroy(h->ev_join);
     if (h->ev_walls) cudaEventDestroy(h->ev_walls);
     if (h->side) cudaStreamDestroy(h->side);
+    cudaFree(h->dslots);
+    cudaFree(h->dbar);
     cudaFree(h->dilf);
     cudaFree(h->dilf_scratch);
     delete h;

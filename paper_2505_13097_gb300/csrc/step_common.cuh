@@ -27,38 +27,22 @@ __device__ __forceinline__ void st_rec(double* p, const double (&v)[N])
 }
 
 template <typename P>
-struct Acc;   // per-lane accumulator of sum theta' (float-float or double)
+struct Acc;   // per-lane accumulator of sum theta' (float-float or fixed point)
 template <>
 struct Acc<float> {
     ff s{0.f, 0.f};
     __device__ void add_ff(const ff& v) { ff_add(s, v.hi); s.lo = __fadd_rn(s.lo, v.lo); }
     __device__ void add_f(float v) { ff_add(s, v); }
     __device__ void add_d(double v) { float h = (float)v; ff_add(s, h); s.lo = __fadd_rn(s.lo, (float)(v - (double)h)); }
-    __device__ double get() const { return ff_to_double(s); }
 };
 template <>
-struct Acc<double> {
-    double s = 0.0;
-    __device__ void add_d(double v) { s += v; }
-    __device__ double get() const { return s; }
+struct Acc<double> {   // exact, on the integer pipe
+    Fx s{0, 0ull};
+    __device__ void add_d(double v) { fx_add(s, to_fixed(v)); }
 };
 
-// m0 accumulator type per precision
-template <typename P> struct M0T;
-template <> struct M0T<float> { using T = ff; };
-template <> struct M0T<double> { using T = double; };
-
-__device__ __forceinline__ void m0_init(ff& a) { a.hi = 0.f; a.lo = 0.f; }
-__device__ __forceinline__ void m0_init(double& a) { a = 0.0; }
-__device__ __forceinline__ void m0_add(ff& a, float v) { ff_add(a, v); }
-__device__ __forceinline__ void m0_add(double& a, double v) { a += v; }
-__device__ __forceinline__ double m0_d(const ff& a) { return ff_to_double(a); }
-__device__ __forceinline__ double m0_d(const double& a) { return a; }
-__device__ __forceinline__ float m0_f(const ff& a) { return a.hi; }
-__device__ __forceinline__ float m0_f(const double& a) { return approx_float(a); }
-
 struct TileSums {
-    double flux = 0.0, phi_sum = 0.0;   // FP64 form
+    Fx flux{0, 0ull};                   // FP64 form
     ff flux_f{0.f, 0.f};                // FP32 form
     int dir_count[4] = {0, 0, 0, 0};   // Dirichlet nodes per wall (adds phi(theta_D)/Ste each)
     int liquid = 0, newton = 0, maxit = 0;
@@ -94,8 +78,8 @@ __device__ __forceinline__ WarpSums warp_tile_sums(const Acc<P>& acc, const Tile
         w.f = float_to_fixed(sf.hi);
         fx_add(w.f, float_to_fixed(sf.lo));
     } else {
-        w.e = to_fixed(warp_sum(acc.get()));
-        w.f = to_fixed(warp_sum(ts.flux));
+        w.e = fx_tree(acc.s);
+        w.f = fx_tree(ts.flux);
     }
     w.nl = warp_sum_i(ts.liquid);
     w.ns = warp_sum_i(ts.shifted);

@@ -24,7 +24,7 @@
 // loads are issued before this row's arithmetic.  Every population is read
 // once per step, plus one halo row of planes 2 and 4 per tile: 20 + 20 bytes
 // per node in FP32, 40 + 40 in FP64.
-#include "step_common.cuh"
+#include "d2q5_row.cuh"
 
 namespace lbm {
 
@@ -55,154 +55,6 @@ __device__ __forceinline__ void d5_ld(const double* p, double (&v)[2])
 }
 __device__ __forceinline__ void d5_ld(const double* p, double (&v)[1]) { v[0] = __ldg(p); }
 
-// ---------------------------------------------------------------- closures
-// A D2Q5 wall node (nx, ny >= 3): q_1 is unknown at x = 0, q_3 at x = nx - 1,
-// q_2 at y = 0, q_4 at y = ny - 1.
-struct Wall5 {
-    unsigned unk;   // bit i: q_i not defined by streaming
-    int wall;       // Dirichlet wall (first of W, E, S, N), -1 if none
-    int sx, sy;     // Eq. (17): the node one step inwards (the diagonal one at a corner)
-};
-
-__device__ __forceinline__ Wall5 wall5_info(int x, int y, const Problem& pb)
-{
-    Wall5 w;
-    const bool W = x == 0, E = x == pb.nx - 1, S = y == 0, N = y == pb.ny - 1;
-    w.unk = (W ? 2u : 0u) | (S ? 4u : 0u) | (E ? 8u : 0u) | (N ? 16u : 0u);
-    const int walls = (W ? 1 : 0) | (E ? 2 : 0) | (S ? 4 : 0) | (N ? 8 : 0);
-    w.wall = -1;
-    for (int k = 0; k < 4; ++k)
-        if (((walls >> k) & 1) && pb.wall_kind[k] == 1) {
-            w.wall = k;
-            break;
-        }
-    w.sx = x + (W ? 1 : (E ? -1 : 0));
-    w.sy = y + (S ? 1 : (N ? -1 : 0));
-    return w;
-}
-
-// The streamed populations of an interior node (x, y), read from the source state.
-template <typename P>
-__device__ __forceinline__ void pulled5(const P* __restrict__ src, const Problem& pb, int x, int y, P (&q)[5])
-{
-    const long long pl = pb.plane, pitch = pb.pitch;
-    const P* r = src + (long long)(y + 1) * pitch + x;
-    q[0] = r[0];
-    q[1] = r[pl - 1];
-    q[2] = r[2 * pl - pitch];
-    q[3] = r[3 * pl + 1];
-    q[4] = r[4 * pl + pitch];
-}
-
-// FP64 form.  q holds the pulled values (unknown entries are overwritten), u
-// the node's own Omega.  Returns the boundary flux (filled q minus Omega that
-// leaves the lattice); wall reports the node's Dirichlet wall or -1.
-__device__ __noinline__ double wall5_closure_d(double* q, const double* u, int x, int y, const Problem& pb,
-                                               const double* __restrict__ src, int& wall)
-{
-    const Wall5 wi = wall5_info(x, y, pb);
-    wall = wi.wall;
-    double out = 0.0, in = 0.0;
-#pragma unroll
-    for (int j = 1; j < 5; ++j)
-        if ((wi.unk >> d2_opp(j)) & 1) out += u[j];
-    if (wi.wall >= 0 || pb.bb_mode == 2) {
-        double m0t;
-        if (wi.wall >= 0) {
-            double th = 0.0;
-#pragma unroll
-            for (int i = 4; i >= 0; --i) th += u[i];
-            m0t = dir_m0_target_d(th, wi.wall, pb);
-        } else {
-            double nq[5];
-            pulled5<double>(src, pb, wi.sx, wi.sy, nq);
-            m0t = 0.0;
-#pragma unroll
-            for (int i = 4; i >= 0; --i) m0t += nq[i];
-        }
-        // the unknown q share what the known ones leave, in proportion to w_i (equal)
-        double known = 0.0;
-        int nu = 0;
-#pragma unroll
-        for (int i = 4; i >= 0; --i) {
-            if ((wi.unk >> i) & 1) ++nu;
-            else known += q[i];
-        }
-        const double r = (m0t - known) / (double)nu;
-#pragma unroll
-        for (int i = 1; i < 5; ++i)
-            if ((wi.unk >> i) & 1) {
-                q[i] = r;
-                in += r;
-            }
-    } else {
-        // bounce-back: the opposite direction is always known on D2Q5 with nx, ny >= 3
-#pragma unroll
-        for (int i = 1; i < 5; ++i)
-            if ((wi.unk >> i) & 1) {
-                const int o = d2_opp(i);
-                q[i] = pb.bb_mode == 0 ? q[o] : u[o];
-                in += q[i];
-            }
-    }
-    return in - out;
-}
-
-// FP32 form with float-float sums.
-__device__ __noinline__ ff wall5_closure_f(float* q, const float* u, int x, int y, const Problem& pb,
-                                           const float* __restrict__ src, int& wall)
-{
-    const Wall5 wi = wall5_info(x, y, pb);
-    wall = wi.wall;
-    ff out{0.f, 0.f}, in{0.f, 0.f};
-#pragma unroll
-    for (int j = 1; j < 5; ++j)
-        if ((wi.unk >> d2_opp(j)) & 1) ff_add(out, u[j]);
-    if (wi.wall >= 0 || pb.bb_mode == 2) {
-        ff m0t{0.f, 0.f};   // target of M0(q), less the state's shift sh (q, u are Omega - w_i sh)
-        if (wi.wall >= 0) {
-            const float sh = __ldg(reinterpret_cast<const float*>(reinterpret_cast<const char*>(src) + pb.tail_off));
-            ff th{0.f, 0.f};
-#pragma unroll
-            for (int i = 4; i >= 0; --i) ff_add(th, u[i]);
-            ff_add(th, sh);
-            m0t = dir_m0_target_f(th, wi.wall, pb);
-            ff_add(m0t, -sh);
-        } else {
-            float nq[5];
-            pulled5<float>(src, pb, wi.sx, wi.sy, nq);
-#pragma unroll
-            for (int i = 4; i >= 0; --i) ff_add(m0t, nq[i]);
-        }
-        ff known{0.f, 0.f};
-        int nu = 0;
-#pragma unroll
-        for (int i = 4; i >= 0; --i) {
-            if ((wi.unk >> i) & 1) ++nu;
-            else ff_add(known, q[i]);
-        }
-        const float r = ((m0t.hi - known.hi) + (m0t.lo - known.lo)) / (float)nu;
-#pragma unroll
-        for (int i = 1; i < 5; ++i)
-            if ((wi.unk >> i) & 1) {
-                q[i] = r;
-                ff_add(in, r);
-            }
-    } else {
-#pragma unroll
-        for (int i = 1; i < 5; ++i)
-            if ((wi.unk >> i) & 1) {
-                const int o = d2_opp(i);
-                q[i] = pb.bb_mode == 0 ? q[o] : u[o];
-                ff_add(in, q[i]);
-            }
-    }
-    ff f{in.hi, in.lo};
-    ff_add(f, -out.hi);
-    f.lo -= out.lo;
-    return f;
-}
-
 // ---------------------------------------------------------------- one row
 // The update of one row of the warp's segment.  qf: pulled q (closed here at
 // wall nodes), u: the nodes' own Omega.  EDGE = false: the caller knows that
@@ -223,9 +75,10 @@ __device__ __forceinline__ void row5_update(const Problem& pb, const P* __restri
     double thn[REC ? N : 1];
     bool newton_k[N], dir_k[N];
     int wall_k[N];
-    typename M0T<P>::T m0[N];
+    double m0[N];       // FP64 form
+    bool sat_k[N];
 #pragma unroll
-    for (int k = 0; k < N; ++k) { dir_k[k] = false; wall_k[k] = -1; }
+    for (int k = 0; k < N; ++k) { dir_k[k] = sat_k[k] = false; wall_k[k] = -1; }
     if constexpr (EDGE) {
         bool any_wall = false;
 #pragma unroll
@@ -241,12 +94,14 @@ __device__ __forceinline__ void row5_update(const Problem& pb, const P* __restri
                     P qq[5], uu[5];
 #pragma unroll
                     for (int i = 0; i < 5; ++i) { qq[i] = qf[i][k]; uu[i] = u[i][k]; }
+                    P nq[5];
+                    if (pb.bb_mode == 2) pulled5_inward<P>(src, pb, x, y, nq);
                     if constexpr (sizeof(P) == 4) {
-                        const ff fl = wall5_closure_f(qq, uu, x, y, pb, src, wall_k[k]);
+                        const ff fl = wall5_closure_f(qq, uu, nq, x, y, pb, wall_k[k], sh);
                         ff_add(ts.flux_f, fl.hi);
                         ts.flux_f.lo += fl.lo;
                     } else {
-                        ts.flux += wall5_closure_d(qq, uu, x, y, pb, src, wall_k[k]);
+                        fx_add(ts.flux, to_fixed(wall5_closure_d(qq, uu, nq, x, y, pb, wall_k[k])));
                     }
                     dir_k[k] = wall_k[k] >= 0;
 #pragma unroll
@@ -269,10 +124,11 @@ __device__ __forceinline__ void row5_update(const Problem& pb, const P* __restri
             for (int i = 4; i >= 0; --i) { tf += u[i][k]; mf += qf[i][k]; }
             tf += sh;   // theta; mf stays M0(q) - sh
         } else {
-            m0_init(m0[k]);
+            double qk[5];
 #pragma unroll
-            for (int i = 4; i >= 0; --i) { tf += approx_float(u[i][k]); m0_add(m0[k], qf[i][k]); }
-            mf = m0_f(m0[k]);
+            for (int i = 4; i >= 0; --i) { tf += approx_float(u[i][k]); qk[i] = qf[i][k]; }
+            m0[k] = sum_q<5>(qk);
+            mf = approx_float(m0[k]);
         }
         const float mt = mf + sh;   // M0(q)
         const float marg = 1e-5f * (1.0f + fabsf(tf));
@@ -297,7 +153,7 @@ __device__ __forceinline__ void row5_update(const Problem& pb, const P* __restri
                 c[k] = (P)(((pb.wall_th_hi[wk] - sh) - oc * mm.hi) + (pb.wall_th_lo[wk] - oc * mm.lo));
                 acc.add_ff(ff{pb.wall_th_hi[wk], pb.wall_th_lo[wk]});
             } else {
-                c[k] = (P)(pb.wall_theta[wk] - omc_d * m0_d(m0[k]));
+                c[k] = (P)(pb.wall_theta[wk] - omc_d * m0[k]);
                 acc.add_d(pb.wall_theta[wk]);
             }
             if constexpr (REC) thn[k] = pb.wall_theta[wk];
@@ -309,10 +165,10 @@ __device__ __forceinline__ void row5_update(const Problem& pb, const P* __restri
                 ts.shifted += 1;
                 if constexpr (REC) thn[k] = (double)mf + (double)sh;
             } else {
-                const double md = m0_d(m0[k]);
-                c[k] = (P)(pb.omega * md);
-                acc.add_d(md);
-                if constexpr (REC) thn[k] = md;
+                c[k] = m0[k];   // omega is in the weight below
+                sat_k[k] = true;
+                acc.add_d(m0[k]);
+                if constexpr (REC) thn[k] = m0[k];
             }
             ts.liquid += sat_liq ? 1 : 0;
         }
@@ -343,11 +199,11 @@ __device__ __forceinline__ void row5_update(const Problem& pb, const P* __restri
                 // FP32 form: the job kernel forms m0 and theta from memory
                 jb.m0 = jb.theta = 0.0;
             } else {
-                double th = 0.0;
+                double uk[5];
 #pragma unroll
-                for (int i = 4; i >= 0; --i) th += u[i][k];
-                jb.m0 = m0_d(m0[k]);
-                jb.theta = th;
+                for (int i = 0; i < 5; ++i) uk[i] = u[i][k];
+                jb.m0 = m0[k];
+                jb.theta = sum_q<5>(uk);
             }
             jobs[slot] = jb;
             ++slot;
@@ -356,13 +212,23 @@ __device__ __forceinline__ void row5_update(const Problem& pb, const P* __restri
         }
     }
 
-    // Omega~_i = (1 - omega) q_i + w_i c
+    // Omega~_i = (1 - omega) q_i + w_i c (FP64: one multiplication, 1/3 = 2/6 and so its rounding)
+    P wc[2][N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        if constexpr (sizeof(P) == 4) {
+            wc[0][k] = w0 * c[k];
+            wc[1][k] = w1 * c[k];
+        } else {
+            wc[1][k] = (sat_k[k] ? pb.omega * w1 : w1) * c[k];
+            wc[0][k] = scale2(wc[1][k], 1);
+        }
+    }
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        const P wi = i == 0 ? w0 : w1;
         P o[N];
 #pragma unroll
-        for (int k = 0; k < N; ++k) o[k] = newton_k[k] ? qf[i][k] : fma(omc, qf[i][k], wi * c[k]);
+        for (int k = 0; k < N; ++k) o[k] = newton_k[k] ? qf[i][k] : fma(omc, qf[i][k], wc[i == 0 ? 0 : 1][k]);
         stv_n(drow + i * pl, o);
     }
     if constexpr (REC) st_rec<N>(rec + (long long)y * pb.pitch + x0, thn);
@@ -382,6 +248,9 @@ __device__ __forceinline__ void row5_update_eebm(const Problem& pb, const P* __r
 {
     const int nx = pb.nx, ny = pb.ny;
     const long long pl = pb.plane;
+    // the state's shift in enthalpy units (FP32 form; 0 in FP64)
+    const P sh = sizeof(P) == 4 ? (P)__ldg(reinterpret_cast<const float*>(reinterpret_cast<const char*>(src) + pb.tail_off))
+                                : (P)0;
     if constexpr (EDGE) {
 #pragma unroll
         for (int k = 0; k < N; ++k) {
@@ -391,12 +260,14 @@ __device__ __forceinline__ void row5_update_eebm(const Problem& pb, const P* __r
                 int wall;
 #pragma unroll
                 for (int i = 0; i < 5; ++i) { qq[i] = qf[i][k]; uu[i] = u[i][k]; }
+                P nq[5];
+                if (pb.bb_mode == 2) pulled5_inward<P>(src, pb, x, y, nq);
                 if constexpr (sizeof(P) == 4) {
-                    const ff fl = wall5_closure_f(qq, uu, x, y, pb, src, wall);
+                    const ff fl = wall5_closure_f(qq, uu, nq, x, y, pb, wall, (float)sh);
                     ff_add(ts.flux_f, fl.hi);
                     ts.flux_f.lo += fl.lo;
                 } else {
-                    ts.flux += wall5_closure_d(qq, uu, x, y, pb, src, wall);
+                    fx_add(ts.flux, to_fixed(wall5_closure_d(qq, uu, nq, x, y, pb, wall)));
                 }
 #pragma unroll
                 for (int i = 0; i < 5; ++i) qf[i][k] = qq[i];
@@ -405,34 +276,38 @@ __device__ __forceinline__ void row5_update_eebm(const Problem& pb, const P* __r
     }
     const P om = (P)1 - omc;
     const P inv_ste = (P)pb.inv_ste;
-    // the state's shift in enthalpy units (FP32 form; 0 in FP64)
-    const P sh = sizeof(P) == 4 ? (P)__ldg(reinterpret_cast<const float*>(reinterpret_cast<const char*>(src) + pb.tail_off))
-                                : (P)0;
     P hs = 0;
     double thn[REC ? N : 1];
 #pragma unroll
     for (int k = 0; k < N; ++k) {
         const bool valid = !EDGE || x0 + k < nx;
         P Hs = 0;   // H less the shift
+        if constexpr (sizeof(P) == 4) {
 #pragma unroll
-        for (int i = 4; i >= 0; --i) Hs += qf[i][k];
+            for (int i = 4; i >= 0; --i) Hs += qf[i][k];
+        } else {
+            P qk[5];
+#pragma unroll
+            for (int i = 0; i < 5; ++i) qk[i] = qf[i][k];
+            Hs = sum_q<5>(qk);
+        }
         if (!valid) {
             Hs = 0;
 #pragma unroll
             for (int i = 0; i < 5; ++i) qf[i][k] = (P)0;
         }
-        hs += Hs;
+        if constexpr (sizeof(P) == 4) hs += Hs;
+        else acc.add_d(Hs);
         if constexpr (sizeof(P) == 4) ts.shifted += valid ? 1 : 0;
         const P H = Hs + sh;
         const P th = eebm_theta(H, inv_ste);
         if constexpr (REC) thn[k] = (double)th;
         // stored values less w_i sh
-        qf[0][k] = fma(omc, qf[0][k], om * (H - ((P)1 - w0) * th - w0 * sh));
+        qf[0][k] = fma(omc, qf[0][k], om * eebm_rest(H, th, w0, sh));
 #pragma unroll
         for (int i = 1; i < 5; ++i) qf[i][k] = fma(omc, qf[i][k], om * w1 * (th - sh));
     }
     if constexpr (sizeof(P) == 4) acc.add_ff(ff{hs, 0.f});
-    else acc.add_d(hs);
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
         P o[N];

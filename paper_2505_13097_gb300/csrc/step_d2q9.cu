@@ -301,7 +301,7 @@ __device__ __forceinline__ void flat_cold_node(const Problem& pb, int pi, const 
         const float om = 1.0f - omc;
         const float H = Hs + sh;
         const float th = eebm_theta(H, (float)pb.inv_ste);
-        d[0] = fmaf(omc, q[0], om * (H - (1.0f - wP[0]) * th - wP[0] * sh));
+        d[0] = fmaf(omc, q[0], om * eebm_rest(H, th, wP[0], sh));
         const float tr = th - sh;
 #pragma unroll
         for (int i = 1; i < 9; ++i) d[i * pl] = fmaf(omc, q[i], om * (i <= 4 ? wP[1] : wP[2]) * tr);
@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(256, LBM_FLAT_MINB) d2q9_flat_kernel(const Ste
                 const float H = Hs + sh;
                 const float th = eebm_theta(H, inv_ste);
                 if constexpr (REC) thn[k] = (double)th;
-                qf[0][k] = fmaf(omc, qf[0][k], om * (H - (1.0f - wP[0]) * th - wP[0] * sh));
+                qf[0][k] = fmaf(omc, qf[0][k], om * eebm_rest(H, th, wP[0], sh));
                 const float tr = th - sh;
 #pragma unroll
                 for (int i = 1; i < 9; ++i) qf[i][k] = fmaf(omc, qf[i][k], om * (i <= 4 ? wP[1] : wP[2]) * tr);

@@ -1,0 +1,949 @@
+// D2Q9 and D2Q5 steps in one resident launch: a cooperative grid keeps its
+// blocks on the SMs for all the steps of a call, one node per thread, the
+// Newton solve of Eq. (14) in place, one grid barrier per step.
+//
+// What bounds it.  A step of a small lattice launched kernel by kernel is a
+// chain of latencies: the wall kernels, the stencil, the side and the last
+// Newton launch and the publication of the statistics, 45 us whatever the size
+// (130 x 64 nodes, FP32).  Here a step ends at one barrier (load, arrival, poll
+// and fence: 4 to 5 us on a lattice of a few hundred nodes), and its sums are
+// added up by a block of their own while the next step runs.  Measured, us per
+// step before and now: D2Q9 FP32 130 x 64 45 / 9.5, 1021 x 777 61 / 18; D2Q9
+// FP64 2048^2 387 / 181; D2Q5 FP32 4096^2 205 / 128, FP64 401^2 116 / 16.
+//
+// A step has two passes over what a block owns, between barriers of the block:
+//  1. plain nodes.  A warp takes a group of 32 N consecutive columns of one of
+//     the rows 1 .. ny-2 (N = 4 in FP32, one 128-bit load per plane, as the
+//     flat kernel; 1 in FP64).  Saturated nodes are updated, the nodes that
+//     need the Newton solve go to a queue in shared memory.
+//  2. items of 32 nodes, one per lane: the queued nodes, gathered densely so
+//     that a solve (a chain of 58 FP64 instructions of 64 cycles) serves full
+//     warps, the rows 0 and ny-1, and the column groups at the W and E walls.
+// Groups of a wave lie side by side (their halo rows and columns meet in L1 and
+// L2), and a block's place in the wave rotates from wave to wave, so that the
+// groups of a front band spread over all SMs.  A lattice of few nodes has no
+// first pass: every node is an item.
+//
+// Memory order.  A step reads state[p] and writes state[p ^ 1].  Every read of
+// a state is a plain load (never the read-only path, which is not coherent
+// with stores of the same launch); the barrier's fences make a step's stores
+// visible and drop stale L1 lines.
+//
+// Arithmetic: that of the kernels in step_d2q9.cu / step_d2q5.cu node by node.
+// FP64 form: the zeroth moment is summed in block floating point with integer
+// instructions (sum_q below) and w_i c takes one multiplication, 10 FP64
+// instructions per D2Q9 node instead of 28: the FP64 pipe, one warp
+// instruction per 64 cycles of an SM quarter, bounds the FP64 form.
+#include <algorithm>
+
+#include "d2q5_row.cuh"
+#include "d2q9_row.cuh"
+
+#ifndef LBM_RES_TF
+#define LBM_RES_TF 768
+#endif
+#ifndef LBM_RES_TD
+#define LBM_RES_TD 640
+#endif
+#ifndef LBM_RES_SCALAR
+#define LBM_RES_SCALAR 8
+#endif
+
+namespace lbm {
+
+// ---------------------------------------------------------------- arguments
+// A warp's, and a block's, sums of one step.
+struct alignas(16) ResidentSlot {
+    Fx e, f;                    // energy terms, boundary flux
+    unsigned liquid, shifted;   // saturated liquid nodes; energy terms added less the shift
+    unsigned dir[4];            // Dirichlet nodes per wall
+    unsigned newton, iters;     // nodes solved, their iterations
+    int maxit;
+    unsigned pad[3];
+};
+
+struct ResidentArgs {
+    Problem pb;                 // by value: constants come from the parameter bank
+    int parity, nsteps;
+    double* rec;                // theta' planes of the steps (ny x pitch each), or NULL
+    DevStats* stats;
+    ResidentSlot* slots;        // kResidentRing sets of one per computing block
+    ResidentBar* bar;
+    int strips, th, tiles;      // first pass: column strips, rows of a tile, tiles (0: no first pass)
+    int nseg;                   // 32-column segments of a row (the items of full rows)
+    int items;                  // second pass: items without the queue
+    int rot;
+    long long wait_ns;
+};
+
+// ---------------------------------------------------------------- grid barrier
+__device__ __forceinline__ unsigned ld_acquire(const unsigned* p)
+{
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+
+// One thread: an arrival for its block (the block has synchronized).
+__device__ __forceinline__ void bar_arrive(unsigned* count)
+{
+    fence_gpu();
+    atomicAdd(count, 1u);
+}
+
+// One thread: waits until *count has reached `target`, for at most limit_ns;
+// false when the wait ran out here or in another block.
+__device__ __forceinline__ bool bar_wait(ResidentBar* b, const unsigned* count, unsigned target, long long limit_ns)
+{
+    unsigned long long t0 = 0;
+    for (unsigned i = 0;; ++i) {
+        if ((int)(ld_acquire(count) - target) >= 0) break;
+        if ((i & 63u) == 63u) {
+            if (ld_acquire(&b->abort)) return false;
+            if (t0 == 0) t0 = global_ns();
+            else if ((long long)(global_ns() - t0) > limit_ns) {
+                atomicExch(&b->abort, 1u);
+                return false;
+            }
+        }
+    }
+    fence_gpu();
+    return true;
+}
+
+// ---------------------------------------------------------------- one node
+template <typename P> struct LaneAcc;
+template <> struct LaneAcc<float> {
+    ff s{0.f, 0.f};
+    __device__ void add(float v) { ff_add(s, v); }
+    __device__ Fx total() const
+    {
+        ff t = s;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float h = __shfl_xor_sync(kFull, t.hi, o), l = __shfl_xor_sync(kFull, t.lo, o);
+            ff_add(t, h);
+            t.lo += l;
+        }
+        Fx f = float_to_fixed(t.hi);
+        fx_add(f, float_to_fixed(t.lo));
+        return f;
+    }
+};
+template <> struct LaneAcc<double> {
+    Fx s{0, 0ull};
+    __device__ void add(double v) { fx_add(s, to_fixed(v)); }
+    __device__ Fx total() const { return fx_tree(s); }
+};
+
+// One item: a node (x, y) per lane, anywhere in the lattice (idle lanes: not
+// valid).  w: the warp's sums in shared memory, where lane 0 adds what few
+// items have.  A resident state has fewer than 2^31 elements (32-bit indices).
+template <typename P, int Q, bool EEBM>
+__device__ __forceinline__ void item_update(const ResidentArgs& a, const P* src, P* dst, double* rec, int x, int y,
+                                            bool valid, int lane, float sh, LaneAcc<P>& acc, ResidentSlot* w)
+{
+    const Problem& pb = a.pb;
+    const int nx = pb.nx, ny = pb.ny, pitch = pb.pitch, plane = (int)pb.plane;
+    const int at = (y + 1) * pitch + x;
+    P u[Q], q[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        u[i] = q[i] = (P)0;
+        if (valid) {
+            u[i] = src[at + i * plane];
+            q[i] = i == 0 ? u[0] : src[at + i * plane - d2_ey(i) * pitch - d2_ex(i)];   // Omega_i(y - e_i)
+        }
+    }
+    int wall = -1;
+    const bool edge = valid && (x == 0 || x == nx - 1 || y == 0 || y == ny - 1);
+    if (__any_sync(kFull, edge)) {
+        Fx fl{0, 0ull};
+        if (edge) {
+            // copies: the closures take addresses, and u, q stay in registers elsewhere
+            P qq[Q], uu[Q];
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                qq[i] = q[i];
+                uu[i] = u[i];
+            }
+            if constexpr (Q == 9) {
+                if constexpr (sizeof(P) == 4) {
+                    const ff t = wall_closure_f(qq, uu, x, y, pb, wall, sh);
+                    fl = float_to_fixed(t.hi);
+                    fx_add(fl, float_to_fixed(t.lo));
+                } else {
+                    fl = to_fixed(wall_closure_d(qq, uu, x, y, pb, wall));
+                }
+            } else {
+                P nq[5];
+                if (pb.bb_mode == 2) pulled5_inward<P>(src, pb, x, y, nq);
+                if constexpr (sizeof(P) == 4) {
+                    const ff t = wall5_closure_f(qq, uu, nq, x, y, pb, wall, sh);
+                    fl = float_to_fixed(t.hi);
+                    fx_add(fl, float_to_fixed(t.lo));
+                } else {
+                    fl = to_fixed(wall5_closure_d(qq, uu, nq, x, y, pb, wall));
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < Q; ++i) q[i] = qq[i];
+        }
+        fl = fx_tree(fl);
+        if (lane == 0) fx_add(w->f, fl);
+    }
+    const P omc = sizeof(P) == 4 ? (P)pb.omc_f : (P)pb.omc;
+    if constexpr (EEBM) {
+        // Algorithm 2: H = M0(q), theta = Theta(H); stored values less w_i sh
+        const P om = (P)1 - omc, w0 = lat_wp<P>(Q, 0);
+        P Hs = (P)0;
+        if constexpr (sizeof(P) == 8) {
+            Hs = sum_q<Q>(q);
+        } else {
+#pragma unroll
+            for (int i = Q - 1; i >= 0; --i) Hs += q[i];
+        }
+        const P H = Hs + (P)sh;
+        const P th = eebm_theta(H, (P)pb.inv_ste);
+        if (valid) {
+            acc.add(Hs);
+            dst[at] = fma(omc, q[0], om * eebm_rest(H, th, w0, (P)sh));
+            const P tr = th - (P)sh;
+#pragma unroll
+            for (int i = 1; i < Q; ++i) dst[at + i * plane] = fma(omc, q[i], om * lat_wp<P>(Q, i) * tr);
+            if (rec) rec[y * pitch + x] = (double)th;
+        }
+        if constexpr (sizeof(P) == 4) {
+            const unsigned n = (unsigned)__popc(__ballot_sync(kFull, valid));
+            if (lane == 0) w->shifted += n;
+        }
+        return;
+    }
+    // saturation from FP32 sums
+    float tf = 0.f;
+    P m0;        // FP32: M0(q) less sh, the plain sum
+    float mt;
+    if constexpr (sizeof(P) == 4) {
+        if constexpr (Q == 9) {
+#pragma unroll
+            for (int i = 0; i < Q; ++i) tf += u[i];
+        } else {
+#pragma unroll
+            for (int i = Q - 1; i >= 0; --i) tf += u[i];
+        }
+        tf += sh;
+        m0 = 0.f;
+#pragma unroll
+        for (int i = Q - 1; i >= 0; --i) m0 += q[i];
+        mt = m0 + sh;
+    } else {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) tf += approx_float(u[i]);
+        m0 = sum_q<Q>(q);
+        mt = approx_float(m0);
+    }
+    const float marg = 1e-5f * (1.0f + fabsf(tf)), thr = pb.sat_f;
+    const bool liq = tf >= thr + marg && mt >= thr + marg;
+    const bool sat = liq || (tf <= -thr - marg && mt <= -thr - marg);
+    const bool dir = wall >= 0;
+    const bool solve = valid && !dir && !sat;
+    const unsigned solving = __ballot_sync(kFull, solve);
+    const bool plain = valid && !dir && sat;
+    {
+        const unsigned n = (unsigned)__popc(__ballot_sync(kFull, plain && liq));
+        const unsigned m = sizeof(P) == 4 ? (unsigned)__popc(__ballot_sync(kFull, plain)) : 0u;
+        if (lane == 0) {
+            w->liquid += n;
+            w->shifted += m;
+        }
+    }
+    if (plain) acc.add(m0);
+    // c = theta' - (1 - omega) m0 (FP32: less omega sh); saturated: theta' = m0, c = omega m0
+    P c = sizeof(P) == 4 ? (P)(pb.omega_f * (float)m0) : m0;
+    double tn = 0.0;
+    if (rec) tn = sizeof(P) == 4 ? widen((float)m0) + widen(sh) : (double)m0;
+    if (__any_sync(kFull, dir)) {
+        // theta' = theta_D
+        Fx e{0, 0ull};
+        if (dir) {
+            if constexpr (sizeof(P) == 4) {
+                ff mm{0.f, 0.f};
+#pragma unroll
+                for (int i = Q - 1; i >= 0; --i) ff_add(mm, q[i]);
+                c = (P)(((pb.wall_th_hi[wall] - sh) - (float)omc * mm.hi) + (pb.wall_th_lo[wall] - (float)omc * mm.lo));
+                e = float_to_fixed(pb.wall_th_hi[wall]);
+                fx_add(e, float_to_fixed(pb.wall_th_lo[wall]));
+            } else {
+                c = (P)(pb.wall_theta[wall] - pb.omc * (double)m0);
+                e = to_fixed(pb.wall_theta[wall]);
+            }
+            tn = pb.wall_theta[wall];
+        }
+        e = fx_tree(e);
+        if (lane == 0) fx_add(w->e, e);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const unsigned b = __ballot_sync(kFull, dir && wall == k);
+            if (lane == 0) w->dir[k] += (unsigned)__popc(b);
+        }
+    }
+    if (solving) {
+        // the local Newton solve of Eq. (14)
+        Fx e{0, 0ull};
+        int it = 0;
+        if (solve) {
+            double m, t, shd = 0.0;
+            if constexpr (sizeof(P) == 4) {
+                ff mm{0.f, 0.f}, tt{0.f, 0.f};
+#pragma unroll
+                for (int i = Q - 1; i >= 0; --i) {
+                    ff_add(tt, u[i]);
+                    ff_add(mm, q[i]);
+                }
+                shd = widen(sh);
+                m = ff_to_double(mm) + shd;
+                t = ff_to_double(tt) + shd;
+            } else {
+                m = (double)m0;
+                t = sum_q<Q>(u);
+            }
+            const Phi pt = phi_parts(t, pb.two_inv_delta);
+            const NewtonOut nr = newton_mixed(m, t, pt, pb);
+            if (!nr.ok || !isfinite(nr.root)) atomicCAS(&a.stats->error, 0, 3);
+            tn = m + (pt.value() - nr.phi_root) * pb.inv_ste;
+            c = (P)((tn - shd) - pb.omc * (m - shd));
+            e = to_fixed(tn + nr.phi_root * pb.inv_ste);
+            it = nr.iters;
+        }
+        e = fx_tree(e);
+        const unsigned its = __reduce_add_sync(kFull, (unsigned)it);
+        const int mx = __reduce_max_sync(kFull, it);
+        if (lane == 0) {
+            fx_add(w->e, e);
+            w->newton += (unsigned)__popc(solving);
+            w->iters += its;
+            w->maxit = max(w->maxit, mx);
+        }
+    }
+    // Omega~_i = (1-omega) q_i + w_i c
+    P wc[3];
+    if constexpr (sizeof(P) == 4) {
+        wc[0] = lat_wp<P>(Q, 0) * c;
+        wc[1] = lat_wp<P>(Q, 1) * c;
+        wc[2] = Q == 9 ? lat_wp<P>(Q, Q - 1) * c : (P)0;
+    } else {
+        // one multiplication: 4/9 and 1/36 are 4 and 1/4 times 1/9 (D2Q5: 1/3 = 2/6),
+        // and so are their roundings
+        const double w1 = lat_wp<double>(Q, 1);
+        const double v = (plain ? pb.omega * w1 : w1) * (double)c;
+        wc[0] = (P)scale2(v, Q == 9 ? 2 : 1);
+        wc[1] = (P)v;
+        wc[2] = Q == 9 ? (P)scale2(v, -2) : (P)0;
+    }
+    if (valid) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) dst[at + i * plane] = fma(omc, q[i], wc[i == 0 ? 0 : (i <= 4 ? 1 : 2)]);
+        if (rec) rec[y * pitch + x] = tn;
+    }
+}
+
+// ---------------------------------------------------------------- plain nodes
+// The columns x0 .. x0 + N - 1 per lane of row y, 1 <= y <= ny-2 (the same for
+// the warp).  Lanes that hold column 0 or nx-1 or reach past nx leave theirs to
+// the second pass (cold).  Nodes to solve: queued, q left for the second pass.
+__device__ __forceinline__ void ld4(const float* p, float (&v)[4])
+{
+    const float4 t = *reinterpret_cast<const float4*>(p);
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
+
+// The queue (dynamic shared memory) has room for every node of kResidentWaves
+// waves of the first pass; the second pass follows that many waves.
+constexpr int kResidentWaves = 8;
+
+struct ResidentQueue {
+    unsigned count;
+    unsigned* node;     // (y << 16) + x
+};
+
+template <int Q, bool EEBM>
+__device__ __forceinline__ void plain_update(const ResidentArgs& a, const float* src, float* dst, double* rec, int x0,
+                                             int y, int lane, float sh, LaneAcc<float>& acc, ResidentSlot* w,
+                                             ResidentQueue* queue)
+{
+    const Problem& pb = a.pb;
+    const int nx = pb.nx, pitch = pb.pitch, plane = (int)pb.plane;
+    const int at = (y + 1) * pitch + x0;
+    const bool cold = x0 == 0 || x0 + 3 >= nx - 1;
+    const float* row = src + at;
+    // every load of a cold lane stays inside the buffer
+    float u[Q][4], q[Q][4];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) ld4(row + i * plane, u[i]);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        float v[4];
+        const float* p = row + i * plane - d2_ey(i) * pitch;
+        if (d2_ey(i) == 0) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[k] = u[i][k];
+        } else {
+            ld4(p, v);
+        }
+        if (d2_ex(i) == 0) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) q[i][k] = v[k];
+        } else if (d2_ex(i) == 1) {
+            q[i][0] = p[-1];
+            q[i][1] = v[0]; q[i][2] = v[1]; q[i][3] = v[2];
+        } else {
+            q[i][0] = v[1]; q[i][1] = v[2]; q[i][2] = v[3];
+            q[i][3] = p[4];
+        }
+    }
+    const float omc = pb.omc_f;
+    if constexpr (EEBM) {
+        const float om = 1.0f - omc, inv_ste = pb.inv_ste_f, w0 = lat_wp<float>(Q, 0);
+        float hs = 0.f;
+        double thn[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            float Hs = 0.f;   // H less the shift
+#pragma unroll
+            for (int i = Q - 1; i >= 0; --i) Hs += q[i][k];
+            hs += Hs;
+            const float H = Hs + sh;
+            const float th = eebm_theta(H, inv_ste);
+            thn[k] = widen(th);
+            q[0][k] = fmaf(omc, q[0][k], om * eebm_rest(H, th, w0, sh));
+            const float tr = th - sh;
+#pragma unroll
+            for (int i = 1; i < Q; ++i) q[i][k] = fmaf(omc, q[i][k], om * lat_wp<float>(Q, i) * tr);
+        }
+        const unsigned n = (unsigned)__popc(__ballot_sync(kFull, !cold));
+        if (lane == 0) w->shifted += 4u * n;
+        if (!cold) {
+            acc.add(hs);
+#pragma unroll
+            for (int i = 0; i < Q; ++i) stv_n(dst + at + i * plane, q[i]);
+            if (rec) st_rec<4>(rec + y * pitch + x0, thn);
+        }
+        return;
+    }
+    const float om_f = pb.omega_f, thr = pb.sat_f;
+    float c[4], m0[4], esum = 0.f;
+    unsigned solve = 0, liquid = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        float tf = 0.f, mf = 0.f;
+        if constexpr (Q == 9) {
+#pragma unroll
+            for (int i = 0; i < Q; ++i) tf += u[i][k];
+        } else {
+#pragma unroll
+            for (int i = Q - 1; i >= 0; --i) tf += u[i][k];
+        }
+        tf += sh;   // theta
+#pragma unroll
+        for (int i = Q - 1; i >= 0; --i) mf += q[i][k];   // M0(q) - sh
+        const float mt = mf + sh;
+        const float marg = 1e-5f * (1.0f + fabsf(tf));
+        const bool liq = tf >= thr + marg && mt >= thr + marg;
+        const bool sat = liq || (tf <= -thr - marg && mt <= -thr - marg);
+        c[k] = om_f * mf;   // c - omega sh = omega (m0 - sh)
+        m0[k] = mf;
+        if (sat) {
+            esum += mf;
+            liquid += liq ? 1u : 0u;
+        } else {
+            solve |= 1u << k;
+        }
+    }
+    if (cold) {
+        solve = liquid = 0u;
+        esum = 0.f;
+    }
+    acc.add(esum);
+    // the warp's counts: liquid, and plain nodes (whose energy terms lack the shift)
+    const unsigned plainc = cold ? 0u : 4u - (unsigned)__popc(solve);
+    const unsigned n = __reduce_add_sync(kFull, liquid | (plainc << 16));
+    if (lane == 0) {
+        w->liquid += n & 0xffffu;
+        w->shifted += n >> 16;
+    }
+    if (!cold) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            const float wi = lat_wp<float>(Q, i);
+            float o[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) o[k] = fmaf(omc, q[i][k], wi * c[k]);
+            stv_n(dst + at + i * plane, o);   // (a queued node's values are replaced by the second pass)
+        }
+        if (rec) {
+            double thn[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) thn[k] = widen(m0[k]) + widen(sh);
+            st_rec<4>(rec + y * pitch + x0, thn);
+        }
+    }
+    if (__any_sync(kFull, solve != 0u)) {
+        const unsigned cnt = (unsigned)__popc(solve);
+        unsigned incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned v = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += v;
+        }
+        unsigned base = 0;
+        if (lane == 31) base = atomicAdd(&queue->count, incl);
+        unsigned slot = __shfl_sync(kFull, base, 31) + incl - cnt;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if ((solve >> k) & 1u) queue->node[slot++] = ((unsigned)y << 16) + (unsigned)(x0 + k);
+    }
+}
+
+// FP64: one column per lane.
+template <int Q, bool EEBM>
+__device__ __forceinline__ void plain_update(const ResidentArgs& a, const double* src, double* dst, double* rec, int x,
+                                             int y, int lane, float sh, LaneAcc<double>& acc, ResidentSlot* w,
+                                             ResidentQueue* queue)
+{
+    const Problem& pb = a.pb;
+    const int nx = pb.nx, pitch = pb.pitch, plane = (int)pb.plane;
+    const int at = (y + 1) * pitch + x;
+    const bool cold = x == 0 || x >= nx - 1;
+    double q[Q];
+    float tf = 0.f;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) q[i] = src[at + i * plane - d2_ey(i) * pitch - d2_ex(i)];
+    if constexpr (!EEBM) {
+        float u[Q];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) u[i] = approx_float(i == 0 ? q[0] : src[at + i * plane]);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) tf += u[i];
+    }
+    const double m0 = sum_q<Q>(q);
+    if constexpr (EEBM) {
+        const double th = eebm_theta(m0, pb.inv_ste), omc = pb.omc, om = 1.0 - omc;
+        if (!cold) {
+            acc.add(m0);
+            dst[at] = fma(omc, q[0], om * eebm_rest(m0, th, lat_wp<double>(Q, 0), 0.0));
+            const double t1 = (om * lat_wp<double>(Q, 1)) * th;
+            const double t2 = Q == 9 ? scale2(t1, -2) : 0.0;
+#pragma unroll
+            for (int i = 1; i < Q; ++i) dst[at + i * plane] = fma(omc, q[i], i <= 4 ? t1 : t2);
+            if (rec) rec[y * pitch + x] = th;
+        }
+        return;
+    }
+    const float mt = approx_float(m0), thr = pb.sat_f;
+    const float marg = 1e-5f * (1.0f + fabsf(tf));
+    const bool liq = tf >= thr + marg && mt >= thr + marg;
+    const bool sat = liq || (tf <= -thr - marg && mt <= -thr - marg);
+    const bool solve = !cold && !sat;
+    const unsigned nliq = (unsigned)__popc(__ballot_sync(kFull, !cold && liq));
+    if (lane == 0) w->liquid += nliq;
+    if (!cold && sat) {
+        // c = omega m0; one multiplication for the three w_i c: 4/9 and 1/36 are 4 and
+        // 1/4 times 1/9 (D2Q5: 1/3 = 2/6), and so are their roundings
+        acc.add(m0);
+        const double v = (pb.omega * lat_wp<double>(Q, 1)) * m0;
+        const double v0 = scale2(v, Q == 9 ? 2 : 1), v2 = Q == 9 ? scale2(v, -2) : 0.0;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) dst[at + i * plane] = fma(pb.omc, q[i], i == 0 ? v0 : (i <= 4 ? v : v2));
+        if (rec) rec[y * pitch + x] = m0;
+    }
+    const unsigned solving = __ballot_sync(kFull, solve);
+    if (solving) {
+        unsigned base = 0;
+        if (lane == 0) base = atomicAdd(&queue->count, (unsigned)__popc(solving));
+        const unsigned slot = __shfl_sync(kFull, base, 0) + (unsigned)__popc(solving & ((1u << lane) - 1u));
+        if (solve) queue->node[slot] = ((unsigned)y << 16) + (unsigned)x;
+    }
+}
+
+// ---------------------------------------------------------------- a block's sums
+// One warp: adds up the block's warps' sums of step s, clears them for step
+// s + 2, and hands the total to the statistics block: the block's next arrival
+// at the barrier releases it.
+static __device__ __noinline__ void resident_emit(const ResidentArgs& a, int s, int nb, int lane, int nwb, ResidentSlot* w)
+{
+    ResidentSlot t = {};
+    if (lane < nwb) {
+        t = w[lane];
+        w[lane] = ResidentSlot{};
+    }
+    t.e = fx_tree(t.e);
+    t.f = fx_tree(t.f);
+    t.liquid = __reduce_add_sync(kFull, t.liquid);
+    t.shifted = __reduce_add_sync(kFull, t.shifted);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) t.dir[k] = __reduce_add_sync(kFull, t.dir[k]);
+    t.newton = __reduce_add_sync(kFull, t.newton);
+    t.iters = __reduce_add_sync(kFull, t.iters);
+    t.maxit = __reduce_max_sync(kFull, t.maxit);
+    // The sets of the next steps have been read (a ring ago: no wait in practice); looked
+    // at for half a ring at once, one lane per set.
+    constexpr int kHalf = kResidentRing / 2;
+    if (s >= kResidentRing && s % kHalf == 0 && lane < kHalf)
+        bar_wait(a.bar, &a.bar->read[(s + lane) % kResidentRing], (unsigned)(s / kResidentRing), a.wait_ns);
+    __syncwarp();
+    if (lane == 0) a.slots[(size_t)(s % kResidentRing) * nb + blockIdx.x] = t;
+}
+
+// ---------------------------------------------------------------- statistics block
+// Adds up the computing blocks' sums of every step while later steps run: warp
+// w takes the steps w, w + W, ... (W warps), each once the arrivals of the step
+// after it are in (those of the last step: the blocks' arrivals at their end).
+// A set of slots is written again kResidentRing steps later, after `read` says
+// that it has been read.
+static __device__ __noinline__ void resident_stats(const ResidentArgs& a, unsigned nb)
+{
+    __shared__ volatile double ring_e[kResidentRing];
+    __shared__ volatile int ring_step[kResidentRing];
+    __shared__ double imax_s[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwb = blockDim.x >> 5;
+    const Problem& pb = a.pb;
+    DevStats* st = a.stats;
+    ResidentBar* bar = a.bar;
+    const double e0 = st->energy;   // of the state before the first step
+    const int have0 = st->have_energy;
+    double imax = 0.0;
+    if (threadIdx.x < kResidentRing) ring_step[threadIdx.x] = -1;
+    __syncthreads();
+    bool ok = true;
+    for (int s = warp; ok && s < a.nsteps; s += nwb) {
+        const int at = s % kResidentRing;
+        int good = 0;
+        if (lane == 0) good = bar_wait(bar, &bar->count, (unsigned)(s + 2) * nb, a.wait_ns);
+        ok = __shfl_sync(kFull, good, 0) != 0;
+        if (!ok) break;
+        const ResidentSlot* set = a.slots + (size_t)at * nb;
+        unsigned long long v[16] = {};   // e 4 limbs, f 4 limbs, dir 4, newton, iters, liquid, shifted
+        int mx = 0;
+        for (unsigned k = lane; k < nb; k += 32) {
+            const uint4* p = reinterpret_cast<const uint4*>(set + k);
+            const uint4 x0 = __ldcg(p), x1 = __ldcg(p + 1), x2 = __ldcg(p + 2), x3 = __ldcg(p + 3), x4 = __ldcg(p + 4);
+            // Fx is {hi, lo}, 8 bytes each
+            v[0] += x0.z; v[1] += x0.w; v[2] += x0.x; v[3] += x0.y;
+            v[4] += x1.z; v[5] += x1.w; v[6] += x1.x; v[7] += x1.y;
+            v[14] += x2.x; v[15] += x2.y;
+            v[8] += x2.z; v[9] += x2.w; v[10] += x3.x; v[11] += x3.y;
+            v[12] += x3.z; v[13] += x3.w;
+            mx = max(mx, (int)x4.x);
+        }
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(kFull, v[k], o);
+        mx = __reduce_max_sync(kFull, mx);
+        if (lane == 0) {
+            fence_gpu();
+            atomicAdd(&bar->read[at], 1u);   // the set is read
+            AccSum es, fs;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                es.limb[j] = v[j];
+                fs.limb[j] = v[4 + j];
+            }
+            double e = acc_read(&es);
+            const double f = acc_read(&fs);
+            double c = (double)v[14];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (v[8 + k]) c += (double)v[8 + k] * pb.wall_phi[k];
+            e += c * pb.inv_ste;
+            if (v[15]) e += (double)v[15] * (double)state_shift(pb, 0);
+            // the previous step's energy, from the warp that has that step
+            double ep = e0;
+            bool have = have0 != 0;
+            if (s > 0) {
+                const int prev = (s - 1) % kResidentRing;
+                unsigned i = 0;
+                while (ring_step[prev] != s - 1) {
+                    if ((++i & 255u) == 0u && ld_acquire(&bar->abort)) {
+                        good = 0;
+                        break;
+                    }
+                }
+                __threadfence_block();
+                ep = ring_e[prev];
+                have = true;
+            }
+            ring_e[at] = e;
+            __threadfence_block();
+            ring_step[at] = s;
+            const double imb = have ? e - ep - f : 0.0;
+            imax = fmax(imax, fabs(imb));
+            if (s + 1 == a.nsteps) {
+                st->energy = e;
+                st->energy_prev = ep;
+                st->imbalance = imb;
+                st->flux = f;
+                st->have_energy = 1;
+                st->newton_nodes = (long long)v[12];
+                st->newton_iters = (long long)v[13];
+                st->newton_max_iter = mx;
+            }
+        }
+        ok = __shfl_sync(kFull, good, 0) != 0;
+    }
+    if (lane == 0) imax_s[warp] = imax;
+    const int all_ok = __syncthreads_and(ok ? 1 : 0);
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < nwb; ++w) imax = fmax(imax, imax_s[w]);
+        if (imax > st->imbalance_max) st->imbalance_max = imax;
+        st->steps += a.nsteps;
+        if (!all_ok) atomicExch(&st->error, 4);   // LBM_ERR_TIMEOUT
+    }
+}
+
+// One block of a size that leaves 80 (FP32) or 96 (FP64) registers a thread.
+template <typename P> constexpr int kResidentThreads = sizeof(P) == 4 ? LBM_RES_TF : LBM_RES_TD;
+
+template <typename P, int Q, bool EEBM>
+__global__ void __launch_bounds__(kResidentThreads<P>, 1) resident_kernel(const __grid_constant__ ResidentArgs a)
+{
+    __shared__ ResidentSlot wsum[2][kResidentThreads<P> / 32];   // by step parity
+    __shared__ ResidentQueue queue;
+    extern __shared__ unsigned queue_nodes[];
+    __shared__ unsigned next_item;
+    __shared__ bool ok_s;
+    constexpr int N = sizeof(P) == 4 ? 4 : 1;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwb = blockDim.x >> 5;
+    const int nb = gridDim.x - 1;   // computing blocks; the last block adds up the statistics
+    if ((int)blockIdx.x == nb) {
+        resident_stats(a, (unsigned)nb);
+    } else {
+        const Problem& pb = a.pb;
+        const int nx = pb.nx, ny = pb.ny;
+        const float sh = sizeof(P) == 4 ? state_shift(pb, 0) : 0.f;   // the same in both buffers
+        const int row_tiles = a.tiles ? a.tiles / a.strips : 0;       // a strip's tiles follow one another
+        const int g = nwb / a.th;                                     // tiles a block takes at a time
+        const int xe = max(N, (nx - 1) / N * N);                      // the E wall's column group
+        if (threadIdx.x == 0) {
+            queue.count = next_item = 0u;
+            queue.node = queue_nodes;
+        }
+        for (int k = threadIdx.x; k < 2 * nwb * (int)(sizeof(ResidentSlot) / 16); k += blockDim.x)
+            reinterpret_cast<uint4*>(k < nwb * (int)(sizeof(ResidentSlot) / 16) ? wsum[0] : wsum[1])
+                [k % (nwb * (int)(sizeof(ResidentSlot) / 16))] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+        bool ok = true;
+        for (int s = 0; ok && s < a.nsteps; ++s) {
+            const int p = (a.parity + s) & 1;
+            const P* src = static_cast<const P*>(pb.state[p]);
+            P* dst = static_cast<P*>(pb.state[p ^ 1]);
+            double* rec = a.rec ? a.rec + (long long)s * ny * pb.pitch : nullptr;
+            ResidentSlot* w = &wsum[s & 1][warp];
+            LaneAcc<P> acc;
+            // the items that are not queued: this block's share of the rows 0 and ny-1 (or of all
+            // rows) and of the W and E column groups
+            unsigned own = a.items > (int)blockIdx.x ? (unsigned)(a.items - 1 - (int)blockIdx.x) / nb + 1u : 0u;
+            int place = blockIdx.x, t0 = 0;
+            do {
+                for (int k = 0; k < kResidentWaves && t0 < a.tiles; ++k, t0 += nb * g) {
+                    // a wave: g tiles of every block, the tiles of a strip dealt round the blocks
+                    const int t = t0 + warp / a.th * nb + place;
+                    place += a.rot;
+                    if (place >= nb) place -= nb;
+                    if (warp / a.th >= g || t >= a.tiles) continue;
+                    const int strip = t / row_tiles;
+                    const int y = 1 + (t - strip * row_tiles) * a.th + warp % a.th;
+                    const int x0 = (strip * 32 + lane) * N;
+                    if (y < ny - 1) plain_update<Q, EEBM>(a, src, dst, rec, x0, y, lane, sh, acc, w, &queue);
+                }
+                if (a.tiles) __syncthreads();
+                const unsigned queued = queue.count;
+                const unsigned total = own + (queued + 31u) / 32u;
+                unsigned it = (unsigned)warp;
+                while (it < total) {
+                    int x = 0, y = 0;
+                    bool valid;
+                    if (it < own) {
+                        const int e = (int)(it * nb + blockIdx.x);
+                        const int rows = a.tiles ? 2 * a.nseg : a.items;
+                        if (e < rows) {
+                            const int r = e / a.nseg;
+                            x = (e - r * a.nseg) * 32 + lane;
+                            y = a.tiles ? (r ? ny - 1 : 0) : r;
+                            valid = x < nx;
+                        } else {
+                            // 2 N columns of 32 / (2 N) rows
+                            const int k = lane % (2 * N);
+                            y = 1 + (e - rows) * (32 / (2 * N)) + lane / (2 * N);
+                            x = k < N ? k : xe + k - N;
+                            valid = y < ny - 1 && x < nx;
+                        }
+                    } else {
+                        const unsigned j = (it - own) * 32u + (unsigned)lane;
+                        valid = j < queued;
+                        if (valid) {
+                            const unsigned n = queue.node[j];
+                            x = (int)(n & 0xffffu);
+                            y = (int)(n >> 16);
+                        }
+                    }
+                    item_update<P, Q, EEBM>(a, src, dst, rec, x, y, valid, lane, sh, acc, w);
+                    // the first items are dealt, the others taken
+                    if (total <= (unsigned)nwb) break;
+                    if (lane == 0) it = (unsigned)nwb + atomicAdd(&next_item, 1u);
+                    it = __shfl_sync(kFull, it, 0);
+                }
+                own = 0u;
+                if (t0 < a.tiles) {
+                    __syncthreads();
+                    if (threadIdx.x == 0) queue.count = next_item = 0u;
+                    __syncthreads();
+                }
+            } while (t0 < a.tiles);
+            const Fx e = acc.total();
+            if (lane == 0) fx_add(w->e, e);
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                queue.count = next_item = 0u;
+                bar_arrive(&a.bar->count);
+                ok_s = s + 1 == a.nsteps || bar_wait(a.bar, &a.bar->count, (unsigned)(s + 1) * nb, a.wait_ns);
+            } else if (warp == 1) {
+                // while thread 0 waits
+                resident_emit(a, s, nb, lane, nwb, wsum[s & 1]);
+            }
+            __syncthreads();
+            ok = ok_s;
+        }
+        if (threadIdx.x == 0) bar_arrive(&a.bar->count);   // the last step's sums are out
+    }
+    // the last block to leave resets the barrier for the next launch
+    __shared__ bool last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        fence_gpu();
+        last = atomicAdd(&a.bar->done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (last) {
+        unsigned* b = reinterpret_cast<unsigned*>(a.bar);
+        for (int k = threadIdx.x; k < (int)(sizeof(ResidentBar) / 4); k += blockDim.x) b[k] = 0u;
+    }
+}
+
+// ---------------------------------------------------------------- launch
+// the queue of a block with a first pass
+template <typename P>
+static size_t resident_smem(bool first_pass)
+{
+    return first_pass ? sizeof(unsigned) * kResidentWaves * kResidentThreads<P> * (sizeof(P) == 4 ? 4 : 1) : 0;
+}
+
+template <typename P, int Q, bool EEBM>
+static cudaError_t resident_go(ResidentArgs& a, int nblocks, int threads, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)nblocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = s;
+    cfg.dynamicSmemBytes = resident_smem<P>(a.tiles > 0);
+    const cudaError_t e = cudaFuncSetAttribute(resident_kernel<P, Q, EEBM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)resident_smem<P>(true));
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;   // every block resident: they wait on one another
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, resident_kernel<P, Q, EEBM>, a);
+}
+
+template <typename P, int Q, bool EEBM>
+static int resident_capacity_t()
+{
+    int dev = 0, sms = 0, per = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(resident_kernel<P, Q, EEBM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)resident_smem<P>(true)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, resident_kernel<P, Q, EEBM>, kResidentThreads<P>,
+                                                      resident_smem<P>(true)) != cudaSuccess)
+        return 0;
+    return sms * per;
+}
+
+template <typename P, int Q>
+static ResidentPlan resident_plan_t(int nx, int ny)
+{
+    ResidentPlan r;
+    const int cap = std::min(resident_capacity_t<P, Q, false>(), resident_capacity_t<P, Q, true>());
+    if (cap < 2 || nx >= 65536 || ny >= 65536) return r;
+    const int most = kResidentThreads<P> / 32, N = sizeof(P) == 4 ? 4 : 1;
+    r.nseg = (nx + 31) / 32;
+    const long long units = (long long)r.nseg * ny;
+    const long long vec = ny > 2 ? (long long)((nx + 32 * N - 1) / (32 * N)) * (ny - 2) : 0;
+    if (units <= (long long)LBM_RES_SCALAR * (cap - 1) || vec == 0) {
+        // few nodes: all of them items, two warps per block, or as many as give every warp one
+        int wpb = 2;
+        while (wpb < most && wpb * (long long)(cap - 1) < units) wpb = std::min(2 * wpb, most);
+        r.items = (int)units;
+        r.blocks = (int)std::min<long long>(cap - 1, (units + wpb - 1) / wpb) + 1;
+        r.threads = wpb * 32;
+    } else {
+        r.strips = (nx + 32 * N - 1) / (32 * N);
+        // tall tiles share their halo rows; short ones spread a front band over the blocks
+        r.th = vec >= 16ll * most * cap ? 8 : 2;
+        r.tiles = r.strips * ((ny - 2 + r.th - 1) / r.th);
+        r.items = 2 * r.nseg + (ny - 2 + 32 / (2 * N) - 1) / (32 / (2 * N));
+        r.blocks = cap;
+        r.threads = most * 32;
+    }
+    r.slots = kResidentRing * (size_t)(r.blocks - 1);
+    r.rot = (int)(0.618 * (r.blocks - 1));
+    return r;
+}
+
+size_t resident_slot_bytes() { return sizeof(ResidentSlot); }
+
+ResidentPlan resident_plan(int precision, int q, int nx, int ny)
+{
+    if (q == 9) return precision == 1 ? resident_plan_t<float, 9>(nx, ny) : resident_plan_t<double, 9>(nx, ny);
+    if (q == 5) return precision == 1 ? resident_plan_t<float, 5>(nx, ny) : resident_plan_t<double, 5>(nx, ny);
+    return ResidentPlan{};
+}
+
+cudaError_t launch_resident(int precision, const ResidentPlan& plan, const Problem& hp, int parity, int nsteps, double* rec,
+                            DevStats* stats, void* slots, ResidentBar* bar, long long wait_ns, cudaStream_t s)
+{
+    ResidentArgs a;
+    a.pb = hp;
+    a.parity = parity;
+    a.nsteps = nsteps;
+    a.rec = rec;
+    a.stats = stats;
+    a.slots = static_cast<ResidentSlot*>(slots);
+    a.bar = bar;
+    a.strips = plan.strips;
+    a.th = plan.th;
+    a.tiles = plan.tiles;
+    a.nseg = plan.nseg;
+    a.items = plan.items;
+    a.rot = plan.rot;
+    a.wait_ns = wait_ns;
+    const bool eebm = hp.method == 1;
+    if (hp.q == 9) {
+        if (precision == 1)
+            return eebm ? resident_go<float, 9, true>(a, plan.blocks, plan.threads, s)
+                        : resident_go<float, 9, false>(a, plan.blocks, plan.threads, s);
+        return eebm ? resident_go<double, 9, true>(a, plan.blocks, plan.threads, s)
+                    : resident_go<double, 9, false>(a, plan.blocks, plan.threads, s);
+    }
+    if (precision == 1)
+        return eebm ? resident_go<float, 5, true>(a, plan.blocks, plan.threads, s)
+                    : resident_go<float, 5, false>(a, plan.blocks, plan.threads, s);
+    return eebm ? resident_go<double, 5, true>(a, plan.blocks, plan.threads, s)
+                : resident_go<double, 5, false>(a, plan.blocks, plan.threads, s);
+}
+
+}  // namespace lbm
