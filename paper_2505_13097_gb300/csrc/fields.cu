@@ -20,6 +20,48 @@ __device__ __forceinline__ bool dirichlet_value(const Problem& pb, int x, int y,
     return false;
 }
 
+// A block's exact sum in thread 0 (256 threads).
+__device__ __forceinline__ Fx block_sum(Fx v)
+{
+    __shared__ Fx part[8];
+    v = fx_tree(v);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < 8; ++w) fx_add(v, part[w]);
+    return v;
+}
+
+// The blocks' exact sums meet in the stripes of one accumulator (S: its offset
+// in a stripe); the last block to arrive (st->ticket, zero before and after)
+// gets the total in its first warp, as a double, and clears the stripes.
+// Returns whether this is that block's first warp.
+template <AccSum StepStripe::*S>
+__device__ __forceinline__ bool last_block_total(DevStats* st, const Fx& v, double& total)
+{
+    __shared__ bool last;
+    if (threadIdx.x == 0) {
+        acc_add_fx(&(st->cur[blockIdx.x % kStripes].*S), v);
+        __threadfence();
+        last = atomicAdd(&st->ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return false;
+    __threadfence();
+    AccSum a;
+    unsigned long long* own = (st->cur[threadIdx.x].*S).limb;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        a.limb[j] = __ldcg(own + j);
+        own[j] = 0ull;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a.limb[j] += __shfl_xor_sync(kFull, a.limb[j], o);
+    }
+    if (threadIdx.x == 0) st->ticket = 0u;
+    total = acc_read(&a);
+    return true;
+}
+
 // The shift s of an FP32 state (its populations are stored less w_i s),
 // written to the tail of both buffers: half the mean over the nodes of the
 // initial M0 (theta0; EEBM: H(theta0)), rounded to a float.  A stored value's
@@ -28,41 +70,40 @@ __device__ __forceinline__ bool dirichlet_value(const Problem& pb, int x, int y,
 // coherently (on the 4096^2 melting workload, 2.45e-5 of theta after 10,000
 // steps against the FP64 form); s = the mean of M0 removes that but makes the
 // values at the melting point (M0 = 0, where phi' is largest) the large ones
-// (max |d phi| 1.04e-4).  Halfway between the two bounds both.  One block; a
-// fixed summation order (deterministic).
-__global__ void __launch_bounds__(1024) shift_kernel(const Problem* dprob, const double* __restrict__ theta0)
+// (max |d phi| 1.04e-4).  Halfway between the two bounds both.  An exact sum
+// over the whole grid, 9 us for 0.5 M nodes: one block took 240 us for 0.8 M
+// and 1.2 ms for 4.2 M.
+__global__ void __launch_bounds__(256) shift_kernel(const Problem* dprob, const double* __restrict__ theta0, DevStats* st)
 {
-    __shared__ double part[1024];
     const Problem& pb = *dprob;
-    const long long n = (long long)pb.nx * pb.ny;
-    double v = 0.0;
-    for (long long k = threadIdx.x; k < n; k += blockDim.x) {
+    const unsigned n = (unsigned)pb.nx * (unsigned)pb.ny;
+    Fx v{0, 0ull};
+    for (unsigned k = blockIdx.x * 256u + threadIdx.x; k < n; k += gridDim.x * 256u) {
         const double th = theta0[k];
-        v += pb.method == 1 ? th + (th > 0.0 ? pb.inv_ste : 0.0) : th;
+        fx_add(v, to_fixed(pb.method == 1 ? th + (th > 0.0 ? pb.inv_ste : 0.0) : th));
     }
-    part[threadIdx.x] = v;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) part[threadIdx.x] += part[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        const float sh = n > 0 ? (float)(0.5 * part[0] / (double)n) : 0.f;
+    v = block_sum(v);
+    double total;
+    if (last_block_total<&StepStripe::flux>(st, v, total) && threadIdx.x == 0) {
+        const float sh = (float)(0.5 * total / (double)n);
         for (int b = 0; b < 2; ++b) *reinterpret_cast<float*>(static_cast<char*>(pb.state[b]) + pb.tail_off) = sh;
     }
 }
 
+// Initial populations; E(0) is summed exactly and published by the last block.
 template <typename P>
-__global__ void init_state_kernel(const Problem* dprob, const double* __restrict__ theta0, int parity, DevStats* st)
+__global__ void __launch_bounds__(256) init_state_kernel(const Problem* dprob, const double* __restrict__ theta0, int parity,
+                                                         DevStats* st)
 {
     const Problem& pb = *dprob;
     P* s = static_cast<P*>(pb.state[parity]);
     // FP32: the populations are stored less w_i sh
     const double sh = sizeof(P) == 4 ? (double)state_shift(pb, parity) : 0.0;
-    const long long n = (long long)pb.nx * pb.ny;
-    double e = 0.0;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(k % pb.nx), y = (int)(k / pb.nx);
+    const unsigned nx = (unsigned)pb.nx, n = nx * (unsigned)pb.ny;
+    Fx e{0, 0ull};
+    for (unsigned k = blockIdx.x * 256u + threadIdx.x; k < n; k += gridDim.x * 256u) {
+        const int y = (int)(k / nx), x = (int)(k - (unsigned)y * nx);
+        const long long at = (long long)(y + 1) * pb.pitch + x;
         double th = theta0[k], td;
         if (dirichlet_value(pb, x, y, td)) th = td;
         if (pb.method == 1) {
@@ -70,24 +111,35 @@ __global__ void init_state_kernel(const Problem* dprob, const double* __restrict
             // and H - (1 - w_0) theta for i = 0
             const double H = th + (th > 0.0 ? pb.inv_ste : 0.0);
             for (int i = 0; i < pb.q; ++i)
-                s[i * pb.plane + (long long)(y + 1) * pb.pitch + x] =
+                s[i * pb.plane + at] =
                     (P)(i == 0 ? H - (1.0 - lat_w(pb.q, 0)) * th - lat_w(pb.q, 0) * sh : lat_w(pb.q, i) * (th - sh));
-            e += H;
+            fx_add(e, to_fixed(H));
             continue;
         }
-        for (int i = 0; i < pb.q; ++i)
-            s[i * pb.plane + (long long)(y + 1) * pb.pitch + x] = (P)(lat_w(pb.q, i) * (th - sh));
+        // one product per weight
+        const P w0 = (P)(lat_w(pb.q, 0) * (th - sh)), w1 = (P)(lat_w(pb.q, 1) * (th - sh));
+        s[at] = w0;
+        for (int i = 1; i < min(pb.q, 5); ++i) s[i * pb.plane + at] = w1;
+        if (pb.q == 9) {
+            const P w2 = (P)(lat_w(9, 5) * (th - sh));
+            for (int i = 5; i < 9; ++i) s[i * pb.plane + at] = w2;
+        }
         if (pb.method == 2) {
             // ILFBM (Algorithm 1): the liquid fraction of the initial phase, plane q
             const double l = th > 0.0 ? 1.0 : 0.0;
-            s[pb.q * pb.plane + (long long)(y + 1) * pb.pitch + x] = (P)l;
-            e += th + l * pb.inv_ste;
+            s[pb.q * pb.plane + at] = (P)l;
+            fx_add(e, to_fixed(th + l * pb.inv_ste));
             continue;
         }
-        e += th + phi_of(th, pb.inv_delta) * pb.inv_ste;
+        fx_add(e, to_fixed(th + phi_of(th, pb.inv_delta) * pb.inv_ste));
     }
-    e = warp_sum(e);
-    if ((threadIdx.x & 31) == 0) acc_add(&my_stripe(st)->energy, e);
+    e = block_sum(e);
+    double total;
+    if (last_block_total<&StepStripe::energy>(st, e, total) && threadIdx.x == 0) {
+        st->energy = total;
+        st->energy_prev = total;
+        st->have_energy = 1;
+    }
 }
 
 __global__ void wall_constants_kernel(Problem* probs, int nprob)
@@ -117,17 +169,6 @@ cudaError_t launch_wall_constants(Problem* dprobs, int nprob, cudaStream_t s)
     return cudaGetLastError();
 }
 
-__global__ void finalize_init_kernel(DevStats* st)
-{
-    AccSum esum = {{0ull, 0ull, 0ull, 0ull}};
-    for (int k = 0; k < kStripes; ++k)
-        for (int j = 0; j < 4; ++j) esum.limb[j] += st->cur[k].energy.limb[j];
-    st->energy = acc_read(&esum);
-    st->energy_prev = st->energy;
-    for (int k = 0; k < kStripes; ++k) acc_clear(&st->cur[k].energy);
-    st->have_energy = 1;
-}
-
 template <typename P>
 __global__ void fields_kernel(const Problem* dprob, int parity, double* theta, double* phi, double* H,
                               double* theta_plane)
@@ -135,9 +176,9 @@ __global__ void fields_kernel(const Problem* dprob, int parity, double* theta, d
     const Problem& pb = *dprob;
     const P* s = static_cast<const P*>(pb.state[parity]);
     const double sh = sizeof(P) == 4 ? (double)state_shift(pb, parity) : 0.0;   // FP32: stored less w_i sh
-    const long long n = (long long)pb.nx * pb.ny;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(k % pb.nx), y = (int)(k / pb.nx);
+    const unsigned nx = (unsigned)pb.nx, n = nx * (unsigned)pb.ny;
+    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        const int y = (int)(k / nx), x = (int)(k - (unsigned)y * nx);
         double th = sh;
         for (int i = pb.q - 1; i >= 0; --i) th += (double)s[i * pb.plane + (long long)(y + 1) * pb.pitch + x];
         if (pb.method == 1) {
@@ -234,7 +275,8 @@ cudaError_t launch_front(int precision, const Problem* dprob, const Problem& hp,
     return cudaGetLastError();
 }
 
-static int grid_for(long long n) { return (int)((n + 255) / 256 < 152 * 16 ? (n + 255) / 256 : 152 * 16); }
+// 256-thread blocks, at most eight per SM (every block adds to the last one's total)
+static int grid_for(long long n) { return (int)((n + 255) / 256 < 152 * 8 ? (n + 255) / 256 : 152 * 8); }
 
 cudaError_t launch_init_state(int precision, const Problem* dprob, const Problem& hp, const double* theta0,
                               int parity, DevStats* st, cudaStream_t s)
@@ -242,18 +284,12 @@ cudaError_t launch_init_state(int precision, const Problem* dprob, const Problem
     const int g = grid_for((long long)hp.nx * hp.ny);
     // FP32 D2Q9 / D2Q5 states carry a shift (FP64 and D1Q3 tails stay zero)
     if (precision == 1 && hp.q != 3) {
-        shift_kernel<<<1, 1024, 0, s>>>(dprob, theta0);
+        shift_kernel<<<g, 256, 0, s>>>(dprob, theta0, st);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     if (precision == 1) init_state_kernel<float><<<g, 256, 0, s>>>(dprob, theta0, parity, st);
     else init_state_kernel<double><<<g, 256, 0, s>>>(dprob, theta0, parity, st);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_finalize_init(DevStats* st, cudaStream_t s)
-{
-    finalize_init_kernel<<<1, 1, 0, s>>>(st);
     return cudaGetLastError();
 }
 

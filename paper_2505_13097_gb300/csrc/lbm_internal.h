@@ -47,6 +47,7 @@ struct DevStats {
     StepStripe cur[kStripes];
     int cur_maxit;                 // largest Newton iteration count
     int error;                     // sticky: lbm_status of a device-detected failure
+    unsigned int ticket;           // last block of the initial-state kernels; zero between launches
     double energy, energy_prev, flux, imbalance, imbalance_max;
     long long steps;
     long long newton_nodes;
@@ -266,7 +267,6 @@ cudaError_t launch_front(int precision, const Problem* dprob, const Problem& hp,
                          cudaStream_t s);
 cudaError_t launch_fields(int precision, const Problem* dprob, const Problem& hp, int parity, double* theta,
                           double* phi, double* H, double* theta_plane, cudaStream_t s);
-cudaError_t launch_finalize_init(DevStats* st, cudaStream_t s);
 // tanh(theta_wall/delta) and phi(theta_wall) of every wall, for nprob problems
 cudaError_t launch_wall_constants(Problem* dprobs, int nprob, cudaStream_t s);
 

@@ -753,7 +753,6 @@ extern "C" lbm_status lbm_stefan_set_ic(lbm_stefan* h, const double* theta0, int
     }
     CUDA_TRY(cudaMemsetAsync(h->dstats, 0, sizeof(DevStats), h->stream));
     CUDA_TRY(lbm::launch_init_state(h->precision, h->dprob, h->hp, src, 0, h->dstats, h->stream));
-    CUDA_TRY(lbm::launch_finalize_init(h->dstats, h->stream));
     if (!on_device) CUDA_TRY(cudaStreamSynchronize(h->stream));
     h->parity = 0;
     h->ic = true;
@@ -1540,7 +1539,6 @@ extern "C" lbm_status lbm_stefan_batch_set_ic(lbm_stefan_batch* b, int k, const 
     }
     CUDA_TRY(cudaMemsetAsync(b->dstats + k, 0, sizeof(DevStats), b->stream));
     CUDA_TRY(lbm::launch_init_state(b->precision, b->dprobs + k, hp, src, 0, b->dstats + k, b->stream));
-    CUDA_TRY(lbm::launch_finalize_init(b->dstats + k, b->stream));
     if (!on_device) CUDA_TRY(cudaStreamSynchronize(b->stream));
     return LBM_OK;
 }
@@ -1602,10 +1600,10 @@ extern "C" lbm_status lbm_stefan_batch_get_fields(lbm_stefan_batch* b, int k, do
     double* dst = on_device ? theta : b->dscratch;
     CUDA_TRY(lbm::launch_fields(b->precision, b->dprobs + k, hp, b->parity, dst, nullptr, nullptr, nullptr, b->stream));
     if (!on_device) CUDA_TRY(cudaMemcpyAsync(theta, b->dscratch, n * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
+    int err = 0;
+    CUDA_TRY(cudaMemcpyAsync(&err, &b->dstats[k].error, sizeof err, cudaMemcpyDeviceToHost, b->stream));
     CUDA_TRY(cudaStreamSynchronize(b->stream));
-    DevStats st;
-    CUDA_TRY(cudaMemcpy(&st, b->dstats + k, sizeof st, cudaMemcpyDeviceToHost));
-    if (st.error) return fail((lbm_status)st.error, "device reported error %d in problem %d", st.error, k);
+    if (err) return fail((lbm_status)err, "device reported error %d in problem %d", err, k);
     return LBM_OK;
 }
 
