@@ -1,6 +1,6 @@
 // ILFBM step (Algorithm 1, the implicit liquid fraction based method of
 // Sec. 3.3), the paper's second comparison scheme, in FP64: D1Q3 in one
-// block (below), D2Q9 and D2Q5 with one launch per inner iteration (at the end).
+// block (below), D2Q9 and D2Q5 in one cooperative launch (at the end).
 //
 // State: f_i (planes 0..q-1, theta = M0(f)) and the liquid fraction l (plane
 // q of the same buffer).  One step:
@@ -26,7 +26,7 @@
 // f^(k) are streamed once, after the loop), and the loop's test is one flag
 // per iteration behind a single barrier (three flags in rotation: the one
 // cleared for the next iteration was last read two iterations earlier).
-#include "lbm_device.cuh"
+#include "resident.cuh"
 
 namespace lbm {
 
@@ -205,35 +205,32 @@ __global__ void __launch_bounds__(kIlfThreads) ilfbm_d1q3_kernel(StepArgs a, int
 
 // ---------------------------------------------------------------- 2D lattices
 // ILFBM on D2Q9 and D2Q5 (Q = 9 or 5; the D2Q5 velocities are D2Q9's first
-// five), FP64.  The inner loop needs a lattice-wide barrier per iteration, so
-// an iteration is one launch; a step is
-//   ilf2_collide   Omega0_i = f_i - (f_i - w_i theta)/tau in place, l^(0) = l
-//   ilf2_s0        S0(y) = sum_i Omega0_i(y - e_i) at the interior nodes
-//   ilf2_iter x maxit
-//                  l^(k)(y) = l(H^(k)(y)), H^(k) = S0(y) + sum_i (w_i/Ste)
-//                  (l - l^(k-1))(y - e_i) + l^(k-1)(y)/Ste at interior nodes, the
-//                  closed streamed populations at wall nodes; a "changed" flag
-//                  per iteration (three in rotation: launch k reads k-1's,
-//                  sets its own and clears k+1's, last read by launch k-1); the
-//                  first launch that finds the previous iteration unchanged
-//                  records it and every later launch returns at once
-//   ilf2_final     f~_i(y) = Omega_i(y - e_i) with the source of l^(K-1) and
-//                  the closures, l~ = l^(K); energy sum theta~ + l~/Ste, flux,
-//                  iteration count, the iteration-limit error; publishes
-// Scratch (nx*ny doubles each): S0, l^(k) x 2, l - l^(k) x 2 (the interior
-// stencil reads the differences, so an iteration spends one FMA per velocity).
-// Node indices stay below 2^31 (the library's size limit), so the column and
-// row come from a 32-bit division.
-struct Ilf2Args {
-    Problem pb;              // by value: the kernels read it from the parameter bank,
-                             // so no store of theirs can alias it
-    int parity;              // state[parity] holds f, then Omega0; f~ goes to state[parity ^ 1]
+// five), FP64, all steps of a call in one cooperative launch.  A step is
+//   first      S0(y) = sum_i Omega0_i(y - e_i), Omega0 the source-free collision, and the
+//              first iterate l^(1)(y) = l(S0 + l/Ste) (its source vanishes)
+//   iterations l^(k)(y) = l(H^(k)(y)), H^(k) = S0(y) + sum_i (w_i/Ste)
+//              (l - l^(k-1))(y - e_i) + l^(k-1)(y)/Ste at interior nodes, the
+//              closed streamed populations at wall nodes, until no l moves by
+//              more than tol
+//   last       f~_i(y) = Omega_i(y - e_i) with the source of l^(K-1) and the
+//              closures, l~ = l^(K); collided in place for the next step
+// with a grid barrier after each.  What bounds it is the chain of some 80
+// barriers per step.  An iterate is a function of l^(k-1) at the node and its
+// neighbours, so it repeats bit for bit where they did not change: only units
+// (32 columns of one row) next to a change are evaluated, the mushy nodes and
+// their surroundings, and the two buffers of l agree everywhere else.  One
+// launch per iteration over all nodes took 2,550 us per step on the 401^2
+// cavity (400 launches, 77 of them with work).
+// Scratch (nx*ny doubles each): S0, l^(k) x 2, l - l^(k) x 2 (the stencil reads
+// the differences, so an iteration spends one FMA per velocity), and a byte per
+// unit for each of three iterations (changed).
+struct Ilf2Args : ResidentCommon {
+    Problem pb;              // by value
+    int parity;
     double* s0;
-    double* lb[2];           // l^(k-1) / l^(k) of iteration k: lb[(k-1) & 1] / lb[k & 1]
-    double* dl[2];           // l - l^(k-1) / l - l^(k), written beside lb: the stencil's input
-    unsigned int* flags;     // [0] done, [1] converged iteration, [2..4] changed per iteration mod 3
-    DevStats* stats;
-    unsigned int* ticket;
+    double* lb[2];           // l^(k) in lb[(base + k) & 1]
+    double* dl[2];           // l - l^(k), likewise
+    unsigned char* chg[3];   // unit changed in iteration k: chg[k % 3]
 };
 
 template <int Q>
@@ -307,174 +304,315 @@ __device__ __forceinline__ double ilf2_streamed(const Problem& pb, const double*
     return in - out;
 }
 
-template <int Q>
-__global__ void __launch_bounds__(256) ilf2_collide(Ilf2Args a)
+// One thread: its block's arrival at the inner barrier number `turn`, `more` if
+// the block moved some l by more than tol, and the wait for the others; any:
+// whether some block did (seen: what this barrier's high bits held after its
+// previous turn).  false: a wait ran out.  Two barriers alternate, so nobody
+// arrives at one again before everybody has read it.
+__device__ __forceinline__ bool inner_barrier(const Ilf2Args& a, unsigned turn, unsigned nb, bool more, unsigned& seen, bool& any)
 {
-    const Problem& pb = a.pb;
-    double* st = static_cast<double*>(pb.state[a.parity]);
-    const long long n = (long long)pb.nx * pb.ny;
-    if (blockIdx.x == 0 && threadIdx.x < 5) a.flags[threadIdx.x] = 0u;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)((unsigned)k % (unsigned)pb.nx), y = (int)((unsigned)k / (unsigned)pb.nx);
-        const long long at = (long long)(y + 1) * pb.pitch + x;
-        double f[Q], th = 0.0;
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            f[i] = st[i * pb.plane + at];
-            th += f[i];
+    unsigned long long* c = &a.bar->inner[turn & 1u];
+    const unsigned long long target = (turn / 2ull + 1ull) * nb;
+    fence_gpu();
+    atomicAdd(c, 1ull | (more ? 1ull << 48 : 0ull));
+    unsigned long long v, t0 = 0;
+    for (unsigned i = 0;; ++i) {
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(c) : "memory");
+        if ((v & 0xffffffffffffull) >= target) break;
+        if ((i & 63u) == 63u) {
+            if (ld_acquire(&a.bar->abort)) return false;
+            if (t0 == 0) t0 = global_ns();
+            else if ((long long)(global_ns() - t0) > a.wait_ns) {
+                atomicExch(&a.bar->abort, 1u);
+                return false;
+            }
         }
-#pragma unroll
-        for (int i = 0; i < Q; ++i) st[i * pb.plane + at] = f[i] - (f[i] - lat_w(Q, i) * th) * pb.omega;
-        a.lb[0][k] = st[Q * pb.plane + at];
-        a.dl[0][k] = 0.0;   // l - l^(0)
     }
+    fence_gpu();
+    any = (unsigned)(v >> 48) != seen;   // (modulo 2^16; a turn adds at most one per block)
+    seen = (unsigned)(v >> 48);
+    return true;
 }
 
-template <int Q>
-__global__ void __launch_bounds__(256) ilf2_s0(Ilf2Args a)
-{
-    const Problem& pb = a.pb;
-    const double* st = static_cast<const double*>(pb.state[a.parity]);
-    const long long n = (long long)pb.nx * pb.ny;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)((unsigned)k % (unsigned)pb.nx), y = (int)((unsigned)k / (unsigned)pb.nx);
-        if (x == 0 || x == pb.nx - 1 || y == 0 || y == pb.ny - 1) continue;
-        double s = 0.0;
-#pragma unroll
-        for (int i = 0; i < Q; ++i)
-            s += st[i * pb.plane + (long long)(y - d2_ey(i) + 1) * pb.pitch + x - d2_ex(i)];
-        a.s0[k] = s;
-    }
-}
+constexpr int kIlf2Threads = 512;
+constexpr int kIlf2Steps = 256;   // steps of one launch
 
 template <int Q>
-__global__ void __launch_bounds__(256) ilf2_iter(Ilf2Args a, int k)
+__global__ void __launch_bounds__(kIlf2Threads, 1) ilf2_kernel(const __grid_constant__ Ilf2Args a)
 {
-    volatile unsigned int* fl = a.flags;
-    if (fl[0]) return;   // converged in an earlier iteration
-    if (k > 1 && fl[2 + (k - 1) % 3] == 0u) {
-        // iteration k - 1 changed nothing: it is the last one
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            fl[1] = (unsigned)(k - 1);
-            fl[0] = 1u;
-        }
+    __shared__ ResidentSlot wsum[2][kIlf2Threads / 32];   // by step parity
+    __shared__ bool ok_s, any_s;
+    const Problem& pb = a.pb;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int nwb = kIlf2Threads / 32;
+    const int nb = gridDim.x - 1;   // computing blocks; the last block adds up the statistics
+    if ((int)blockIdx.x == nb) {
+        resident_stats(a, pb, (unsigned)nb);
+        bar_leave(a.bar);
         return;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) fl[2 + (k + 1) % 3] = 0u;
-    const Problem& pb = a.pb;
-    const double* st = static_cast<const double*>(pb.state[a.parity]);
-    const double* lq = st + Q * pb.plane;
-    const double* lp = a.lb[(k - 1) & 1];
-    const double* dp = a.dl[(k - 1) & 1];
-    double* ln = a.lb[k & 1];
-    double* dn = a.dl[k & 1];
-    const long long n = (long long)pb.nx * pb.ny;
-    bool more = false;
-    for (long long nd = blockIdx.x * (long long)blockDim.x + threadIdx.x; nd < n; nd += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)((unsigned)nd % (unsigned)pb.nx), y = (int)((unsigned)nd / (unsigned)pb.nx);
-        const int wk = ilf2_dirichlet(pb, x, y);
-        double lk;
-        if (wk >= 0) {
-            lk = pb.wall_theta[wk] > 0.0 ? 1.0 : 0.0;
-        } else {
-            double H;
-            if (x > 0 && x < pb.nx - 1 && y > 0 && y < pb.ny - 1) {
-                H = a.s0[nd];
+    const int nx = pb.nx, ny = pb.ny;
+    const int nseg = (nx + 31) / 32, units = nseg * ny;
+    const int W = nb * nwb, w0 = warp * nb + (int)blockIdx.x;   // units w0, w0 + W, ...: neighbours on other SMs
+    const double om = pb.omega, inv_ste = pb.inv_ste;
+    unsigned turn = 0, seen[2] = {0u, 0u};
+    bool ok = true;
+    // every thread: the inner barrier; false: a wait ran out
+    auto barrier = [&](bool more, bool& any) -> bool {
+        const int m = __syncthreads_or(more ? 1 : 0);
+        if (threadIdx.x == 0) {
+            bool some = false;
+            ok_s = inner_barrier(a, turn, (unsigned)nb, m != 0, seen[turn & 1u], some);
+            any_s = some;
+        }
+        ++turn;
+        __syncthreads();
+        any = any_s;
+        return ok_s;
+    };
+    if (threadIdx.x < 2 * nwb) wsum[threadIdx.x / nwb][threadIdx.x % nwb] = ResidentSlot{};
+    // the launch's first step: collide its state in place, l^(0) = l
+    {
+        double* st = static_cast<double*>(pb.state[a.parity]);
+        for (int u = w0; u < units; u += W) {
+            const int y = u / nseg, x = (u - y * nseg) * 32 + lane;
+            if (x >= nx) continue;
+            const long long at = (long long)(y + 1) * pb.pitch + x;
+            double f[Q], th = 0.0;
 #pragma unroll
-                for (int i = 0; i < Q; ++i) {
-                    const long long sn = (long long)(y - d2_ey(i)) * pb.nx + x - d2_ex(i);
-                    H += lat_w(Q, i) * pb.inv_ste * dp[sn];
-                }
-            } else {
-                double q[Q];
-                (void)ilf2_streamed<Q>(pb, st, lp, x, y, q, false);
-                H = 0.0;
-#pragma unroll
-                for (int i = 0; i < Q; ++i) H += q[i];
+            for (int i = 0; i < Q; ++i) {
+                f[i] = st[i * pb.plane + at];
+                th += f[i];
             }
-            H += lp[nd] * pb.inv_ste;
-            lk = ilf_lever(H, pb.ste, pb.inv_ste);
-        }
-        more |= fabs(lk - lp[nd]) > pb.tol;
-        ln[nd] = lk;
-        dn[nd] = lq[(long long)(y + 1) * pb.pitch + x] - lk;
-    }
-    if (__any_sync(kFull, more) && (threadIdx.x & 31) == 0) fl[2 + k % 3] = 1u;
-}
-
-template <int Q>
-__global__ void __launch_bounds__(256) ilf2_final(Ilf2Args a, int maxit)
-{
-    const Problem& pb = a.pb;
-    const volatile unsigned int* fl = a.flags;
-    const bool done = fl[0] != 0u;
-    const int K = done ? (int)fl[1] : maxit;
-    const bool conv = done || fl[2 + maxit % 3] == 0u;
-    const double* st = static_cast<const double*>(pb.state[a.parity]);
-    double* dst = static_cast<double*>(pb.state[a.parity ^ 1]);
-    const double* lp = a.lb[(K - 1) & 1];
-    const double* ln = a.lb[K & 1];
-    DevStats* sts = &a.stats[pb.stats];
-    const long long n = (long long)pb.nx * pb.ny;
-    double e = 0.0, fx = 0.0;
-    for (long long nd = blockIdx.x * (long long)blockDim.x + threadIdx.x; nd < n; nd += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)((unsigned)nd % (unsigned)pb.nx), y = (int)((unsigned)nd / (unsigned)pb.nx);
-        double q[Q];
-        fx += ilf2_streamed<Q>(pb, st, lp, x, y, q, true);
-        const long long at = (long long)(y + 1) * pb.pitch + x;
-        double th = 0.0;
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            dst[i * pb.plane + at] = q[i];
-            th += q[i];
+            for (int i = 0; i < Q; ++i) st[i * pb.plane + at] = f[i] - (f[i] - lat_w(Q, i) * th) * om;
+            a.lb[0][(long long)y * nx + x] = st[Q * pb.plane + at];
         }
-        dst[Q * pb.plane + at] = ln[nd];
-        e += th + ln[nd] * pb.inv_ste;
+        bool any;
+        ok = barrier(false, any);
     }
-    e = warp_sum(e);
-    fx = warp_sum(fx);
-    if ((threadIdx.x & 31) == 0) {
-        acc_add(&my_stripe(sts)->energy, e);
-        acc_add(&my_stripe(sts)->flux, fx);
+    int base = 0;
+    for (int s = 0; ok && s < a.nsteps; ++s) {
+        const int p = (a.parity + s) & 1;
+        const double* st = static_cast<const double*>(pb.state[p]);
+        double* dst = static_cast<double*>(pb.state[p ^ 1]);
+        const double* lq = st + Q * pb.plane;
+        // first iterate: l - l^(0) = 0
+        bool more = false, any = true;
+        for (int u = w0; u < units; u += W) {
+            const int y = u / nseg, x = (u - y * nseg) * 32 + lane;
+            bool changed = false;
+            if (x < nx) {
+                const long long nd = (long long)y * nx + x;
+                const double lp = a.lb[base][nd];
+                const int wk = ilf2_dirichlet(pb, x, y);
+                double lk;
+                if (wk >= 0) {
+                    lk = pb.wall_theta[wk] > 0.0 ? 1.0 : 0.0;
+                } else {
+                    double H;
+                    if (x > 0 && x < nx - 1 && y > 0 && y < ny - 1) {
+                        H = 0.0;
+#pragma unroll
+                        for (int i = 0; i < Q; ++i)
+                            H += st[i * pb.plane + (long long)(y - d2_ey(i) + 1) * pb.pitch + x - d2_ex(i)];
+                        a.s0[nd] = H;
+                    } else {
+                        double q[Q];
+                        (void)ilf2_streamed<Q>(pb, st, a.lb[base], x, y, q, false);
+                        H = 0.0;
+#pragma unroll
+                        for (int i = 0; i < Q; ++i) H += q[i];
+                    }
+                    H += lp * inv_ste;
+                    lk = ilf_lever(H, pb.ste, inv_ste);
+                }
+                more |= fabs(lk - lp) > pb.tol;
+                changed = lk != lp;
+                a.lb[base ^ 1][nd] = lk;
+                a.dl[base][nd] = 0.0;
+                a.dl[base ^ 1][nd] = lq[(long long)(y + 1) * pb.pitch + x] - lk;
+            }
+            const bool c = __any_sync(kFull, changed);
+            if (lane == 0) {
+                a.chg[1][u] = c;
+                a.chg[2][u] = 0;
+            }
+        }
+        ok = barrier(more, any);
+        int k = 1;
+        while (ok && any && k < pb.maxit) {
+            ++k;
+            const double* lp = a.lb[(base + k - 1) & 1];
+            const double* dp = a.dl[(base + k - 1) & 1];
+            double* ln = a.lb[(base + k) & 1];
+            double* dn = a.dl[(base + k) & 1];
+            const unsigned char* prev = a.chg[(k - 1) % 3];
+            unsigned char* cur = a.chg[k % 3];
+            unsigned char* next = a.chg[(k + 1) % 3];
+            more = false;
+            for (int u0 = w0; u0 < units; u0 += 32 * W) {
+                // a lane per unit: is it next to a change of iteration k - 1?
+                const long long ul = (long long)u0 + (long long)lane * W;
+                bool active = false;
+                if (ul < units) {
+                    const int u = (int)ul, y = u / nseg, sg = u - y * nseg;
+                    unsigned f = 0;
+#pragma unroll
+                    for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
+                        for (int dx = -1; dx <= 1; ++dx)
+                            if (y + dy >= 0 && y + dy < ny && sg + dx >= 0 && sg + dx < nseg) f |= prev[u + dy * nseg + dx];
+                    active = f != 0u;
+                    next[u] = 0;
+                }
+                unsigned todo = __ballot_sync(kFull, active);
+                while (todo) {
+                    const int l = __ffs(todo) - 1;
+                    todo &= todo - 1;
+                    const int u = u0 + l * W, y = u / nseg, x = (u - y * nseg) * 32 + lane;
+                    bool changed = false;
+                    if (x < nx) {
+                        const long long nd = (long long)y * nx + x;
+                        const double l0 = lp[nd];
+                        const int wk = ilf2_dirichlet(pb, x, y);
+                        if (wk < 0) {
+                            double H;
+                            if (x > 0 && x < nx - 1 && y > 0 && y < ny - 1) {
+                                H = a.s0[nd];
+#pragma unroll
+                                for (int i = 0; i < Q; ++i)
+                                    H += lat_w(Q, i) * inv_ste * dp[nd - (long long)d2_ey(i) * nx - d2_ex(i)];
+                            } else {
+                                double q[Q];
+                                (void)ilf2_streamed<Q>(pb, st, lp, x, y, q, false);
+                                H = 0.0;
+#pragma unroll
+                                for (int i = 0; i < Q; ++i) H += q[i];
+                            }
+                            H += l0 * inv_ste;
+                            const double lk = ilf_lever(H, pb.ste, inv_ste);
+                            more |= fabs(lk - l0) > pb.tol;
+                            changed = lk != l0;
+                            ln[nd] = lk;
+                            dn[nd] = lq[(long long)(y + 1) * pb.pitch + x] - lk;
+                        } else {   // its wall's phase since the first iterate
+                            ln[nd] = l0;
+                            dn[nd] = dp[nd];
+                        }
+                    }
+                    if (__any_sync(kFull, changed) && lane == 0) cur[u] = 1;
+                }
+            }
+            ok = barrier(more, any);
+        }
+        if (!ok) break;
+        // f~ with the source of l^(k-1), l~ = l^(k); collided for the launch's next step
+        const double* lp = a.lb[(base + k - 1) & 1];
+        const double* dp = a.dl[(base + k - 1) & 1];
+        const double* ln = a.lb[(base + k) & 1];
+        const bool last = s + 1 == a.nsteps;
+        Fx e{0, 0ull}, fx{0, 0ull};
+        for (int u = w0; u < units; u += W) {
+            const int y = u / nseg, x = (u - y * nseg) * 32 + lane;
+            if (x >= nx) continue;
+            const long long nd = (long long)y * nx + x, at = (long long)(y + 1) * pb.pitch + x;
+            double q[Q];
+            if (x > 0 && x < nx - 1 && y > 0 && y < ny - 1) {
+#pragma unroll
+                for (int i = 0; i < Q; ++i)
+                    q[i] = st[i * pb.plane + at - (long long)d2_ey(i) * pb.pitch - d2_ex(i)] +
+                           lat_w(Q, i) * inv_ste * dp[nd - (long long)d2_ey(i) * nx - d2_ex(i)];
+            } else {
+                fx_add(fx, to_fixed(ilf2_streamed<Q>(pb, st, lp, x, y, q, true)));
+            }
+            double th = 0.0;
+#pragma unroll
+            for (int i = 0; i < Q; ++i) th += q[i];
+#pragma unroll
+            for (int i = 0; i < Q; ++i)
+                dst[i * pb.plane + at] = last ? q[i] : q[i] - (q[i] - lat_w(Q, i) * th) * om;
+            const double l = ln[nd];
+            dst[Q * pb.plane + at] = l;
+            fx_add(e, to_fixed(th + l * inv_ste));
+        }
+        e = fx_tree(e);
+        fx = fx_tree(fx);
+        if (lane == 0) {
+            ResidentSlot* w = &wsum[s & 1][warp];
+            w->e = e;
+            w->f = fx;
+            w->maxit = k;   // inner iterations of the step
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            if (any && blockIdx.x == 0) atomicOr(&a.stats->error, 3);   // LBM_ERR_NEWTON: the inner loop reached its limit
+            bar_arrive(&a.bar->count);
+            ok_s = last || bar_wait(a.bar, &a.bar->count, (unsigned)(s + 1) * nb, a.wait_ns);
+        } else if (warp == 1) {
+            resident_emit(a, s, nb, lane, nwb, wsum[s & 1]);   // while thread 0 waits
+        }
+        __syncthreads();
+        ok = ok_s;
+        base = (base + k) & 1;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        atomicMax(&sts->cur_maxit, K);
-        if (!conv) atomicOr(&sts->error, 3);   // LBM_ERR_NEWTON: the inner loop reached its limit
-    }
-    finish_launch(a.stats, 1, a.ticket);
+    if (threadIdx.x == 0) bar_arrive(&a.bar->count);   // the last step's sums are out
+    bar_leave(a.bar);
 }
 
-template <int Q>
-static cudaError_t ilf2_step(const Ilf2Args& a, int maxit, int grid, cudaStream_t s)
+static size_t ilf2_units(int nx, int ny) { return (size_t)((nx + 31) / 32) * ny; }
+// nx*ny doubles x 5, then three bytes per unit
+size_t ilfbm_2d_scratch(int nx, int ny) { return sizeof(double) * 5 * (size_t)nx * ny + 3 * ilf2_units(nx, ny); }
+
+int ilfbm_2d_blocks(int q, int nx, int ny)
 {
-    ilf2_collide<Q><<<grid, 256, 0, s>>>(a);
-    ilf2_s0<Q><<<grid, 256, 0, s>>>(a);
-    for (int k = 1; k <= maxit; ++k) ilf2_iter<Q><<<grid, 256, 0, s>>>(a, k);
-    ilf2_final<Q><<<grid, 256, 0, s>>>(a, maxit);
-    return cudaGetLastError();
+    int dev = 0, sms = 0, per = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        (q == 9 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, ilf2_kernel<9>, kIlf2Threads, 0)
+                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, ilf2_kernel<5>, kIlf2Threads, 0)) != cudaSuccess)
+        return 0;
+    const long long want = ((long long)ilf2_units(nx, ny) + kIlf2Threads / 32 - 1) / (kIlf2Threads / 32) + 1;
+    return (int)(want < (long long)sms * per ? want : (long long)sms * per);
 }
 
-cudaError_t launch_ilfbm_2d(const Problem& hp, int parity, double* scratch,
-                            unsigned int* flags, DevStats* stats, unsigned int* ticket, cudaStream_t s)
+cudaError_t launch_ilfbm_2d(const Problem& hp, int parity, int nsteps, void* scratch, DevStats* stats, void* slots,
+                            ResidentBar* bar, long long wait_ns, cudaStream_t s)
 {
+    const int blocks = ilfbm_2d_blocks(hp.q, hp.nx, hp.ny);
+    if (blocks < 2) return cudaErrorCooperativeLaunchTooLarge;
     Ilf2Args a;
+    const size_t n = (size_t)hp.nx * hp.ny, units = ilf2_units(hp.nx, hp.ny);
+    double* d = static_cast<double*>(scratch);
     a.pb = hp;
-    a.parity = parity;
-    const long long n = (long long)hp.nx * hp.ny;
-    a.s0 = scratch;
-    a.lb[0] = scratch + n;
-    a.lb[1] = scratch + 2 * n;
-    a.dl[0] = scratch + 3 * n;
-    a.dl[1] = scratch + 4 * n;
-    a.flags = flags;
     a.stats = stats;
-    a.ticket = ticket;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long want = (n + 255) / 256;
-    const int grid = (int)(want < (long long)sms * 8 ? want : (long long)sms * 8);
-    return hp.q == 9 ? ilf2_step<9>(a, hp.maxit, grid, s) : ilf2_step<5>(a, hp.maxit, grid, s);
+    a.slots = static_cast<ResidentSlot*>(slots);
+    a.bar = bar;
+    a.wait_ns = wait_ns;
+    a.s0 = d;
+    a.lb[0] = d + n;
+    a.lb[1] = d + 2 * n;
+    a.dl[0] = d + 3 * n;
+    a.dl[1] = d + 4 * n;
+    for (int k = 0; k < 3; ++k) a.chg[k] = reinterpret_cast<unsigned char*>(d + 5 * n) + k * units;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kIlf2Threads);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;   // every block resident: they wait on one another
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    while (nsteps > 0) {
+        a.parity = parity;
+        a.nsteps = nsteps < kIlf2Steps ? nsteps : kIlf2Steps;
+        const cudaError_t e = hp.q == 9 ? cudaLaunchKernelEx(&cfg, ilf2_kernel<9>, a) : cudaLaunchKernelEx(&cfg, ilf2_kernel<5>, a);
+        if (e != cudaSuccess) return e;
+        parity ^= a.nsteps & 1;
+        nsteps -= a.nsteps;
+    }
+    return cudaSuccess;
 }
 
 static size_t ilfbm_smem(int nx) { return (size_t)9 * nx * sizeof(double); }

@@ -154,6 +154,9 @@ struct ResidentBar {
     unsigned int count, pad0[31];          // arrivals of the computing blocks since the launch
     unsigned int abort, done, pad1[30];    // a wait ran out; blocks that have left
     unsigned int read[kResidentRing];      // per set: times the statistics block has read it
+    // 2D ILFBM: inner iterations, two barriers in turn (arrivals in the low 48 bits, blocks
+    // with a change above the tolerance in the high 16)
+    unsigned long long inner[2];
 };
 // How a resident launch covers a lattice; blocks == 0: it does not.
 struct ResidentPlan {
@@ -255,10 +258,13 @@ bool d1q3_fused_fits(int precision, int nx);
 // ILFBM (Algorithm 1) on D1Q3, FP64, one block over the whole lattice (ilfbm.cu)
 cudaError_t launch_ilfbm_d1q3(const StepArgs& a, const Problem& hp, int nsteps, cudaStream_t s);
 bool ilfbm_d1q3_fits(int nx);
-// one ILFBM step on D2Q9 / D2Q5 (hp.q), FP64: scratch holds 5 nx*ny doubles,
-// flags 5 unsigned ints; publishes the step statistics (hp: the host copy, passed by value)
-cudaError_t launch_ilfbm_2d(const Problem& hp, int parity, double* scratch,
-                            unsigned int* flags, DevStats* stats, unsigned int* ticket, cudaStream_t s);
+// nsteps ILFBM steps on D2Q9 / D2Q5 (hp.q), FP64, in one cooperative launch; scratch:
+// ilfbm_2d_scratch bytes, slots and bar as for launch_resident (ilfbm_2d_blocks - 1 slots
+// per set); hp: the host copy, passed by value
+size_t ilfbm_2d_scratch(int nx, int ny);
+int ilfbm_2d_blocks(int q, int nx, int ny);
+cudaError_t launch_ilfbm_2d(const Problem& hp, int parity, int nsteps, void* scratch, DevStats* stats, void* slots,
+                            ResidentBar* bar, long long wait_ns, cudaStream_t s);
 
 // Field and state kernels (fields.cu)
 cudaError_t launch_init_state(int precision, const Problem* dprob, const Problem& hp, const double* theta0,

@@ -84,8 +84,8 @@ struct lbm_stefan {
     int parity = 0;
     bool ic = false;
     int adj_tile_h = lbm::kAdjTileH;   // rows per warp tile of the D2Q9 adjoint
-    unsigned int* dilf = nullptr;      // 2D ILFBM: inner-loop flags (done, iteration, changed x 3)
-    double* dilf_scratch = nullptr;    // 2D ILFBM: S0, two l iterates, two l differences (5 nx*ny)
+    void* dilf = nullptr;              // 2D ILFBM: S0, two l iterates, two l differences, changed units
+    void* dilf_slots = nullptr;        // 2D ILFBM: the steps' sums
     bool flat = false;                 // FP32 D2Q9: the flat and wall kernels
     bool use_tma = false;              // FP32 D2Q9: the TMA row-pipeline kernel (for the wait test hook)
     lbm::TmaMaps tma;
@@ -730,9 +730,15 @@ extern "C" lbm_status lbm_stefan_set_method(lbm_stefan* h, int method)
                 h->state_bytes = need;
                 h->hp.tail_off = (long long)(need - kStateTail);
             }
-            if (!h->dilf) CUDA_TRY(cudaMalloc(&h->dilf, 8 * sizeof(unsigned int)));
-            if (!h->dilf_scratch)
-                CUDA_TRY(cudaMalloc(&h->dilf_scratch, 5 * sizeof(double) * (size_t)h->hp.nx * h->hp.ny));
+            if (!h->dilf) {
+                const size_t slots = (size_t)lbm::kResidentRing * std::max(1, lbm::ilfbm_2d_blocks(h->hp.q, h->hp.nx, h->hp.ny));
+                CUDA_TRY(cudaMalloc(&h->dilf, lbm::ilfbm_2d_scratch(h->hp.nx, h->hp.ny)));
+                if (!h->dilf_slots) CUDA_TRY(cudaMalloc(&h->dilf_slots, slots * lbm::resident_slot_bytes()));
+                if (!h->dbar) {
+                    CUDA_TRY(cudaMalloc(&h->dbar, sizeof(lbm::ResidentBar)));
+                    CUDA_TRY(cudaMemset(h->dbar, 0, sizeof(lbm::ResidentBar)));
+                }
+            }
         }
     }
     h->hp.method = method;
@@ -795,14 +801,10 @@ extern "C" lbm_status lbm_stefan_step(lbm_stefan* h, int nsteps)
         return LBM_OK;
     }
     if (h->hp.method == LBM_ILFBM) {
-        // 2D: one launch per inner iteration (newton_max_iter of them, those
-        // after convergence return at once), framed by the collision and the
-        // final streaming
-        for (int k = 0; k < nsteps; ++k) {
-            CUDA_TRY(lbm::launch_ilfbm_2d(h->hp, h->parity, h->dilf_scratch, h->dilf, h->dstats, h->dticket,
-                                          h->stream));
-            h->parity ^= 1;
-        }
+        // 2D: one cooperative launch, a barrier per inner iteration
+        CUDA_TRY(lbm::launch_ilfbm_2d(h->hp, h->parity, nsteps, h->dilf, h->dstats, h->dilf_slots, h->dbar, kResidentWaitNs,
+                                      h->stream));
+        h->parity ^= nsteps & 1;
         return LBM_OK;
     }
     if (h->p.lattice == LBM_D1Q3 && lbm::d1q3_fused_fits(h->precision, h->hp.nx)) {
@@ -1252,7 +1254,7 @@ extern "C" void lbm_stefan_destroy(lbm_stefan* h)
     cudaFree(h->dslots);
     cudaFree(h->dbar);
     cudaFree(h->dilf);
-    cudaFree(h->dilf_scratch);
+    cudaFree(h->dilf_slots);
     delete h;
 }
 
