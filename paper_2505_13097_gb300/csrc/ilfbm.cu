@@ -317,7 +317,7 @@ __device__ __forceinline__ bool inner_barrier(const Ilf2Args& a, unsigned turn, 
     atomicAdd(c, 1ull | (more ? 1ull << 48 : 0ull));
     unsigned long long v, t0 = 0;
     for (unsigned i = 0;; ++i) {
-        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(c) : "memory");
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(c) : "memory");
         if ((v & 0xffffffffffffull) >= target) break;
         if ((i & 63u) == 63u) {
             if (ld_acquire(&a.bar->abort)) return false;

@@ -34,6 +34,12 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p)
     return v;
 }
 
+__device__ __forceinline__ unsigned ld_relaxed(const unsigned* p)
+{
+    unsigned v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
 // One thread: an arrival for its block (the block has synchronized).
@@ -44,14 +50,15 @@ __device__ __forceinline__ void bar_arrive(unsigned* count)
 }
 
 // One thread: waits until *count has reached `target`, for at most limit_ns;
-// false when the wait ran out here or in another block.
+// false when the wait ran out here or in another block.  The polls are relaxed
+// (an acquiring load drops the SM's L1 lines each time); one fence follows.
 __device__ __forceinline__ bool bar_wait(ResidentBar* b, const unsigned* count, unsigned target, long long limit_ns)
 {
     unsigned long long t0 = 0;
     for (unsigned i = 0;; ++i) {
-        if ((int)(ld_acquire(count) - target) >= 0) break;
+        if ((int)(ld_relaxed(count) - target) >= 0) break;
         if ((i & 63u) == 63u) {
-            if (ld_acquire(&b->abort)) return false;
+            if (ld_relaxed(&b->abort)) return false;
             if (t0 == 0) t0 = global_ns();
             else if ((long long)(global_ns() - t0) > limit_ns) {
                 atomicExch(&b->abort, 1u);
