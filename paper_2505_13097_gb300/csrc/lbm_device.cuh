@@ -105,7 +105,10 @@ __device__ __forceinline__ double ff_to_double(const ff& a) { return widen(a.hi)
 // the melting plateau [0, 1/Ste], H - 1/Ste above it.
 __device__ __forceinline__ double eebm_theta(double H, double inv_ste)
 {
-    return H < 0.0 ? H : (H > inv_ste ? H - inv_ste : 0.0);
+    // (sign and order from the bits: an FP64 comparison takes the FP64 pipe)
+    const long long b = __double_as_longlong(H);
+    if (b < 0) return H;
+    return b > __double_as_longlong(inv_ste) ? H - inv_ste : 0.0;
 }
 __device__ __forceinline__ float eebm_theta(float H, float inv_ste)
 {
@@ -613,6 +616,9 @@ __device__ __forceinline__ void acc_clear(Acc128* a)
     va->hi = 0ll;
 }
 
+// a fixed-point value as a double
+__device__ __forceinline__ double fx_value(const Fx& v) { return (double)v.hi * 16.0 + (double)v.lo * 0x1p-60; }
+
 // The per-step sums (AccSum): return-less additions of the four limbs, so a
 // thread never waits for them.
 __device__ __forceinline__ void acc_add_fx(AccSum* a, const Fx& v)
@@ -766,7 +772,7 @@ __device__ __forceinline__ void publish_stats_warp(DevStats* st, const Problem* 
 // Last-block pattern: every block calls this after its warps have added their
 // partial sums; the block that arrives last publishes the statistics of all
 // problems (one thread per problem) and resets the ticket.  No block waits.
-__device__ __forceinline__ void finish_launch(DevStats* stats, int nprob, unsigned int* ticket)
+__device__ __forceinline__ void finish_launch(DevStats* stats, int nprob, unsigned int* ticket, const Problem* probs)
 {
     __shared__ bool last;
     __syncthreads();
@@ -778,7 +784,7 @@ __device__ __forceinline__ void finish_launch(DevStats* stats, int nprob, unsign
     __syncthreads();
     if (last) {
         __threadfence();
-        for (int p = threadIdx.x; p < nprob; p += blockDim.x) publish_stats(&stats[p], nullptr);
+        for (int p = threadIdx.x; p < nprob; p += blockDim.x) publish_stats(&stats[p], &probs[p]);
         __threadfence();
         __syncthreads();
         if (threadIdx.x == 0) *ticket = 0u;

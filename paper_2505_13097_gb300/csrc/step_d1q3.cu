@@ -6,92 +6,108 @@
 //    memory and runs many steps per launch, synchronizing the block between
 //    steps.  A 512-node lattice is far too small to fill the GPU, so the
 //    per-step cost is launch latency unless the steps are fused.
-// Moments are summed in FP64 for both storage precisions (three terms).
+// Moments are summed exactly from both storage precisions (three terms).
 // EEBM (Algorithm 2) runs in the same kernels (method 1 of the problem).
-#include "lbm_device.cuh"
+#include "step_common.cuh"
 
 namespace lbm {
 
 struct NodeOut {
     double theta_new;   // theta' of the node
-    double energy;      // theta' + phi(theta')/Ste
+    Fx energy;          // theta' + phi(theta')/Ste, a saturated liquid node's less 1/Ste
     double flux;        // boundary flux contribution
+    int liquid;         // 1 at a saturated liquid node
     int newton;         // 1 if the Newton iteration ran
     int iters;
     bool fail;
 };
 
 // One node: u = Omega(x) at time t, ql/qr = Omega_1(x-1), Omega_2(x+1) (ignored at walls).
+// One block's SM issues one FP64 warp instruction in 19 cycles (64 for a lone
+// warp), so a saturated node spends four: the moment is summed with integers
+// (sum_q), the test for saturation runs on FP32 sums, w_i c takes one
+// multiplication (2/3 is 4 times 1/6, and so is its rounding) and the energy is
+// fixed point.
 template <typename P>
 __device__ __forceinline__ NodeOut d1q3_node(const Problem& pb, int x, const P (&u)[3], P ql, P qr, P (&o)[3])
 {
     NodeOut r;
     r.flux = 0.0;
+    r.liquid = 0;
     r.newton = 0;
     r.iters = 0;
     r.fail = false;
-    double q[3] = {(double)u[0], (double)ql, (double)qr};
-    const double th = (double)u[0] + (double)u[1] + (double)u[2];
+    auto dbl = [](P v) -> double {
+        if constexpr (sizeof(P) == 4) return widen(v);
+        else return v;
+    };
+    const double ud[3] = {dbl(u[0]), dbl(u[1]), dbl(u[2])};
+    double q[3] = {ud[0], dbl(ql), dbl(qr)};
     bool dir = false;
     double thd = 0.0;
+    int side = 0;
     const bool west = x == 0, east = x == pb.nx - 1;
     if (west || east) {
         // nx >= 2: the west node misses q_1 (e = +1), the east node q_2 (e = -1) (Sec. 4.2)
-        const int side = west ? 0 : 1;
+        side = west ? 0 : 1;
         const int iu = west ? 1 : 2, io = west ? 2 : 1;
-        const double out = (double)u[io];   // Omega leaving through this wall
+        const double out = ud[io];   // Omega leaving through this wall
         if (pb.wall_kind[side] == 1) {
             dir = true;
             thd = pb.wall_theta[side];
             // Eq. (16): the single unknown closes M0(q), with M0(q) from Eq. (14) at theta' = theta_D
             // (EEBM: the wall value's enthalpy, Algorithm 2 keeps H = M0)
-            const double m0t = pb.method == 1 ? pb.wall_H[side]
-                                              : thd + (phi_of(thd, pb.inv_delta) - phi_of(th, pb.inv_delta)) * pb.inv_ste;
+            const double m0t = dir_m0_target_d(ud[0] + ud[1] + ud[2], side, pb);
             q[iu] = (double)(P)(m0t - q[0] - q[io]);
         } else {
             // bounce-back q_iu = q_io (Sec. 4.2.2), or link-wise q_iu = Omega_io at the node
-            q[iu] = pb.bb_mode == 0 ? q[io] : (double)u[io];
+            q[iu] = pb.bb_mode == 0 ? q[io] : out;
         }
         r.flux = q[iu] - out;
     }
-    const double m0 = q[2] + q[1] + q[0];
+    const double m0 = sum_q<3>(q);
+    const double omc = pb.omc, w1 = d1_w(1);
     if (pb.method == 1) {
         // EEBM (Algorithm 2): H = M0(q), theta = Theta(H), relaxation toward
         // w_i theta (i != 0) and H - (1 - w_0) theta (i = 0); the energy is H
-        const double H = m0, t = eebm_theta(H, pb.inv_ste), om = pb.omega, omc = 1.0 - pb.omega;
-        o[0] = (P)(omc * q[0] + om * (H - (1.0 - d1_w(0)) * t));
-        o[1] = (P)(omc * q[1] + om * d1_w(1) * t);
-        o[2] = (P)(omc * q[2] + om * d1_w(2) * t);
+        const double t = eebm_theta(m0, pb.inv_ste), om = pb.omega;
+        o[0] = (P)fma(omc, q[0], om * eebm_rest(m0, t, d1_w(0), 0.0));
+        const double v = (om * w1) * t;
+        o[1] = (P)fma(omc, q[1], v);
+        o[2] = (P)fma(omc, q[2], v);
         r.theta_new = t;
-        r.energy = H;
+        r.energy = to_fixed(m0);
         return r;
     }
-    double tn, phn;
+    const float tf = (approx_float(ud[0]) + approx_float(ud[1])) + approx_float(ud[2]), mf = approx_float(m0);
+    const float thr = (float)kSat * pb.delta_f, marg = 1e-5f * (1.0f + fabsf(tf));
+    const bool liq = tf >= thr + marg && mf >= thr + marg;
+    const bool sat = liq || (tf <= -thr - marg && mf <= -thr - marg);
+    double v;   // w_1 c, c = theta' - (1 - omega) m0
     if (dir) {
-        tn = thd;
-        phn = phi_of(thd, pb.inv_delta);
+        v = w1 * (thd - omc * m0);
+        r.theta_new = thd;
+        r.energy = to_fixed(thd + pb.wall_phi[side] * pb.inv_ste);
+    } else if (sat) {
+        v = (pb.omega * w1) * m0;
+        r.theta_new = m0;
+        r.energy = to_fixed(m0);
+        r.liquid = liq ? 1 : 0;
     } else {
-        const double thr = kSat * pb.delta;
-        if ((th >= thr && m0 >= thr) || (th <= -thr && m0 <= -thr)) {
-            tn = m0;
-            phn = m0 > 0.0 ? 1.0 : 0.0;
-        } else {
-            const Phi pt = phi_parts(th, pb.two_inv_delta);
-            const double pth = pt.value();
-            NewtonOut nr = newton_mixed(m0, th, pt, pb);
-            r.fail = !nr.ok || !isfinite(nr.root);
-            tn = m0 + (pth - nr.phi_root) * pb.inv_ste;
-            phn = nr.phi_root;
-            r.newton = 1;
-            r.iters = nr.iters;
-        }
+        const double th = sum_q<3>(ud);
+        const Phi pt = phi_parts(th, pb.two_inv_delta);
+        const NewtonOut nr = newton_mixed(m0, th, pt, pb);
+        r.fail = !nr.ok || !isfinite(nr.root);
+        const double tn = m0 + (pt.value() - nr.phi_root) * pb.inv_ste;
+        v = w1 * (tn - omc * m0);
+        r.theta_new = tn;
+        r.energy = to_fixed(tn + nr.phi_root * pb.inv_ste);
+        r.newton = 1;
+        r.iters = nr.iters;
     }
-    const double cc = tn - (1.0 - pb.omega) * m0;
-    const double omc = 1.0 - pb.omega;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) o[i] = (P)(omc * q[i] + d1_w(i) * cc);
-    r.theta_new = tn;
-    r.energy = tn + phn * pb.inv_ste;
+    o[0] = (P)fma(omc, q[0], scale2(v, 2));
+    o[1] = (P)fma(omc, q[1], v);
+    o[2] = (P)fma(omc, q[2], v);
     return r;
 }
 
@@ -104,8 +120,8 @@ __global__ void __launch_bounds__(128) d1q3_step_kernel(StepArgs a)
     P* dst = static_cast<P*>(pb.state[a.parity ^ 1]);
     const long long pl = pb.plane, row = pb.pitch;   // row 0 of a plane starts at +pitch
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    double e = 0.0, f = 0.0;
-    int nn = 0, mi = 0;
+    Fx e{0, 0ull}, f{0, 0ull};
+    int nn = 0, mi = 0, nl = 0;
     if (x < pb.nx) {
         P u[3], o[3];
         for (int i = 0; i < 3; ++i) u[i] = src[i * pl + row + x];
@@ -116,105 +132,70 @@ __global__ void __launch_bounds__(128) d1q3_step_kernel(StepArgs a)
         if (a.rec) a.rec[x] = r.theta_new;
         if (r.fail) atomicOr(&st->error, 3);
         e = r.energy;
-        f = r.flux;
+        f = to_fixed(r.flux);
         nn = r.newton;
         mi = r.iters;
+        nl = r.liquid;
     }
-    e = warp_sum(e);
-    f = warp_sum(f);
+    e = fx_tree(e);
+    f = fx_tree(f);
     nn = warp_sum_i(nn);
+    nl = warp_sum_i(nl);
     mi = warp_max_i(mi);
     if ((threadIdx.x & 31) == 0) {
-        acc_add(&my_stripe(st)->energy, e);
-        acc_add(&my_stripe(st)->flux, f);
+        acc_add_fx(&my_stripe(st)->energy, e);
+        acc_add_fx(&my_stripe(st)->flux, f);
         if (nn) atomicAdd(&my_stripe(st)->newton, (unsigned long long)nn);
+        if (nl) atomicAdd(&my_stripe(st)->liquid, (unsigned long long)nl);
         if (mi) atomicMax(&st->cur_maxit, mi);
     }
-    finish_launch(a.stats, 1, a.ticket);
+    finish_launch(a.stats, 1, a.ticket, a.probs);
 }
 
-constexpr int kFusedThreads = 512;
+constexpr int kFusedThreads = 512;               // computing threads
 constexpr int kFusedWarps = kFusedThreads / 32;
 
 // One block keeps the lattice in shared memory and runs `nsteps` steps.  A
-// step ends at a single barrier: the warps' partial sums go to a per-step
-// parity half of a small array, and thread 0 sums them in a fixed warp order
-// (deterministic) after the barrier while the others start the next step; a
-// warp writes that half again only two steps later, after the next barrier,
-// which thread 0 reaches only when it has read it.  Thread 0 keeps the
-// statistics in registers and writes them once at the end.
+// step ends at a single barrier.  The warps' sums go to a per-step parity half
+// of a small array; a warp of its own adds them up and keeps the statistics
+// while the others run the next step (a half is written again two steps later,
+// after a barrier that warp reaches only when it has read it).  What bounds a
+// step is the longest warp's chain: a Newton solve, 58 FP64 instructions of 64
+// cycles and the FP32 stage, about 3.4 us; the saturated warps run beside it.
+// 512 nodes with a front: 15.3 us per step with a library tanh and FP64 sums,
+// 9.3 with the shorter solve alone.
 template <typename P>
-__global__ void __launch_bounds__(kFusedThreads) d1q3_fused_kernel(StepArgs a, int nsteps, double* rec)
+__global__ void __launch_bounds__(kFusedThreads + 32)
+    d1q3_fused_kernel(StepArgs a, const __grid_constant__ Problem pb, int nsteps, double* rec)
 {
     extern __shared__ unsigned char smem_raw[];
-    const Problem& pb = a.probs[0];
+    __shared__ Fx red_e[2][kFusedWarps], red_f[2][kFusedWarps];
+    __shared__ int red_n[2][kFusedWarps], red_m[2][kFusedWarps], red_l[2][kFusedWarps], red_i[2][kFusedWarps];
     DevStats* st = &a.stats[pb.stats];
     const int n = pb.nx;
     P* buf[2] = {reinterpret_cast<P*>(smem_raw), reinterpret_cast<P*>(smem_raw) + 3 * n};
-    __shared__ double red_e[2][kFusedWarps], red_f[2][kFusedWarps];
-    __shared__ int red_n[2][kFusedWarps], red_m[2][kFusedWarps];
     const long long pl = pb.plane, row = pb.pitch;
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     const P* src = static_cast<const P*>(pb.state[a.parity]);
     for (int x = threadIdx.x; x < n; x += blockDim.x)
         for (int i = 0; i < 3; ++i) buf[0][i * n + x] = src[i * pl + row + x];
-    // thread 0: the statistics carried across the steps of this launch
-    double E = 0.0, imb = 0.0, imb_max = 0.0, flux = 0.0, E_prev = 0.0;
-    int have = 0, last_n = 0, last_m = 0;
-    if (threadIdx.x == 0) {
-        E = st->energy;
-        E_prev = st->energy_prev;
-        imb = st->imbalance;
-        imb_max = st->imbalance_max;
-        flux = st->flux;
-        have = st->have_energy;
-        last_n = (int)st->newton_nodes;
-        last_m = st->newton_max_iter;
-    }
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    bool fail = false;
     __syncthreads();
-    int cur = 0;
-    for (int s = 0; s < nsteps; ++s) {
-        const P* in = buf[cur];
-        P* out = buf[cur ^ 1];
-        double e = 0.0, f = 0.0;
-        int nn = 0, mi = 0;
-        for (int x = threadIdx.x; x < n; x += blockDim.x) {
-            P u[3] = {in[x], in[n + x], in[2 * n + x]}, o[3];
-            const P ql = x > 0 ? in[n + x - 1] : (P)0;
-            const P qr = x < n - 1 ? in[2 * n + x + 1] : (P)0;
-            NodeOut r = d1q3_node<P>(pb, x, u, ql, qr, o);
-            out[x] = o[0];
-            out[n + x] = o[1];
-            out[2 * n + x] = o[2];
-            if (rec) rec[(long long)s * pb.pitch + x] = r.theta_new;
-            e += r.energy;
-            f += r.flux;
-            nn += r.newton;
-            mi = max(mi, r.iters);
-            fail |= r.fail;
-        }
-        e = warp_sum(e);
-        f = warp_sum(f);
-        nn = warp_sum_i(nn);
-        mi = warp_max_i(mi);
-        const int h = s & 1;
-        if (l == 0) {
-            red_e[h][w] = e;
-            red_f[h][w] = f;
-            red_n[h][w] = nn;
-            red_m[h][w] = mi;
-        }
-        __syncthreads();   // the step's writes of `out` and of the partial sums are complete
-        if (threadIdx.x == 0) {
-            double es = 0.0, fs = 0.0;
-            int nsum = 0, mmax = 0;
-            for (int k = 0; k < kFusedWarps; ++k) {
-                es += red_e[h][k];
-                fs += red_f[h][k];
-                nsum += red_n[h][k];
-                mmax = max(mmax, red_m[h][k]);
-            }
+    if (w == kFusedWarps) {
+        // the statistics, carried across the steps of this launch
+        double E = st->energy, E_prev = st->energy_prev, imb = st->imbalance, imb_max = st->imbalance_max, flux = st->flux;
+        int have = st->have_energy, last_n = (int)st->newton_nodes, last_m = st->newton_max_iter;
+        long long last_i = st->newton_iters;
+        for (int s = 0; s < nsteps; ++s) {
+            __syncthreads();   // the sums of step s are in
+            const int h = s & 1;
+            const bool mine = l < kFusedWarps;
+            const Fx e = fx_tree(mine ? red_e[h][l] : Fx{0, 0ull});
+            const Fx f = fx_tree(mine ? red_f[h][l] : Fx{0, 0ull});
+            last_n = __reduce_add_sync(kFull, mine ? red_n[h][l] : 0);
+            last_i = __reduce_add_sync(kFull, mine ? red_i[h][l] : 0);
+            last_m = __reduce_max_sync(kFull, mine ? red_m[h][l] : 0);
+            const int nl = __reduce_add_sync(kFull, mine ? red_l[h][l] : 0);
+            const double es = fx_value(e) + (double)nl * pb.inv_ste, fs = fx_value(f);
             if (have) {
                 imb = es - E - fs;
                 if (fabs(imb) > imb_max) imb_max = fabs(imb);
@@ -223,26 +204,74 @@ __global__ void __launch_bounds__(kFusedThreads) d1q3_fused_kernel(StepArgs a, i
             E = es;
             flux = fs;
             have = 1;
-            last_n = nsum;
-            last_m = mmax;
         }
-        cur ^= 1;
+        if (l == 0) {
+            st->energy = E;
+            st->energy_prev = E_prev;
+            st->imbalance = imb;
+            st->imbalance_max = imb_max;
+            st->flux = flux;
+            st->have_energy = have;
+            st->steps += nsteps;
+            st->newton_nodes = last_n;
+            st->newton_iters = last_i;
+            st->newton_max_iter = last_m;
+        }
+    } else {
+        bool fail = false;
+        int cur = 0;
+        for (int s = 0; s < nsteps; ++s) {
+            const P* in = buf[cur];
+            P* out = buf[cur ^ 1];
+            Fx e{0, 0ull}, f{0, 0ull};
+            int nn = 0, mi = 0, nl = 0, ni = 0;
+            bool wall = false;
+            for (int x = threadIdx.x; x < n; x += kFusedThreads) {
+                P u[3] = {in[x], in[n + x], in[2 * n + x]}, o[3];
+                const P ql = x > 0 ? in[n + x - 1] : (P)0;
+                const P qr = x < n - 1 ? in[2 * n + x + 1] : (P)0;
+                NodeOut r = d1q3_node<P>(pb, x, u, ql, qr, o);
+                out[x] = o[0];
+                out[n + x] = o[1];
+                out[2 * n + x] = o[2];
+                if (rec) rec[(long long)s * pb.pitch + x] = r.theta_new;
+                fx_add(e, r.energy);
+                if (x == 0 || x == n - 1) {
+                    fx_add(f, to_fixed(r.flux));
+                    wall = true;
+                }
+                nn += r.newton;
+                nl += r.liquid;
+                ni += r.iters;
+                mi = max(mi, r.iters);
+                fail |= r.fail;
+            }
+            e = fx_tree(e);
+            if (__any_sync(kFull, wall)) f = fx_tree(f);
+            nn = __reduce_add_sync(kFull, nn);
+            nl = __reduce_add_sync(kFull, nl);
+            if (nn) {
+                ni = __reduce_add_sync(kFull, ni);
+                mi = __reduce_max_sync(kFull, mi);
+            }
+            const int h = s & 1;
+            if (l == 0) {
+                red_e[h][w] = e;
+                red_f[h][w] = f;
+                red_n[h][w] = nn;
+                red_l[h][w] = nl;
+                red_i[h][w] = ni;
+                red_m[h][w] = mi;
+            }
+            __syncthreads();   // the step's writes of `out` and of the sums are complete
+            cur ^= 1;
+        }
+        if (fail) atomicOr(&st->error, 3);
     }
-    if (fail) atomicOr(&st->error, 3);
-    if (threadIdx.x == 0) {
-        st->energy = E;
-        st->energy_prev = E_prev;
-        st->imbalance = imb;
-        st->imbalance_max = imb_max;
-        st->flux = flux;
-        st->have_energy = have;
-        st->steps += nsteps;
-        st->newton_nodes = last_n;
-        st->newton_max_iter = last_m;
-    }
+    __syncthreads();
     P* dst = static_cast<P*>(pb.state[a.parity ^ (nsteps & 1)]);
     for (int x = threadIdx.x; x < n; x += blockDim.x)
-        for (int i = 0; i < 3; ++i) dst[i * pl + row + x] = buf[cur][i * n + x];
+        for (int i = 0; i < 3; ++i) dst[i * pl + row + x] = buf[nsteps & 1][i * n + x];
 }
 
 static size_t fused_smem(int precision, int nx) { return (size_t)2 * 3 * nx * (precision == 1 ? 4 : 8); }
@@ -267,11 +296,11 @@ cudaError_t launch_d1q3_fused(int precision, const StepArgs& a, const Problem& h
     if (precision == 1) {
         e = cudaFuncSetAttribute(d1q3_fused_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
-        d1q3_fused_kernel<float><<<1, kFusedThreads, sm, s>>>(b, nsteps, rec);
+        d1q3_fused_kernel<float><<<1, kFusedThreads + 32, sm, s>>>(b, hp, nsteps, rec);
     } else {
         e = cudaFuncSetAttribute(d1q3_fused_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
-        d1q3_fused_kernel<double><<<1, kFusedThreads, sm, s>>>(b, nsteps, rec);
+        d1q3_fused_kernel<double><<<1, kFusedThreads + 32, sm, s>>>(b, hp, nsteps, rec);
     }
     return cudaGetLastError();
 }
