@@ -14,165 +14,229 @@
 // bounce-back as for IREBM; a Dirichlet node's liquid fraction is that of its
 // wall value, [theta_D > 0].
 //
-// Every inner iteration streams the whole lattice, and the loop's test is a
-// maximum over the lattice, so the iterations of a step are separated by
-// lattice-wide barriers.  D1Q3: a lattice of the paper's sizes (N <= 1601) fits
-// in one thread block's shared memory (72 bytes per node): one block runs
-// all steps of a call, its barriers are __syncthreads, and HBM is touched
-// only at the start and the end of the call.  The inner loop is bound by the
-// block's FP64 issue rate (FP64 is scarce on this GPU), so it is cut to what
-// changes between iterations: the source-free part of the collision is formed
-// once per step, an iteration forms only H^(k) and l^(k) (the populations
-// f^(k) are streamed once, after the loop), and the loop's test is one flag
-// per iteration behind a single barrier (three flags in rotation: the one
-// cleared for the next iteration was last read two iterations earlier).
+// The loop's test is a maximum over the lattice, so the iterations of a step
+// are separated by lattice-wide barriers.  D1Q3: a lattice of the paper's sizes
+// (N <= 1601) fits in one thread block's shared memory (72 bytes per node): one
+// block runs all steps of a call, its barriers are __syncthreads, and HBM is
+// touched only at the start and the end of the call.  The block's SM issues one
+// FP64 warp instruction in 19 cycles, which bounds what all nodes do, and a lone
+// warp one in 64, which bounds an inner iteration.  So
+//  * an iterate is a function of l^(k-1) at the node and its neighbours and
+//    repeats bit for bit where they did not change: an iteration evaluates only
+//    segments of 32 nodes next to a change (the mushy zone is a node or two wide;
+//    the two buffers of l agree everywhere else);
+//  * the source-free sum S0 of the streamed populations is formed once per step,
+//    an iteration adds the three source terms;
+//  * the first iterate has no source; the last streaming adds it only near a
+//    change, and collides for the next step;
+//  * sums are fixed point, comparisons work on the bits, and a warp of its own
+//    adds up the statistics while the next step runs.
+// 801 nodes: 86 us per step with every node in every iteration.
 #include "resident.cuh"
 
 namespace lbm {
 
-constexpr int kIlfThreads = 512;
+constexpr int kIlfThreads = 512;                // computing threads
 constexpr int kIlfWarps = kIlfThreads / 32;
+constexpr int kIlfSegs = 96;                    // segments of 32 nodes, at most (2,844 nodes)
 
 __device__ __forceinline__ double ilf_lever(double H, double ste, double inv_ste)
 {
-    return H < 0.0 ? 0.0 : (H > inv_ste ? 1.0 : ste * H);
+    // sign and order from the bits
+    const long long b = __double_as_longlong(H);
+    if ((b & 0x7fffffffffffffffll) > 0x7ff0000000000000ll) return H;   // NaN
+    return b < 0 ? 0.0 : (b > __double_as_longlong(inv_ste) ? 1.0 : ste * H);
 }
 
-__global__ void __launch_bounds__(kIlfThreads) ilfbm_d1q3_kernel(StepArgs a, int nsteps)
+// |d| > tol, tol > 0 (NaN: no)
+__device__ __forceinline__ bool ilf_above(double d, double tol)
+{
+    const long long b = __double_as_longlong(d) & 0x7fffffffffffffffll;
+    return b > __double_as_longlong(tol) && b <= 0x7ff0000000000000ll;
+}
+
+__global__ void __launch_bounds__(kIlfThreads + 32) ilfbm_d1q3_kernel(StepArgs a, const __grid_constant__ Problem pb, int nsteps)
 {
     extern __shared__ double sm[];
-    __shared__ double red_e[2][kIlfWarps], red_f[2][kIlfWarps];   // per-step partial sums, step parity
-    __shared__ int s_more[3];   // "some node changed by more than tol", iteration gk uses gk % 3
-    const Problem& pb = a.probs[0];
+    __shared__ Fx red_e[2][kIlfWarps], red_f[2][kIlfWarps];   // per-step sums, step parity
+    __shared__ unsigned char chg[3][kIlfSegs + 2];            // segment changed in iteration k: chg[k % 3][segment + 1]
+    __shared__ unsigned char ever[kIlfSegs + 2];              // ... in some iteration of the step
     DevStats* st = &a.stats[pb.stats];
-    const int n = pb.nx;
-    double* o = sm;              // f_i at time t, then Omega_i without the source: f_i - (f_i - w_i theta)/tau
-    double* fn = sm + 3 * n;     // f~ of the step (the buffers swap roles every step)
+    const int n = pb.nx, nseg = (n + 31) / 32;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool stats_warp = w == kIlfWarps;   // no nodes; takes part in the barriers
+    const int seg0 = stats_warp ? nseg : w;
+    double* o = sm;              // Omega_i of the step without the source
+    double* fn = sm + 3 * n;     // next step's; during the iterations: l - l^(k) (two buffers), S0
     double* el = sm + 6 * n;     // l at time t
-    double* lb[2] = {el + n, el + 2 * n};   // l^(k-1) and l^(k), alternating
+    double* lb[2] = {el + n, el + 2 * n};   // l^(k), alternating
     const long long pl = pb.plane, row = pb.pitch;
-    const double* src = static_cast<const double*>(pb.state[a.parity]);
-    // the state at time t: f_i and l
-    for (int x = threadIdx.x; x < n; x += blockDim.x) {
-        for (int i = 0; i < 3; ++i) o[i * n + x] = src[i * pl + row + x];
-        el[x] = src[3 * pl + row + x];
-    }
     const double om = pb.omega, ste = pb.ste, inv_ste = pb.inv_ste, tol = pb.tol;
-    const double w0 = d1_w(0), w1 = d1_w(1), w2 = d1_w(2);
-    const double c0 = w0 * inv_ste, c1 = w1 * inv_ste, c2 = w2 * inv_ste;
+    const double w1 = d1_w(1);
+    const double c0 = d1_w(0) * inv_ste, c1 = w1 * inv_ste;   // (w_i/Ste)
     const bool dirW = pb.wall_kind[0] == 1, dirE = pb.wall_kind[1] == 1;
     const double thW = pb.wall_theta[0], thE = pb.wall_theta[1];
     const bool mirror = pb.bb_mode == 0;
-    bool failed = false;
-    unsigned gk = 0;   // inner iterations so far in this launch: selects the flag
-    // thread 0: the statistics carried across the steps of this launch
-    double E = 0.0, E_prev = 0.0, imb = 0.0, imb_max = 0.0, flux = 0.0;
-    int have = 0, last_it = 0;
-    if (threadIdx.x == 0) {
-        E = st->energy;
-        E_prev = st->energy_prev;
-        imb = st->imbalance;
-        imb_max = st->imbalance_max;
-        flux = st->flux;
-        have = st->have_energy;
-        last_it = st->newton_max_iter;
+    // Omega_i = f_i - (f_i - w_i theta) omega, theta = sum f_i: in this form (1 - omega and
+    // omega w_i do not appear as rounded factors) theta does not drift over many steps
+    auto collide = [&](const double (&f)[3], double th, double (&g)[3]) {
+        g[0] = fma(-om, fma(-d1_w(0), th, f[0]), f[0]);
+        g[1] = fma(-om, fma(-w1, th, f[1]), f[1]);
+        g[2] = fma(-om, fma(-w1, th, f[2]), f[2]);
+    };
+    // the state at time t: f_i, collided, and l
+    const double* src = static_cast<const double*>(pb.state[a.parity]);
+    for (int x = threadIdx.x; x < n; x += blockDim.x) {
+        const double f[3] = {src[row + x], src[pl + row + x], src[2 * pl + row + x]};
+        double g[3];
+        collide(f, sum_q<3>(f), g);
+        for (int i = 0; i < 3; ++i) o[i * n + x] = g[i];
+        lb[0][x] = src[3 * pl + row + x];
     }
-    if (threadIdx.x < 3) s_more[threadIdx.x] = 0;
+    if (threadIdx.x < kIlfSegs + 2) chg[0][threadIdx.x] = chg[1][threadIdx.x] = chg[2][threadIdx.x] = ever[threadIdx.x] = 0;
+    bool failed = false;
+    // the statistics warp: carried across the steps of this launch
+    double E = st->energy, E_prev = st->energy_prev, imb = st->imbalance, imb_max = st->imbalance_max, flux = st->flux;
+    int have = st->have_energy, last_it = st->newton_max_iter;
     __syncthreads();
+    int base = 0;
     for (int s = 0; s < nsteps; ++s) {
-        // moments and the source-free part of the collision (the same in every
-        // inner iteration); l^(0) = l
-        for (int x = threadIdx.x; x < n; x += blockDim.x) {
-            const double f0 = o[x], f1 = o[n + x], f2 = o[2 * n + x];
-            const double th = f0 + f1 + f2;
-            o[x] = f0 - (f0 - w0 * th) * om;
-            o[n + x] = f1 - (f1 - w1 * th) * om;
-            o[2 * n + x] = f2 - (f2 - w2 * th) * om;
-            lb[0][x] = el[x];
-        }
-        __syncthreads();
-        // streamed f^(k)(y) from Omega_i(x) = o_i(x) + (w_i/Ste)(l(x) - l^(k-1)(x)),
-        // the closures on the unknown one at a wall; returns the three values
-        auto stream = [&](int y, const double* lp, double& q0, double& q1, double& q2) {
-            q0 = o[y] + c0 * (el[y] - lp[y]);
-            q1 = y > 0 ? o[n + y - 1] + c1 * (el[y - 1] - lp[y - 1]) : 0.0;
-            q2 = y < n - 1 ? o[2 * n + y + 1] + c2 * (el[y + 1] - lp[y + 1]) : 0.0;
-            if (y == 0)   // west wall: f_1 (e = +1) is unknown
-                q1 = dirW ? thW - q0 - q2 : (mirror ? q2 : o[2 * n] + c2 * (el[0] - lp[0]));
-            if (y == n - 1)   // east wall: f_2 (e = -1) is unknown
-                q2 = dirE ? thE - q0 - q1 : (mirror ? q1 : o[n + n - 1] + c1 * (el[n - 1] - lp[n - 1]));
-        };
-        int it = 0, cur = 0;
-        bool conv = false;
-        while (!conv && it < pb.maxit) {   // it, gk, cur and conv are the same in every thread
-            const double* lp = lb[cur];
-            double* ln = lb[cur ^ 1];
-            const int slot = gk % 3;
-            ++it;
-            ++gk;
-            // H^(k) = M0(f^(k)) + l^(k-1)/Ste and the lever rule; Dirichlet nodes keep
-            // the phase of their wall value
-            bool more = false;
-            for (int y = threadIdx.x; y < n; y += blockDim.x) {
+        double* S0 = fn + 2 * n;
+        // first iterate: l^(0) = l, no source
+        bool more = false;
+        for (int sg = seg0; sg < nseg; sg += kIlfWarps) {
+            const int y = sg * 32 + lane;
+            bool changed = false;
+            if (y < n) {
+                const double l0 = lb[base][y];
+                el[y] = l0;
                 double lk;
                 if (y == 0 && dirW) {
                     lk = thW > 0.0 ? 1.0 : 0.0;
                 } else if (y == n - 1 && dirE) {
                     lk = thE > 0.0 ? 1.0 : 0.0;
                 } else {
-                    double q0, q1, q2;
-                    stream(y, lp, q0, q1, q2);
-                    lk = ilf_lever(q0 + q1 + q2 + lp[y] * inv_ste, ste, inv_ste);
+                    double q[3] = {o[y], y > 0 ? o[n + y - 1] : 0.0, y < n - 1 ? o[2 * n + y + 1] : 0.0};
+                    if (y == 0) q[1] = mirror ? q[2] : o[2 * n];
+                    if (y == n - 1) q[2] = mirror ? q[1] : o[n + n - 1];
+                    const double sum = sum_q<3>(q);
+                    S0[y] = sum;
+                    lk = ilf_lever(fma(l0, inv_ste, sum), ste, inv_ste);
                 }
-                more |= fabs(lk - lp[y]) > tol;
-                ln[y] = lk;
+                const double d = l0 - lk;
+                more |= ilf_above(d, tol);
+                changed = lk != l0;
+                lb[base ^ 1][y] = lk;
+                fn[base * n + y] = 0.0;
+                fn[(base ^ 1) * n + y] = d;
             }
-            // flag of this iteration; thread 0 clears the next iteration's flag, last read
-            // two iterations ago (every thread read it before the previous barrier) and
-            // next set after this iteration's barrier
-            if (more) s_more[slot] = 1;
-            if (threadIdx.x == 0) s_more[(slot + 1) % 3] = 0;
-            __syncthreads();
-            conv = s_more[slot] == 0;
-            cur ^= 1;
+            const bool c = __any_sync(kFull, changed);
+            if (lane == 0) {
+                chg[1][sg + 1] = ever[sg + 1] = c;
+                chg[2][sg + 1] = 0;
+            }
         }
-        failed |= !conv;
-        // f~ = f^(k) (streamed with the source of l^(k-1)) into the other buffer,
-        // l~ = l^(k); the boundary flux is filled minus leaving at the two walls
-        const double* lp = lb[cur ^ 1];
-        const double* ln = lb[cur];
-        double e = 0.0, fl = 0.0;
-        for (int y = threadIdx.x; y < n; y += blockDim.x) {
-            double q0, q1, q2;
-            stream(y, lp, q0, q1, q2);
-            if (y == 0) fl += q1 - (o[2 * n] + c2 * (el[0] - lp[0]));
-            if (y == n - 1) fl += q2 - (o[n + n - 1] + c1 * (el[n - 1] - lp[n - 1]));
-            fn[y] = q0;
-            fn[n + y] = q1;
-            fn[2 * n + y] = q2;
-            e += (q0 + q1 + q2) + ln[y] * inv_ste;
+        bool any = __syncthreads_or(more ? 1 : 0) != 0;
+        int k = 1;
+        while (any && k < pb.maxit) {   // k and any are the same in every thread
+            ++k;
+            const int pv = (base + k - 1) & 1;
+            const double* lp = lb[pv];
+            const double* dp = fn + pv * n;
+            double* ln = lb[pv ^ 1];
+            double* dn = fn + (pv ^ 1) * n;
+            const unsigned char* prev = chg[(k - 1) % 3];
+            unsigned char* cur = chg[k % 3];
+            unsigned char* next = chg[(k + 1) % 3];
+            more = false;
+            for (int sg = seg0; sg < nseg; sg += kIlfWarps) {
+                bool changed = false;
+                if (prev[sg] | prev[sg + 1] | prev[sg + 2]) {
+                    const int y = sg * 32 + lane;
+                    if (y < n) {
+                        const double l0 = lp[y];
+                        double lk = l0;   // a Dirichlet node keeps its wall's phase
+                        if (!((y == 0 && dirW) || (y == n - 1 && dirE))) {
+                            // S0 and the source terms c_i (l - l^(k-1)); a wall's unknown one is
+                            // the opposite one's, mirrored or of the node itself
+                            const double d0 = dp[y];
+                            double d1 = y > 0 ? dp[y - 1] : 0.0, d2 = y < n - 1 ? dp[y + 1] : 0.0;
+                            if (y == 0) d1 = mirror ? d2 : d0;
+                            if (y == n - 1) d2 = mirror ? d1 : d0;
+                            double H = fma(c0, d0, S0[y]);
+                            H = fma(c1, d1, H);
+                            H = fma(c1, d2, H);
+                            lk = ilf_lever(fma(l0, inv_ste, H), ste, inv_ste);
+                        }
+                        more |= ilf_above(lk - l0, tol);
+                        changed = lk != l0;
+                        ln[y] = lk;
+                        dn[y] = el[y] - lk;
+                    }
+                    changed = __any_sync(kFull, changed);
+                }
+                if (lane == 0) {
+                    next[sg + 1] = 0;
+                    if (changed) cur[sg + 1] = ever[sg + 1] = 1;
+                }
+            }
+            any = __syncthreads_or(more ? 1 : 0) != 0;
         }
-        e = warp_sum(e);
-        fl = warp_sum(fl);
+        failed |= any;
+        // f~ with the source of l^(k-1), l~ = l^(k); the boundary flux is filled minus leaving
+        // at the two walls; collided for the launch's next step
+        const double* lp = lb[(base + k - 1) & 1];
+        const double* ln = lb[(base + k) & 1];
+        const bool last = s + 1 == nsteps;
+        Fx e{0, 0ull}, fl{0, 0ull};
+        bool wall = false;
+        for (int sg = seg0; sg < nseg; sg += kIlfWarps) {
+            const int y = sg * 32 + lane;
+            if (y >= n) continue;
+            const bool near = (ever[sg] | ever[sg + 1] | ever[sg + 2]) != 0;
+            double q0 = o[y], q1 = y > 0 ? o[n + y - 1] : 0.0, q2 = y < n - 1 ? o[2 * n + y + 1] : 0.0;
+            double o1 = o[n + y], o2 = o[2 * n + y];   // leaving at a wall
+            if (near) {
+                const double d0 = el[y] - lp[y];
+                q0 = fma(c0, d0, q0);
+                if (y > 0) q1 = fma(c1, el[y - 1] - lp[y - 1], q1);
+                if (y < n - 1) q2 = fma(c1, el[y + 1] - lp[y + 1], q2);
+                o1 = fma(c1, d0, o1);
+                o2 = fma(c1, d0, o2);
+            }
+            if (y == 0) {   // west wall: f_1 (e = +1) is unknown
+                q1 = dirW ? thW - q0 - q2 : (mirror ? q2 : o2);
+                fx_add(fl, to_fixed(q1 - o2));
+                wall = true;
+            }
+            if (y == n - 1) {   // east wall: f_2 (e = -1) is unknown
+                q2 = dirE ? thE - q0 - q1 : (mirror ? q1 : o1);
+                fx_add(fl, to_fixed(q2 - o1));
+                wall = true;
+            }
+            const double q[3] = {q0, q1, q2};
+            const double th = sum_q<3>(q);
+            fx_add(e, to_fixed(fma(ln[y], inv_ste, th)));
+            double g[3] = {q0, q1, q2};
+            if (!last) collide(q, th, g);
+            for (int i = 0; i < 3; ++i) fn[i * n + y] = g[i];
+        }
+        e = fx_tree(e);
+        if (__any_sync(kFull, wall)) fl = fx_tree(fl);
         const int h = s & 1;
-        if ((threadIdx.x & 31) == 0) {
-            red_e[h][threadIdx.x >> 5] = e;
-            red_f[h][threadIdx.x >> 5] = fl;
+        if (lane == 0 && !stats_warp) {
+            red_e[h][w] = e;
+            red_f[h][w] = fl;
         }
-        __syncthreads();   // every read of o, el and l^(k-1) of this step is done
-        for (int y = threadIdx.x; y < n; y += blockDim.x) el[y] = ln[y];
+        __syncthreads();   // the next step's populations and the sums are complete
         double* t = o;
         o = fn;
         fn = t;
-        if (threadIdx.x == 0) {
-            // the warps' sums in a fixed order; a half of red_* is written again two
-            // steps later, after the next step's barriers, which thread 0 reaches
-            // only after this
-            double es = 0.0, fs = 0.0;
-            for (int k = 0; k < kIlfWarps; ++k) {
-                es += red_e[h][k];
-                fs += red_f[h][k];
-            }
+        base = (base + k) & 1;
+        if (stats_warp) {
+            const bool mine = lane < kIlfWarps;
+            const double es = fx_value(fx_tree(mine ? red_e[h][lane] : Fx{0, 0ull}));
+            const double fs = fx_value(fx_tree(mine ? red_f[h][lane] : Fx{0, 0ull}));
             if (have) {
                 imb = es - E - fs;
                 if (fabs(imb) > imb_max) imb_max = fabs(imb);
@@ -181,10 +245,10 @@ __global__ void __launch_bounds__(kIlfThreads) ilfbm_d1q3_kernel(StepArgs a, int
             E = es;
             flux = fs;
             have = 1;
-            last_it = it;
+            last_it = k;
         }
     }
-    if (threadIdx.x == 0) {
+    if (stats_warp && lane == 0) {
         st->energy = E;
         st->energy_prev = E_prev;
         st->imbalance = imb;
@@ -194,12 +258,12 @@ __global__ void __launch_bounds__(kIlfThreads) ilfbm_d1q3_kernel(StepArgs a, int
         st->steps += nsteps;
         st->newton_nodes = 0;
         st->newton_max_iter = last_it;   // inner iterations of the last step
+        if (failed) atomicOr(&st->error, 3);   // LBM_ERR_NEWTON: inner loop at its limit
     }
-    if (failed && threadIdx.x == 0) atomicOr(&st->error, 3);   // LBM_ERR_NEWTON: inner loop at its limit
     double* dst = static_cast<double*>(pb.state[a.parity ^ (nsteps & 1)]);
     for (int x = threadIdx.x; x < n; x += blockDim.x) {
         for (int i = 0; i < 3; ++i) dst[i * pl + row + x] = o[i * n + x];
-        dst[3 * pl + row + x] = el[x];
+        dst[3 * pl + row + x] = lb[base][x];
     }
 }
 
@@ -624,7 +688,7 @@ cudaError_t launch_ilfbm_d1q3(const StepArgs& a, const Problem& hp, int nsteps, 
     const size_t sm = ilfbm_smem(hp.nx);
     cudaError_t e = cudaFuncSetAttribute(ilfbm_d1q3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    ilfbm_d1q3_kernel<<<1, kIlfThreads, sm, s>>>(a, nsteps);
+    ilfbm_d1q3_kernel<<<1, kIlfThreads + 32, sm, s>>>(a, hp, nsteps);
     return cudaGetLastError();
 }
 
