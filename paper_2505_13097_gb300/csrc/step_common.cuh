@@ -174,6 +174,7 @@ struct NewtonResult {
     int sidx = -1;   // -1: no node (an idle lane)
 };
 
+// (FP32: the energy term lacks the state's shift, as at saturated nodes.)
 template <typename P, bool REC, int Q>
 __device__ __forceinline__ NewtonResult newton_job_apply(const NewtonJob& jb, const Problem& pb, int parity,
                                                          double* rec, DevStats* stats)
@@ -189,33 +190,31 @@ __device__ __forceinline__ NewtonResult newton_job_apply(const NewtonJob& jb, co
     P qv[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) qv[i] = __ldcg(d + i * pb.plane);
-    double m0, th, sh = 0.0;
+    double mm, tt, sh = 0.0, shz = 0.0;   // m0 and theta less the shift
     if constexpr (sizeof(P) == 4) {
         // FP32 form: the job carries only the node; m0 = M0(q) from the stored
         // unrelaxed q_i and theta = M0(f) = sum of the node's Omega_i(t) (the
         // step's source state), both as float-float sums in the order the
         // step kernel uses (last plane first), plus the state's shift s
         const P* sv = static_cast<const P*>(pb.state[parity]) + at;
-        ff mm{0.f, 0.f}, t{0.f, 0.f};
+        ff m{0.f, 0.f}, t{0.f, 0.f};
 #pragma unroll
         for (int i = Q - 1; i >= 0; --i) {
             ff_add(t, __ldg(sv + i * pb.plane));
-            ff_add(mm, qv[i]);
+            ff_add(m, qv[i]);
         }
         sh = widen(state_shift(pb, parity));
-        m0 = ff_to_double(mm) + sh;
-        th = ff_to_double(t) + sh;
+        shz = sh * pb.two_inv_delta;
+        mm = ff_to_double(m);
+        tt = ff_to_double(t);
     } else {
-        m0 = jb.m0;
-        th = jb.theta;
+        mm = jb.m0;
+        tt = jb.theta;
     }
-    const Phi pt = phi_parts(th, pb.two_inv_delta);
-    const double pth = pt.value();
-    const NewtonOut nr = newton_mixed(m0, th, pt, pb);
-    if (!nr.ok || !isfinite(nr.root)) atomicCAS(&stats[r.sidx].error, 0, 3);
-    const double tn = m0 + (pth - nr.phi_root) * pb.inv_ste;
+    const NewtonNode nr = newton_mixed(mm, tt, sh, shz, pb);
+    if (!nr.ok) atomicCAS(&stats[r.sidx].error, 0, 3);
     // c = theta' - (1-omega) m0; stored values less w_i s: c - omega s
-    const P c = (P)((tn - sh) - pb.omc * (m0 - sh));
+    const P c = (P)fma(-pb.omc, mm, nr.tns);
     const P omc = sizeof(P) == 4 ? (P)pb.omc_f : (P)pb.omc;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -223,8 +222,8 @@ __device__ __forceinline__ NewtonResult newton_job_apply(const NewtonJob& jb, co
         d[i * pb.plane] = fma(omc, qv[i], wi * c);
     }
     (void)x;
-    if (REC) rec[(long long)y * pb.pitch + x] = tn;
-    r.e = to_fixed(tn + nr.phi_root * pb.inv_ste);
+    if (REC) rec[(long long)y * pb.pitch + x] = nr.tns + sh;
+    r.e = to_fixed(nr.ens);
     r.it = nr.iters;
     return r;
 }
@@ -234,6 +233,7 @@ __device__ __forceinline__ NewtonResult newton_job_apply(const NewtonJob& jb, co
 // largest iteration count once.  A warp whose jobs are of one problem (a single
 // problem always) sums by a tree, about 60 instructions; the loop over the 32
 // lanes, some 1,100, is left to warps that straddle problems.
+template <typename P>
 __device__ __forceinline__ void newton_group_add(const NewtonResult& r, DevStats* stats)
 {
     const int lane = threadIdx.x & 31;
@@ -257,6 +257,7 @@ __device__ __forceinline__ void newton_group_add(const NewtonResult& r, DevStats
             StepStripe* c = my_stripe(st);
             acc_add_fx(&c->energy, sum);
             atomicAdd(&c->newton, (unsigned long long)__popc(have));
+            if (sizeof(P) == 4) atomicAdd(&c->shifted, (unsigned long long)__popc(have));
             atomicAdd(&c->iters, (unsigned long long)its);
             atomicMax(&st->cur_maxit, mx);
         }
@@ -283,6 +284,7 @@ __device__ __forceinline__ void newton_group_add(const NewtonResult& r, DevStats
         StepStripe* c = my_stripe(st);
         acc_add_fx(&c->energy, sum);
         atomicAdd(&c->newton, (unsigned long long)n);
+        if (sizeof(P) == 4) atomicAdd(&c->shifted, (unsigned long long)n);
         atomicAdd(&c->iters, (unsigned long long)its);
         atomicMax(&st->cur_maxit, mx);
     }

@@ -94,14 +94,11 @@ __device__ __forceinline__ NodeOut d1q3_node(const Problem& pb, int x, const P (
         r.energy = to_fixed(m0);
         r.liquid = liq ? 1 : 0;
     } else {
-        const double th = sum_q<3>(ud);
-        const Phi pt = phi_parts(th, pb.two_inv_delta);
-        const NewtonOut nr = newton_mixed(m0, th, pt, pb);
-        r.fail = !nr.ok || !isfinite(nr.root);
-        const double tn = m0 + (pt.value() - nr.phi_root) * pb.inv_ste;
-        v = w1 * (tn - omc * m0);
-        r.theta_new = tn;
-        r.energy = to_fixed(tn + nr.phi_root * pb.inv_ste);
+        const NewtonNode nr = newton_mixed(m0, sum_q<3>(ud), 0.0, 0.0, pb);
+        r.fail = !nr.ok;
+        v = w1 * fma(-omc, m0, nr.tns);
+        r.theta_new = nr.tns;
+        r.energy = to_fixed(nr.ens);
         r.newton = 1;
         r.iters = nr.iters;
     }
@@ -160,8 +157,8 @@ constexpr int kFusedWarps = kFusedThreads / 32;
 // of a small array; a warp of its own adds them up and keeps the statistics
 // while the others run the next step (a half is written again two steps later,
 // after a barrier that warp reaches only when it has read it).  What bounds a
-// step is the longest warp's chain: a Newton solve, 58 FP64 instructions of 64
-// cycles and the FP32 stage, about 3.4 us; the saturated warps run beside it.
+// step is the longest warp's chain: a Newton solve, 43 FP64 instructions of 64
+// cycles and the FP32 stage; the saturated warps run beside it.
 // 512 nodes with a front: 15.3 us per step with a library tanh and FP64 sums,
 // 9.3 with the shorter solve alone.
 template <typename P>

@@ -805,7 +805,7 @@ __device__ __forceinline__ void newton_job_group(const JobArgs& a, const NewtonJ
         const NewtonJob jb = jobs[j];
         r = newton_job_apply<P, REC, Q>(jb, a.probs[jb.prob], a.parity, a.rec, a.stats);
     }
-    newton_group_add(r, a.stats);
+    newton_group_add<P>(r, a.stats);
 }
 
 template <typename P, bool REC, int Q>

@@ -17,7 +17,7 @@
 //     flat kernel; 1 in FP64).  Saturated nodes are updated, the nodes that
 //     need the Newton solve go to a queue in shared memory.
 //  2. items of 32 nodes, one per lane: the queued nodes, gathered densely so
-//     that a solve (a chain of 58 FP64 instructions of 64 cycles) serves full
+//     that a solve (a chain of 43 FP64 instructions of 64 cycles) serves full
 //     warps, the rows 0 and ny-1, and the column groups at the W and E walls.
 // Groups of a wave lie side by side (their halo rows and columns meet in L1 and
 // L2), and a block's place in the wave rotates from wave to wave, so that the
@@ -244,27 +244,27 @@ __device__ __forceinline__ void item_update(const ResidentArgs& a, const P* src,
         Fx e{0, 0ull};
         int it = 0;
         if (solve) {
-            double m, t, shd = 0.0;
+            double mm, tt, shd = 0.0, shz = 0.0;   // m0 and theta less the shift
             if constexpr (sizeof(P) == 4) {
-                ff mm{0.f, 0.f}, tt{0.f, 0.f};
+                ff fm{0.f, 0.f}, ft{0.f, 0.f};
 #pragma unroll
                 for (int i = Q - 1; i >= 0; --i) {
-                    ff_add(tt, u[i]);
-                    ff_add(mm, q[i]);
+                    ff_add(ft, u[i]);
+                    ff_add(fm, q[i]);
                 }
                 shd = widen(sh);
-                m = ff_to_double(mm) + shd;
-                t = ff_to_double(tt) + shd;
+                shz = shd * pb.two_inv_delta;
+                mm = ff_to_double(fm);
+                tt = ff_to_double(ft);
             } else {
-                m = (double)m0;
-                t = sum_q<Q>(u);
+                mm = (double)m0;
+                tt = sum_q<Q>(u);
             }
-            const Phi pt = phi_parts(t, pb.two_inv_delta);
-            const NewtonOut nr = newton_mixed(m, t, pt, pb);
-            if (!nr.ok || !isfinite(nr.root)) atomicCAS(&a.stats->error, 0, 3);
-            tn = m + (pt.value() - nr.phi_root) * pb.inv_ste;
-            c = (P)((tn - shd) - pb.omc * (m - shd));
-            e = to_fixed(tn + nr.phi_root * pb.inv_ste);
+            const NewtonNode nr = newton_mixed(mm, tt, shd, shz, pb);
+            if (!nr.ok) atomicCAS(&a.stats->error, 0, 3);
+            tn = nr.tns + shd;
+            c = (P)fma(-pb.omc, mm, nr.tns);
+            e = to_fixed(nr.ens);   // FP32: less the shift
             it = nr.iters;
         }
         e = fx_tree(e);
@@ -273,6 +273,7 @@ __device__ __forceinline__ void item_update(const ResidentArgs& a, const P* src,
         if (lane == 0) {
             fx_add(w->e, e);
             w->newton += (unsigned)__popc(solving);
+            if (sizeof(P) == 4) w->shifted += (unsigned)__popc(solving);
             w->iters += its;
             w->maxit = max(w->maxit, mx);
         }
