@@ -36,6 +36,8 @@
 // phi(theta(t+1)) - phi(theta(t)) = sinh(x1 - x0) / (2 cosh x0 cosh x1),
 // x = theta/delta, both free of cancellation; wall nodes in FP64.
 // FP64 form: everything in FP64 with the formulas of the gather above.
+#include <algorithm>
+
 #include "lbm_device.cuh"
 
 namespace lbm {
@@ -654,6 +656,156 @@ __global__ void adj_links_kernel(const __grid_constant__ AdjArgs g, int corners_
         if ((t.link_mask >> j) & 1) aout[j * pb.plane + ro] = (P)(t.nu + link[j]);
 }
 
+// ---------------------------------------------------------------- D2Q9 flat kernel, FP32
+// One launch per reverse step.  For a node y away from the walls
+// D_j(y) = (1 - omega) a_j(y) + mu(y), so a tile's outputs
+//   lambda_j(x) = nu(x) + (1 - omega) a_j(x + e_j) + mu(x + e_j)
+// need one number per neighbour node beyond loads that are in L1 already: the
+// block evaluates mu of its 64 x 16 nodes and the ring around them (1.16
+// evaluations per node; the marching kernel's tiles of 4 rows at 1024^2 take
+// 1.5, with the shuffles of six planes), keeps them in shared memory and
+// gathers.  Outputs whose neighbourhood holds a wall node (the two outermost
+// rows and columns) are gathered by the last blocks, one node per thread with
+// the general node terms and the link-wise terms of adj_links_kernel: a few
+// thousand nodes beside the tiles, instead of a launch of their own after them.
+// Measured per step, marching and link kernels / this one: 44 / 31 us at 1024^2,
+// 119 / 97 us at 2048^2.  (FP64, and lattices beyond 32-bit indices: marching.)
+constexpr int kAdjFlatW = 64, kAdjFlatH = 16, kAdjFlatThreads = 512;
+constexpr int kAdjMuW = kAdjFlatW + 2, kAdjMuH = kAdjFlatH + 2;
+
+__device__ __forceinline__ bool adj_has_links(const Problem& pb, unsigned bmask, unsigned unk)
+{
+    for (int w = 0; w < 4; ++w)
+        if (((bmask >> w) & 1u) && pb.wall_kind[w] == 1) return false;
+    bool any = false;
+    for (int i = 1; i < 9; ++i)
+        if (((unk >> i) & 1u) && (pb.bb_mode == 1 || ((unk >> d2_opp(i)) & 1u))) any = true;
+    return any;
+}
+
+__global__ void __launch_bounds__(kAdjFlatThreads, 2) adj_flat_kernel(const __grid_constant__ AdjArgs g, int ntx, int ntiles)
+{
+    __shared__ float mu_s[kAdjMuH * kAdjMuW];
+    __shared__ double wall_sums[5 * kWarpsPerBlock * 32];
+    const Problem& pb = g.pb;
+    const AdjConst& c = g.c;
+    const int nx = pb.nx, ny = pb.ny, pitch = pb.pitch, plane = (int)pb.plane;
+    const float* ain = static_cast<const float*>(g.adj_in);
+    float* aout = static_cast<float*>(g.adj_out);
+    const float omc = c.omc_f;
+    DevStats* st = g.stats;
+    const int tid = threadIdx.x;
+    if ((int)blockIdx.x < ntiles) {
+        // outputs 2 <= x <= nx-3, 2 <= y <= ny-3
+        const int x0 = 2 + (int)(blockIdx.x % ntx) * kAdjFlatW, y0 = 2 + (int)(blockIdx.x / ntx) * kAdjFlatH;
+        float nu[2] = {0.f, 0.f}, gs = 0.f;
+        auto node = [&](int x, int y, float& mu, float& nuv, float& gsv) {
+            const float* p = ain + (y + 1) * pitch + x;
+            const float A = d2_wf(0) * __ldg(p) +
+                            d2_wf(1) * ((__ldg(p + plane) + __ldg(p + 2 * plane)) + (__ldg(p + 3 * plane) + __ldg(p + 4 * plane))) +
+                            d2_wf(5) * ((__ldg(p + 5 * plane) + __ldg(p + 6 * plane)) + (__ldg(p + 7 * plane) + __ldg(p + 8 * plane)));
+            interior_terms(A, __ldg(g.theta_t + y * pitch + x), __ldg(g.theta_t1 + y * pitch + x), c, mu, nuv, gsv);
+        };
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int lx = tid % kAdjFlatW, ly = tid / kAdjFlatW + 8 * k, x = x0 + lx, y = y0 + ly;
+            if (x <= nx - 3 && y <= ny - 3) {
+                float mu;
+                node(x, y, mu, nu[k], gs);
+                mu_s[(ly + 1) * kAdjMuW + lx + 1] = mu;
+            }
+        }
+        // the ring around the tile (as far as the last outputs' neighbours)
+        const int wx = min(kAdjFlatW, nx - 2 - x0), hy = min(kAdjFlatH, ny - 2 - y0);   // outputs of this tile
+        const int ring = 2 * (wx + 2) + 2 * hy;
+        if (tid < ring) {
+            int lx, ly;
+            if (tid < wx + 2) { lx = tid; ly = 0; }
+            else if (tid < 2 * (wx + 2)) { lx = tid - (wx + 2); ly = hy + 1; }
+            else if (tid < 2 * (wx + 2) + hy) { lx = 0; ly = tid - 2 * (wx + 2) + 1; }
+            else { lx = wx + 1; ly = tid - 2 * (wx + 2) - hy + 1; }
+            float mu, nuv, gsv = 0.f;
+            node(x0 + lx - 1, y0 + ly - 1, mu, nuv, gsv);
+            mu_s[ly * kAdjMuW + lx] = mu;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int lx = tid % kAdjFlatW, ly = tid / kAdjFlatW + 8 * k, x = x0 + lx, y = y0 + ly;
+            if (x > nx - 3 || y > ny - 3) continue;
+            const int at = (y + 1) * pitch + x;
+            const float* m = mu_s + (ly + 1) * kAdjMuW + lx + 1;
+#pragma unroll
+            for (int j = 0; j < 9; ++j) {
+                const float a = __ldg(ain + j * plane + at + d2_ey(j) * pitch + d2_ex(j));
+                aout[j * plane + at] = nu[k] + fmaf(omc, a, m[d2_ey(j) * kAdjMuW + d2_ex(j)]);
+            }
+        }
+        const double v = warp_sum((double)gs);
+        if ((tid & 31) == 0 && v != 0.0) acc_add(&st->g_ste, v);
+        return;
+    }
+    // the two outermost rows (all columns), then the two outermost columns of the rows between
+    if (tid >= kWarpsPerBlock * 32) return;
+    AdjSums<float> sums;
+    sums.gs = 0.f;
+    sums.wall = wall_sums + tid;
+    for (int k = 0; k < 5; ++k) sums.wall[k * kWarpsPerBlock * 32] = 0.0;
+    const int k = ((int)blockIdx.x - ntiles) * kWarpsPerBlock * 32 + tid;
+    const int rows = min(4, ny), mid = max(0, ny - 4), cols = min(4, nx);
+    int x = -1, y = 0;
+    if (k < rows * nx) {
+        const int r = k / nx;
+        x = k - r * nx;
+        y = r < 2 ? r : ny - rows + r;
+    } else if (k < rows * nx + cols * mid) {
+        const int q = (k - rows * nx) / cols, e = (k - rows * nx) - q * cols;
+        y = 2 + q;
+        x = e < 2 ? e : nx - cols + e;
+    }
+    if (x >= 0) {
+        const int at = (y + 1) * pitch + x;
+        auto mask = [&](int xx, int yy) -> unsigned {
+            return (xx == 0 ? 1u : 0u) | (xx == nx - 1 ? 2u : 0u) | (yy == 0 ? 4u : 0u) | (yy == ny - 1 ? 8u : 0u);
+        };
+        float nu = 0.f, lam[9];
+        for (int j = 0; j < 9; ++j) {
+            const int xx = x + d2_ex(j), yy = y + d2_ey(j);
+            lam[j] = 0.f;
+            if (xx < 0 || xx >= nx || yy < 0 || yy >= ny) continue;
+            float a[9][1], d[9][1];
+            for (int i = 0; i < 9; ++i) a[i][0] = __ldg(ain + i * plane + (yy + 1) * pitch + xx);
+            const float v = node_row_terms<float, 1>(pb, c, a, 0, __ldg(g.theta_t + yy * pitch + xx),
+                                                     __ldg(g.theta_t1 + yy * pitch + xx), mask(xx, yy), j == 0, d, sums);
+            if (j == 0) nu = v;
+#pragma unroll
+            for (int i = 0; i < 9; ++i)
+                if (i == j) lam[j] = d[i][0];
+        }
+        for (int j = 0; j < 9; ++j) aout[j * plane + at] = nu + lam[j];
+        const unsigned bmask = mask(x, y);
+        const unsigned unk = ((bmask & 1u) ? 0x122u : 0u) | ((bmask & 2u) ? 0x0c8u : 0u) | ((bmask & 4u) ? 0x064u : 0u) |
+                             ((bmask & 8u) ? 0x190u : 0u);
+        if (unk && adj_has_links(pb, bmask, unk)) {
+            double a[9], link[9];
+            for (int i = 0; i < 9; ++i) {
+                a[i] = (double)__ldg(ain + i * plane + at);
+                link[i] = 0.0;
+            }
+            const NodeTerms t = node_terms(pb, a, link, g.theta_t[y * pitch + x], g.theta_t1[y * pitch + x], x, y);
+            for (int j = 1; j < 9; ++j)
+                if ((t.link_mask >> j) & 1) aout[j * plane + at] = (float)(t.nu + link[j]);
+        }
+    }
+    for (int w = 0; w < 4; ++w) {
+        if (pb.wall_kind[w] != 1) continue;
+        const double v = warp_sum(sums.wall[(1 + w) * kWarpsPerBlock * 32]);
+        if ((tid & 31) == 0 && v != 0.0) acc_add(&st->g_wall[w], v);
+    }
+    const double v = warp_sum((double)sums.gs + sums.wall[0]);
+    if ((tid & 31) == 0 && v != 0.0) acc_add(&st->g_ste, v);
+}
+
 // ---------------------------------------------------------------- seed and finish
 template <int Q, typename P>
 __global__ void adj_seed_kernel(const Problem* dprob, const double* __restrict__ thT, const double* __restrict__ target,
@@ -726,6 +878,14 @@ cudaError_t launch_adj_seed(int precision, const Problem* dprob, const Problem& 
 
 cudaError_t launch_adj_step(int precision, const AdjArgs& a, const Problem& hp, cudaStream_t s)
 {
+    if (hp.q == 9 && precision == 1 && hp.plane * 9 < 1ll << 31) {   // (32-bit indices)
+        const int ntx = hp.nx > 4 ? (hp.nx - 4 + kAdjFlatW - 1) / kAdjFlatW : 0;
+        const int nty = hp.ny > 4 ? (hp.ny - 4 + kAdjFlatH - 1) / kAdjFlatH : 0;
+        const long long ring = (long long)std::min(4, hp.ny) * hp.nx + (long long)std::min(4, hp.nx) * std::max(0, hp.ny - 4);
+        const int edge = (int)((ring + kWarpsPerBlock * 32 - 1) / (kWarpsPerBlock * 32));
+        adj_flat_kernel<<<ntx * nty + edge, kAdjFlatThreads, 0, s>>>(a, ntx, ntx * nty);
+        return cudaGetLastError();
+    }
     if (hp.q == 9) {
         const int blocks = (a.ntiles + kWarpsPerBlock - 1) / kWarpsPerBlock;
         if (precision == 1) adj_march_kernel<float><<<blocks, kWarpsPerBlock * 32, 0, s>>>(a);
