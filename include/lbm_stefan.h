@@ -9,7 +9,7 @@
  * streaming, the boundary closures of Sec. 4.2 on q, the zeroth moment, the
  * local Newton solve of Eq. (14), the source of Eq. (13), and the next
  * collision.  D2Q9 and D2Q5 lattices up to 2^25 nodes (FP32 D2Q9; its EEBM
- * 2^23) or 2^31 elements of a state (the other forms) run all the steps of a
+ * 2^24) or 2^31 elements of a state (the other forms) run all the steps of a
  * call, up to 8,192, in one cooperative launch whose blocks stay on the GPU and
  * meet at a barrier after every step.  Kernel launches per step otherwise: D2Q9 with FP32 populations, four on
  * the legacy default stream (the nodes on or next to a wall in two, rows 1 .. ny-2

@@ -475,14 +475,14 @@ static cudaError_t run_resident(lbm_stefan* h, int nsteps, int parity, double* r
 #define LBM_RESIDENT 1
 #endif
 // The largest lattice that steps in resident launches (measured us per step, separate
-// kernels / resident).  FP32 D2Q9 IREBM: 235 / 231 at 4096^2, 850 / 871 at 8192^2; EEBM,
-// which has no Newton work to hide: 69 / 60 at 2048^2, 202 / 215 at 4096^2.  FP64 and
-// D2Q5 gain at every size (D2Q9 FP64 966 / 658 and D2Q5 FP32 183 / 128 at 4096^2): the
-// bound is that of the 32-bit indices, 2^31 elements of a state.
+// kernels / resident).  FP32 D2Q9 IREBM: 235 / 221 at 4096^2, 473 / 443 at 8192 x 4096,
+// 849 / 855 at 8192^2; EEBM, which has no Newton work to hide: 69 / 56 at 2048^2, 202 / 201
+// at 4096^2.  FP64 and D2Q5 gain at every size (D2Q9 FP64 966 / 658 and D2Q5 FP32 183 / 128
+// at 4096^2): the bound is that of the 32-bit indices, 2^31 elements of a state.
 static long long resident_max_nodes(int lattice, int precision, int method)
 {
     if (!LBM_RESIDENT) return 0;
-    if (lattice == LBM_D2Q9 && precision == LBM_FP32) return method == LBM_EEBM ? 1ll << 23 : 1ll << 25;
+    if (lattice == LBM_D2Q9 && precision == LBM_FP32) return method == LBM_EEBM ? 1ll << 24 : 1ll << 25;
     return 1ll << 31;
 }
 

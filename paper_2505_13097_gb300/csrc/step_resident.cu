@@ -40,12 +40,6 @@
 #include "d2q9_row.cuh"
 #include "resident.cuh"
 
-#ifndef LBM_RES_TF
-#define LBM_RES_TF 768
-#endif
-#ifndef LBM_RES_TD
-#define LBM_RES_TD 640
-#endif
 #ifndef LBM_RES_SCALAR
 #define LBM_RES_SCALAR 8
 #endif
@@ -311,8 +305,10 @@ __device__ __forceinline__ void ld4(const float* p, float (&v)[4])
 }
 
 // The queue (dynamic shared memory) has room for every node of kResidentWaves
-// waves of the first pass; the second pass follows that many waves.
-constexpr int kResidentWaves = 8;
+// waves of the first pass; the second pass follows that many waves.  FP32: 64 and
+// 96 KB; more costs L1 (4096^2 with 16 waves 232 us instead of 220), FP64 48 KB
+// (2048^2 with 8 / 16 waves: 161 / 154 us).
+template <typename P> constexpr int kResidentWaves = sizeof(P) == 4 ? 8 : 16;
 
 struct ResidentQueue {
     unsigned count;
@@ -518,13 +514,17 @@ __device__ __forceinline__ void plain_update(const ResidentArgs& a, const double
     }
 }
 
-// One block of a size that leaves 80 (FP32) or 96 (FP64) registers a thread.
-template <typename P> constexpr int kResidentThreads = sizeof(P) == 4 ? LBM_RES_TF : LBM_RES_TD;
+// One block per SM.  D2Q9 in FP32: 512 threads leave 128 registers, without spills,
+// and 16 warps take two 8-row tiles at a time (us per step with 768 / 512 threads:
+// 4096^2 227 / 221, EEBM 2048^2 60 / 56); D2Q5 in FP32 streams less per node and wants
+// the warps (4096^2, 768 / 640: 127 / 141), and so does FP64, whose sums are integer
+// work beside the FP64 pipe (2048^2, 768 / 640: 161 / 180).
+template <typename P, int Q> constexpr int kResidentThreads = sizeof(P) == 4 && Q == 9 ? 512 : 768;
 
 template <typename P, int Q, bool EEBM>
-__global__ void __launch_bounds__(kResidentThreads<P>, 1) resident_kernel(const __grid_constant__ ResidentArgs a)
+__global__ void __launch_bounds__(kResidentThreads<P, Q>, 1) resident_kernel(const __grid_constant__ ResidentArgs a)
 {
-    __shared__ ResidentSlot wsum[2][kResidentThreads<P> / 32];   // by step parity
+    __shared__ ResidentSlot wsum[2][kResidentThreads<P, Q> / 32];   // by step parity
     __shared__ ResidentQueue queue;
     extern __shared__ unsigned queue_nodes[];
     __shared__ unsigned next_item;
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(kResidentThreads<P>, 1) resident_kernel(const 
             unsigned own = a.items > (int)blockIdx.x ? (unsigned)(a.items - 1 - (int)blockIdx.x) / nb + 1u : 0u;
             int place = blockIdx.x, t0 = 0;
             do {
-                for (int k = 0; k < kResidentWaves && t0 < a.tiles; ++k, t0 += nb * g) {
+                for (int k = 0; k < kResidentWaves<P> && t0 < a.tiles; ++k, t0 += nb * g) {
                     // a wave: g tiles of every block, the tiles of a strip dealt round the blocks
                     const int t = t0 + warp / a.th * nb + place;
                     place += a.rot;
@@ -638,10 +638,10 @@ __global__ void __launch_bounds__(kResidentThreads<P>, 1) resident_kernel(const 
 
 // ---------------------------------------------------------------- launch
 // the queue of a block with a first pass
-template <typename P>
+template <typename P, int Q>
 static size_t resident_smem(bool first_pass)
 {
-    return first_pass ? sizeof(unsigned) * kResidentWaves * kResidentThreads<P> * (sizeof(P) == 4 ? 4 : 1) : 0;
+    return first_pass ? sizeof(unsigned) * kResidentWaves<P> * kResidentThreads<P, Q> * (sizeof(P) == 4 ? 4 : 1) : 0;
 }
 
 template <typename P, int Q, bool EEBM>
@@ -651,9 +651,9 @@ static cudaError_t resident_go(ResidentArgs& a, int nblocks, int threads, cudaSt
     cfg.gridDim = dim3((unsigned)nblocks);
     cfg.blockDim = dim3((unsigned)threads);
     cfg.stream = s;
-    cfg.dynamicSmemBytes = resident_smem<P>(a.tiles > 0);
+    cfg.dynamicSmemBytes = resident_smem<P, Q>(a.tiles > 0);
     const cudaError_t e = cudaFuncSetAttribute(resident_kernel<P, Q, EEBM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)resident_smem<P>(true));
+                                               (int)resident_smem<P, Q>(true));
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeCooperative;   // every block resident: they wait on one another
@@ -670,9 +670,9 @@ static int resident_capacity_t()
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaFuncSetAttribute(resident_kernel<P, Q, EEBM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)resident_smem<P>(true)) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, resident_kernel<P, Q, EEBM>, kResidentThreads<P>,
-                                                      resident_smem<P>(true)) != cudaSuccess)
+                             (int)resident_smem<P, Q>(true)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, resident_kernel<P, Q, EEBM>, kResidentThreads<P, Q>,
+                                                      resident_smem<P, Q>(true)) != cudaSuccess)
         return 0;
     return sms * per;
 }
@@ -683,7 +683,7 @@ static ResidentPlan resident_plan_t(int nx, int ny)
     ResidentPlan r;
     const int cap = std::min(resident_capacity_t<P, Q, false>(), resident_capacity_t<P, Q, true>());
     if (cap < 2 || nx >= 65536 || ny >= 65536) return r;
-    const int most = kResidentThreads<P> / 32, N = sizeof(P) == 4 ? 4 : 1;
+    const int most = kResidentThreads<P, Q> / 32, N = sizeof(P) == 4 ? 4 : 1;
     r.nseg = (nx + 31) / 32;
     const long long units = (long long)r.nseg * ny;
     const long long vec = ny > 2 ? (long long)((nx + 32 * N - 1) / (32 * N)) * (ny - 2) : 0;
@@ -701,7 +701,10 @@ static ResidentPlan resident_plan_t(int nx, int ny)
         r.tiles = r.strips * ((ny - 2 + r.th - 1) / r.th);
         r.items = 2 * r.nseg + (ny - 2 + 32 / (2 * N) - 1) / (32 / (2 * N));
         r.blocks = cap;
-        r.threads = most * 32;
+        // as many warps as the waves need, so that all have as many units
+        const long long waves = (vec + (long long)(cap - 1) * most - 1) / ((long long)(cap - 1) * most);
+        const long long per = (vec + (cap - 1) * waves - 1) / ((cap - 1) * waves);
+        r.threads = 32 * (int)std::min<long long>(most, (per + r.th - 1) / r.th * r.th);
     }
     r.slots = kResidentRing * (size_t)(r.blocks - 1);
     r.rot = (int)(0.618 * (r.blocks - 1));
