@@ -245,6 +245,13 @@ size_t resident_slot_bytes();
 cudaError_t launch_resident(int precision, const ResidentPlan& plan, const Problem& hp, int parity, int nsteps, double* rec,
                             DevStats* stats, void* slots, ResidentBar* bar, long long wait_ns, cudaStream_t s);
 
+// FP32 D2Q9 batches in one cooperative launch; units: (problem, kind, strip or side,
+// first row); sums: resident_batch_bytes, zero before the first launch
+int resident_batch_blocks();
+size_t resident_batch_bytes(int count);
+cudaError_t launch_resident_batch(const Problem* probs, int count, const int4* units, int nunits, int blocks, int parity,
+                                  int nsteps, DevStats* stats, void* sums, ResidentBar* bar, long long wait_ns, cudaStream_t s);
+
 // D2Q5 launchers (step_d2q5.cu): one tile per warp over a.nslots tiles
 cudaError_t launch_d2q5_step(int precision, const StepArgs& a, cudaStream_t s);
 int d2q5_segment_width(int precision);   // nodes per warp segment

@@ -149,6 +149,11 @@ struct lbm_stefan_batch {
     cudaStream_t side = nullptr;       // split step (stream of its own): the left halves' Newton solves
     cudaEvent_t ev_fork = nullptr, ev_half = nullptr, ev_join = nullptr;
     cudaEvent_t ev_walls = nullptr;   // split step: the wall kernels are done (list A's wall part is final)
+    int res_blocks = 0;               // FP32: steps in resident launches of this many blocks (0: separate kernels)
+    int4* dunits = nullptr;            // their units, a problem's in a row: column groups, wall rows, tiles
+    int nunits = 0;
+    void* dsums = nullptr;
+    lbm::ResidentBar* dbar = nullptr;
     GraphCache graph;
 };
 
@@ -1302,6 +1307,24 @@ static lbm_status batch_build_flat_tables(lbm_stefan_batch* b, int schedule)
             rows.push_back(make_int2(k, 2 * seg + 1));
         }
     }
+    std::vector<int4> units;
+    if (b->res_blocks > 0)
+        for (int k : order) {
+            const Problem& pb = b->hp[k];
+            const int nsegs = pb.pitch / lbm::kTmaW;
+            for (int y0 = 1; y0 < pb.ny - 1; y0 += 32) units.push_back(make_int4(k, 2, 0, y0));
+            for (int seg = 0; seg < nsegs; ++seg)
+                for (int y : {0, pb.ny - 1}) units.push_back(make_int4(k, 1, seg, y));
+            for (int y0 = 0; y0 < pb.ny - 1 && pb.ny > 2; y0 += 8)
+                for (int seg = 0; seg < nsegs; ++seg) units.push_back(make_int4(k, 0, seg, y0));
+        }
+    cudaFree(b->dunits);
+    b->dunits = nullptr;
+    if (!units.empty()) {
+        CUDA_TRY(cudaMalloc(&b->dunits, sizeof(int4) * units.size()));
+        CUDA_TRY(cudaMemcpy(b->dunits, units.data(), sizeof(int4) * units.size(), cudaMemcpyHostToDevice));
+    }
+    b->nunits = (int)units.size();
     cudaFree(b->dftiles);
     cudaFree(b->dwrows);
     cudaFree(b->dcrows);
@@ -1438,6 +1461,28 @@ static cudaError_t batch_launch_one(lbm_stefan_batch* b, int parity)
                                    b->stream);
 }
 
+// nsteps steps by resident launches; false with *e == cudaSuccess: take the separate
+// kernels (the batch has none, or the grid does not fit here and nothing ran).
+static bool batch_run_resident(lbm_stefan_batch* b, int nsteps, cudaError_t* e)
+{
+    *e = cudaSuccess;
+    while (b->res_blocks > 0 && nsteps > 0) {
+        const int n = std::min(nsteps, kResidentSteps);
+        *e = lbm::launch_resident_batch(b->dprobs, b->count, b->dunits, b->nunits, b->res_blocks, b->parity, n, b->dstats,
+                                        b->dsums, b->dbar, kResidentWaitNs, b->stream);
+        if (*e == cudaErrorCooperativeLaunchTooLarge) {
+            (void)cudaGetLastError();
+            *e = cudaSuccess;
+            b->res_blocks = 0;
+            return false;
+        }
+        if (*e != cudaSuccess) return false;
+        b->parity ^= n & 1;
+        nsteps -= n;
+    }
+    return b->res_blocks > 0;
+}
+
 extern "C" lbm_status lbm_stefan_batch_create(int count, const lbm_stefan_problem* probs, int precision,
                                               double newton_tol, int newton_max_iter, void* cuda_stream,
                                               lbm_stefan_batch** out)
@@ -1517,6 +1562,22 @@ extern "C" lbm_status lbm_stefan_batch_create(int count, const lbm_stefan_proble
         base += 2 * sz;
     }
     b->use_flat = precision == LBM_FP32;
+    if (b->use_flat && LBM_RESIDENT) {
+        bool fits = true;   // 32-bit indices, 16-bit coordinates
+        for (const Problem& pb : b->hp) fits = fits && 9 * pb.plane < 1ll << 31 && pb.nx < 65536 && pb.ny < 65536;
+        if (fits) b->res_blocks = lbm::resident_batch_blocks();
+        if (b->res_blocks < 2) b->res_blocks = 0;
+    }
+    if (b->res_blocks > 0) {
+        e = cudaMalloc(&b->dsums, lbm::resident_batch_bytes(count));
+        if (e == cudaSuccess) e = cudaMemset(b->dsums, 0, lbm::resident_batch_bytes(count));
+        if (e == cudaSuccess) e = cudaMalloc(&b->dbar, sizeof(lbm::ResidentBar));
+        if (e == cudaSuccess) e = cudaMemset(b->dbar, 0, sizeof(lbm::ResidentBar));
+        if (e != cudaSuccess) {
+            lbm_stefan_batch_destroy(b);
+            return fail(LBM_ERR_CUDA, "batch allocation failed: %s", cudaGetErrorString(e));
+        }
+    }
     cudaGetLastError();
     lbm_status s = batch_build_schedule(b, 16, 1);
     if (s != LBM_OK) {
@@ -1569,6 +1630,9 @@ extern "C" lbm_status lbm_stefan_batch_step(lbm_stefan_batch* b, int nsteps)
     NvtxRange r("lbm_stefan_batch_step");
     if (!b) return fail(LBM_ERR_ARG, "NULL handle");
     if (nsteps < 0) return fail(LBM_ERR_ARG, "nsteps must be >= 0");
+    cudaError_t re;
+    if (batch_run_resident(b, nsteps, &re)) return LBM_OK;
+    CUDA_TRY(re);
     int left = nsteps;
     if (b->parity == 1 && left > 0) {
         CUDA_TRY(batch_launch_one(b, 1));
@@ -1671,13 +1735,18 @@ extern "C" lbm_status lbm_stefan_batch_autotune(lbm_stefan_batch* b, int trial_s
             st = batch_build_schedule(b, hs, sc);
             if (st != LBM_OK) break;
             // one untimed warm-up step, then the timed trial
-            if (batch_launch_one(b, b->parity) != cudaSuccess) { st = fail(LBM_ERR_CUDA, "autotune launch failed"); break; }
-            b->parity ^= 1;
+            auto trial = [&](int n) -> bool {
+                cudaError_t re;
+                if (batch_run_resident(b, n, &re)) return true;
+                for (int k = 0; k < n && re == cudaSuccess; ++k) {
+                    re = batch_launch_one(b, b->parity);
+                    b->parity ^= 1;
+                }
+                return re == cudaSuccess;
+            };
+            if (!trial(1)) { st = fail(LBM_ERR_CUDA, "autotune launch failed"); break; }
             cudaEventRecord(e0, b->stream);
-            for (int k = 0; k < trial_steps; ++k) {
-                if (batch_launch_one(b, b->parity) != cudaSuccess) { st = fail(LBM_ERR_CUDA, "autotune launch failed"); break; }
-                b->parity ^= 1;
-            }
+            if (!trial(trial_steps)) { st = fail(LBM_ERR_CUDA, "autotune launch failed"); break; }
             cudaEventRecord(e1, b->stream);
             cudaEventSynchronize(e1);
             float ms = 0.f;
@@ -1719,6 +1788,9 @@ extern "C" void lbm_stefan_batch_destroy(lbm_stefan_batch* b)
     cudaFree(b->dftiles);
     cudaFree(b->dwrows);
     cudaFree(b->dcrows);
+    cudaFree(b->dunits);
+    cudaFree(b->dsums);
+    cudaFree(b->dbar);
     if (b->ev_fork) cudaEventDestroy(b->ev_fork);
     if (b->ev_half) cudaEventDestroy(b->ev_half);
     if (b->ev_join) cudaEventDestroy(b->ev_join);

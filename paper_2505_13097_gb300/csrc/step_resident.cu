@@ -86,10 +86,9 @@ template <> struct LaneAcc<double> {
 // valid).  w: the warp's sums in shared memory, where lane 0 adds what few
 // items have.  A resident state has fewer than 2^31 elements (32-bit indices).
 template <typename P, int Q, bool EEBM>
-__device__ __forceinline__ void item_update(const ResidentArgs& a, const P* src, P* dst, double* rec, int x, int y,
+__device__ __forceinline__ void item_update(const Problem& pb, DevStats* st, const P* src, P* dst, double* rec, int x, int y,
                                             bool valid, int lane, float sh, LaneAcc<P>& acc, ResidentSlot* w)
 {
-    const Problem& pb = a.pb;
     const int nx = pb.nx, ny = pb.ny, pitch = pb.pitch, plane = (int)pb.plane;
     const int at = (y + 1) * pitch + x;
     P u[Q], q[Q];
@@ -255,7 +254,7 @@ __device__ __forceinline__ void item_update(const ResidentArgs& a, const P* src,
                 tt = sum_q<Q>(u);
             }
             const NewtonNode nr = newton_mixed(mm, tt, shd, shz, pb);
-            if (!nr.ok) atomicCAS(&a.stats->error, 0, 3);
+            if (!nr.ok) atomicCAS(&st->error, 0, 3);
             tn = nr.tns + shd;
             c = (P)fma(-pb.omc, mm, nr.tns);
             e = to_fixed(nr.ens);   // FP32: less the shift
@@ -316,11 +315,10 @@ struct ResidentQueue {
 };
 
 template <int Q, bool EEBM>
-__device__ __forceinline__ void plain_update(const ResidentArgs& a, const float* src, float* dst, double* rec, int x0,
+__device__ __forceinline__ void plain_update(const Problem& pb, const float* src, float* dst, double* rec, int x0,
                                              int y, int lane, float sh, LaneAcc<float>& acc, ResidentSlot* w,
                                              ResidentQueue* queue)
 {
-    const Problem& pb = a.pb;
     const int nx = pb.nx, pitch = pb.pitch, plane = (int)pb.plane;
     const int at = (y + 1) * pitch + x0;
     const bool cold = x0 == 0 || x0 + 3 >= nx - 1;
@@ -455,11 +453,10 @@ __device__ __forceinline__ void plain_update(const ResidentArgs& a, const float*
 
 // FP64: one column per lane.
 template <int Q, bool EEBM>
-__device__ __forceinline__ void plain_update(const ResidentArgs& a, const double* src, double* dst, double* rec, int x,
+__device__ __forceinline__ void plain_update(const Problem& pb, const double* src, double* dst, double* rec, int x,
                                              int y, int lane, float sh, LaneAcc<double>& acc, ResidentSlot* w,
                                              ResidentQueue* queue)
 {
-    const Problem& pb = a.pb;
     const int nx = pb.nx, pitch = pb.pitch, plane = (int)pb.plane;
     const int at = (y + 1) * pitch + x;
     const bool cold = x == 0 || x >= nx - 1;
@@ -571,7 +568,7 @@ __global__ void __launch_bounds__(kResidentThreads<P, Q>, 1) resident_kernel(con
                     const int strip = t / row_tiles;
                     const int y = 1 + (t - strip * row_tiles) * a.th + warp % a.th;
                     const int x0 = (strip * 32 + lane) * N;
-                    if (y < ny - 1) plain_update<Q, EEBM>(a, src, dst, rec, x0, y, lane, sh, acc, w, &queue);
+                    if (y < ny - 1) plain_update<Q, EEBM>(pb, src, dst, rec, x0, y, lane, sh, acc, w, &queue);
                 }
                 if (a.tiles) __syncthreads();
                 const unsigned queued = queue.count;
@@ -604,7 +601,7 @@ __global__ void __launch_bounds__(kResidentThreads<P, Q>, 1) resident_kernel(con
                             y = (int)(n >> 16);
                         }
                     }
-                    item_update<P, Q, EEBM>(a, src, dst, rec, x, y, valid, lane, sh, acc, w);
+                    item_update<P, Q, EEBM>(pb, a.stats, src, dst, rec, x, y, valid, lane, sh, acc, w);
                     // the first items are dealt, the others taken
                     if (total <= (unsigned)nwb) break;
                     if (lane == 0) it = (unsigned)nwb + atomicAdd(&next_item, 1u);
@@ -634,6 +631,220 @@ __global__ void __launch_bounds__(kResidentThreads<P, Q>, 1) resident_kernel(con
         if (threadIdx.x == 0) bar_arrive(&a.bar->count);   // the last step's sums are out
     }
     bar_leave(a.bar);
+}
+
+// ---------------------------------------------------------------- batches, FP32 D2Q9
+// Many problems in one resident launch.  A warp takes a whole unit of one
+// problem: a tile of 128 columns x 8 rows, whose nodes to solve it queues for
+// itself and solves right after the rows (280 of a vertical front's tile fill
+// nine warps' worth densely), so that solves, bound by latency and the FP64 pipe,
+// and streaming run side by side on every SM; a stretch of an S or N row; or 32
+// rows of the W and E column groups.  Sums go to the unit's problem by atomics,
+// in sets by step parity that the statistics block reads, clears and publishes
+// while the next step runs.  256 problems of 64^2 to 1024^2 (58.6 M nodes, 3.9 M of
+// them solved), us per step: 1,440 by separate kernels, whose solves came after the
+// streaming for the most part; 1,320 here with the units dealt to the warps, 1,025
+// with a counter per block (a front's tile lasts several times a plain one's).
+struct ResidentBatchArgs : ResidentCommon {
+    const Problem* probs;
+    int count;                  // problems
+    const int4* units;          // (problem, kind: 0 tile, 1 row, 2 column groups; strip or side; first row)
+    int nunits, parity;
+    StepStripe* acc;            // 2 x count x kBatchStripes
+    int* maxit;                 // 2 x count
+};
+
+constexpr int kBatchThreads = 512, kBatchWarps = kBatchThreads / 32;
+constexpr int kBatchStripes = 4;
+
+// Adds the warp's sums to its problem's and clears them.
+__device__ __forceinline__ void batch_flush(StepStripe* c, int* maxit, LaneAcc<float>& acc, ResidentSlot* w, int lane)
+{
+    const Fx e = acc.total();
+    acc = LaneAcc<float>{};
+    if (lane == 0) {
+        fx_add(w->e, e);
+        acc_add_fx(&c->energy, w->e);
+        acc_add_fx(&c->flux, w->f);
+        if (w->liquid) atomicAdd(&c->liquid, (unsigned long long)w->liquid);
+        if (w->shifted) atomicAdd(&c->shifted, (unsigned long long)w->shifted);
+        for (int k = 0; k < 4; ++k)
+            if (w->dir[k]) atomicAdd(&c->dir[k], (unsigned long long)w->dir[k]);
+        if (w->newton) {
+            atomicAdd(&c->newton, (unsigned long long)w->newton);
+            atomicAdd(&c->iters, (unsigned long long)w->iters);
+            atomicMax(maxit, w->maxit);
+        }
+        *w = ResidentSlot{};
+    }
+    __syncwarp();
+}
+
+// The statistics block: a thread per problem.
+static __device__ __noinline__ void batch_stats(const ResidentBatchArgs& a, unsigned nb, bool* ok_s)
+{
+    bool ok = true;
+    for (int s = 0; ok && s < a.nsteps; ++s) {
+        if (threadIdx.x == 0) *ok_s = bar_wait(a.bar, &a.bar->count, (unsigned)(s + 1) * nb, a.wait_ns);
+        __syncthreads();
+        ok = *ok_s;
+        if (!ok) break;
+        for (int p = threadIdx.x; p < a.count; p += blockDim.x) {
+            StepStripe* c = a.acc + ((size_t)(s & 1) * a.count + p) * kBatchStripes;
+            int* mx = a.maxit + (size_t)(s & 1) * a.count + p;
+            StatSums t = {};
+            for (int k = 0; k < kBatchStripes; ++k) stripe_take(c + k, t);
+            DevStats* st = &a.stats[a.probs[p].stats];
+            st->cur_maxit = *reinterpret_cast<volatile int*>(mx);
+            *reinterpret_cast<volatile int*>(mx) = 0;
+            __threadfence();
+            publish_totals(st, &a.probs[p], t);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) bar_arrive(&a.bar->read[0]);   // the step's set is read and clear
+    }
+    if (!ok && threadIdx.x == 0)
+        for (int p = 0; p < a.count; ++p) atomicExch(&a.stats[p].error, 4);   // LBM_ERR_TIMEOUT
+}
+
+__global__ void __launch_bounds__(kBatchThreads, 1) resident_batch_kernel(const __grid_constant__ ResidentBatchArgs a)
+{
+    __shared__ ResidentSlot wsum[kBatchWarps];
+    __shared__ ResidentQueue queues[kBatchWarps];
+    __shared__ unsigned next_unit;
+    __shared__ bool ok_s;
+    extern __shared__ unsigned batch_nodes[];   // 1,024 per warp: a tile's nodes
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nb = gridDim.x - 1;   // computing blocks; the last block publishes the statistics
+    if ((int)blockIdx.x == nb) {
+        batch_stats(a, (unsigned)nb, &ok_s);
+        bar_leave(a.bar);
+        return;
+    }
+    ResidentSlot* w = &wsum[warp];
+    ResidentQueue* queue = &queues[warp];
+    if (lane == 0) {
+        *w = ResidentSlot{};
+        queue->count = 0u;
+        queue->node = batch_nodes + warp * 1024;
+        next_unit = 0u;
+    }
+    __syncthreads();
+    const int rot = (int)(0.618f * nb);
+    bool ok = true;
+    for (int s = 0; ok && s < a.nsteps; ++s) {
+        const int p = (a.parity + s) & 1;
+        LaneAcc<float> acc;
+        // a block's units are dealt (one of every nb in a row, at a rotating place) and its warps
+        // take them from a counter: a front's tile lasts several times a plain one's
+        for (;;) {
+            unsigned i = 0;
+            if (lane == 0) i = atomicAdd(&next_unit, 1u);
+            i = __shfl_sync(kFull, i, 0);
+            const int u = (int)i * nb + (int)((blockIdx.x + i * (unsigned)rot) % (unsigned)nb);
+            if ((int)i * nb >= a.nunits) break;
+            if (u >= a.nunits) continue;
+            const int4 e = __ldg(a.units + u);
+            const Problem& pb = a.probs[e.x];
+            DevStats* st = &a.stats[pb.stats];
+            const float* src = static_cast<const float*>(pb.state[p]);
+            float* dst = static_cast<float*>(pb.state[p ^ 1]);
+            const float sh = state_shift(pb, 0);   // the same in both buffers
+            const int nx = pb.nx, ny = pb.ny;
+            if (e.y == 0) {
+                const int x0 = e.z * 128 + 4 * lane;
+                for (int y = max(e.w, 1); y < min(e.w + 8, ny - 1); ++y)
+                    plain_update<9, false>(pb, src, dst, nullptr, x0, y, lane, sh, acc, w, queue);
+                __syncwarp();
+            }
+            // the items: the tile's queue; 4 stretches of 32 nodes of a row; 8 times 4 rows of the
+            // W and E column groups
+            const unsigned queued = e.y == 0 ? queue->count : 0u;
+            const int items = e.y == 0 ? (int)((queued + 31u) / 32u) : (e.y == 1 ? 4 : 8);
+            const int xe = max(4, (nx - 1) / 4 * 4);
+            for (int i = 0; i < items; ++i) {
+                int x, y;
+                bool valid;
+                if (e.y == 0) {
+                    const unsigned j = (unsigned)(i * 32 + lane);
+                    valid = j < queued;
+                    const unsigned n = valid ? queue->node[j] : 0u;
+                    x = (int)(n & 0xffffu);
+                    y = (int)(n >> 16);
+                } else if (e.y == 1) {
+                    x = e.z * 128 + i * 32 + lane;
+                    y = e.w;
+                    valid = x < nx;
+                } else {
+                    const int k = lane & 7;
+                    y = e.w + 4 * i + (lane >> 3);
+                    x = k < 4 ? k : xe + k - 4;
+                    valid = y < ny - 1 && x < nx;
+                }
+                if (!__any_sync(kFull, valid)) continue;
+                item_update<float, 9, false>(pb, st, src, dst, nullptr, x, y, valid, lane, sh, acc, w);
+            }
+            __syncwarp();
+            if (lane == 0) queue->count = 0u;
+            const size_t c = (size_t)(s & 1) * a.count + e.x;
+            batch_flush(a.acc + c * kBatchStripes + u % kBatchStripes, a.maxit + c, acc, w, lane);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            next_unit = 0u;
+            bar_arrive(&a.bar->count);
+            // the next step adds to the set of step s - 1
+            ok_s = s + 1 == a.nsteps || (bar_wait(a.bar, &a.bar->count, (unsigned)(s + 1) * nb, a.wait_ns) &&
+                                         bar_wait(a.bar, &a.bar->read[0], (unsigned)s, a.wait_ns));
+        }
+        __syncthreads();
+        ok = ok_s;
+    }
+    bar_leave(a.bar);
+}
+
+static size_t batch_smem() { return sizeof(unsigned) * 1024 * kBatchWarps; }
+
+int resident_batch_blocks()
+{
+    int dev = 0, sms = 0, per = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(resident_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)batch_smem()) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, resident_batch_kernel, kBatchThreads, batch_smem()) != cudaSuccess)
+        return 0;
+    return sms * per;
+}
+
+size_t resident_batch_bytes(int count) { return (size_t)2 * count * (kBatchStripes * sizeof(StepStripe) + sizeof(int)); }
+
+cudaError_t launch_resident_batch(const Problem* probs, int count, const int4* units, int nunits, int blocks, int parity,
+                                  int nsteps, DevStats* stats, void* sums, ResidentBar* bar, long long wait_ns, cudaStream_t s)
+{
+    ResidentBatchArgs a;
+    a.nsteps = nsteps;
+    a.stats = stats;
+    a.slots = nullptr;
+    a.bar = bar;
+    a.wait_ns = wait_ns;
+    a.probs = probs;
+    a.count = count;
+    a.units = units;
+    a.nunits = nunits;
+    a.parity = parity;
+    a.acc = static_cast<StepStripe*>(sums);
+    a.maxit = reinterpret_cast<int*>(a.acc + (size_t)2 * count * kBatchStripes);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kBatchThreads);
+    cfg.dynamicSmemBytes = batch_smem();
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;   // every block resident: they wait on one another
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, resident_batch_kernel, a);
 }
 
 // ---------------------------------------------------------------- launch
