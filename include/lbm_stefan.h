@@ -10,8 +10,9 @@
  * local Newton solve of Eq. (14), the source of Eq. (13), and the next
  * collision.  D2Q9 and D2Q5 lattices up to 2^25 nodes (FP32 D2Q9; its EEBM
  * 2^24) or 2^31 elements of a state (the other forms) run all the steps of a
- * call, up to 8,192, in one cooperative launch whose blocks stay on the GPU and
- * meet at a barrier after every step.  Kernel launches per step otherwise: D2Q9 with FP32 populations, four on
+ * call in cooperative launches (of up to 2^32 node updates and 8,192 steps) whose
+ * blocks stay on the GPU and meet at a barrier after every step; so do FP32
+ * batches.  Kernel launches per step otherwise: D2Q9 with FP32 populations, four on
  * the legacy default stream (the nodes on or next to a wall in two, rows 1 .. ny-2
  * of every 128-column strip, then the kernel that solves the list of nodes
  * that need the Newton iteration and publishes the step), six on a stream of

@@ -32,6 +32,8 @@
 //  * sums are fixed point, comparisons work on the bits, and a warp of its own
 //    adds up the statistics while the next step runs.
 // 801 nodes: 86 us per step with every node in every iteration.
+#include <algorithm>
+
 #include "resident.cuh"
 
 namespace lbm {
@@ -399,7 +401,7 @@ __device__ __forceinline__ bool inner_barrier(const Ilf2Args& a, unsigned turn, 
 }
 
 constexpr int kIlf2Threads = 512;
-constexpr int kIlf2Steps = 256;   // steps of one launch
+constexpr int kIlf2Steps = 256;   // steps of one launch, at most (and 2^24 node updates: some 50 ms)
 
 template <int Q>
 __global__ void __launch_bounds__(kIlf2Threads, 1) ilf2_kernel(const __grid_constant__ Ilf2Args a)
@@ -668,9 +670,10 @@ cudaError_t launch_ilfbm_2d(const Problem& hp, int parity, int nsteps, void* scr
     at[0].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
+    const int most = (int)std::max<size_t>(2, std::min<size_t>(kIlf2Steps, ((size_t)1 << 24) / n));
     while (nsteps > 0) {
         a.parity = parity;
-        a.nsteps = nsteps < kIlf2Steps ? nsteps : kIlf2Steps;
+        a.nsteps = nsteps < most ? nsteps : most;
         const cudaError_t e = hp.q == 9 ? cudaLaunchKernelEx(&cfg, ilf2_kernel<9>, a) : cudaLaunchKernelEx(&cfg, ilf2_kernel<5>, a);
         if (e != cudaSuccess) return e;
         parity ^= a.nsteps & 1;

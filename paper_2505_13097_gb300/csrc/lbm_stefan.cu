@@ -454,24 +454,34 @@ static cudaError_t launch_one(lbm_stefan* h, int parity, double* rec)
     return lbm::launch_d1q3_step(h->precision, a, h->hp, h->stream);
 }
 
-// Bound of a wait at the resident step's barrier, and the most steps of one launch.
+// Bound of a wait at the resident step's barrier.
 constexpr long long kResidentWaitNs = 5000000000LL;
-constexpr int kResidentSteps = 8192;
 
-// nsteps steps by resident launches from state[parity] on; theta' planes to
-// rec, if given.  cudaErrorCooperativeLaunchTooLarge (nothing ran): the grid
-// does not fit, take the separate kernels.
-static cudaError_t run_resident(lbm_stefan* h, int nsteps, int parity, double* rec)
+// Steps of one resident launch: 2^32 node updates (some 60 ms), so that other streams
+// get the GPU in between; at most 8,192.
+static int resident_steps(long long nodes) { return (int)std::max(32ll, std::min(8192ll, (1ll << 32) / std::max(1ll, nodes))); }
+
+// *nsteps steps by resident launches from state[*parity] on, theta' planes to *rec, if
+// given; the three advance with every launch.  cudaErrorCooperativeLaunchTooLarge: the grid
+// does not fit, take the separate kernels for the steps that are left.
+static cudaError_t run_resident(lbm_stefan* h, int* nsteps, int* parity, double** rec)
 {
     const long long plane = (long long)h->hp.ny * h->hp.pitch;
-    while (nsteps > 0) {
-        const int n = std::min(nsteps, kResidentSteps);
-        const cudaError_t e = lbm::launch_resident(h->precision, h->res, h->hp, parity, n, rec, h->dstats, h->dslots, h->dbar,
+    const int most = resident_steps((long long)h->hp.nx * h->hp.ny);
+    while (*nsteps > 0) {
+        const int n = std::min(*nsteps, most);
+        const cudaError_t e = lbm::launch_resident(h->precision, h->res, h->hp, *parity, n, *rec, h->dstats, h->dslots, h->dbar,
                                                    kResidentWaitNs, h->stream);
-        if (e != cudaSuccess) return e;
-        parity ^= n & 1;
-        nsteps -= n;
-        if (rec) rec += n * plane;
+        if (e != cudaSuccess) {
+            if (e == cudaErrorCooperativeLaunchTooLarge) {
+                (void)cudaGetLastError();
+                h->res.blocks = 0;
+            }
+            return e;
+        }
+        *parity ^= n & 1;
+        *nsteps -= n;
+        if (*rec) *rec += n * plane;
     }
     return cudaSuccess;
 }
@@ -818,18 +828,13 @@ extern "C" lbm_status lbm_stefan_step(lbm_stefan* h, int nsteps)
         h->parity ^= nsteps & 1;
         return LBM_OK;
     }
-    if (resident_on(h)) {
-        const cudaError_t e = run_resident(h, nsteps, h->parity, nullptr);
-        if (e == cudaSuccess) {
-            h->parity ^= nsteps & 1;
-            return LBM_OK;
-        }
-        if (e != cudaErrorCooperativeLaunchTooLarge) CUDA_TRY(e);
-        (void)cudaGetLastError();
-        h->res.blocks = 0;
-    }
     int left = nsteps;
-    if (h->parity == 1) {
+    if (resident_on(h)) {
+        double* no_rec = nullptr;
+        const cudaError_t e = run_resident(h, &left, &h->parity, &no_rec);
+        if (e != cudaErrorCooperativeLaunchTooLarge) CUDA_TRY(e);
+    }
+    if (h->parity == 1 && left > 0) {
         CUDA_TRY(launch_one(h, 1, nullptr));
         h->parity = 0;
         --left;
@@ -930,15 +935,9 @@ extern "C" lbm_status lbm_stefan_step_record(lbm_stefan* h, int nsteps, double* 
         h->parity ^= nsteps & 1;
         return LBM_OK;
     }
-    if (resident_on(h) && nsteps > 0) {
-        const cudaError_t e = run_resident(h, nsteps, h->parity, traj);
-        if (e == cudaSuccess) {
-            h->parity ^= nsteps & 1;
-            return LBM_OK;
-        }
+    if (resident_on(h)) {
+        const cudaError_t e = run_resident(h, &nsteps, &h->parity, &traj);
         if (e != cudaErrorCooperativeLaunchTooLarge) CUDA_TRY(e);
-        (void)cudaGetLastError();
-        h->res.blocks = 0;
     }
     for (int k = 0; k < nsteps; ++k) {
         CUDA_TRY(launch_one(h, h->parity, traj + k * plane));
@@ -1163,13 +1162,16 @@ static cudaError_t segment_launches(lbm_stefan* h, int nsteps, double* traj, voi
     cudaError_t e = lbm::launch_fields(h->precision, h->dprob, h->hp, parity0, nullptr, nullptr, nullptr, traj,
                                        h->stream);
     int par = parity0;
+    int left = nsteps;
+    double* rec = traj + plane;
     if (resident_on(h) && e == cudaSuccess) {
-        e = run_resident(h, nsteps, par, traj + plane);
-    } else {
-        for (int k = 0; k < nsteps && e == cudaSuccess; ++k) {
-            e = launch_one(h, par, traj + (k + 1) * plane);
-            par ^= 1;
-        }
+        e = run_resident(h, &left, &par, &rec);
+        if (e == cudaErrorCooperativeLaunchTooLarge) e = cudaSuccess;   // the steps that are left:
+    }
+    for (; left > 0 && e == cudaSuccess; --left) {
+        e = launch_one(h, par, rec);
+        par ^= 1;
+        rec += plane;
     }
     void* buf[2] = {a, b};
     int cur = 0;
@@ -1461,26 +1463,25 @@ static cudaError_t batch_launch_one(lbm_stefan_batch* b, int parity)
                                    b->stream);
 }
 
-// nsteps steps by resident launches; false with *e == cudaSuccess: take the separate
-// kernels (the batch has none, or the grid does not fit here and nothing ran).
-static bool batch_run_resident(lbm_stefan_batch* b, int nsteps, cudaError_t* e)
+// *nsteps steps by resident launches (none if the batch has none); what is left in
+// *nsteps with cudaSuccess is for the separate kernels (the grid does not fit here).
+static cudaError_t batch_run_resident(lbm_stefan_batch* b, int* nsteps)
 {
-    *e = cudaSuccess;
-    while (b->res_blocks > 0 && nsteps > 0) {
-        const int n = std::min(nsteps, kResidentSteps);
-        *e = lbm::launch_resident_batch(b->dprobs, b->count, b->dunits, b->nunits, b->res_blocks, b->parity, n, b->dstats,
-                                        b->dsums, b->dbar, kResidentWaitNs, b->stream);
-        if (*e == cudaErrorCooperativeLaunchTooLarge) {
+    const int most = resident_steps((long long)b->total_nodes);
+    while (b->res_blocks > 0 && *nsteps > 0) {
+        const int n = std::min(*nsteps, most);
+        const cudaError_t e = lbm::launch_resident_batch(b->dprobs, b->count, b->dunits, b->nunits, b->res_blocks, b->parity, n,
+                                                         b->dstats, b->dsums, b->dbar, kResidentWaitNs, b->stream);
+        if (e == cudaErrorCooperativeLaunchTooLarge) {
             (void)cudaGetLastError();
-            *e = cudaSuccess;
             b->res_blocks = 0;
-            return false;
+            break;
         }
-        if (*e != cudaSuccess) return false;
+        if (e != cudaSuccess) return e;
         b->parity ^= n & 1;
-        nsteps -= n;
+        *nsteps -= n;
     }
-    return b->res_blocks > 0;
+    return cudaSuccess;
 }
 
 extern "C" lbm_status lbm_stefan_batch_create(int count, const lbm_stefan_problem* probs, int precision,
@@ -1630,10 +1631,8 @@ extern "C" lbm_status lbm_stefan_batch_step(lbm_stefan_batch* b, int nsteps)
     NvtxRange r("lbm_stefan_batch_step");
     if (!b) return fail(LBM_ERR_ARG, "NULL handle");
     if (nsteps < 0) return fail(LBM_ERR_ARG, "nsteps must be >= 0");
-    cudaError_t re;
-    if (batch_run_resident(b, nsteps, &re)) return LBM_OK;
-    CUDA_TRY(re);
     int left = nsteps;
+    CUDA_TRY(batch_run_resident(b, &left));
     if (b->parity == 1 && left > 0) {
         CUDA_TRY(batch_launch_one(b, 1));
         b->parity = 0;
@@ -1736,9 +1735,8 @@ extern "C" lbm_status lbm_stefan_batch_autotune(lbm_stefan_batch* b, int trial_s
             if (st != LBM_OK) break;
             // one untimed warm-up step, then the timed trial
             auto trial = [&](int n) -> bool {
-                cudaError_t re;
-                if (batch_run_resident(b, n, &re)) return true;
-                for (int k = 0; k < n && re == cudaSuccess; ++k) {
+                cudaError_t re = batch_run_resident(b, &n);
+                for (; n > 0 && re == cudaSuccess; --n) {
                     re = batch_launch_one(b, b->parity);
                     b->parity ^= 1;
                 }
