@@ -661,17 +661,27 @@ __global__ void adj_links_kernel(const __grid_constant__ AdjArgs g, int corners_
 // D_j(y) = (1 - omega) a_j(y) + mu(y), so a tile's outputs
 //   lambda_j(x) = nu(x) + (1 - omega) a_j(x + e_j) + mu(x + e_j)
 // need one number per neighbour node beyond loads that are in L1 already: the
-// block evaluates mu of its 64 x 16 nodes and the ring around them (1.16
-// evaluations per node; the marching kernel's tiles of 4 rows at 1024^2 take
-// 1.5, with the shuffles of six planes), keeps them in shared memory and
-// gathers.  Outputs whose neighbourhood holds a wall node (the two outermost
-// rows and columns) are gathered by the last blocks, one node per thread with
-// the general node terms and the link-wise terms of adj_links_kernel: a few
-// thousand nodes beside the tiles, instead of a launch of their own after them.
-// Measured per step, marching and link kernels / this one: 44 / 31 us at 1024^2,
-// 119 / 97 us at 2048^2.  (FP64, and lattices beyond 32-bit indices: marching.)
-constexpr int kAdjFlatW = 64, kAdjFlatH = 16, kAdjFlatThreads = 512;
-constexpr int kAdjMuW = kAdjFlatW + 2, kAdjMuH = kAdjFlatH + 2;
+// block evaluates mu of its 64 x 16 nodes, four consecutive columns per thread
+// (vector loads and stores: 12 memory instructions per node instead of 38), and
+// of the ring around them (1.16 evaluations per node; the marching kernel's tiles
+// of 4 rows at 1024^2 take 1.5, with the shuffles of six planes), keeps them in
+// shared memory and gathers.  Outputs whose neighbourhood holds a wall node (the
+// two outermost rows and columns) are gathered by the first blocks, one node per
+// thread with the general node terms and the link-wise terms of adj_links_kernel:
+// a few thousand nodes beside the tiles, instead of a launch of their own after
+// them (as the last blocks they were a tail of their own).
+// Measured per step, marching and link kernels / this one with a column per thread
+// and the wall nodes last / as it stands: 44 / 31.1 / 23.8 us at 1024^2, 119 / 97 /
+// 74 us at 2048^2.  The wall nodes first gave 5 and 11 us of it, the vectors 2 and 12.
+// FP64, lattices beyond 32-bit indices, buffers off 16 bytes: marching.
+constexpr int kAdjFlatW = 64, kAdjFlatH = 16, kAdjFlatThreads = 256;
+constexpr int kAdjMuW = kAdjFlatW + 8, kAdjMuH = kAdjFlatH + 2;   // column x - x0 at x - x0 + 4 (16-byte rows)
+
+__device__ __forceinline__ void adj_ld4(const float* p, float (&v)[4])
+{
+    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
 
 __device__ __forceinline__ bool adj_has_links(const Problem& pb, unsigned bmask, unsigned unk)
 {
@@ -683,9 +693,9 @@ __device__ __forceinline__ bool adj_has_links(const Problem& pb, unsigned bmask,
     return any;
 }
 
-__global__ void __launch_bounds__(kAdjFlatThreads, 2) adj_flat_kernel(const __grid_constant__ AdjArgs g, int ntx, int ntiles)
+__global__ void __launch_bounds__(kAdjFlatThreads, 3) adj_flat_kernel(const __grid_constant__ AdjArgs g, int ntx, int nedge)
 {
-    __shared__ float mu_s[kAdjMuH * kAdjMuW];
+    __shared__ __align__(16) float mu_s[kAdjMuH * kAdjMuW];
     __shared__ double wall_sums[5 * kWarpsPerBlock * 32];
     const Problem& pb = g.pb;
     const AdjConst& c = g.c;
@@ -695,50 +705,109 @@ __global__ void __launch_bounds__(kAdjFlatThreads, 2) adj_flat_kernel(const __gr
     const float omc = c.omc_f;
     DevStats* st = g.stats;
     const int tid = threadIdx.x;
-    if ((int)blockIdx.x < ntiles) {
-        // outputs 2 <= x <= nx-3, 2 <= y <= ny-3
-        const int x0 = 2 + (int)(blockIdx.x % ntx) * kAdjFlatW, y0 = 2 + (int)(blockIdx.x / ntx) * kAdjFlatH;
-        float nu[2] = {0.f, 0.f}, gs = 0.f;
-        auto node = [&](int x, int y, float& mu, float& nuv, float& gsv) {
-            const float* p = ain + (y + 1) * pitch + x;
-            const float A = d2_wf(0) * __ldg(p) +
-                            d2_wf(1) * ((__ldg(p + plane) + __ldg(p + 2 * plane)) + (__ldg(p + 3 * plane) + __ldg(p + 4 * plane))) +
-                            d2_wf(5) * ((__ldg(p + 5 * plane) + __ldg(p + 6 * plane)) + (__ldg(p + 7 * plane) + __ldg(p + 8 * plane)));
-            interior_terms(A, __ldg(g.theta_t + y * pitch + x), __ldg(g.theta_t1 + y * pitch + x), c, mu, nuv, gsv);
+    if ((int)blockIdx.x >= nedge) {
+        const int tile = (int)blockIdx.x - nedge;
+        // outputs 2 <= x <= nx-3, 2 <= y <= ny-3 of the columns x0 .. x0 + 63
+        const int x0 = tile % ntx * kAdjFlatW, y0 = 2 + tile / ntx * kAdjFlatH;
+        auto weigh = [](float a0, float a1, float a2, float a3, float a4, float a5, float a6, float a7, float a8) {
+            return d2_wf(0) * a0 + d2_wf(1) * ((a1 + a2) + (a3 + a4)) + d2_wf(5) * ((a5 + a6) + (a7 + a8));
         };
+        const int lx = (tid % (kAdjFlatW / 4)) * 4, ly = tid / (kAdjFlatW / 4), x = x0 + lx, y = y0 + ly;
+        const int at = (y + 1) * pitch + x;
+        // every load of these four columns stays inside the planes (their rows are whole segments)
+        const bool mine = x < nx && y <= ny - 3;
+        float nu[4] = {0.f, 0.f, 0.f, 0.f}, gs = 0.f;
+        float a0[4], a1[4], a3[4];   // planes 0, 1, 3 of this row serve the gather as well
+        if (mine) {
+            float a2[4], a4[4], a5[4], a6[4], a7[4], a8[4];
+            adj_ld4(ain + at, a0);
+            adj_ld4(ain + plane + at, a1);
+            adj_ld4(ain + 2 * plane + at, a2);
+            adj_ld4(ain + 3 * plane + at, a3);
+            adj_ld4(ain + 4 * plane + at, a4);
+            adj_ld4(ain + 5 * plane + at, a5);
+            adj_ld4(ain + 6 * plane + at, a6);
+            adj_ld4(ain + 7 * plane + at, a7);
+            adj_ld4(ain + 8 * plane + at, a8);
+            double t0[4], t1[4];
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int lx = tid % kAdjFlatW, ly = tid / kAdjFlatW + 8 * k, x = x0 + lx, y = y0 + ly;
-            if (x <= nx - 3 && y <= ny - 3) {
-                float mu;
-                node(x, y, mu, nu[k], gs);
-                mu_s[(ly + 1) * kAdjMuW + lx + 1] = mu;
+            for (int k = 0; k < 4; k += 2) {
+                const double2 u = __ldg(reinterpret_cast<const double2*>(g.theta_t + y * pitch + x + k));
+                const double2 v = __ldg(reinterpret_cast<const double2*>(g.theta_t1 + y * pitch + x + k));
+                t0[k] = u.x; t0[k + 1] = u.y;
+                t1[k] = v.x; t1[k + 1] = v.y;
+            }
+            float mu[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                float gsk = 0.f;
+                interior_terms(weigh(a0[k], a1[k], a2[k], a3[k], a4[k], a5[k], a6[k], a7[k], a8[k]), t0[k], t1[k], c, mu[k], nu[k],
+                               gsk);
+                if (x + k >= 2 && x + k <= nx - 3) gs += gsk;   // (the others are counted by the first blocks)
+            }
+            *reinterpret_cast<float4*>(mu_s + (ly + 1) * kAdjMuW + lx + 4) = make_float4(mu[0], mu[1], mu[2], mu[3]);
+        }
+        // the ring around the tile: the rows below and above, the columns beside
+        const int hy = min(kAdjFlatH, ny - 2 - y0);   // rows of outputs
+        if (tid < 2 * (kAdjFlatW + 2) + 2 * hy) {
+            int rx, ry;
+            if (tid < 2 * (kAdjFlatW + 2)) {
+                ry = tid < kAdjFlatW + 2 ? -1 : hy;
+                rx = tid % (kAdjFlatW + 2) - 1;
+            } else {
+                const int k = tid - 2 * (kAdjFlatW + 2);
+                rx = k < hy ? -1 : kAdjFlatW;
+                ry = k < hy ? k : k - hy;
+            }
+            const int xx = x0 + rx, yy = y0 + ry;
+            if (xx >= 1 && xx <= nx - 2) {
+                const float* q = ain + (yy + 1) * pitch + xx;
+                float mu, nuv, gsv = 0.f;
+                interior_terms(weigh(__ldg(q), __ldg(q + plane), __ldg(q + 2 * plane), __ldg(q + 3 * plane), __ldg(q + 4 * plane),
+                                     __ldg(q + 5 * plane), __ldg(q + 6 * plane), __ldg(q + 7 * plane), __ldg(q + 8 * plane)),
+                               __ldg(g.theta_t + yy * pitch + xx), __ldg(g.theta_t1 + yy * pitch + xx), c, mu, nuv, gsv);
+                mu_s[(ry + 1) * kAdjMuW + rx + 4] = mu;
             }
         }
-        // the ring around the tile (as far as the last outputs' neighbours)
-        const int wx = min(kAdjFlatW, nx - 2 - x0), hy = min(kAdjFlatH, ny - 2 - y0);   // outputs of this tile
-        const int ring = 2 * (wx + 2) + 2 * hy;
-        if (tid < ring) {
-            int lx, ly;
-            if (tid < wx + 2) { lx = tid; ly = 0; }
-            else if (tid < 2 * (wx + 2)) { lx = tid - (wx + 2); ly = hy + 1; }
-            else if (tid < 2 * (wx + 2) + hy) { lx = 0; ly = tid - 2 * (wx + 2) + 1; }
-            else { lx = wx + 1; ly = tid - 2 * (wx + 2) - hy + 1; }
-            float mu, nuv, gsv = 0.f;
-            node(x0 + lx - 1, y0 + ly - 1, mu, nuv, gsv);
-            mu_s[ly * kAdjMuW + lx] = mu;
-        }
         __syncthreads();
+        if (mine) {
+            const bool whole = x >= 2 && x + 3 <= nx - 3;
+            // the six values of mu of rows y - 1, y, y + 1 around the four columns
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int lx = tid % kAdjFlatW, ly = tid / kAdjFlatW + 8 * k, x = x0 + lx, y = y0 + ly;
-            if (x > nx - 3 || y > ny - 3) continue;
-            const int at = (y + 1) * pitch + x;
-            const float* m = mu_s + (ly + 1) * kAdjMuW + lx + 1;
+            for (int dy = -1; dy <= 1; ++dy) {
+                const float* m = mu_s + (ly + 1 + dy) * kAdjMuW + lx + 4;
+                const float4 mv = *reinterpret_cast<const float4*>(m);
+                const float mm[6] = {m[-1], mv.x, mv.y, mv.z, mv.w, m[4]};
 #pragma unroll
-            for (int j = 0; j < 9; ++j) {
-                const float a = __ldg(ain + j * plane + at + d2_ey(j) * pitch + d2_ex(j));
-                aout[j * plane + at] = nu[k] + fmaf(omc, a, m[d2_ey(j) * kAdjMuW + d2_ex(j)]);
+                for (int j = 0; j < 9; ++j) {
+                    if (d2_ey(j) != dy) continue;
+                    const float* q = ain + j * plane + at + dy * pitch;
+                    float v[4], n[4];
+                    if (j == 0 || j == 1 || j == 3) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) v[k] = j == 0 ? a0[k] : (j == 1 ? a1[k] : a3[k]);
+                    } else {
+                        adj_ld4(q, v);
+                    }
+                    if (d2_ex(j) == 0) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) n[k] = v[k];
+                    } else if (d2_ex(j) == 1) {
+                        n[0] = v[1]; n[1] = v[2]; n[2] = v[3]; n[3] = __ldg(q + 4);
+                    } else {
+                        n[0] = __ldg(q - 1); n[1] = v[0]; n[2] = v[1]; n[3] = v[2];
+                    }
+                    float o[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) o[k] = nu[k] + fmaf(omc, n[k], mm[1 + k + d2_ex(j)]);
+                    if (whole) {
+                        *reinterpret_cast<float4*>(aout + j * plane + at) = make_float4(o[0], o[1], o[2], o[3]);
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (x + k >= 2 && x + k <= nx - 3) aout[j * plane + at + k] = o[k];
+                    }
+                }
             }
         }
         const double v = warp_sum((double)gs);
@@ -751,7 +820,7 @@ __global__ void __launch_bounds__(kAdjFlatThreads, 2) adj_flat_kernel(const __gr
     sums.gs = 0.f;
     sums.wall = wall_sums + tid;
     for (int k = 0; k < 5; ++k) sums.wall[k * kWarpsPerBlock * 32] = 0.0;
-    const int k = ((int)blockIdx.x - ntiles) * kWarpsPerBlock * 32 + tid;
+    const int k = (int)blockIdx.x * kWarpsPerBlock * 32 + tid;
     const int rows = min(4, ny), mid = max(0, ny - 4), cols = min(4, nx);
     int x = -1, y = 0;
     if (k < rows * nx) {
@@ -878,12 +947,15 @@ cudaError_t launch_adj_seed(int precision, const Problem* dprob, const Problem& 
 
 cudaError_t launch_adj_step(int precision, const AdjArgs& a, const Problem& hp, cudaStream_t s)
 {
-    if (hp.q == 9 && precision == 1 && hp.plane * 9 < 1ll << 31) {   // (32-bit indices)
-        const int ntx = hp.nx > 4 ? (hp.nx - 4 + kAdjFlatW - 1) / kAdjFlatW : 0;
+    // the flat form: 32-bit indices, vector loads and stores
+    const bool aligned = (((uintptr_t)a.adj_in | (uintptr_t)a.adj_out | (uintptr_t)a.theta_t | (uintptr_t)a.theta_t1) & 15) == 0 &&
+                         hp.pitch % 4 == 0;
+    if (hp.q == 9 && precision == 1 && hp.plane * 9 < 1ll << 31 && aligned) {
+        const int ntx = hp.nx > 4 ? (hp.nx - 2 + kAdjFlatW - 1) / kAdjFlatW : 0;   // columns 0 .. nx-3
         const int nty = hp.ny > 4 ? (hp.ny - 4 + kAdjFlatH - 1) / kAdjFlatH : 0;
         const long long ring = (long long)std::min(4, hp.ny) * hp.nx + (long long)std::min(4, hp.nx) * std::max(0, hp.ny - 4);
         const int edge = (int)((ring + kWarpsPerBlock * 32 - 1) / (kWarpsPerBlock * 32));
-        adj_flat_kernel<<<ntx * nty + edge, kAdjFlatThreads, 0, s>>>(a, ntx, ntx * nty);
+        adj_flat_kernel<<<edge + ntx * nty, kAdjFlatThreads, 0, s>>>(a, ntx, edge);
         return cudaGetLastError();
     }
     if (hp.q == 9) {

@@ -55,3 +55,34 @@ def test_flat_reverse_step(shape, bb_mode, wi):
     # sums over the nodes of terms of the same accuracy (Ste's up to 1/Ste^2 each)
     assert np.max(np.abs(gw - hw)) <= 1e-4 * (np.max(np.abs(y)) * nx * ny)
     assert abs(gs - hs) <= 1e-4 * nx * ny / 0.2 ** 2
+
+
+@pytest.mark.parametrize("shape", [(67, 19), (133, 37)])
+def test_state_buffers_on_8_bytes(shape):
+    """Adjoint states that are not on 16 bytes take the marching kernel: the same
+    function in other FP32 roundings, 2e-6 of the largest value (above)."""
+    import torch
+    from paper_2505_13097_gb300 import solver
+    nx, ny = shape
+    rng = np.random.Generator(np.random.PCG64(nx))
+    S = solver.Stefan(2, nx, ny, 0.8, 0.02, 0.2, workloads.FP32, {"W": (1, 0.9)})
+    planes = S.new_theta_planes(2)
+    planes.zero_()
+    th = rng.uniform(-0.2, 0.2, (ny, nx))
+    planes[0, :, :nx] = torch.tensor(th, device="cuda")
+    planes[1, :, :nx] = torch.tensor(th + rng.uniform(-0.01, 0.01, (ny, nx)), device="cuda")
+    lam = torch.tensor(rng.uniform(-1, 1, (9, ny, nx)), device="cuda").float()
+    n, out = 9 * (ny + 2) * S.row_stride, []
+    for off in (0, 8):
+        size = S.new_state_buffer().numel()
+        a, b = (torch.zeros(size + 16, dtype=torch.uint8, device="cuda")[off:off + size] for _ in range(2))
+        assert a.data_ptr() % 16 == off and b.data_ptr() % 16 == off
+
+        def view(buf):
+            return buf[:4 * n].view(torch.float32).view(9, ny + 2, S.row_stride)[:, 1:-1, :nx]
+        view(a)[:] = lam
+        S.adjoint_step(planes[0], planes[1], a, b)
+        S.sync()
+        out.append(view(b).double().cpu().numpy())
+    S.close()
+    assert np.max(np.abs(out[0] - out[1])) <= 2e-6 * np.max(np.abs(out[0]))
