@@ -1,10 +1,9 @@
 """Benchmark of the IREBM time step on GB300 (one JSON line on stdout).
 
 Headline: D2Q9 MLUPS of the step in the FP32 form (FP32 populations, FP64
-Newton; five launches per step: rows 1 .. ny-2 of the left and the right
-half of the strips, and on a second stream the wall nodes and the Newton
-solves of the left half beside the right half, then the right half's) on the 4096 x 4096 melting workload, timed with CUDA events on
-the launching stream over --steps steps after --warmup untimed steps.  The
+Newton; the steps run in resident cooperative launches of up to 2^32 node
+updates; lattices of more than 2^25 nodes: six launches per step) on the
+4096 x 4096 melting workload, timed with CUDA events on the launching stream over --steps steps after --warmup untimed steps.  The
 timed window sits at the middle of the 10,000-step job (the state is first
 advanced, untimed, to step 5,000 - (warmup + steps)/2) so the Newton front band
 has its average width.  The state (1.2 GB) is larger than L2 (129 MB), so
@@ -12,7 +11,7 @@ every step reads and writes HBM; no flush is needed.
 
 Also reported: the FP64 form on the same workload, the 2048^2 FP64 corner
 workload for Ste in {0.01, 0.1, 1}, EEBM (Algorithm 2) on the same window, 256
-batched problems in one persistent graph-captured launch per step, the
+batched problems advanced together, the
 adjoint/forward time ratio on 1024^2 with sqrt(T) checkpointing, the 512-node
 D1Q3 workload (all steps of a call in one launch), the paper's 2D cavity on D2Q5 (4096^2, Eq. 17
 closure; IREBM FP32 and FP64, EEBM), the paper's 1D bar (N = 801) and its 2D
@@ -49,6 +48,20 @@ FLAT_TRAFFIC_PER_NODE = (77219072 + 29094656) / 2086920
 FLAT_TRAFFIC_NOTE = ("ncu capture of one launch (left half of the strips) on the 2048^2 melting workload at "
                      "step 301: 77.2 MB read + 29.1 MB written for 2,086,920 nodes, 50.9 B per node; writes "
                      "still in L2 when the launch ends are written back during the next; scaled by nodes")
+
+
+# DRAM bytes per node and step of the resident D2Q9 FP32 kernel (ncu, a smaller case), None: not captured
+RESIDENT_TRAFFIC_PER_NODE = None
+RESIDENT_TRAFFIC_NOTE = None
+
+
+def resident_launches(nx, ny, steps):
+    """Launches of `steps` FP32 D2Q9 IREBM steps that run resident (up to 2^25
+    nodes; a launch runs up to 2^32 node updates, 32 to 8,192 steps); None for
+    larger lattices, whose steps are separate kernels."""
+    if nx * ny > 1 << 25:
+        return None
+    return -(-steps // max(32, min(8192, (1 << 32) // (nx * ny))))
 
 
 def flat_nodes(nx, ny):
@@ -172,10 +185,11 @@ def bench_single(torch, solver, case, steps, warmup, stream, barrier=None, centr
         barrier()
     ms = time_steps(torch, S, steps, stream)
     st = S.stats()
-    # per-kernel device times (CUDA events between the two launches of a step)
+    # per-kernel device times of the separate kernels (lbm_stefan_step_timed; resident steps have one kernel)
     if case.lattice == 2 and case.precision == 1:
         k0, k1, kf = S.step_timed(min(steps, 50), flat=True)
         st["kernel_ms"], st["flat_ms"] = (k0, k1), kf
+        st["resident_launches"] = resident_launches(case.nx, case.ny, steps)
     else:
         st["kernel_ms"] = S.step_timed(min(steps, 50)) if case.lattice in (2, 3) else None
     S.close()
@@ -192,6 +206,7 @@ def bench_eebm(torch, solver, case, steps, warmup, stream, nodes, irebm_ms):
     ms = time_steps(torch, S, steps, stream)
     k = S.step_timed(min(steps, 50))
     S.close()
+    # kernel_*: the separate stencil kernel (step_timed); mlups is of the resident steps
     return {"mlups": nodes * steps / ms / 1e3, "ms_per_step": ms / steps, "kernel_ms": k[0],
             "kernel_gbs": BYTES_FP32 * nodes / (k[0] * 1e-3) / 1e9, "irebm_over_eebm": irebm_ms / ms}
 
@@ -207,6 +222,7 @@ def bench_d2q5(torch, solver, workloads, steps, warmup, stream, peak, n=4096, fp
         ms, st = bench_single(torch, solver, c, steps, warmup, stream, centre=centre)
         k_step, k_job = st["kernel_ms"]
         gbs = bpn * nodes / (k_step * 1e-3) / 1e9
+        # kernel_*: the separate kernels (step_timed); mlups and whole_step_gbs are of the resident steps
         out[tag] = {"workload": c.name, "mlups": nodes * steps / ms / 1e3, "ms_per_step": ms / steps,
                     "kernel": "d2q5_step_kernel<%s,false>" % ("float" if prec == workloads.FP32 else "double"),
                     "kernel_ms": k_step, "job_kernel_ms": k_job, "bytes_per_node": bpn,
@@ -626,13 +642,37 @@ def run_gpu(args):
     value = job_mlups(world, nodes, args.steps, ms_max)
     per_step_ms = ms / args.steps
     k_step_ms, k_job_ms = st["kernel_ms"]
-    # the dominant kernel: the flat kernel, two launches per step (the left and the
-    # right half of the strips), timed with events on the handle's stream around each
-    # launch (the wall kernel and the left half's Newton solves run beside the right
-    # half on a second stream); 72 algorithmic bytes per node it updates
-    fnodes = flat_nodes(case.nx, case.ny)
-    flat_launch_ms = st["flat_ms"] / 2
-    achieved = BYTES_FP32 * (fnodes / 2) / (flat_launch_ms * 1e-3) / 1e9
+    launches = st.get("resident_launches")
+    if launches:
+        # the dominant kernel: the resident kernel, whose launches fill the timed window
+        achieved = BYTES_FP32 * nodes / (per_step_ms * 1e-3) / 1e9
+        roof = {"kernel": "resident_kernel<float,9,false> (all steps of a launch: streaming, wall nodes, Newton solves, a "
+                          "grid barrier per step)",
+                "units_per_launch": nodes * args.steps / launches, "kernel_ms": ms / launches, "launches": launches,
+                "traffic": RESIDENT_TRAFFIC_PER_NODE * nodes * args.steps / launches if RESIDENT_TRAFFIC_PER_NODE else None,
+                "traffic_note": RESIDENT_TRAFFIC_NOTE, "flat_kernel_ms": st["flat_ms"] / 2,
+                "timing": "kernel_ms: the timed window by its launches (the same kernel throughout; one event pair); "
+                          "flat_kernel_ms, step_kernels_ms, second_kernel_ms: the separate kernels that larger lattices "
+                          "run, 50 steps launched one by one right after the window"}
+    else:
+        # the flat kernel, two launches per step (the left and the right half of the strips),
+        # timed with events on the handle's stream around each launch (the wall kernel and the
+        # left half's Newton solves run beside the right half on a second stream); 72
+        # algorithmic bytes per node it updates
+        fnodes = flat_nodes(case.nx, case.ny)
+        flat_launch_ms = st["flat_ms"] / 2
+        achieved = BYTES_FP32 * (fnodes / 2) / (flat_launch_ms * 1e-3) / 1e9
+        roof = {"kernel": "d2q9_flat_kernel<false,false> (two launches per step: the left and the right "
+                          "half of the strips; d2q9_wall_kernel<false>, d2q9_wall_cols_kernel<false> and "
+                          "the left half's newton_jobs_kernel<float,false,9> on a second stream)",
+                # dram__bytes_read.sum + dram__bytes_write.sum of one launch of this kernel in an ncu
+                # capture, per launch at this node count
+                "traffic": FLAT_TRAFFIC_PER_NODE * fnodes / 2, "traffic_note": FLAT_TRAFFIC_NOTE,
+                "units_per_launch": fnodes / 2, "kernel_ms": flat_launch_ms, "launches_per_step": 6,
+                "timing": "kernel_ms: mean of the flat launches' CUDA-event times (on the handle's "
+                          "stream) over 50 steps launched one by one right after the timed window; "
+                          "step_kernels_ms: every launch but the last job launch, same steps; "
+                          "whole_step: the timed window (graph replays)"}
 
     extra = {}
     if rank == 0 and not args.quick:
@@ -686,27 +726,13 @@ def run_gpu(args):
                                       args.window_step if args.window_step is not None else case.steps // 2),
                        "l2": "state 1.2 GB > 129 MB L2 (no flush needed)", "parallelism": "replicas" if world > 1 else "1 GPU"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                         "frac": achieved / peak,
-                         # dram__bytes_read.sum + dram__bytes_write.sum of one launch of this kernel in an ncu
-                         # capture, per launch at this node count (None: not captured since the kernel changed)
-                         "traffic": FLAT_TRAFFIC_PER_NODE * fnodes / 2 if FLAT_TRAFFIC_PER_NODE else None,
-                         "traffic_note": FLAT_TRAFFIC_NOTE,
-                         "bytes_per_node": BYTES_FP32, "units_per_launch": fnodes / 2,
-                         "kernel": "d2q9_flat_kernel<false,false> (two launches per step: the left and the right "
-                                   "half of the strips; d2q9_wall_kernel<false>, d2q9_wall_cols_kernel<false> and "
-                                   "the left half's newton_jobs_kernel<float,false,9> on a second stream)",
-                         "kernel_ms": flat_launch_ms,
-                         "launches_per_step": 6,
+                         "frac": achieved / peak, "bytes_per_node": BYTES_FP32, **roof,
                          "step_kernels_ms": k_step_ms,
                          "second_kernel": "newton_jobs_kernel<float,false,9> (the last job launch: the rest of "
                                           "the left half's list, the right half's, the publication)",
                          "second_kernel_ms": k_job_ms,
                          "whole_step_gbs": BYTES_FP32 * nodes / (per_step_ms * 1e-3) / 1e9,
                          "whole_step_frac": BYTES_FP32 * nodes / (per_step_ms * 1e-3) / 1e9 / peak,
-                         "timing": "kernel_ms: mean of the flat launches' CUDA-event times (on the handle's "
-                                   "stream) over 50 steps launched one by one right after the timed window; "
-                                   "step_kernels_ms: every launch but the last job launch, same steps; "
-                                   "whole_step: the timed window (graph replays)",
                          "peak_source": peak_kind},
             "error_vs_oracle": errs.get("melt_2d_fp32"),
             "cpu_baseline": cpu_baseline_sample(workloads) if (world == 1 and not args.no_cpu) else None,
@@ -715,7 +741,8 @@ def run_gpu(args):
                     "what": "lbm_stefan_set_state from a pinned host copy of the state at the start of the "
                             "headline's window (all populations), %d steps, lbm_stefan_get_fields to pinned host "
                             "theta; wall clock" % args.steps},
-            "gpu_launches": 6 * args.steps,   # two flat halves, two wall kernels, two Newton launches
+            # resident launches, or per step two flat halves, two wall kernels, two Newton launches
+            "gpu_launches": launches or 6 * args.steps,
             "clocks": clk.summary(),
             "energy_imbalance_last_step": st["imbalance"],
             "newton_nodes_last_step": st["newton_nodes"],
