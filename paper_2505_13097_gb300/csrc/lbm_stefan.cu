@@ -85,7 +85,7 @@ struct lbm_stefan {
     bool ic = false;
     int adj_tile_h = lbm::kAdjTileH;   // rows per warp tile of the D2Q9 adjoint
     void* dilf = nullptr;              // 2D ILFBM: S0, two l iterates, two l differences, changed units
-    void* dilf_slots = nullptr;        // 2D ILFBM: the steps' sums
+    void* dilf_slots = nullptr;        // 2D ILFBM: barrier and sums of its own, where dslots has no room for them
     bool flat = false;                 // FP32 D2Q9: the flat and wall kernels
     bool use_tma = false;              // FP32 D2Q9: the TMA row-pipeline kernel (for the wait test hook)
     lbm::TmaMaps tma;
@@ -94,8 +94,8 @@ struct lbm_stefan {
     cudaEvent_t ev_fork = nullptr, ev_half = nullptr, ev_join = nullptr;
     cudaEvent_t ev_walls = nullptr;   // split step: the wall kernels are done (list A's wall part is final)
     lbm::ResidentPlan res;             // D2Q9 / D2Q5: the resident step (blocks 0: the step's separate kernels)
-    void* dslots = nullptr;            // its per-warp sums
-    lbm::ResidentBar* dbar = nullptr;  // its barrier
+    lbm::ResidentBar* dbar = nullptr;  // its barrier, then
+    void* dslots = nullptr;            // the blocks' sums (one allocation)
     GraphCache graph;
     // captured adjoint segments (lbm_stefan_adjoint_segment): recompute + reverse
     // steps for one (length, trajectory, adjoint buffers) combination each
@@ -454,6 +454,9 @@ static cudaError_t launch_one(lbm_stefan* h, int parity, double* rec)
     return lbm::launch_d1q3_step(h->precision, a, h->hp, h->stream);
 }
 
+// What a barrier takes before the sums of its launch.
+constexpr size_t kBarBytes = (sizeof(lbm::ResidentBar) + 255) / 256 * 256;
+
 // Bound of a wait at the resident step's barrier.
 constexpr long long kResidentWaitNs = 5000000000LL;
 
@@ -491,8 +494,8 @@ static cudaError_t run_resident(lbm_stefan* h, int* nsteps, int* parity, double*
 #endif
 // The largest lattice that steps in resident launches (measured us per step, separate
 // kernels / resident).  FP32 D2Q9 IREBM: 235 / 221 at 4096^2, 473 / 443 at 8192 x 4096,
-// 849 / 855 at 8192^2; EEBM, which has no Newton work to hide: 69 / 56 at 2048^2, 202 / 201
-// at 4096^2.  FP64 and D2Q5 gain at every size (D2Q9 FP64 966 / 658 and D2Q5 FP32 183 / 128
+// 849 / 855 at 8192^2; EEBM, which has no Newton work to hide: 69 / 56 at 2048^2, 203 / 199
+// at 4096^2.  FP64 and D2Q5 gain at every size (D2Q9 FP64 966 / 547 and D2Q5 FP32 183 / 124
 // at 4096^2): the bound is that of the 32-bit indices, 2^31 elements of a state.
 static long long resident_max_nodes(int lattice, int precision, int method)
 {
@@ -657,9 +660,9 @@ extern "C" lbm_status lbm_stefan_create(const lbm_stefan_params* p, void* cuda_s
         (long long)p->nx * p->ny <= resident_max_nodes(p->lattice, p->precision, LBM_IREBM)) {
         const lbm::ResidentPlan plan = lbm::resident_plan(p->precision, q, p->nx, p->ny);
         if (plan.blocks > 0) {
-            e = cudaMalloc(&h->dslots, plan.slots * lbm::resident_slot_bytes());
-            if (e == cudaSuccess) e = cudaMalloc(&h->dbar, sizeof(lbm::ResidentBar));
+            e = cudaMalloc((void**)&h->dbar, kBarBytes + plan.slots * lbm::resident_slot_bytes());
             if (e == cudaSuccess) e = cudaMemset(h->dbar, 0, sizeof(lbm::ResidentBar));
+            h->dslots = reinterpret_cast<char*>(h->dbar) + kBarBytes;
             h->res = plan;
         }
     }
@@ -730,7 +733,7 @@ extern "C" lbm_status lbm_stefan_set_method(lbm_stefan* h, int method)
                 cudaError_t e = cudaSuccess;
                 for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
                     e = cudaMalloc(&nb[k], need);
-                    if (e == cudaSuccess) e = cudaMemset(nb[k], 0, need);
+                    if (e == cudaSuccess) e = cudaMemsetAsync(nb[k], 0, need, h->stream);
                 }
                 if (e != cudaSuccess) {
                     cudaFree(nb[0]);
@@ -746,13 +749,13 @@ extern "C" lbm_status lbm_stefan_set_method(lbm_stefan* h, int method)
                 h->hp.tail_off = (long long)(need - kStateTail);
             }
             if (!h->dilf) {
-                const size_t slots = (size_t)lbm::kResidentRing * std::max(1, lbm::ilfbm_2d_blocks(h->hp.q, h->hp.nx, h->hp.ny));
-                CUDA_TRY(cudaMalloc(&h->dilf, lbm::ilfbm_2d_scratch(h->hp.nx, h->hp.ny)));
-                if (!h->dilf_slots) CUDA_TRY(cudaMalloc(&h->dilf_slots, slots * lbm::resident_slot_bytes()));
-                if (!h->dbar) {
-                    CUDA_TRY(cudaMalloc(&h->dbar, sizeof(lbm::ResidentBar)));
-                    CUDA_TRY(cudaMemset(h->dbar, 0, sizeof(lbm::ResidentBar)));
+                const int blocks = lbm::ilfbm_2d_blocks(h->hp.q, h->hp.nx, h->hp.ny);
+                const size_t slots = (size_t)lbm::kResidentRing * std::max(1, blocks - 1);
+                if (slots > h->res.slots && !h->dilf_slots) {
+                    CUDA_TRY(cudaMalloc(&h->dilf_slots, kBarBytes + slots * lbm::resident_slot_bytes()));
+                    CUDA_TRY(cudaMemsetAsync(h->dilf_slots, 0, sizeof(lbm::ResidentBar), h->stream));
                 }
+                CUDA_TRY(cudaMalloc(&h->dilf, lbm::ilfbm_2d_scratch(h->hp.nx, h->hp.ny)));
             }
         }
     }
@@ -817,8 +820,9 @@ extern "C" lbm_status lbm_stefan_step(lbm_stefan* h, int nsteps)
     }
     if (h->hp.method == LBM_ILFBM) {
         // 2D: one cooperative launch, a barrier per inner iteration
-        CUDA_TRY(lbm::launch_ilfbm_2d(h->hp, h->parity, nsteps, h->dilf, h->dstats, h->dilf_slots, h->dbar, kResidentWaitNs,
-                                      h->stream));
+        char* own = static_cast<char*>(h->dilf_slots);
+        CUDA_TRY(lbm::launch_ilfbm_2d(h->hp, h->parity, nsteps, h->dilf, h->dstats, own ? own + kBarBytes : h->dslots,
+                                      own ? reinterpret_cast<lbm::ResidentBar*>(own) : h->dbar, kResidentWaitNs, h->stream));
         h->parity ^= nsteps & 1;
         return LBM_OK;
     }
@@ -1258,7 +1262,6 @@ extern "C" void lbm_stefan_destroy(lbm_stefan* h)
     if (h->ev_join) cudaEventDestroy(h->ev_join);
     if (h->ev_walls) cudaEventDestroy(h->ev_walls);
     if (h->side) cudaStreamDestroy(h->side);
-    cudaFree(h->dslots);
     cudaFree(h->dbar);
     cudaFree(h->dilf);
     cudaFree(h->dilf_slots);

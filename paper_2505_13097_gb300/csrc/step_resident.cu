@@ -8,8 +8,9 @@
 // (130 x 64 nodes, FP32).  Here a step ends at one barrier (load, arrival, poll
 // and fence: 4 to 5 us on a lattice of a few hundred nodes), and its sums are
 // added up by a block of their own while the next step runs.  Measured, us per
-// step before and now: D2Q9 FP32 130 x 64 45 / 9.5, 1021 x 777 61 / 18; D2Q9
-// FP64 2048^2 387 / 181; D2Q5 FP32 4096^2 205 / 128, FP64 401^2 116 / 16.
+// step before and now: D2Q9 FP32 130 x 64 45 / 9, 1021 x 777 61 / 16.5, 4096^2
+// 232 / 217; D2Q9 FP64 2048^2 387 / 151; D2Q5 FP32 4096^2 205 / 124, FP64 401^2
+// 116 / 17.
 //
 // A step has two passes over what a block owns, between barriers of the block:
 //  1. plain nodes.  A warp takes a group of 32 N consecutive columns of one of
@@ -31,7 +32,7 @@
 //
 // Arithmetic: that of the kernels in step_d2q9.cu / step_d2q5.cu node by node.
 // FP64 form: the zeroth moment is summed in block floating point with integer
-// instructions (sum_q below) and w_i c takes one multiplication, 10 FP64
+// instructions (sum_q) and w_i c takes one multiplication, 10 FP64
 // instructions per D2Q9 node instead of 28: the FP64 pipe, one warp
 // instruction per 64 cycles of an SM quarter, bounds the FP64 form.
 #include <algorithm>
