@@ -9,7 +9,7 @@
 // and fence: 4 to 5 us on a lattice of a few hundred nodes), and its sums are
 // added up by a block of their own while the next step runs.  Measured, us per
 // step before and now: D2Q9 FP32 130 x 64 45 / 9, 1021 x 777 61 / 16.5, 4096^2
-// 232 / 217; D2Q9 FP64 2048^2 387 / 151; D2Q5 FP32 4096^2 205 / 124, FP64 401^2
+// 232 / 214; D2Q9 FP64 2048^2 387 / 150; D2Q5 FP32 4096^2 205 / 123, FP64 401^2
 // 116 / 17.
 //
 // A step has two passes over what a block owns, between barriers of the block:
