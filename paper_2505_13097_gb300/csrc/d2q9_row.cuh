@@ -191,12 +191,11 @@ __device__ __forceinline__ void row_update(const Problem& pb, int y, int x0, int
     double thn[REC ? N : 1];
     bool newton_k[N];
     double m0[N];       // FP64 form
-    bool sat_k[N];
     bool any_wall = false;
     bool dir_k[N];
     int wall_k[N];
 #pragma unroll
-    for (int k = 0; k < N; ++k) { dir_k[k] = sat_k[k] = false; wall_k[k] = -1; }
+    for (int k = 0; k < N; ++k) { dir_k[k] = false; wall_k[k] = -1; }
     if constexpr (EDGE) {
 #pragma unroll
         for (int k = 0; k < N; ++k) {
@@ -289,8 +288,7 @@ __device__ __forceinline__ void row_update(const Problem& pb, int y, int x0, int
                 ts.shifted += 1;
                 if constexpr (REC) thn[k] = (double)mf + (double)sh;
             } else {
-                c[k] = m0[k];   // omega is in the weight below
-                sat_k[k] = true;
+                c[k] = (P)(pb.omega * m0[k]);
                 acc.add_d(m0[k]);
                 if constexpr (REC) thn[k] = m0[k];
             }
@@ -346,7 +344,7 @@ __device__ __forceinline__ void row_update(const Problem& pb, int y, int x0, int
             wc[2][k] = wP[2] * c[k];
         } else {
             // one multiplication: 4/9 and 1/36 are 4 and 1/4 times 1/9, and so are their roundings
-            wc[1][k] = (sat_k[k] ? pb.omega * wP[1] : wP[1]) * c[k];
+            wc[1][k] = wP[1] * c[k];
             wc[0][k] = scale2(wc[1][k], 2);
             wc[2][k] = scale2(wc[1][k], -2);
         }

@@ -24,9 +24,9 @@ struct NodeOut {
 
 // One node: u = Omega(x) at time t, ql/qr = Omega_1(x-1), Omega_2(x+1) (ignored at walls).
 // One block's SM issues one FP64 warp instruction in 19 cycles (64 for a lone
-// warp), so a saturated node spends four: the moment is summed with integers
+// warp), so a saturated node spends five: the moment is summed with integers
 // (sum_q), the test for saturation runs on FP32 sums, w_i c takes one
-// multiplication (2/3 is 4 times 1/6, and so is its rounding) and the energy is
+// multiplication by a weight (2/3 is 4 times 1/6, and so is its rounding) and the energy is
 // fixed point.
 template <typename P>
 __device__ __forceinline__ NodeOut d1q3_node(const Problem& pb, int x, const P (&u)[3], P ql, P qr, P (&o)[3])
@@ -89,7 +89,7 @@ __device__ __forceinline__ NodeOut d1q3_node(const Problem& pb, int x, const P (
         r.theta_new = thd;
         r.energy = to_fixed(thd + pb.wall_phi[side] * pb.inv_ste);
     } else if (sat) {
-        v = (pb.omega * w1) * m0;
+        v = w1 * fma(-omc, m0, m0);   // (not (omega w_1) m0: a constant's rounding would enter every step)
         r.theta_new = m0;
         r.energy = to_fixed(m0);
         r.liquid = liq ? 1 : 0;

@@ -76,9 +76,8 @@ __device__ __forceinline__ void row5_update(const Problem& pb, const P* __restri
     bool newton_k[N], dir_k[N];
     int wall_k[N];
     double m0[N];       // FP64 form
-    bool sat_k[N];
 #pragma unroll
-    for (int k = 0; k < N; ++k) { dir_k[k] = sat_k[k] = false; wall_k[k] = -1; }
+    for (int k = 0; k < N; ++k) { dir_k[k] = false; wall_k[k] = -1; }
     if constexpr (EDGE) {
         bool any_wall = false;
 #pragma unroll
@@ -165,8 +164,7 @@ __device__ __forceinline__ void row5_update(const Problem& pb, const P* __restri
                 ts.shifted += 1;
                 if constexpr (REC) thn[k] = (double)mf + (double)sh;
             } else {
-                c[k] = m0[k];   // omega is in the weight below
-                sat_k[k] = true;
+                c[k] = (P)(pb.omega * m0[k]);
                 acc.add_d(m0[k]);
                 if constexpr (REC) thn[k] = m0[k];
             }
@@ -220,7 +218,7 @@ __device__ __forceinline__ void row5_update(const Problem& pb, const P* __restri
             wc[0][k] = w0 * c[k];
             wc[1][k] = w1 * c[k];
         } else {
-            wc[1][k] = (sat_k[k] ? pb.omega * w1 : w1) * c[k];
+            wc[1][k] = w1 * c[k];
             wc[0][k] = scale2(wc[1][k], 1);
         }
     }

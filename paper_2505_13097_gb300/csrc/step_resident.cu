@@ -32,7 +32,7 @@
 //
 // Arithmetic: that of the kernels in step_d2q9.cu / step_d2q5.cu node by node.
 // FP64 form: the zeroth moment is summed in block floating point with integer
-// instructions (sum_q) and w_i c takes one multiplication, 10 FP64
+// instructions (sum_q) and w_i c takes two multiplications, 11 FP64
 // instructions per D2Q9 node instead of 28: the FP64 pipe, one warp
 // instruction per 64 cycles of an SM quarter, bounds the FP64 form.
 #include <algorithm>
@@ -205,7 +205,7 @@ __device__ __forceinline__ void item_update(const Problem& pb, DevStats* st, con
     }
     if (plain) acc.add(m0);
     // c = theta' - (1 - omega) m0 (FP32: less omega sh); saturated: theta' = m0, c = omega m0
-    P c = sizeof(P) == 4 ? (P)(pb.omega_f * (float)m0) : m0;
+    P c = sizeof(P) == 4 ? (P)(pb.omega_f * (float)m0) : (P)(pb.omega * (double)m0);
     double tn = 0.0;
     if (rec) tn = sizeof(P) == 4 ? widen((float)m0) + widen(sh) : (double)m0;
     if (__any_sync(kFull, dir)) {
@@ -281,8 +281,7 @@ __device__ __forceinline__ void item_update(const Problem& pb, DevStats* st, con
     } else {
         // one multiplication: 4/9 and 1/36 are 4 and 1/4 times 1/9 (D2Q5: 1/3 = 2/6),
         // and so are their roundings
-        const double w1 = lat_wp<double>(Q, 1);
-        const double v = (plain ? pb.omega * w1 : w1) * (double)c;
+        const double v = lat_wp<double>(Q, 1) * (double)c;
         wc[0] = (P)scale2(v, Q == 9 ? 2 : 1);
         wc[1] = (P)v;
         wc[2] = Q == 9 ? (P)scale2(v, -2) : (P)0;
@@ -494,10 +493,13 @@ __device__ __forceinline__ void plain_update(const Problem& pb, const double* sr
     const unsigned nliq = (unsigned)__popc(__ballot_sync(kFull, !cold && liq));
     if (lane == 0) w->liquid += nliq;
     if (!cold && sat) {
-        // c = omega m0; one multiplication for the three w_i c: 4/9 and 1/36 are 4 and
-        // 1/4 times 1/9 (D2Q5: 1/3 = 2/6), and so are their roundings
+        // w_i c, c = omega m0: one multiplication by a weight, 4/9 and 1/36 being 4 and 1/4
+        // times 1/9 (D2Q5: 1/3 = 2/6), and so their roundings.  Not (omega w_i) m0, which would
+        // save the other one: the rounding of omega w_i, up to 2^-53 of it whatever m0, would
+        // enter every node at every step (at tau = 0.62 the coefficients would miss a sum of 1
+        // by 1.4e-16 on D2Q9, 2.2e-16 on D2Q5, against 0.9e-16 by the weights alone)
         acc.add(m0);
-        const double v = (pb.omega * lat_wp<double>(Q, 1)) * m0;
+        const double v = lat_wp<double>(Q, 1) * (pb.omega * m0);
         const double v0 = scale2(v, Q == 9 ? 2 : 1), v2 = Q == 9 ? scale2(v, -2) : 0.0;
 #pragma unroll
         for (int i = 0; i < Q; ++i) dst[at + i * plane] = fma(pb.omc, q[i], i == 0 ? v0 : (i <= 4 ? v : v2));
