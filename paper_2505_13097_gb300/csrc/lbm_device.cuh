@@ -216,12 +216,14 @@ __device__ __forceinline__ double exp_neg(double w)
     return __hiloint2double(__double2hiint(e) + ((n >> 8) << 20), __double2loint(e));
 }
 
-// 1/d for d in [1, 2]: an FP32 reciprocal (relative error e < 2^-21) and one
-// third-order step, r0 (1 + e + e^2), remainder e^3 < 2^-63.
-__device__ __forceinline__ double rcp_1_2(double d)
+// 1/(1 + E) for E in [0, 1]: an FP32 reciprocal r0 (relative error e < 2^-21) and
+// one third-order step, r0 (1 + e + e^2), remainder e^3 < 2^-63.  e = (1 - r0) - E r0,
+// whose difference is exact, so 1 + E is not rounded: half an ulp of the result
+// (with e from the rounded sum an ulp and a half, which theta' inherits over Ste).
+__device__ __forceinline__ double logistic(double E)
 {
-    const double r0 = widen(__frcp_rn(trunc_float(d)));
-    double e = fma(-d, r0, 1.0);
+    const double r0 = widen(__frcp_rn(1.0f + trunc_float(E)));
+    double e = fma(-E, r0, 1.0 - r0);
     e = fma(e, e, e);
     return fma(r0, e, r0);
 }
@@ -251,7 +253,7 @@ __device__ __forceinline__ Phi phi_z(double z)
         p.r = nan ? z : 1.0;
     } else {
         p.E = exp_neg(__hiloint2double(h, __double2loint(z)));
-        p.r = rcp_1_2(1.0 + p.E);
+        p.r = logistic(p.E);
     }
     return p;
 }
@@ -320,8 +322,8 @@ static __device__ __noinline__ NewtonOut newton_solve(double m0, double theta, d
 }
 
 // Mixed-precision form of the same solve (same root, same stopping rule), for
-// m0 = mm + sh and theta = tt + sh (sh: the state's shift, 0 in FP64; shz =
-// 2 sh / delta), as theta' = m0 + (phi(theta) - phi(root))/Ste.
+// m0 = mm + sh and theta = tt + sh (SHIFTED: sh is the state's shift; else 0, the
+// FP64 form), as theta' = m0 + (phi(theta) - phi(root))/Ste.
 //  1. FP32 Newton for the step u = x - theta.  The equation is
 //     u - (m0 - theta) + (phi(theta + u) - phi(theta))/Ste = 0 with the
 //     difference of phi from expm1 (no cancellation: with b = 2u/delta and
@@ -345,9 +347,13 @@ static __device__ __noinline__ NewtonOut newton_solve(double m0, double theta, d
 // quarter, so only differences of phi are formed (phi = r, or 1 - r for x < 0,
 // and the sides agree as a rule), the arguments of phi and theta' come in one
 // fused operation each, and the energy theta' + phi(theta')/Ste is
-// m0 + phi(theta)/Ste: 43 FP64 instructions per node with the sums before and the
-// collision after (236 with the library's tanh, conversion instructions and FP64
-// corrections; counted per warp on the front band of a 1021 x 777 lattice).
+// m0 + phi(theta)/Ste: 43 FP64 instructions (44 with a shift) per node with the
+// sums before and the collision after (236 with the library's tanh, conversion
+// instructions and FP64 corrections; counted per warp on the front band of a
+// 1021 x 777 lattice).  Error of theta' against 113-bit arithmetic, theta within
+// 19.5 delta, m0 - theta from 1e-12 to 1/Ste, Ste 0.01 to 1, in units of
+// 2^-53/Ste: at most 2.0, standard deviation at most 0.37 (with the library's tanh
+// and FP64 corrections from an FP32-accurate start 2.2 and 0.41).
 struct NewtonNode {
     double tns;      // theta' - sh
     double ens;      // theta' + phi(theta')/Ste - sh
@@ -360,11 +366,14 @@ __device__ __forceinline__ double flip_sign(double v, bool neg)
     return __hiloint2double(__double2hiint(v) ^ (neg ? (int)0x80000000 : 0), __double2loint(v));
 }
 
-__device__ __forceinline__ NewtonNode newton_mixed(double mm, double tt, double sh, double shz, const Problem& pb)
+template <bool SHIFTED>
+__device__ __forceinline__ NewtonNode newton_mixed(double mm, double tt, double sh, const Problem& pb)
 {
     const double inv_ste = pb.inv_ste, tid = pb.two_inv_delta;
     const int maxit = pb.maxit;
-    const double z = fma(tt, tid, shz);
+    // theta first: near the band the shift cancels exactly (2 sh/delta would round by its own
+    // size, up to 100 times that of z, and phi(theta) with it)
+    const double z = (SHIFTED ? tt + sh : tt) * tid;
     const Phi pt = phi_z(z);
     const double dmd = mm - tt;   // m0 - theta
     const float isf = pb.inv_ste_f, idf2 = 2.0f * pb.inv_delta_f;
@@ -430,8 +439,10 @@ __device__ __forceinline__ NewtonNode newton_mixed(double mm, double tt, double 
         for (int j = 0; j < 3; ++j) {
             const double z0 = fma(ud, tid, z);
             const Phi p = phi_z(z0);
-            double dphi = flip_sign(p.r, p.neg) - bt;   // phi(x) - phi(theta)
-            if (p.neg != pt.neg) dphi += p.neg ? 1.0 : -1.0;
+            // phi(x) - phi(theta); across 0 the 1 goes to r(x) first, where it is exact
+            double a = flip_sign(p.r, p.neg);
+            if (p.neg != pt.neg) a += p.neg ? 1.0 : -1.0;
+            const double dphi = a - bt;
             const double s = p.s();
             const double F = fma(dphi, inv_ste, ud - dmd);
             const double Fp = fma(s, pb.two_inv_delta_ste, 1.0);
@@ -467,8 +478,11 @@ __device__ __forceinline__ NewtonNode newton_mixed(double mm, double tt, double 
             ud += d;
         }
     }
-    const NewtonOut r = newton_solve(mm + sh, tt + sh, phi_theta, inv_ste, pb.inv_delta, pb.tol, maxit);
-    out.tns = fma(phi_theta - r.phi_root, inv_ste, mm);
+    // theta' from the m0 that the root was found for: inside the band it hardly depends on it
+    const double m0 = SHIFTED ? mm + sh : mm;
+    const NewtonOut r = newton_solve(m0, SHIFTED ? tt + sh : tt, phi_theta, inv_ste, pb.inv_delta, pb.tol, maxit);
+    out.tns = fma(phi_theta - r.phi_root, inv_ste, m0);
+    if (SHIFTED) out.tns -= sh;
     out.iters = r.iters + k;
     out.ok = r.ok && out.iters <= maxit && isfinite(r.root);
     return out;

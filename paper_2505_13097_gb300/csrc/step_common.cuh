@@ -190,7 +190,7 @@ __device__ __forceinline__ NewtonResult newton_job_apply(const NewtonJob& jb, co
     P qv[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) qv[i] = __ldcg(d + i * pb.plane);
-    double mm, tt, sh = 0.0, shz = 0.0;   // m0 and theta less the shift
+    double mm, tt, sh = 0.0;   // m0 and theta less the shift
     if constexpr (sizeof(P) == 4) {
         // FP32 form: the job carries only the node; m0 = M0(q) from the stored
         // unrelaxed q_i and theta = M0(f) = sum of the node's Omega_i(t) (the
@@ -204,14 +204,13 @@ __device__ __forceinline__ NewtonResult newton_job_apply(const NewtonJob& jb, co
             ff_add(m, qv[i]);
         }
         sh = widen(state_shift(pb, parity));
-        shz = sh * pb.two_inv_delta;
         mm = ff_to_double(m);
         tt = ff_to_double(t);
     } else {
         mm = jb.m0;
         tt = jb.theta;
     }
-    const NewtonNode nr = newton_mixed(mm, tt, sh, shz, pb);
+    const NewtonNode nr = newton_mixed<sizeof(P) == 4>(mm, tt, sh, pb);
     if (!nr.ok) atomicCAS(&stats[r.sidx].error, 0, 3);
     // c = theta' - (1-omega) m0; stored values less w_i s: c - omega s
     const P c = (P)fma(-pb.omc, mm, nr.tns);

@@ -94,7 +94,7 @@ __device__ __forceinline__ NodeOut d1q3_node(const Problem& pb, int x, const P (
         r.energy = to_fixed(m0);
         r.liquid = liq ? 1 : 0;
     } else {
-        const NewtonNode nr = newton_mixed(m0, sum_q<3>(ud), 0.0, 0.0, pb);
+        const NewtonNode nr = newton_mixed<false>(m0, sum_q<3>(ud), 0.0, pb);
         r.fail = !nr.ok;
         v = w1 * fma(-omc, m0, nr.tns);
         r.theta_new = nr.tns;

@@ -238,7 +238,7 @@ __device__ __forceinline__ void item_update(const Problem& pb, DevStats* st, con
         Fx e{0, 0ull};
         int it = 0;
         if (solve) {
-            double mm, tt, shd = 0.0, shz = 0.0;   // m0 and theta less the shift
+            double mm, tt, shd = 0.0;   // m0 and theta less the shift
             if constexpr (sizeof(P) == 4) {
                 ff fm{0.f, 0.f}, ft{0.f, 0.f};
 #pragma unroll
@@ -247,14 +247,13 @@ __device__ __forceinline__ void item_update(const Problem& pb, DevStats* st, con
                     ff_add(fm, q[i]);
                 }
                 shd = widen(sh);
-                shz = shd * pb.two_inv_delta;
                 mm = ff_to_double(fm);
                 tt = ff_to_double(ft);
             } else {
                 mm = (double)m0;
                 tt = sum_q<Q>(u);
             }
-            const NewtonNode nr = newton_mixed(mm, tt, shd, shz, pb);
+            const NewtonNode nr = newton_mixed<sizeof(P) == 4>(mm, tt, shd, pb);
             if (!nr.ok) atomicCAS(&st->error, 0, 3);
             tn = nr.tns + shd;
             c = (P)fma(-pb.omc, mm, nr.tns);
