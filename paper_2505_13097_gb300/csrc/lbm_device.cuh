@@ -281,7 +281,10 @@ struct NewtonOut {
 static __device__ __noinline__ NewtonOut newton_solve(double m0, double theta, double phi_theta, double inv_ste,
                                                       double inv_delta, double tol, int maxit)
 {
-    double lo = m0 + (phi_theta - 1.0) * inv_ste, hi = m0 + phi_theta * inv_ste;
+    // (widened by their rounding: a root at an end, as that of a node that leaves the band at
+    // once, must not fall outside: bisecting towards it takes more steps than maxit)
+    const double slack = 0x1p-51 * (fabs(m0) + inv_ste);
+    double lo = m0 + (phi_theta - 1.0) * inv_ste - slack, hi = m0 + phi_theta * inv_ste + slack;
     double x = theta;
     double step_old = hi - lo, step = step_old;
     NewtonOut r;
@@ -381,7 +384,8 @@ __device__ __forceinline__ NewtonNode newton_mixed(double mm, double tt, double 
     const float dm0 = trunc_float(dmd);
     const float dm = pt.neg ? -dm0 : dm0;            // mirrored to theta >= 0
     const float E = trunc_float(pt.E), r0 = trunc_float(pt.r);
-    float lo = dm + (r0 - 1.0f) * isf, hi = dm + r0 * isf;
+    const float slack = 0x1p-21f * (fabsf(dm) + isf);   // rounding of the bracket, as in newton_solve
+    float lo = dm + (r0 - 1.0f) * isf - slack, hi = dm + r0 * isf + slack;
     const float small = 1e-3f * pb.delta_f, di = idf2 * isf;
     // the first iterate from x = theta (F = -dm there) needs no exponential
     float u = __fdividef(dm, fmaf(E * r0 * r0, di, 1.0f));
