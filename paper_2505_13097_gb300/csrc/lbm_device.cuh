@@ -393,7 +393,8 @@ __device__ __forceinline__ NewtonNode newton_mixed(double mm, double tt, double 
     else hi = fminf(hi, 0.0f);
     if (!(u >= lo && u <= hi)) u = 0.5f * (lo + hi);
     float step_prev = fabsf(u);
-    int k = 1;
+    // an update below the FP32 resolution of x is no iteration (a node in equilibrium: m0 = theta)
+    int k = idf2 * step_prev <= 0x1p-23f * zf ? 0 : 1;
     for (; k < 16 && step_prev > small; ++k) {
         const float b = idf2 * u, ab = fabsf(b);
         float D, dph;   // phi(theta + u) - phi(theta), phi'(theta + u) delta / 2
