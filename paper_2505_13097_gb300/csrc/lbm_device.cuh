@@ -88,12 +88,12 @@ __device__ __forceinline__ float trunc_float(double d)
 
 // A float as a double with integer operations (a conversion instruction runs
 // on the FP64 pipe, an SM's narrowest: 64 cycles of a quarter's issue slots).
-// Exact; subnormal floats give 0.
+// Exact; infinities, NaN and subnormal floats take the conversion.
 __device__ __forceinline__ double widen(float f)
 {
     const unsigned b = __float_as_uint(f);
     const unsigned e = (b >> 23) & 0xffu;
-    if (e == 0xffu) return (double)f;   // infinity, NaN
+    if (e == 0xffu || (e == 0u && (b << 1) != 0u)) return (double)f;
     const unsigned hi = e == 0u ? 0u : (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20));
     return __hiloint2double((int)hi, e == 0u ? 0 : (int)(b << 29));
 }
