@@ -57,8 +57,10 @@ __device__ __forceinline__ bool ilf_above(double d, double tol)
     return b > __double_as_longlong(tol) && b <= 0x7ff0000000000000ll;
 }
 
-__global__ void __launch_bounds__(kIlfThreads + 32) ilfbm_d1q3_kernel(StepArgs a, const __grid_constant__ Problem pb, int nsteps)
+template <bool DEV>
+__global__ void __launch_bounds__(kIlfThreads + 32) ilfbm_d1q3_kernel(StepArgs a, const __grid_constant__ Problem pbv, int nsteps)
 {
+    const Problem& pb = DEV ? a.probs[0] : pbv;   // (device: for launches that a caller's graph keeps)
     extern __shared__ double sm[];
     __shared__ Fx red_e[2][kIlfWarps], red_f[2][kIlfWarps];   // per-step sums, step parity
     __shared__ unsigned char chg[3][kIlfSegs + 2];            // segment changed in iteration k: chg[k % 3][segment + 1]
@@ -686,12 +688,13 @@ static size_t ilfbm_smem(int nx) { return (size_t)9 * nx * sizeof(double); }
 
 bool ilfbm_d1q3_fits(int nx) { return ilfbm_smem(nx) <= 200 * 1024; }
 
-cudaError_t launch_ilfbm_d1q3(const StepArgs& a, const Problem& hp, int nsteps, cudaStream_t s)
+cudaError_t launch_ilfbm_d1q3(const StepArgs& a, const Problem& hp, int nsteps, bool from_device, cudaStream_t s)
 {
     const size_t sm = ilfbm_smem(hp.nx);
-    cudaError_t e = cudaFuncSetAttribute(ilfbm_d1q3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const auto kernel = from_device ? ilfbm_d1q3_kernel<true> : ilfbm_d1q3_kernel<false>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    ilfbm_d1q3_kernel<<<1, kIlfThreads + 32, sm, s>>>(a, hp, nsteps);
+    kernel<<<1, kIlfThreads + 32, sm, s>>>(a, hp, nsteps);
     return cudaGetLastError();
 }
 

@@ -256,14 +256,15 @@ cudaError_t launch_resident_batch(const Problem* probs, int count, const int4* u
 cudaError_t launch_d2q5_step(int precision, const StepArgs& a, cudaStream_t s);
 int d2q5_segment_width(int precision);   // nodes per warp segment
 
-// D1Q3 launchers (step_d1q3.cu)
+// D1Q3 launchers (step_d1q3.cu); from_device: the kernel reads the problem from a.probs, not
+// from the copy passed by value (launches that a caller's graph keeps)
 cudaError_t launch_d1q3_step(int precision, const StepArgs& a, const Problem& hp, cudaStream_t s);
 cudaError_t launch_d1q3_fused(int precision, const StepArgs& a, const Problem& hp, int nsteps, int start_parity,
-                              double* rec, cudaStream_t s);
+                              double* rec, bool from_device, cudaStream_t s);
 bool d1q3_fused_fits(int precision, int nx);
 
 // ILFBM (Algorithm 1) on D1Q3, FP64, one block over the whole lattice (ilfbm.cu)
-cudaError_t launch_ilfbm_d1q3(const StepArgs& a, const Problem& hp, int nsteps, cudaStream_t s);
+cudaError_t launch_ilfbm_d1q3(const StepArgs& a, const Problem& hp, int nsteps, bool from_device, cudaStream_t s);
 bool ilfbm_d1q3_fits(int nx);
 // nsteps ILFBM steps on D2Q9 / D2Q5 (hp.q), FP64, in one cooperative launch; scratch:
 // ilfbm_2d_scratch bytes, slots and bar as for launch_resident (ilfbm_2d_blocks - 1 slots

@@ -510,6 +510,20 @@ static bool resident_on(const lbm_stefan* h)
            (long long)h->hp.nx * h->hp.ny <= resident_max_nodes(h->p.lattice, h->precision, h->hp.method);
 }
 
+// Whether the caller is capturing the handle's stream.  A graph of the caller's outlives
+// this call, and its launches are to see the walls and Ste of each replay (set_bc,
+// set_ste): they read the problem on the device, which the resident kernels do not.
+static bool caller_captures(const lbm_stefan* h)
+{
+    if (h->stream == nullptr || h->stream == cudaStreamLegacy) return false;   // never capture
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
 static lbm_status check_stats_error(lbm_stefan* h, DevStats* out)
 {
     DevStats st;
@@ -810,11 +824,12 @@ extern "C" lbm_status lbm_stefan_step(lbm_stefan* h, int nsteps)
     if (nsteps < 0) return fail(LBM_ERR_ARG, "nsteps must be >= 0");
     if (!h->ic) return fail(LBM_ERR_STATE, "set_ic must come before step");
     if (nsteps == 0) return LBM_OK;
+    const bool captured = caller_captures(h);
     if (h->hp.method == LBM_ILFBM && h->p.lattice == LBM_D1Q3) {
         // all steps in one launch (one block over the lattice, whose barriers
         // separate the inner iterations)
         StepArgs a = single_args(h, h->parity, nullptr);
-        CUDA_TRY(lbm::launch_ilfbm_d1q3(a, h->hp, nsteps, h->stream));
+        CUDA_TRY(lbm::launch_ilfbm_d1q3(a, h->hp, nsteps, captured, h->stream));
         h->parity ^= nsteps & 1;
         return LBM_OK;
     }
@@ -828,12 +843,12 @@ extern "C" lbm_status lbm_stefan_step(lbm_stefan* h, int nsteps)
     }
     if (h->p.lattice == LBM_D1Q3 && lbm::d1q3_fused_fits(h->precision, h->hp.nx)) {
         StepArgs a = single_args(h, h->parity, nullptr);
-        CUDA_TRY(lbm::launch_d1q3_fused(h->precision, a, h->hp, nsteps, h->parity, nullptr, h->stream));
+        CUDA_TRY(lbm::launch_d1q3_fused(h->precision, a, h->hp, nsteps, h->parity, nullptr, captured, h->stream));
         h->parity ^= nsteps & 1;
         return LBM_OK;
     }
     int left = nsteps;
-    if (resident_on(h)) {
+    if (resident_on(h) && !captured) {
         double* no_rec = nullptr;
         const cudaError_t e = run_resident(h, &left, &h->parity, &no_rec);
         if (e != cudaErrorCooperativeLaunchTooLarge) CUDA_TRY(e);
@@ -844,7 +859,7 @@ extern "C" lbm_status lbm_stefan_step(lbm_stefan* h, int nsteps)
         --left;
     }
     // graphs only on a non-default stream (capture is not allowed on the legacy stream)
-    if (h->stream != nullptr && left >= kGraphSteps) {
+    if (h->stream != nullptr && left >= kGraphSteps && !captured) {
         if (!h->graph.exec) {
             lbm_status s = capture_graph(h);
             if (s != LBM_OK) return s;
@@ -935,11 +950,11 @@ extern "C" lbm_status lbm_stefan_step_record(lbm_stefan* h, int nsteps, double* 
     const long long plane = (long long)h->hp.ny * h->hp.pitch;
     if (h->p.lattice == LBM_D1Q3 && lbm::d1q3_fused_fits(h->precision, h->hp.nx)) {
         StepArgs a = single_args(h, h->parity, nullptr);
-        CUDA_TRY(lbm::launch_d1q3_fused(h->precision, a, h->hp, nsteps, h->parity, traj, h->stream));
+        CUDA_TRY(lbm::launch_d1q3_fused(h->precision, a, h->hp, nsteps, h->parity, traj, caller_captures(h), h->stream));
         h->parity ^= nsteps & 1;
         return LBM_OK;
     }
-    if (resident_on(h)) {
+    if (resident_on(h) && !caller_captures(h)) {
         const cudaError_t e = run_resident(h, &nsteps, &h->parity, &traj);
         if (e != cudaErrorCooperativeLaunchTooLarge) CUDA_TRY(e);
     }

@@ -161,10 +161,11 @@ constexpr int kFusedWarps = kFusedThreads / 32;
 // cycles and the FP32 stage; the saturated warps run beside it.
 // 512 nodes with a front: 15.3 us per step with a library tanh and FP64 sums,
 // 9.3 with the shorter solve alone.
-template <typename P>
+template <typename P, bool DEV>
 __global__ void __launch_bounds__(kFusedThreads + 32)
-    d1q3_fused_kernel(StepArgs a, const __grid_constant__ Problem pb, int nsteps, double* rec)
+    d1q3_fused_kernel(StepArgs a, const __grid_constant__ Problem pbv, int nsteps, double* rec)
 {
+    const Problem& pb = DEV ? a.probs[0] : pbv;
     extern __shared__ unsigned char smem_raw[];
     __shared__ Fx red_e[2][kFusedWarps], red_f[2][kFusedWarps];
     __shared__ int red_n[2][kFusedWarps], red_m[2][kFusedWarps], red_l[2][kFusedWarps], red_i[2][kFusedWarps];
@@ -284,21 +285,16 @@ cudaError_t launch_d1q3_step(int precision, const StepArgs& a, const Problem& hp
 }
 
 cudaError_t launch_d1q3_fused(int precision, const StepArgs& a, const Problem& hp, int nsteps, int start_parity,
-                              double* rec, cudaStream_t s)
+                              double* rec, bool from_device, cudaStream_t s)
 {
     StepArgs b = a;
     b.parity = start_parity;
     const size_t sm = fused_smem(precision, hp.nx);
-    cudaError_t e;
-    if (precision == 1) {
-        e = cudaFuncSetAttribute(d1q3_fused_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-        d1q3_fused_kernel<float><<<1, kFusedThreads + 32, sm, s>>>(b, hp, nsteps, rec);
-    } else {
-        e = cudaFuncSetAttribute(d1q3_fused_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-        d1q3_fused_kernel<double><<<1, kFusedThreads + 32, sm, s>>>(b, hp, nsteps, rec);
-    }
+    const auto kernel = precision == 1 ? (from_device ? d1q3_fused_kernel<float, true> : d1q3_fused_kernel<float, false>)
+                                       : (from_device ? d1q3_fused_kernel<double, true> : d1q3_fused_kernel<double, false>);
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    kernel<<<1, kFusedThreads + 32, sm, s>>>(b, hp, nsteps, rec);
     return cudaGetLastError();
 }
 
