@@ -167,10 +167,10 @@ __global__ void __launch_bounds__(128) adj_step_kernel(const __grid_constant__ A
     }
     for (int w = 0; w < 4; ++w) {
         const double v = warp_sum(gw[w]);
-        if ((threadIdx.x & 31) == 0) acc_add(&st->g_wall[w], v);
+        if ((threadIdx.x & 31) == 0) adj_add(st, w, v);
     }
     gs = warp_sum(gs);
-    if ((threadIdx.x & 31) == 0) acc_add(&st->g_ste, gs);
+    if ((threadIdx.x & 31) == 0) adj_add(st, 4, gs);
 }
 
 // ---------------------------------------------------------------- D2Q9 node terms
@@ -598,10 +598,10 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, LBM_ADJ_MIN_BLOCKS) adj_m
     for (int w = 0; w < 4; ++w) {
         if (pb.wall_kind[w] != 1) continue;
         const double v = warp_sum(sums.wall[(1 + w) * kWarpsPerBlock * 32]);
-        if ((threadIdx.x & 31) == 0 && v != 0.0) acc_add(&st->g_wall[w], v);
+        if ((threadIdx.x & 31) == 0 && v != 0.0) adj_add(st, w, v);
     }
     gs_total = warp_sum(gs_total);
-    if ((threadIdx.x & 31) == 0 && gs_total != 0.0) acc_add(&st->g_ste, gs_total);
+    if ((threadIdx.x & 31) == 0 && gs_total != 0.0) adj_add(st, 4, gs_total);
 }
 
 // Link-wise bounce-back terms (Sec. 4.2): at a boundary node whose q_i is
@@ -811,7 +811,7 @@ __global__ void __launch_bounds__(kAdjFlatThreads, 3) adj_flat_kernel(const __gr
             }
         }
         const double v = warp_sum((double)gs);
-        if ((tid & 31) == 0 && v != 0.0) acc_add(&st->g_ste, v);
+        if ((tid & 31) == 0 && v != 0.0) adj_add(st, 4, v);
         return;
     }
     // the two outermost rows (all columns), then the two outermost columns of the rows between
@@ -869,10 +869,10 @@ __global__ void __launch_bounds__(kAdjFlatThreads, 3) adj_flat_kernel(const __gr
     for (int w = 0; w < 4; ++w) {
         if (pb.wall_kind[w] != 1) continue;
         const double v = warp_sum(sums.wall[(1 + w) * kWarpsPerBlock * 32]);
-        if ((tid & 31) == 0 && v != 0.0) acc_add(&st->g_wall[w], v);
+        if ((tid & 31) == 0 && v != 0.0) adj_add(st, w, v);
     }
     const double v = warp_sum((double)sums.gs + sums.wall[0]);
-    if ((tid & 31) == 0 && v != 0.0) acc_add(&st->g_ste, v);
+    if ((tid & 31) == 0 && v != 0.0) adj_add(st, 4, v);
 }
 
 // ---------------------------------------------------------------- seed and finish
@@ -893,7 +893,7 @@ __global__ void adj_seed_kernel(const Problem* dprob, const double* __restrict__
         for (int i = 0; i < Q; ++i) a[i * pb.plane + (long long)(y + 1) * pb.pitch + x] = (P)s;
     }
     L = warp_sum(L);
-    if ((threadIdx.x & 31) == 0) acc_add(&st->loss, L);
+    if ((threadIdx.x & 31) == 0) adj_add(st, 5, L);
 }
 
 template <int Q, typename P>
@@ -925,7 +925,7 @@ __global__ void adj_finish_kernel(const Problem* dprob, const void* adj0, double
     }
     for (int w = 0; w < 4; ++w) {
         const double v = warp_sum(gw[w]);
-        if ((threadIdx.x & 31) == 0) acc_add(&st->g_wall[w], v);
+        if ((threadIdx.x & 31) == 0) adj_add(st, w, v);
     }
 }
 

@@ -219,7 +219,7 @@ __device__ __forceinline__ void row_update(const Problem& pb, int y, int x0, int
                     ff_add(ts.flux_f, fl.hi);
                     ts.flux_f.lo += fl.lo;
                 } else {
-                    fx_add(ts.flux, to_fixed(wall_closure_d(qq, uu, x, y, pb, wall_k[k])));
+                    ts.add_flux(wall_closure_d(qq, uu, x, y, pb, wall_k[k]));
                 }
                 dir_k[k] = wall_k[k] >= 0;
 #pragma unroll
@@ -413,7 +413,7 @@ __device__ __forceinline__ void row_update_eebm(const Problem& pb, int y, int x0
                         ff_add(ts.flux_f, fl.hi);
                         ts.flux_f.lo += fl.lo;
                     } else {
-                        fx_add(ts.flux, to_fixed(wall_closure_d(qq, uu, x, y, pb, wall)));
+                        ts.add_flux(wall_closure_d(qq, uu, x, y, pb, wall));
                     }
 #pragma unroll
                     for (int i = 0; i < 9; ++i) qf[i][k] = qq[i];

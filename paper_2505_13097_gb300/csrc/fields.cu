@@ -20,13 +20,14 @@ __device__ __forceinline__ bool dirichlet_value(const Problem& pb, int x, int y,
     return false;
 }
 
-// A block's exact sum in thread 0 (256 threads).
-__device__ __forceinline__ Fx block_sum(Fx v)
+// A block's exact sum in thread 0 (256 threads); mag: the largest fx_mag of the
+// thread's terms, lost: some thread's has no fixed-point value.
+__device__ __forceinline__ Fx block_sum(Fx v, unsigned mag, bool& lost)
 {
     __shared__ Fx part[8];
     v = fx_tree(v);
     if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
-    __syncthreads();
+    lost = __syncthreads_or(mag >= kFxMag ? 1 : 0) != 0;
     if (threadIdx.x == 0)
         for (int w = 1; w < 8; ++w) fx_add(v, part[w]);
     return v;
@@ -34,14 +35,15 @@ __device__ __forceinline__ Fx block_sum(Fx v)
 
 // The blocks' exact sums meet in the stripes of one accumulator (S: its offset
 // in a stripe); the last block to arrive (st->ticket, zero before and after)
-// gets the total in its first warp, as a double, and clears the stripes.
-// Returns whether this is that block's first warp.
+// gets the total in its first warp, as a double (NaN if a block lost a term), and
+// clears the stripes.  Returns whether this is that block's first warp.
 template <AccSum StepStripe::*S>
-__device__ __forceinline__ bool last_block_total(DevStats* st, const Fx& v, double& total)
+__device__ __forceinline__ bool last_block_total(DevStats* st, const Fx& v, bool lost, double& total)
 {
     __shared__ bool last;
     if (threadIdx.x == 0) {
         acc_add_fx(&(st->cur[blockIdx.x % kStripes].*S), v);
+        if (lost) atomicOr(&st->cur_lost, kLostEnergy);
         __threadfence();
         last = atomicAdd(&st->ticket, 1u) == gridDim.x - 1;
     }
@@ -57,8 +59,12 @@ __device__ __forceinline__ bool last_block_total(DevStats* st, const Fx& v, doub
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) a.limb[j] += __shfl_xor_sync(kFull, a.limb[j], o);
     }
-    if (threadIdx.x == 0) st->ticket = 0u;
-    total = acc_read(&a);
+    total = __ldcg(&st->cur_lost) ? nan_d() : acc_read(&a);
+    __syncwarp();
+    if (threadIdx.x == 0) {
+        st->ticket = 0u;
+        st->cur_lost = 0u;
+    }
     return true;
 }
 
@@ -78,13 +84,26 @@ __global__ void __launch_bounds__(256) shift_kernel(const Problem* dprob, const 
     const Problem& pb = *dprob;
     const unsigned n = (unsigned)pb.nx * (unsigned)pb.ny;
     Fx v{0, 0ull};
+    unsigned mag = 0u;
     for (unsigned k = blockIdx.x * 256u + threadIdx.x; k < n; k += gridDim.x * 256u) {
-        const double th = theta0[k];
-        fx_add(v, to_fixed(pb.method == 1 ? th + (th > 0.0 ? pb.inv_ste : 0.0) : th));
+        const double th = theta0[k], m = pb.method == 1 ? th + (th > 0.0 ? pb.inv_ste : 0.0) : th;
+        fx_add(v, to_fixed(m));
+        mag = max(mag, fx_mag(m));
     }
-    v = block_sum(v);
+    bool lost;
+    v = block_sum(v, mag, lost);
     double total;
-    if (last_block_total<&StepStripe::flux>(st, v, total) && threadIdx.x == 0) {
+    const bool mine = last_block_total<&StepStripe::flux>(st, v, lost, total);
+    if (mine && isnan(total)) {
+        // a term without a fixed-point value: the plain sum, which may be NaN, infinite or huge
+        total = 0.0;
+        for (unsigned k = threadIdx.x; k < n; k += 32u) {
+            const double th = theta0[k];
+            total += pb.method == 1 ? th + (th > 0.0 ? pb.inv_ste : 0.0) : th;
+        }
+        total = warp_sum(total);
+    }
+    if (mine && threadIdx.x == 0) {
         const float sh = (float)(0.5 * total / (double)n);
         for (int b = 0; b < 2; ++b) *reinterpret_cast<float*>(static_cast<char*>(pb.state[b]) + pb.tail_off) = sh;
     }
@@ -101,6 +120,11 @@ __global__ void __launch_bounds__(256) init_state_kernel(const Problem* dprob, c
     const double sh = sizeof(P) == 4 ? (double)state_shift(pb, parity) : 0.0;
     const unsigned nx = (unsigned)pb.nx, n = nx * (unsigned)pb.ny;
     Fx e{0, 0ull};
+    unsigned mag = 0u;
+    auto add = [&](double v) {
+        fx_add(e, to_fixed(v));
+        mag = max(mag, fx_mag(v));
+    };
     for (unsigned k = blockIdx.x * 256u + threadIdx.x; k < n; k += gridDim.x * 256u) {
         const int y = (int)(k / nx), x = (int)(k - (unsigned)y * nx);
         const long long at = (long long)(y + 1) * pb.pitch + x;
@@ -113,7 +137,7 @@ __global__ void __launch_bounds__(256) init_state_kernel(const Problem* dprob, c
             for (int i = 0; i < pb.q; ++i)
                 s[i * pb.plane + at] =
                     (P)(i == 0 ? H - (1.0 - lat_w(pb.q, 0)) * th - lat_w(pb.q, 0) * sh : lat_w(pb.q, i) * (th - sh));
-            fx_add(e, to_fixed(H));
+            add(H);
             continue;
         }
         // one product per weight
@@ -128,14 +152,15 @@ __global__ void __launch_bounds__(256) init_state_kernel(const Problem* dprob, c
             // ILFBM (Algorithm 1): the liquid fraction of the initial phase, plane q
             const double l = th > 0.0 ? 1.0 : 0.0;
             s[pb.q * pb.plane + at] = (P)l;
-            fx_add(e, to_fixed(th + l * pb.inv_ste));
+            add(th + l * pb.inv_ste);
             continue;
         }
-        fx_add(e, to_fixed(th + phi_of(th, pb.inv_delta) * pb.inv_ste));
+        add(th + phi_of(th, pb.inv_delta) * pb.inv_ste);
     }
-    e = block_sum(e);
+    bool lost;
+    e = block_sum(e, mag, lost);
     double total;
-    if (last_block_total<&StepStripe::energy>(st, e, total) && threadIdx.x == 0) {
+    if (last_block_total<&StepStripe::energy>(st, e, lost, total) && threadIdx.x == 0) {
         st->energy = total;
         st->energy_prev = total;
         st->have_energy = 1;

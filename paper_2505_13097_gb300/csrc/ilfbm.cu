@@ -63,6 +63,7 @@ __global__ void __launch_bounds__(kIlfThreads + 32) ilfbm_d1q3_kernel(StepArgs a
     const Problem& pb = DEV ? a.probs[0] : pbv;   // (device: for launches that a caller's graph keeps)
     extern __shared__ double sm[];
     __shared__ Fx red_e[2][kIlfWarps], red_f[2][kIlfWarps];   // per-step sums, step parity
+    __shared__ unsigned red_b[2][kIlfWarps];                  // kLostEnergy, kLostFlux
     __shared__ unsigned char chg[3][kIlfSegs + 2];            // segment changed in iteration k: chg[k % 3][segment + 1]
     __shared__ unsigned char ever[kIlfSegs + 2];              // ... in some iteration of the step
     DevStats* st = &a.stats[pb.stats];
@@ -193,6 +194,7 @@ __global__ void __launch_bounds__(kIlfThreads + 32) ilfbm_d1q3_kernel(StepArgs a
         const double* ln = lb[(base + k) & 1];
         const bool last = s + 1 == nsteps;
         Fx e{0, 0ull}, fl{0, 0ull};
+        unsigned emag = 0u, fmag = 0u;
         bool wall = false;
         for (int sg = seg0; sg < nseg; sg += kIlfWarps) {
             const int y = sg * 32 + lane;
@@ -211,24 +213,30 @@ __global__ void __launch_bounds__(kIlfThreads + 32) ilfbm_d1q3_kernel(StepArgs a
             if (y == 0) {   // west wall: f_1 (e = +1) is unknown
                 q1 = dirW ? thW - q0 - q2 : (mirror ? q2 : o2);
                 fx_add(fl, to_fixed(q1 - o2));
+                fmag = max(fmag, fx_mag(q1 - o2));
                 wall = true;
             }
             if (y == n - 1) {   // east wall: f_2 (e = -1) is unknown
                 q2 = dirE ? thE - q0 - q1 : (mirror ? q1 : o1);
                 fx_add(fl, to_fixed(q2 - o1));
+                fmag = max(fmag, fx_mag(q2 - o1));
                 wall = true;
             }
             const double q[3] = {q0, q1, q2};
             const double th = sum_q<3>(q);
-            fx_add(e, to_fixed(fma(ln[y], inv_ste, th)));
+            const double H = fma(ln[y], inv_ste, th);
+            fx_add(e, to_fixed(H));
+            emag = max(emag, fx_mag(H));
             double g[3] = {q0, q1, q2};
             if (!last) collide(q, th, g);
             for (int i = 0; i < 3; ++i) fn[i * n + y] = g[i];
         }
         e = fx_tree(e);
         if (__any_sync(kFull, wall)) fl = fx_tree(fl);
+        const unsigned lost = __reduce_or_sync(kFull, (emag >= kFxMag ? kLostEnergy : 0u) | (fmag >= kFxMag ? kLostFlux : 0u));
         const int h = s & 1;
         if (lane == 0 && !stats_warp) {
+            red_b[h][w] = lost;
             red_e[h][w] = e;
             red_f[h][w] = fl;
         }
@@ -239,8 +247,10 @@ __global__ void __launch_bounds__(kIlfThreads + 32) ilfbm_d1q3_kernel(StepArgs a
         base = (base + k) & 1;
         if (stats_warp) {
             const bool mine = lane < kIlfWarps;
-            const double es = fx_value(fx_tree(mine ? red_e[h][lane] : Fx{0, 0ull}));
-            const double fs = fx_value(fx_tree(mine ? red_f[h][lane] : Fx{0, 0ull}));
+            const unsigned b = __reduce_or_sync(kFull, mine ? red_b[h][lane] : 0u);
+            const double ev = fx_value(fx_tree(mine ? red_e[h][lane] : Fx{0, 0ull}));
+            const double fv = fx_value(fx_tree(mine ? red_f[h][lane] : Fx{0, 0ull}));
+            const double es = b & kLostEnergy ? nan_d() : ev, fs = b & kLostFlux ? nan_d() : fv;
             if (have) {
                 imb = es - E - fs;
                 if (fabs(imb) > imb_max) imb_max = fabs(imb);
@@ -581,6 +591,7 @@ __global__ void __launch_bounds__(kIlf2Threads, 1) ilf2_kernel(const __grid_cons
         const double* ln = a.lb[(base + k) & 1];
         const bool last = s + 1 == a.nsteps;
         Fx e{0, 0ull}, fx{0, 0ull};
+        unsigned emag = 0u, fmag = 0u;
         for (int u = w0; u < units; u += W) {
             const int y = u / nseg, x = (u - y * nseg) * 32 + lane;
             if (x >= nx) continue;
@@ -592,7 +603,9 @@ __global__ void __launch_bounds__(kIlf2Threads, 1) ilf2_kernel(const __grid_cons
                     q[i] = st[i * pb.plane + at - (long long)d2_ey(i) * pb.pitch - d2_ex(i)] +
                            lat_w(Q, i) * inv_ste * dp[nd - (long long)d2_ey(i) * nx - d2_ex(i)];
             } else {
-                fx_add(fx, to_fixed(ilf2_streamed<Q>(pb, st, lp, x, y, q, true)));
+                const double f = ilf2_streamed<Q>(pb, st, lp, x, y, q, true);
+                fx_add(fx, to_fixed(f));
+                fmag = max(fmag, fx_mag(f));
             }
             double th = 0.0;
 #pragma unroll
@@ -602,15 +615,19 @@ __global__ void __launch_bounds__(kIlf2Threads, 1) ilf2_kernel(const __grid_cons
                 dst[i * pb.plane + at] = last ? q[i] : q[i] - (q[i] - lat_w(Q, i) * th) * om;
             const double l = ln[nd];
             dst[Q * pb.plane + at] = l;
-            fx_add(e, to_fixed(th + l * inv_ste));
+            const double H = th + l * inv_ste;
+            fx_add(e, to_fixed(H));
+            emag = max(emag, fx_mag(H));
         }
         e = fx_tree(e);
         fx = fx_tree(fx);
+        const unsigned lost = __reduce_or_sync(kFull, (emag >= kFxMag ? kLostEnergy : 0u) | (fmag >= kFxMag ? kLostFlux : 0u));
         if (lane == 0) {
             ResidentSlot* w = &wsum[s & 1][warp];
             w->e = e;
             w->f = fx;
             w->maxit = k;   // inner iterations of the step
+            w->lost = lost;
         }
         __syncthreads();
         if (threadIdx.x == 0) {

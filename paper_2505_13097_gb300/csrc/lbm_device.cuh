@@ -601,7 +601,13 @@ struct Fx {
 
 // With integer operations only (an FP64 conversion costs 64 cycles of an SM
 // quarter): v = m 2^(e - 1075), scaled by 2^60.  Bits below 2^-60 are dropped;
-// values of 2^66 and more, infinities and NaN give 0 (the solves report them).
+// values of 2^67 and more, infinities and NaN have no fixed-point value and give
+// 0: the caller keeps the largest fx_mag of its terms beside the sum, and one that
+// reaches kFxMag makes the published sum NaN.
+constexpr unsigned kFxMag = (1023u + 67u) << 20;
+__device__ __forceinline__ unsigned fx_mag(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+__device__ __forceinline__ double nan_d() { return __longlong_as_double(0x7ff8000000000000ll); }
+
 __device__ __forceinline__ Fx to_fixed(double v)
 {
     Fx f{0, 0ull};
@@ -611,7 +617,7 @@ __device__ __forceinline__ Fx to_fixed(double v)
     const int sh = e - 1015;   // m * 2^(e - 1075 + 60)
     unsigned long long lo = 0, hi = 0;
     if (sh >= 0) {
-        if (sh >= 74) return f;
+        if (sh >= 75) return f;
         lo = sh < 64 ? m << sh : 0ull;
         hi = sh == 0 ? 0ull : (sh < 64 ? m >> (64 - sh) : m << (sh - 64));
     } else if (sh > -64 && e != 0) {
@@ -684,11 +690,12 @@ __device__ __forceinline__ Fx float_to_fixed(float v)
     return f;
 }
 
-// Add v into the 128-bit fixed-point accumulator.
-__device__ __forceinline__ void acc_add(Acc128* a, double v)
+// Add v to an adjoint accumulator (0..3: g_wall, 4: g_ste, 5: loss).
+__device__ __forceinline__ void adj_add(DevStats* st, int k, double v)
 {
     if (v == 0.0) return;
-    acc_add_fx(a, to_fixed(v));
+    if (fx_mag(v) >= kFxMag) atomicOr(&st->g_lost, 1u << k);
+    else acc_add_fx(k < 4 ? &st->g_wall[k] : (k == 4 ? &st->g_ste : &st->loss), to_fixed(v));
 }
 
 __device__ __forceinline__ double acc_read(const Acc128* a)
@@ -719,12 +726,6 @@ __device__ __forceinline__ void acc_add_fx(AccSum* a, const Fx& v)
     atomicAdd(&a->limb[1], lo >> 32);
     atomicAdd(&a->limb[2], hi & 0xffffffffull);
     atomicAdd(&a->limb[3], hi >> 32);
-}
-
-__device__ __forceinline__ void acc_add(AccSum* a, double v)
-{
-    if (v == 0.0) return;
-    acc_add_fx(a, to_fixed(v));
 }
 
 // sum_k limb[k] 2^(32k) modulo 2^128, as a double
@@ -797,6 +798,7 @@ __device__ __forceinline__ void publish_totals(DevStats* st, const Problem* pb, 
     const double e_old = __ldcg(&st->energy), imax = __ldcg(&st->imbalance_max);
     const long long steps = __ldcg(&st->steps);
     const int cmax = __ldcg(&st->cur_maxit);
+    const unsigned lost = __ldcg(&st->cur_lost);
     double inv_ste = 0.0, wphi[4] = {0.0, 0.0, 0.0, 0.0};
     float shift = 0.0f;
     if (pb) {
@@ -811,8 +813,8 @@ __device__ __forceinline__ void publish_totals(DevStats* st, const Problem* pb, 
         esum.limb[j] = s.e[j];
         fsum.limb[j] = s.f[j];
     }
-    double e = acc_read(&esum);
-    const double f = acc_read(&fsum);
+    double e = lost & kLostEnergy ? nan_d() : acc_read(&esum);
+    const double f = lost & kLostFlux ? nan_d() : acc_read(&fsum);
     if (pb) {
         double c = (double)s.liquid;
 #pragma unroll
@@ -833,6 +835,7 @@ __device__ __forceinline__ void publish_totals(DevStats* st, const Problem* pb, 
     __stcg(&st->newton_iters, (long long)s.iters);
     __stcg(&st->newton_max_iter, cmax);
     __stcg(&st->cur_maxit, 0);
+    if (lost) __stcg(&st->cur_lost, 0u);
 }
 
 // Publish one problem's step statistics and clear its stripes (one thread of

@@ -48,6 +48,8 @@ struct DevStats {
     int cur_maxit;                 // largest Newton iteration count
     int error;                     // sticky: lbm_status of a device-detected failure
     unsigned int ticket;           // last block of the initial-state kernels; zero between launches
+    unsigned int cur_lost;         // bits: the step's sums miss a term that has no fixed-point value
+                                   // (kLostEnergy, kLostFlux): published as NaN
     double energy, energy_prev, flux, imbalance, imbalance_max;
     long long steps;
     long long newton_nodes;
@@ -58,7 +60,9 @@ struct DevStats {
     Acc128 g_wall[4];
     Acc128 g_ste;
     Acc128 loss;
+    unsigned int g_lost;           // bits, in their order: accumulators that miss such a term
 };
+constexpr unsigned kLostEnergy = 1u, kLostFlux = 2u;
 
 // Device view of one problem.  Populations are stored as q planes (SoA);
 // plane i starts at base + i * plane; each plane has ny + 2 rows of `pitch`

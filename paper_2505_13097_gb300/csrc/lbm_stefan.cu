@@ -534,7 +534,11 @@ static lbm_status check_stats_error(lbm_stefan* h, DevStats* out)
     return LBM_OK;
 }
 
-static double acc_host(const lbm::Acc128& a) { return (double)a.hi * 16.0 + (double)a.lo * 0x1p-60; }
+// an adjoint accumulator (bit k of `lost`: it misses a term without a fixed-point value)
+static double acc_host(const lbm::Acc128& a, unsigned lost, int k)
+{
+    return (lost >> k) & 1u ? std::nan("") : (double)a.hi * 16.0 + (double)a.lo * 0x1p-60;
+}
 
 // ------------------------------------------------------------------ one problem
 
@@ -1095,12 +1099,13 @@ extern "C" lbm_status lbm_stefan_adjoint_seed(lbm_stefan* h, const double* theta
     if (h && h->p.lattice == LBM_D2Q5) return fail(LBM_ERR_ARG, "the adjoint covers D1Q3 and D2Q9");
     if (h && h->hp.method != LBM_IREBM) return fail(LBM_ERR_STATE, "the adjoint is that of the IREBM step");
     if (!h || !theta_T || !phi_target || !adj) return fail(LBM_ERR_ARG, "NULL argument");
-    CUDA_TRY(cudaMemsetAsync(&h->dstats->g_wall, 0, sizeof(lbm::Acc128) * 6, h->stream));
+    constexpr size_t sums0 = offsetof(DevStats, g_wall), sums1 = offsetof(DevStats, g_lost) + sizeof(DevStats::g_lost);
+    CUDA_TRY(cudaMemsetAsync(reinterpret_cast<char*>(h->dstats) + sums0, 0, sums1 - sums0, h->stream));
     CUDA_TRY(lbm::launch_adj_seed(h->precision, h->dprob, h->hp, theta_T, phi_target, adj, h->dstats, h->stream));
     if (loss) {
         DevStats st;
         lbm_status s = check_stats_error(h, &st);
-        *loss = acc_host(st.loss);
+        *loss = acc_host(st.loss, st.g_lost, 5);
         return s;
     }
     return LBM_OK;
@@ -1254,8 +1259,8 @@ extern "C" lbm_status lbm_stefan_adjoint_finish(lbm_stefan* h, const void* adj0,
     DevStats st;
     lbm_status s = check_stats_error(h, &st);
     if (g_wall)
-        for (int k = 0; k < 4; ++k) g_wall[k] = h->hp.wall_kind[k] == LBM_DIRICHLET ? acc_host(st.g_wall[k]) : 0.0;
-    if (g_ste) *g_ste = acc_host(st.g_ste);
+        for (int k = 0; k < 4; ++k) g_wall[k] = h->hp.wall_kind[k] == LBM_DIRICHLET ? acc_host(st.g_wall[k], st.g_lost, k) : 0.0;
+    if (g_ste) *g_ste = acc_host(st.g_ste, st.g_lost, 4);
     return s;
 }
 

@@ -15,7 +15,8 @@ struct alignas(16) ResidentSlot {
     unsigned dir[4];            // Dirichlet nodes per wall
     unsigned newton, iters;     // nodes solved, their iterations
     int maxit;
-    unsigned pad[3];
+    unsigned lost;              // kLostEnergy, kLostFlux (FP64 forms)
+    unsigned pad[2];
 };
 
 struct ResidentCommon {
@@ -106,6 +107,7 @@ static __device__ __noinline__ void resident_emit(const ResidentCommon& a, int s
     t.newton = __reduce_add_sync(kFull, t.newton);
     t.iters = __reduce_add_sync(kFull, t.iters);
     t.maxit = __reduce_max_sync(kFull, t.maxit);
+    t.lost = __reduce_or_sync(kFull, t.lost);
     // The sets of the next steps have been read (a ring ago: no wait in practice); looked
     // at for half a ring at once, one lane per set.
     constexpr int kHalf = kResidentRing / 2;
@@ -144,6 +146,7 @@ static __device__ __noinline__ void resident_stats(const ResidentCommon& a, cons
         const ResidentSlot* set = a.slots + (size_t)at * nb;
         unsigned long long v[16] = {};   // e 4 limbs, f 4 limbs, dir 4, newton, iters, liquid, shifted
         int mx = 0;
+        unsigned lost = 0;
         for (unsigned k = lane; k < nb; k += 32) {
             const uint4* p = reinterpret_cast<const uint4*>(set + k);
             const uint4 x0 = __ldcg(p), x1 = __ldcg(p + 1), x2 = __ldcg(p + 2), x3 = __ldcg(p + 3), x4 = __ldcg(p + 4);
@@ -154,12 +157,14 @@ static __device__ __noinline__ void resident_stats(const ResidentCommon& a, cons
             v[8] += x2.z; v[9] += x2.w; v[10] += x3.x; v[11] += x3.y;
             v[12] += x3.z; v[13] += x3.w;
             mx = max(mx, (int)x4.x);
+            lost |= x4.y;
         }
 #pragma unroll
         for (int k = 0; k < 16; ++k)
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(kFull, v[k], o);
         mx = __reduce_max_sync(kFull, mx);
+        lost = __reduce_or_sync(kFull, lost);
         if (lane == 0) {
             fence_gpu();
             atomicAdd(&bar->read[at], 1u);   // the set is read
@@ -169,8 +174,8 @@ static __device__ __noinline__ void resident_stats(const ResidentCommon& a, cons
                 es.limb[j] = v[j];
                 fs.limb[j] = v[4 + j];
             }
-            double e = acc_read(&es);
-            const double f = acc_read(&fs);
+            double e = lost & kLostEnergy ? nan_d() : acc_read(&es);
+            const double f = lost & kLostFlux ? nan_d() : acc_read(&fs);
             double c = (double)v[14];
 #pragma unroll
             for (int k = 0; k < 4; ++k)

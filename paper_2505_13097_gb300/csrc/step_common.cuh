@@ -38,11 +38,22 @@ struct Acc<float> {
 template <>
 struct Acc<double> {   // exact, on the integer pipe
     Fx s{0, 0ull};
-    __device__ void add_d(double v) { fx_add(s, to_fixed(v)); }
+    unsigned mag = 0u;
+    __device__ void add_d(double v)
+    {
+        fx_add(s, to_fixed(v));
+        mag = max(mag, fx_mag(v));
+    }
 };
 
 struct TileSums {
     Fx flux{0, 0ull};                   // FP64 form
+    unsigned flux_mag = 0u;
+    __device__ void add_flux(double v)
+    {
+        fx_add(flux, to_fixed(v));
+        flux_mag = max(flux_mag, fx_mag(v));
+    }
     ff flux_f{0.f, 0.f};                // FP32 form
     int dir_count[4] = {0, 0, 0, 0};   // Dirichlet nodes per wall (adds phi(theta_D)/Ste each)
     int liquid = 0, newton = 0, maxit = 0;
@@ -56,6 +67,7 @@ struct WarpSums {
     int nl = 0;        // saturated liquid nodes
     int nd[4] = {0, 0, 0, 0};   // Dirichlet nodes per wall
     int ns = 0;        // energy terms added less the state's shift
+    unsigned lost = 0u;   // kLostEnergy, kLostFlux (FP64 form)
 };
 
 template <typename P>
@@ -80,6 +92,7 @@ __device__ __forceinline__ WarpSums warp_tile_sums(const Acc<P>& acc, const Tile
     } else {
         w.e = fx_tree(acc.s);
         w.f = fx_tree(ts.flux);
+        w.lost = __reduce_or_sync(kFull, (acc.mag >= kFxMag ? kLostEnergy : 0u) | (ts.flux_mag >= kFxMag ? kLostFlux : 0u));
     }
     w.nl = warp_sum_i(ts.liquid);
     w.ns = warp_sum_i(ts.shifted);
@@ -94,6 +107,7 @@ __device__ __forceinline__ void add_sums(WarpSums& a, const WarpSums& b)
     fx_add(a.f, b.f);
     a.nl += b.nl;
     a.ns += b.ns;
+    a.lost |= b.lost;
 #pragma unroll
     for (int k = 0; k < 4; ++k) a.nd[k] += b.nd[k];
 }
@@ -107,6 +121,7 @@ __device__ __forceinline__ void emit_sums(const WarpSums& w, DevStats* st)
     acc_add_fx(&c->flux, w.f);
     if (w.nl) atomicAdd(&c->liquid, (unsigned long long)w.nl);
     if (w.ns) atomicAdd(&c->shifted, (unsigned long long)w.ns);
+    if (w.lost) atomicOr(&st->cur_lost, w.lost);
 #pragma unroll
     for (int k = 0; k < 4; ++k)
         if (w.nd[k]) atomicAdd(&c->dir[k], (unsigned long long)w.nd[k]);

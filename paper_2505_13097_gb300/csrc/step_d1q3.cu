@@ -14,7 +14,7 @@ namespace lbm {
 
 struct NodeOut {
     double theta_new;   // theta' of the node
-    Fx energy;          // theta' + phi(theta')/Ste, a saturated liquid node's less 1/Ste
+    double energy;      // theta' + phi(theta')/Ste, a saturated liquid node's less 1/Ste
     double flux;        // boundary flux contribution
     int liquid;         // 1 at a saturated liquid node
     int newton;         // 1 if the Newton iteration ran
@@ -76,7 +76,7 @@ __device__ __forceinline__ NodeOut d1q3_node(const Problem& pb, int x, const P (
         o[1] = (P)fma(omc, q[1], v);
         o[2] = (P)fma(omc, q[2], v);
         r.theta_new = t;
-        r.energy = to_fixed(m0);
+        r.energy = m0;
         return r;
     }
     const float tf = (approx_float(ud[0]) + approx_float(ud[1])) + approx_float(ud[2]), mf = approx_float(m0);
@@ -87,18 +87,18 @@ __device__ __forceinline__ NodeOut d1q3_node(const Problem& pb, int x, const P (
     if (dir) {
         v = w1 * (thd - omc * m0);
         r.theta_new = thd;
-        r.energy = to_fixed(thd + pb.wall_phi[side] * pb.inv_ste);
+        r.energy = thd + pb.wall_phi[side] * pb.inv_ste;
     } else if (sat) {
         v = w1 * fma(-omc, m0, m0);   // (not (omega w_1) m0: a constant's rounding would enter every step)
         r.theta_new = m0;
-        r.energy = to_fixed(m0);
+        r.energy = m0;
         r.liquid = liq ? 1 : 0;
     } else {
         const NewtonNode nr = newton_mixed<false>(m0, sum_q<3>(ud), 0.0, pb);
         r.fail = !nr.ok;
         v = w1 * fma(-omc, m0, nr.tns);
         r.theta_new = nr.tns;
-        r.energy = to_fixed(nr.ens);
+        r.energy = nr.ens;
         r.newton = 1;
         r.iters = nr.iters;
     }
@@ -118,6 +118,7 @@ __global__ void __launch_bounds__(128) d1q3_step_kernel(StepArgs a)
     const long long pl = pb.plane, row = pb.pitch;   // row 0 of a plane starts at +pitch
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     Fx e{0, 0ull}, f{0, 0ull};
+    unsigned lost = 0u;
     int nn = 0, mi = 0, nl = 0;
     if (x < pb.nx) {
         P u[3], o[3];
@@ -128,8 +129,9 @@ __global__ void __launch_bounds__(128) d1q3_step_kernel(StepArgs a)
         for (int i = 0; i < 3; ++i) dst[i * pl + row + x] = o[i];
         if (a.rec) a.rec[x] = r.theta_new;
         if (r.fail) atomicOr(&st->error, 3);
-        e = r.energy;
+        e = to_fixed(r.energy);
         f = to_fixed(r.flux);
+        lost = (fx_mag(r.energy) >= kFxMag ? kLostEnergy : 0u) | (fx_mag(r.flux) >= kFxMag ? kLostFlux : 0u);
         nn = r.newton;
         mi = r.iters;
         nl = r.liquid;
@@ -139,12 +141,14 @@ __global__ void __launch_bounds__(128) d1q3_step_kernel(StepArgs a)
     nn = warp_sum_i(nn);
     nl = warp_sum_i(nl);
     mi = warp_max_i(mi);
+    lost = __reduce_or_sync(kFull, lost);
     if ((threadIdx.x & 31) == 0) {
         acc_add_fx(&my_stripe(st)->energy, e);
         acc_add_fx(&my_stripe(st)->flux, f);
         if (nn) atomicAdd(&my_stripe(st)->newton, (unsigned long long)nn);
         if (nl) atomicAdd(&my_stripe(st)->liquid, (unsigned long long)nl);
         if (mi) atomicMax(&st->cur_maxit, mi);
+        if (lost) atomicOr(&st->cur_lost, lost);
     }
     finish_launch(a.stats, 1, a.ticket, a.probs);
 }
@@ -169,6 +173,7 @@ __global__ void __launch_bounds__(kFusedThreads + 32)
     extern __shared__ unsigned char smem_raw[];
     __shared__ Fx red_e[2][kFusedWarps], red_f[2][kFusedWarps];
     __shared__ int red_n[2][kFusedWarps], red_m[2][kFusedWarps], red_l[2][kFusedWarps], red_i[2][kFusedWarps];
+    __shared__ unsigned red_b[2][kFusedWarps];   // kLostEnergy, kLostFlux
     DevStats* st = &a.stats[pb.stats];
     const int n = pb.nx;
     P* buf[2] = {reinterpret_cast<P*>(smem_raw), reinterpret_cast<P*>(smem_raw) + 3 * n};
@@ -193,7 +198,9 @@ __global__ void __launch_bounds__(kFusedThreads + 32)
             last_i = __reduce_add_sync(kFull, mine ? red_i[h][l] : 0);
             last_m = __reduce_max_sync(kFull, mine ? red_m[h][l] : 0);
             const int nl = __reduce_add_sync(kFull, mine ? red_l[h][l] : 0);
-            const double es = fx_value(e) + (double)nl * pb.inv_ste, fs = fx_value(f);
+            const unsigned lost = __reduce_or_sync(kFull, mine ? red_b[h][l] : 0u);
+            const double es = lost & kLostEnergy ? nan_d() : fx_value(e) + (double)nl * pb.inv_ste;
+            const double fs = lost & kLostFlux ? nan_d() : fx_value(f);
             if (have) {
                 imb = es - E - fs;
                 if (fabs(imb) > imb_max) imb_max = fabs(imb);
@@ -222,6 +229,7 @@ __global__ void __launch_bounds__(kFusedThreads + 32)
             const P* in = buf[cur];
             P* out = buf[cur ^ 1];
             Fx e{0, 0ull}, f{0, 0ull};
+            unsigned emag = 0u, fmag = 0u;
             int nn = 0, mi = 0, nl = 0, ni = 0;
             bool wall = false;
             for (int x = threadIdx.x; x < n; x += kFusedThreads) {
@@ -233,9 +241,11 @@ __global__ void __launch_bounds__(kFusedThreads + 32)
                 out[n + x] = o[1];
                 out[2 * n + x] = o[2];
                 if (rec) rec[(long long)s * pb.pitch + x] = r.theta_new;
-                fx_add(e, r.energy);
+                fx_add(e, to_fixed(r.energy));
+                emag = max(emag, fx_mag(r.energy));
                 if (x == 0 || x == n - 1) {
                     fx_add(f, to_fixed(r.flux));
+                    fmag = max(fmag, fx_mag(r.flux));
                     wall = true;
                 }
                 nn += r.newton;
@@ -252,8 +262,11 @@ __global__ void __launch_bounds__(kFusedThreads + 32)
                 ni = __reduce_add_sync(kFull, ni);
                 mi = __reduce_max_sync(kFull, mi);
             }
+            const unsigned lost =
+                __reduce_or_sync(kFull, (emag >= kFxMag ? kLostEnergy : 0u) | (fmag >= kFxMag ? kLostFlux : 0u));
             const int h = s & 1;
             if (l == 0) {
+                red_b[h][w] = lost;
                 red_e[h][w] = e;
                 red_f[h][w] = f;
                 red_n[h][w] = nn;

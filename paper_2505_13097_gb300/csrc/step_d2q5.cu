@@ -100,7 +100,7 @@ __device__ __forceinline__ void row5_update(const Problem& pb, const P* __restri
                         ff_add(ts.flux_f, fl.hi);
                         ts.flux_f.lo += fl.lo;
                     } else {
-                        fx_add(ts.flux, to_fixed(wall5_closure_d(qq, uu, nq, x, y, pb, wall_k[k])));
+                        ts.add_flux(wall5_closure_d(qq, uu, nq, x, y, pb, wall_k[k]));
                     }
                     dir_k[k] = wall_k[k] >= 0;
 #pragma unroll
@@ -265,7 +265,7 @@ __device__ __forceinline__ void row5_update_eebm(const Problem& pb, const P* __r
                     ff_add(ts.flux_f, fl.hi);
                     ts.flux_f.lo += fl.lo;
                 } else {
-                    fx_add(ts.flux, to_fixed(wall5_closure_d(qq, uu, nq, x, y, pb, wall)));
+                    ts.add_flux(wall5_closure_d(qq, uu, nq, x, y, pb, wall));
                 }
 #pragma unroll
                 for (int i = 0; i < 5; ++i) qf[i][k] = qq[i];

@@ -63,6 +63,7 @@ template <typename P> struct LaneAcc;
 template <> struct LaneAcc<float> {
     ff s{0.f, 0.f};
     __device__ void add(float v) { ff_add(s, v); }
+    __device__ bool lost() const { return false; }
     __device__ Fx total() const
     {
         ff t = s;
@@ -79,7 +80,13 @@ template <> struct LaneAcc<float> {
 };
 template <> struct LaneAcc<double> {
     Fx s{0, 0ull};
-    __device__ void add(double v) { fx_add(s, to_fixed(v)); }
+    unsigned mag = 0u;
+    __device__ void add(double v)
+    {
+        fx_add(s, to_fixed(v));
+        mag = max(mag, fx_mag(v));
+    }
+    __device__ bool lost() const { return __any_sync(kFull, mag >= kFxMag); }
     __device__ Fx total() const { return fx_tree(s); }
 };
 
@@ -105,6 +112,7 @@ __device__ __forceinline__ void item_update(const Problem& pb, DevStats* st, con
     const bool edge = valid && (x == 0 || x == nx - 1 || y == 0 || y == ny - 1);
     if (__any_sync(kFull, edge)) {
         Fx fl{0, 0ull};
+        unsigned mag = 0u;
         if (edge) {
             // copies: the closures take addresses, and u, q stay in registers elsewhere
             P qq[Q], uu[Q];
@@ -119,7 +127,9 @@ __device__ __forceinline__ void item_update(const Problem& pb, DevStats* st, con
                     fl = float_to_fixed(t.hi);
                     fx_add(fl, float_to_fixed(t.lo));
                 } else {
-                    fl = to_fixed(wall_closure_d(qq, uu, x, y, pb, wall));
+                    const double t = wall_closure_d(qq, uu, x, y, pb, wall);
+                    fl = to_fixed(t);
+                    mag = fx_mag(t);
                 }
             } else {
                 P nq[5];
@@ -129,14 +139,20 @@ __device__ __forceinline__ void item_update(const Problem& pb, DevStats* st, con
                     fl = float_to_fixed(t.hi);
                     fx_add(fl, float_to_fixed(t.lo));
                 } else {
-                    fl = to_fixed(wall5_closure_d(qq, uu, nq, x, y, pb, wall));
+                    const double t = wall5_closure_d(qq, uu, nq, x, y, pb, wall);
+                    fl = to_fixed(t);
+                    mag = fx_mag(t);
                 }
             }
 #pragma unroll
             for (int i = 0; i < Q; ++i) q[i] = qq[i];
         }
         fl = fx_tree(fl);
-        if (lane == 0) fx_add(w->f, fl);
+        const bool lost = sizeof(P) == 8 && __any_sync(kFull, mag >= kFxMag);
+        if (lane == 0) {
+            fx_add(w->f, fl);
+            if (lost) w->lost |= kLostFlux;
+        }
     }
     const P omc = sizeof(P) == 4 ? (P)pb.omc_f : (P)pb.omc;
     if constexpr (EEBM) {
@@ -617,7 +633,11 @@ __global__ void __launch_bounds__(kResidentThreads<P, Q>, 1) resident_kernel(con
                 }
             } while (t0 < a.tiles);
             const Fx e = acc.total();
-            if (lane == 0) fx_add(w->e, e);
+            const bool lost = acc.lost();
+            if (lane == 0) {
+                fx_add(w->e, e);
+                if (lost) w->lost |= kLostEnergy;
+            }
             __syncthreads();
             if (threadIdx.x == 0) {
                 queue.count = next_item = 0u;
