@@ -60,8 +60,8 @@ typedef enum {
     LBM_ERR_ARG = 1,     /* invalid argument (sizes, tau <= 1/2, Ste <= 0, delta <= 0, NULL, ...) */
     LBM_ERR_CUDA = 2,    /* a CUDA runtime call failed */
     LBM_ERR_NEWTON = 3,  /* a node's Newton solve hit its iteration limit, or a value was not finite */
-    LBM_ERR_TIMEOUT = 4, /* a bounded device wait ran out (the TMA row-pipeline kernel's waits for its row
-                            loads: FP32 D2Q9 batches, and single problems under lbm_stefan_set_wait_test) */
+    LBM_ERR_TIMEOUT = 4, /* a bounded device wait ran out: at a barrier of a resident launch (5 s), or for a
+                            row load of the TMA row-pipeline kernel (lbm_stefan_set_wait_test) */
     LBM_ERR_STATE = 5    /* call out of order (e.g. step before set_ic) */
 } lbm_status;
 
@@ -197,6 +197,20 @@ lbm_status lbm_stefan_step_timed(lbm_stefan* h, int nsteps, double* ms_kernels);
  * a value outside [-1, 2] or a wait limit outside (0, 60] s. */
 lbm_status lbm_stefan_set_wait_test(lbm_stefan* h, double wait_limit_s, int withhold_load);
 
+/* Test hook of the resident launches, whose blocks wait for one another at
+ * barriers in device memory.  wait_limit_s in (0, 60] bounds every such wait
+ * (default 5 s).  withhold >= 0: the first block does not arrive at that barrier
+ * of each launch (0: after the launch's first step; LBM_ILFBM: an inner
+ * iteration's), so the waits for it run out, the launch ends normally and the next
+ * synchronizing call returns LBM_ERR_TIMEOUT; the state is undefined until the
+ * next set_ic, which also clears the error.  max_blocks > 0: a launch of more
+ * blocks is refused as on a device that its grid does not fit, and the handle
+ * steps by the separate kernels from then on.  max_steps > 0: at most that many
+ * steps per launch.  (5.0, -1, 0, 0) restore normal launches.
+ * LBM_ERR_ARG for values outside these ranges.  The same for batches (set_ic of
+ * every problem after LBM_ERR_TIMEOUT). */
+lbm_status lbm_stefan_set_launch_test(lbm_stefan* h, double wait_limit_s, int withhold, int max_blocks, int max_steps);
+
 /* Advance nsteps steps and write theta(t+1), ..., theta(t+nsteps) to
  * theta_traj (device, nsteps planes of ny*row_stride doubles, row_stride from
  * lbm_stefan_layout).  Used to recompute a checkpoint segment for the adjoint. */
@@ -318,6 +332,7 @@ lbm_status lbm_stefan_batch_set_ic(lbm_stefan_batch* b, int k, const double* the
 lbm_status lbm_stefan_batch_step(lbm_stefan_batch* b, int nsteps);
 lbm_status lbm_stefan_batch_get_fields(lbm_stefan_batch* b, int k, double* theta, int on_device);
 lbm_status lbm_stefan_batch_get_stats(lbm_stefan_batch* b, int k, lbm_stefan_stats* out);
+lbm_status lbm_stefan_batch_set_launch_test(lbm_stefan_batch* b, double wait_limit_s, int withhold, int max_blocks, int max_steps);
 /* Time candidate schedules (FP64: and tile heights) for trial_steps steps
  * each and keep the fastest; the state is saved and restored around the
  * trials.  chosen_tile_h receives the chosen height (FP32: 8; may be NULL). */

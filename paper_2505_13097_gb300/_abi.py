@@ -66,6 +66,7 @@ SIGNATURES = {
     "lbm_stefan_step": (_S, [_V, _I]),
     "lbm_stefan_step_timed": (_S, [_V, _I, _D]),
     "lbm_stefan_set_wait_test": (_S, [_V, ctypes.c_double, _I]),
+    "lbm_stefan_set_launch_test": (_S, [_V, ctypes.c_double, _I, _I, _I]),
     "lbm_stefan_step_record": (_S, [_V, _I, _V]),
     "lbm_stefan_sync": (_S, [_V]),
     "lbm_stefan_get_fields": (_S, [_V, _V, _V, _V, _I]),
@@ -88,6 +89,7 @@ SIGNATURES = {
     "lbm_stefan_batch_step": (_S, [_V, _I]),
     "lbm_stefan_batch_get_fields": (_S, [_V, _I, _V, _I]),
     "lbm_stefan_batch_get_stats": (_S, [_V, _I, ctypes.POINTER(lbm_stefan_stats)]),
+    "lbm_stefan_batch_set_launch_test": (_S, [_V, ctypes.c_double, _I, _I, _I]),
     "lbm_stefan_batch_autotune": (_S, [_V, _I, ctypes.POINTER(ctypes.c_int)]),
     "lbm_stefan_batch_set_schedule": (_S, [_V, _I, _I]),
     "lbm_stefan_batch_destroy": (None, [_V]),

@@ -392,7 +392,7 @@ __device__ __forceinline__ bool inner_barrier(const Ilf2Args& a, unsigned turn, 
     unsigned long long* c = &a.bar->inner[turn & 1u];
     const unsigned long long target = (turn / 2ull + 1ull) * nb;
     fence_gpu();
-    atomicAdd(c, 1ull | (more ? 1ull << 48 : 0ull));
+    if ((int)turn != a.withhold || blockIdx.x != 0) atomicAdd(c, 1ull | (more ? 1ull << 48 : 0ull));
     unsigned long long v, t0 = 0;
     for (unsigned i = 0;; ++i) {
         asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(c) : "memory");
@@ -662,10 +662,10 @@ int ilfbm_2d_blocks(int q, int nx, int ny)
 }
 
 cudaError_t launch_ilfbm_2d(const Problem& hp, int parity, int nsteps, void* scratch, DevStats* stats, void* slots,
-                            ResidentBar* bar, long long wait_ns, cudaStream_t s)
+                            ResidentBar* bar, const ResidentLimits& lim, cudaStream_t s)
 {
     const int blocks = ilfbm_2d_blocks(hp.q, hp.nx, hp.ny);
-    if (blocks < 2) return cudaErrorCooperativeLaunchTooLarge;
+    if (blocks < 2 || lim.refuses(blocks)) return cudaErrorCooperativeLaunchTooLarge;
     Ilf2Args a;
     const size_t n = (size_t)hp.nx * hp.ny, units = ilf2_units(hp.nx, hp.ny);
     double* d = static_cast<double*>(scratch);
@@ -673,7 +673,8 @@ cudaError_t launch_ilfbm_2d(const Problem& hp, int parity, int nsteps, void* scr
     a.stats = stats;
     a.slots = static_cast<ResidentSlot*>(slots);
     a.bar = bar;
-    a.wait_ns = wait_ns;
+    a.wait_ns = lim.wait_ns;
+    a.withhold = lim.withhold;
     a.s0 = d;
     a.lb[0] = d + n;
     a.lb[1] = d + 2 * n;
@@ -689,7 +690,8 @@ cudaError_t launch_ilfbm_2d(const Problem& hp, int parity, int nsteps, void* scr
     at[0].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    const int most = (int)std::max<size_t>(2, std::min<size_t>(kIlf2Steps, ((size_t)1 << 24) / n));
+    int most = (int)std::max<size_t>(2, std::min<size_t>(kIlf2Steps, ((size_t)1 << 24) / n));
+    if (lim.max_steps > 0) most = std::min(most, lim.max_steps);
     while (nsteps > 0) {
         a.parity = parity;
         a.nsteps = nsteps < most ? nsteps : most;

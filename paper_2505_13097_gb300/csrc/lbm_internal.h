@@ -162,6 +162,15 @@ struct ResidentBar {
     // with a change above the tolerance in the high 16)
     unsigned long long inner[2];
 };
+// Bound of a resident launch's waits, and the test hook of these launches
+// (lbm_stefan_set_launch_test).
+struct ResidentLimits {
+    long long wait_ns = 5000000000LL;
+    int withhold = -1;       // >= 0: block 0 does not arrive at its launch's barrier of that number
+    int max_blocks = 0;      // > 0: larger grids are refused, as by a device they do not fit
+    int max_steps = 0;       // > 0: steps of one launch, at most
+    bool refuses(int blocks) const { return max_blocks > 0 && blocks > max_blocks; }
+};
 // How a resident launch covers a lattice; blocks == 0: it does not.
 struct ResidentPlan {
     int blocks = 0, threads = 0;   // blocks: the computing ones and one for the statistics
@@ -247,14 +256,15 @@ cudaError_t launch_newton_jobs(int precision, int q, const JobArgs& a, cudaStrea
 ResidentPlan resident_plan(int precision, int q, int nx, int ny);
 size_t resident_slot_bytes();
 cudaError_t launch_resident(int precision, const ResidentPlan& plan, const Problem& hp, int parity, int nsteps, double* rec,
-                            DevStats* stats, void* slots, ResidentBar* bar, long long wait_ns, cudaStream_t s);
+                            DevStats* stats, void* slots, ResidentBar* bar, const ResidentLimits& lim, cudaStream_t s);
 
 // FP32 D2Q9 batches in one cooperative launch; units: (problem, kind, strip or side,
 // first row); sums: resident_batch_bytes, zero before the first launch
 int resident_batch_blocks();
 size_t resident_batch_bytes(int count);
 cudaError_t launch_resident_batch(const Problem* probs, int count, const int4* units, int nunits, int blocks, int parity,
-                                  int nsteps, DevStats* stats, void* sums, ResidentBar* bar, long long wait_ns, cudaStream_t s);
+                                  int nsteps, DevStats* stats, void* sums, ResidentBar* bar, const ResidentLimits& lim,
+                                  cudaStream_t s);
 
 // D2Q5 launchers (step_d2q5.cu): one tile per warp over a.nslots tiles
 cudaError_t launch_d2q5_step(int precision, const StepArgs& a, cudaStream_t s);
@@ -276,7 +286,7 @@ bool ilfbm_d1q3_fits(int nx);
 size_t ilfbm_2d_scratch(int nx, int ny);
 int ilfbm_2d_blocks(int q, int nx, int ny);
 cudaError_t launch_ilfbm_2d(const Problem& hp, int parity, int nsteps, void* scratch, DevStats* stats, void* slots,
-                            ResidentBar* bar, long long wait_ns, cudaStream_t s);
+                            ResidentBar* bar, const ResidentLimits& lim, cudaStream_t s);
 
 // Field and state kernels (fields.cu)
 cudaError_t launch_init_state(int precision, const Problem* dprob, const Problem& hp, const double* theta0,

@@ -90,6 +90,7 @@ struct lbm_stefan {
     bool use_tma = false;              // FP32 D2Q9: the TMA row-pipeline kernel (for the wait test hook)
     lbm::TmaMaps tma;
     int withhold_load = -1;            // test hook of the TMA kernel's row loads (-1: off)
+    lbm::ResidentLimits lim;           // bound of the resident launches' waits, their test hook
     cudaStream_t side = nullptr;       // split FP32 D2Q9 step: stream of the left half's Newton solves
     cudaEvent_t ev_fork = nullptr, ev_half = nullptr, ev_join = nullptr;
     cudaEvent_t ev_walls = nullptr;   // split step: the wall kernels are done (list A's wall part is final)
@@ -154,6 +155,7 @@ struct lbm_stefan_batch {
     int nunits = 0;
     void* dsums = nullptr;
     lbm::ResidentBar* dbar = nullptr;
+    lbm::ResidentLimits lim;
     GraphCache graph;
 };
 
@@ -457,12 +459,13 @@ static cudaError_t launch_one(lbm_stefan* h, int parity, double* rec)
 // What a barrier takes before the sums of its launch.
 constexpr size_t kBarBytes = (sizeof(lbm::ResidentBar) + 255) / 256 * 256;
 
-// Bound of a wait at the resident step's barrier.
-constexpr long long kResidentWaitNs = 5000000000LL;
-
 // Steps of one resident launch: 2^32 node updates (some 60 ms), so that other streams
 // get the GPU in between; at most 8,192.
-static int resident_steps(long long nodes) { return (int)std::max(32ll, std::min(8192ll, (1ll << 32) / std::max(1ll, nodes))); }
+static int resident_steps(long long nodes, const lbm::ResidentLimits& lim)
+{
+    const int n = (int)std::max(32ll, std::min(8192ll, (1ll << 32) / std::max(1ll, nodes)));
+    return lim.max_steps > 0 ? std::min(n, lim.max_steps) : n;
+}
 
 // *nsteps steps by resident launches from state[*parity] on, theta' planes to *rec, if
 // given; the three advance with every launch.  cudaErrorCooperativeLaunchTooLarge: the grid
@@ -470,11 +473,11 @@ static int resident_steps(long long nodes) { return (int)std::max(32ll, std::min
 static cudaError_t run_resident(lbm_stefan* h, int* nsteps, int* parity, double** rec)
 {
     const long long plane = (long long)h->hp.ny * h->hp.pitch;
-    const int most = resident_steps((long long)h->hp.nx * h->hp.ny);
+    const int most = resident_steps((long long)h->hp.nx * h->hp.ny, h->lim);
     while (*nsteps > 0) {
         const int n = std::min(*nsteps, most);
         const cudaError_t e = lbm::launch_resident(h->precision, h->res, h->hp, *parity, n, *rec, h->dstats, h->dslots, h->dbar,
-                                                   kResidentWaitNs, h->stream);
+                                                   h->lim, h->stream);
         if (e != cudaSuccess) {
             if (e == cudaErrorCooperativeLaunchTooLarge) {
                 (void)cudaGetLastError();
@@ -841,7 +844,7 @@ extern "C" lbm_status lbm_stefan_step(lbm_stefan* h, int nsteps)
         // 2D: one cooperative launch, a barrier per inner iteration
         char* own = static_cast<char*>(h->dilf_slots);
         CUDA_TRY(lbm::launch_ilfbm_2d(h->hp, h->parity, nsteps, h->dilf, h->dstats, own ? own + kBarBytes : h->dslots,
-                                      own ? reinterpret_cast<lbm::ResidentBar*>(own) : h->dbar, kResidentWaitNs, h->stream));
+                                      own ? reinterpret_cast<lbm::ResidentBar*>(own) : h->dbar, h->lim, h->stream));
         h->parity ^= nsteps & 1;
         return LBM_OK;
     }
@@ -1046,6 +1049,32 @@ extern "C" lbm_status lbm_stefan_set_wait_test(lbm_stefan* h, double wait_limit_
     h->graph.reset();   // captured launches carry the old values
     h->reset_seg_graphs();
     return LBM_OK;
+}
+
+static lbm_status set_limits(lbm::ResidentLimits& lim, double wait_limit_s, int withhold, int max_blocks, int max_steps)
+{
+    if (!(wait_limit_s > 0.0) || !(wait_limit_s <= 60.0)) return fail(LBM_ERR_ARG, "wait_limit_s must be in (0, 60]");
+    if (withhold < -1 || max_blocks < 0 || max_steps < 0)
+        return fail(LBM_ERR_ARG, "withhold must be >= -1, max_blocks and max_steps >= 0");
+    lim.wait_ns = (long long)(wait_limit_s * 1e9);
+    lim.withhold = withhold;
+    lim.max_blocks = max_blocks;
+    lim.max_steps = max_steps;
+    return LBM_OK;
+}
+
+extern "C" lbm_status lbm_stefan_set_launch_test(lbm_stefan* h, double wait_limit_s, int withhold, int max_blocks, int max_steps)
+{
+    if (!h) return fail(LBM_ERR_ARG, "NULL handle");
+    h->reset_seg_graphs();   // captured launches carry the old values
+    return set_limits(h->lim, wait_limit_s, withhold, max_blocks, max_steps);
+}
+
+extern "C" lbm_status lbm_stefan_batch_set_launch_test(lbm_stefan_batch* b, double wait_limit_s, int withhold, int max_blocks,
+                                                       int max_steps)
+{
+    if (!b) return fail(LBM_ERR_ARG, "NULL handle");
+    return set_limits(b->lim, wait_limit_s, withhold, max_blocks, max_steps);
 }
 
 extern "C" lbm_status lbm_stefan_layout(lbm_stefan* h, size_t* state_bytes, int* row_stride)
@@ -1490,11 +1519,11 @@ static cudaError_t batch_launch_one(lbm_stefan_batch* b, int parity)
 // *nsteps with cudaSuccess is for the separate kernels (the grid does not fit here).
 static cudaError_t batch_run_resident(lbm_stefan_batch* b, int* nsteps)
 {
-    const int most = resident_steps((long long)b->total_nodes);
+    const int most = resident_steps((long long)b->total_nodes, b->lim);
     while (b->res_blocks > 0 && *nsteps > 0) {
         const int n = std::min(*nsteps, most);
         const cudaError_t e = lbm::launch_resident_batch(b->dprobs, b->count, b->dunits, b->nunits, b->res_blocks, b->parity, n,
-                                                         b->dstats, b->dsums, b->dbar, kResidentWaitNs, b->stream);
+                                                         b->dstats, b->dsums, b->dbar, b->lim, b->stream);
         if (e == cudaErrorCooperativeLaunchTooLarge) {
             (void)cudaGetLastError();
             b->res_blocks = 0;

@@ -25,6 +25,7 @@ struct ResidentCommon {
     ResidentSlot* slots;        // kResidentRing sets of one per computing block
     ResidentBar* bar;
     long long wait_ns;          // bound of a wait
+    int withhold;               // test hook: block 0 does not arrive at this barrier of the launch (-1: off)
 };
 
 // ---------------------------------------------------------------- grid barrier
@@ -72,19 +73,22 @@ __device__ __forceinline__ bool bar_wait(ResidentBar* b, const unsigned* count, 
 }
 
 // Every block at its end: the last one resets the barrier for the next launch.
-__device__ __forceinline__ void bar_leave(ResidentBar* bar)
+// Returns whether this is that block and a wait of the launch ran out.
+__device__ __forceinline__ bool bar_leave(ResidentBar* bar)
 {
-    __shared__ bool last;
+    __shared__ bool last, failed;
     __syncthreads();
     if (threadIdx.x == 0) {
         fence_gpu();
         last = atomicAdd(&bar->done, 1u) == gridDim.x - 1;
+        failed = last && ld_acquire(&bar->abort) != 0u;
     }
     __syncthreads();
     if (last) {
         unsigned* b = reinterpret_cast<unsigned*>(bar);
         for (int k = threadIdx.x; k < (int)(sizeof(ResidentBar) / 4); k += blockDim.x) b[k] = 0u;
     }
+    return failed;
 }
 
 // ---------------------------------------------------------------- a block's sums

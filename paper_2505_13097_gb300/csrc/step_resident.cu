@@ -641,7 +641,7 @@ __global__ void __launch_bounds__(kResidentThreads<P, Q>, 1) resident_kernel(con
             __syncthreads();
             if (threadIdx.x == 0) {
                 queue.count = next_item = 0u;
-                bar_arrive(&a.bar->count);
+                if (s != a.withhold || blockIdx.x != 0) bar_arrive(&a.bar->count);
                 ok_s = s + 1 == a.nsteps || bar_wait(a.bar, &a.bar->count, (unsigned)(s + 1) * nb, a.wait_ns);
             } else if (warp == 1) {
                 // while thread 0 waits
@@ -729,6 +729,16 @@ static __device__ __noinline__ void batch_stats(const ResidentBatchArgs& a, unsi
         for (int p = 0; p < a.count; ++p) atomicExch(&a.stats[p].error, 4);   // LBM_ERR_TIMEOUT
 }
 
+// A block at its end; after a wait that ran out the last one clears the sums that
+// nobody has read, so that the next launch does not add to them.
+static __device__ __noinline__ void batch_leave(const ResidentBatchArgs& a)
+{
+    if (!bar_leave(a.bar)) return;
+    unsigned long long* w = reinterpret_cast<unsigned long long*>(a.acc);
+    for (size_t k = threadIdx.x; k < (size_t)2 * a.count * kBatchStripes * (sizeof(StepStripe) / 8); k += blockDim.x) w[k] = 0ull;
+    for (int k = threadIdx.x; k < 2 * a.count; k += blockDim.x) a.maxit[k] = 0;
+}
+
 __global__ void __launch_bounds__(kBatchThreads, 1) resident_batch_kernel(const __grid_constant__ ResidentBatchArgs a)
 {
     __shared__ ResidentSlot wsum[kBatchWarps];
@@ -740,7 +750,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) resident_batch_kernel(const 
     const int nb = gridDim.x - 1;   // computing blocks; the last block publishes the statistics
     if ((int)blockIdx.x == nb) {
         batch_stats(a, (unsigned)nb, &ok_s);
-        bar_leave(a.bar);
+        batch_leave(a);
         return;
     }
     ResidentSlot* w = &wsum[warp];
@@ -814,7 +824,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) resident_batch_kernel(const 
         __syncthreads();
         if (threadIdx.x == 0) {
             next_unit = 0u;
-            bar_arrive(&a.bar->count);
+            if (s != a.withhold || blockIdx.x != 0) bar_arrive(&a.bar->count);
             // the next step adds to the set of step s - 1
             ok_s = s + 1 == a.nsteps || (bar_wait(a.bar, &a.bar->count, (unsigned)(s + 1) * nb, a.wait_ns) &&
                                          bar_wait(a.bar, &a.bar->read[0], (unsigned)s, a.wait_ns));
@@ -822,7 +832,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) resident_batch_kernel(const 
         __syncthreads();
         ok = ok_s;
     }
-    bar_leave(a.bar);
+    batch_leave(a);
 }
 
 static size_t batch_smem() { return sizeof(unsigned) * 1024 * kBatchWarps; }
@@ -841,14 +851,17 @@ int resident_batch_blocks()
 size_t resident_batch_bytes(int count) { return (size_t)2 * count * (kBatchStripes * sizeof(StepStripe) + sizeof(int)); }
 
 cudaError_t launch_resident_batch(const Problem* probs, int count, const int4* units, int nunits, int blocks, int parity,
-                                  int nsteps, DevStats* stats, void* sums, ResidentBar* bar, long long wait_ns, cudaStream_t s)
+                                  int nsteps, DevStats* stats, void* sums, ResidentBar* bar, const ResidentLimits& lim,
+                                  cudaStream_t s)
 {
+    if (lim.refuses(blocks)) return cudaErrorCooperativeLaunchTooLarge;
     ResidentBatchArgs a;
     a.nsteps = nsteps;
     a.stats = stats;
     a.slots = nullptr;
     a.bar = bar;
-    a.wait_ns = wait_ns;
+    a.wait_ns = lim.wait_ns;
+    a.withhold = lim.withhold;
     a.probs = probs;
     a.count = count;
     a.units = units;
@@ -954,8 +967,9 @@ ResidentPlan resident_plan(int precision, int q, int nx, int ny)
 }
 
 cudaError_t launch_resident(int precision, const ResidentPlan& plan, const Problem& hp, int parity, int nsteps, double* rec,
-                            DevStats* stats, void* slots, ResidentBar* bar, long long wait_ns, cudaStream_t s)
+                            DevStats* stats, void* slots, ResidentBar* bar, const ResidentLimits& lim, cudaStream_t s)
 {
+    if (lim.refuses(plan.blocks)) return cudaErrorCooperativeLaunchTooLarge;
     ResidentArgs a;
     a.pb = hp;
     a.parity = parity;
@@ -970,7 +984,8 @@ cudaError_t launch_resident(int precision, const ResidentPlan& plan, const Probl
     a.nseg = plan.nseg;
     a.items = plan.items;
     a.rot = plan.rot;
-    a.wait_ns = wait_ns;
+    a.wait_ns = lim.wait_ns;
+    a.withhold = lim.withhold;
     const bool eebm = hp.method == 1;
     if (hp.q == 9) {
         if (precision == 1)

@@ -120,6 +120,12 @@ class Stefan:
         load is withheld this FP32 D2Q9 handle steps with that kernel (-1: off)."""
         check(self.lib.lbm_stefan_set_wait_test(self.h, float(wait_limit_s), int(withhold_load)))
 
+    def set_launch_test(self, wait_limit_s=5.0, withhold=-1, max_blocks=0, max_steps=0):
+        """Test hook of the resident launches: bound of their waits, a barrier at which
+        the first block does not arrive (-1: none), the largest grid and the most steps
+        of a launch (0: no limit)."""
+        check(self.lib.lbm_stefan_set_launch_test(self.h, float(wait_limit_s), int(withhold), int(max_blocks), int(max_steps)))
+
     def step_record(self, n, traj):
         """traj: CUDA float64 tensor holding at least n planes of ny x row_stride."""
         if not _is_cuda_tensor(traj) or traj.dtype != torch.float64:
@@ -263,6 +269,11 @@ class StefanBatch:
         s = _abi.lbm_stefan_stats()
         check(self.lib.lbm_stefan_batch_get_stats(self.h, int(k), ctypes.byref(s)))
         return s.as_dict()
+
+    def set_launch_test(self, wait_limit_s=5.0, withhold=-1, max_blocks=0, max_steps=0):
+        """Test hook of the resident launches, as Stefan.set_launch_test."""
+        check(self.lib.lbm_stefan_batch_set_launch_test(self.h, float(wait_limit_s), int(withhold), int(max_blocks),
+                                                        int(max_steps)))
 
     def autotune(self, trial_steps=20):
         th = ctypes.c_int()
