@@ -393,14 +393,14 @@ __device__ __forceinline__ bool inner_barrier(const Ilf2Args& a, unsigned turn, 
     const unsigned long long target = (turn / 2ull + 1ull) * nb;
     fence_gpu();
     if ((int)turn != a.withhold || blockIdx.x != 0) atomicAdd(c, 1ull | (more ? 1ull << 48 : 0ull));
-    unsigned long long v, t0 = 0;
+    unsigned long long v;
+    WaitClock clock;
     for (unsigned i = 0;; ++i) {
-        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(c) : "memory");
+        v = ld_relaxed(c);
         if ((v & 0xffffffffffffull) >= target) break;
         if ((i & 63u) == 63u) {
             if (ld_acquire(&a.bar->abort)) return false;
-            if (t0 == 0) t0 = global_ns();
-            else if ((long long)(global_ns() - t0) > a.wait_ns) {
+            if (wait_over(a.bar, v, clock, a.wait_ns)) {
                 atomicExch(&a.bar->abort, 1u);
                 return false;
             }

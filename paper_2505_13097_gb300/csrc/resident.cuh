@@ -51,18 +51,47 @@ __device__ __forceinline__ void bar_arrive(unsigned* count)
     atomicAdd(count, 1u);
 }
 
-// One thread: waits until *count has reached `target`, for at most limit_ns;
-// false when the wait ran out here or in another block.  The polls are relaxed
-// (an acquiring load drops the SM's L1 lines each time); one fence follows.
+__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long* p)
+{
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// The bound of a wait: limit_ns without an arrival at any barrier of the launch.
+// Counted from the wait's start it would end correct runs: a warp of the
+// statistics block waits for as many steps as the block has warps, each of up to
+// newton_max_iter barriers in the 2D ILFBM launch.
+struct WaitClock {
+    unsigned long long t0 = 0, seen = 0;
+};
+
+// Now and then during a wait for *word: whether it has run out (arrivals are looked
+// at once per limit, so that it runs out after one to two limits).
+__device__ __forceinline__ bool wait_over(ResidentBar* b, unsigned long long word, WaitClock& c, long long limit_ns)
+{
+    const unsigned long long now = global_ns();
+    if (c.t0 != 0 && (long long)(now - c.t0) <= limit_ns) return false;
+    // counters that only grow during a launch
+    const unsigned long long seen = word + ld_relaxed(&b->count) + ld_relaxed(&b->inner[0]) + ld_relaxed(&b->inner[1]);
+    const bool over = c.t0 != 0 && seen == c.seen;
+    c.t0 = now;
+    c.seen = seen;
+    return over;
+}
+
+// One thread: waits until *count has reached `target`; false when the wait ran out
+// here or in another block.  The polls are relaxed (an acquiring load drops the
+// SM's L1 lines each time); one fence follows.
 __device__ __forceinline__ bool bar_wait(ResidentBar* b, const unsigned* count, unsigned target, long long limit_ns)
 {
-    unsigned long long t0 = 0;
+    WaitClock clock;
     for (unsigned i = 0;; ++i) {
-        if ((int)(ld_relaxed(count) - target) >= 0) break;
+        const unsigned v = ld_relaxed(count);
+        if ((int)(v - target) >= 0) break;
         if ((i & 63u) == 63u) {
             if (ld_relaxed(&b->abort)) return false;
-            if (t0 == 0) t0 = global_ns();
-            else if ((long long)(global_ns() - t0) > limit_ns) {
+            if (wait_over(b, v, clock, limit_ns)) {
                 atomicExch(&b->abort, 1u);
                 return false;
             }

@@ -80,6 +80,26 @@ def test_batch_after_a_timeout(withhold):
         assert np.array_equal(x[2], y[2])
 
 
+@pytest.mark.parametrize("lattice,limit,steps,maxit", [(2, 0.002, 100, 400), (3, 0.005, 2, 20000)])
+def test_a_long_step_is_no_timeout(lattice, limit, steps, maxit):
+    """The bound counts from the last arrival of any block: a launch whose steps (D2Q5: many
+    inner iterations) or whose statistics' waits (16 steps ahead) last longer runs to its end."""
+    import torch
+    from paper_2505_13097_gb300 import solver
+    out = []
+    for w in (limit, 5.0):
+        S = solver.Stefan(lattice, 200, 150, 0.84, 0.01, 0.0521, 0, {"W": (1, -2.0), "S": (1, -2.0)},
+                          stream=torch.cuda.Stream(), newton_tol=1e-12, newton_max_iter=maxit)
+        S.set_method("ILFBM")
+        S.set_launch_test(wait_limit_s=w)
+        S.set_ic(_field(200, 150) + 0.7)
+        S.step(steps)
+        out.append((S.stats(), S.theta()))
+        S.close()
+    assert out[0][0]["newton_max_iter"] > 20 and out[0][0] == out[1][0]
+    assert np.array_equal(out[0][1], out[1][1])
+
+
 def test_hook_rejects_bad_values():
     from paper_2505_13097_gb300 import _abi, solver
     c = workloads.melt_2d(n=64, steps=1)
