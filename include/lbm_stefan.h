@@ -205,8 +205,9 @@ lbm_status lbm_stefan_set_wait_test(lbm_stefan* h, double wait_limit_s, int with
  * synchronizing call returns LBM_ERR_TIMEOUT; the state is undefined until the
  * next set_ic, which also clears the error.  max_blocks > 0: a launch of more
  * blocks is refused as on a device that its grid does not fit, and the handle
- * steps by the separate kernels from then on.  max_steps > 0: at most that many
- * steps per launch.  (5.0, -1, 0, 0) restore normal launches.
+ * steps by the separate kernels from then on (2D LBM_ILFBM: by grids halved until
+ * one fits; none of 2 blocks or more: LBM_ERR_CUDA).  max_steps > 0: at most that
+ * many steps per launch.  (5.0, -1, 0, 0) restore normal launches.
  * LBM_ERR_ARG for values outside these ranges.  The same for batches (set_ic of
  * every problem after LBM_ERR_TIMEOUT). */
 lbm_status lbm_stefan_set_launch_test(lbm_stefan* h, double wait_limit_s, int withhold, int max_blocks, int max_steps);

@@ -656,16 +656,14 @@ int ilfbm_2d_blocks(int q, int nx, int ny)
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         (q == 9 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, ilf2_kernel<9>, kIlf2Threads, 0)
                 : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, ilf2_kernel<5>, kIlf2Threads, 0)) != cudaSuccess)
-        return 0;
+        return 2;
     const long long want = ((long long)ilf2_units(nx, ny) + kIlf2Threads / 32 - 1) / (kIlf2Threads / 32) + 1;
-    return (int)(want < (long long)sms * per ? want : (long long)sms * per);
+    return (int)std::max(2ll, std::min(want, (long long)sms * per));
 }
 
-cudaError_t launch_ilfbm_2d(const Problem& hp, int parity, int nsteps, void* scratch, DevStats* stats, void* slots,
-                            ResidentBar* bar, const ResidentLimits& lim, cudaStream_t s)
+cudaError_t launch_ilfbm_2d(const Problem& hp, int* parity, int* nsteps, int* blocks, void* scratch, DevStats* stats,
+                            void* slots, ResidentBar* bar, const ResidentLimits& lim, cudaStream_t s)
 {
-    const int blocks = ilfbm_2d_blocks(hp.q, hp.nx, hp.ny);
-    if (blocks < 2 || lim.refuses(blocks)) return cudaErrorCooperativeLaunchTooLarge;
     Ilf2Args a;
     const size_t n = (size_t)hp.nx * hp.ny, units = ilf2_units(hp.nx, hp.ny);
     double* d = static_cast<double*>(scratch);
@@ -682,7 +680,6 @@ cudaError_t launch_ilfbm_2d(const Problem& hp, int parity, int nsteps, void* scr
     a.dl[1] = d + 4 * n;
     for (int k = 0; k < 3; ++k) a.chg[k] = reinterpret_cast<unsigned char*>(d + 5 * n) + k * units;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3(kIlf2Threads);
     cfg.stream = s;
     cudaLaunchAttribute at[1];
@@ -692,13 +689,23 @@ cudaError_t launch_ilfbm_2d(const Problem& hp, int parity, int nsteps, void* scr
     cfg.numAttrs = 1;
     int most = (int)std::max<size_t>(2, std::min<size_t>(kIlf2Steps, ((size_t)1 << 24) / n));
     if (lim.max_steps > 0) most = std::min(most, lim.max_steps);
-    while (nsteps > 0) {
-        a.parity = parity;
-        a.nsteps = nsteps < most ? nsteps : most;
-        const cudaError_t e = hp.q == 9 ? cudaLaunchKernelEx(&cfg, ilf2_kernel<9>, a) : cudaLaunchKernelEx(&cfg, ilf2_kernel<5>, a);
+    while (*nsteps > 0) {
+        a.parity = *parity;
+        a.nsteps = std::min(*nsteps, most);
+        cfg.gridDim = dim3((unsigned)*blocks);
+        cudaError_t e = cudaErrorCooperativeLaunchTooLarge;
+        if (!lim.refuses(*blocks))
+            e = hp.q == 9 ? cudaLaunchKernelEx(&cfg, ilf2_kernel<9>, a) : cudaLaunchKernelEx(&cfg, ilf2_kernel<5>, a);
+        if (e == cudaErrorCooperativeLaunchTooLarge && *blocks > 2) {
+            // the grid does not fit here (SMs held back from this process): the kernel's blocks
+            // take the lattice in strides, so any number of them will do
+            (void)cudaGetLastError();
+            *blocks = std::max(2, *blocks / 2);
+            continue;
+        }
         if (e != cudaSuccess) return e;
-        parity ^= a.nsteps & 1;
-        nsteps -= a.nsteps;
+        *parity ^= a.nsteps & 1;
+        *nsteps -= a.nsteps;
     }
     return cudaSuccess;
 }

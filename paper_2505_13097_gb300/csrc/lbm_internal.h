@@ -280,13 +280,14 @@ bool d1q3_fused_fits(int precision, int nx);
 // ILFBM (Algorithm 1) on D1Q3, FP64, one block over the whole lattice (ilfbm.cu)
 cudaError_t launch_ilfbm_d1q3(const StepArgs& a, const Problem& hp, int nsteps, bool from_device, cudaStream_t s);
 bool ilfbm_d1q3_fits(int nx);
-// nsteps ILFBM steps on D2Q9 / D2Q5 (hp.q), FP64, in one cooperative launch; scratch:
-// ilfbm_2d_scratch bytes, slots and bar as for launch_resident (ilfbm_2d_blocks - 1 slots
-// per set); hp: the host copy, passed by value
+// *nsteps ILFBM steps on D2Q9 / D2Q5 (hp.q), FP64, from state[*parity] on, by cooperative
+// launches (nsteps and parity advance with each); scratch: ilfbm_2d_scratch bytes, slots and
+// bar as for launch_resident (*blocks - 1 slots per set); hp: the host copy, passed by value.
+// *blocks: the grid, ilfbm_2d_blocks at first; halved where it does not fit
 size_t ilfbm_2d_scratch(int nx, int ny);
 int ilfbm_2d_blocks(int q, int nx, int ny);
-cudaError_t launch_ilfbm_2d(const Problem& hp, int parity, int nsteps, void* scratch, DevStats* stats, void* slots,
-                            ResidentBar* bar, const ResidentLimits& lim, cudaStream_t s);
+cudaError_t launch_ilfbm_2d(const Problem& hp, int* parity, int* nsteps, int* blocks, void* scratch, DevStats* stats,
+                            void* slots, ResidentBar* bar, const ResidentLimits& lim, cudaStream_t s);
 
 // Field and state kernels (fields.cu)
 cudaError_t launch_init_state(int precision, const Problem* dprob, const Problem& hp, const double* theta0,

@@ -86,6 +86,7 @@ struct lbm_stefan {
     int adj_tile_h = lbm::kAdjTileH;   // rows per warp tile of the D2Q9 adjoint
     void* dilf = nullptr;              // 2D ILFBM: S0, two l iterates, two l differences, changed units
     void* dilf_slots = nullptr;        // 2D ILFBM: barrier and sums of its own, where dslots has no room for them
+    int ilf_blocks = 0;                // 2D ILFBM: blocks of a launch
     bool flat = false;                 // FP32 D2Q9: the flat and wall kernels
     bool use_tma = false;              // FP32 D2Q9: the TMA row-pipeline kernel (for the wait test hook)
     lbm::TmaMaps tma;
@@ -770,8 +771,8 @@ extern "C" lbm_status lbm_stefan_set_method(lbm_stefan* h, int method)
                 h->hp.tail_off = (long long)(need - kStateTail);
             }
             if (!h->dilf) {
-                const int blocks = lbm::ilfbm_2d_blocks(h->hp.q, h->hp.nx, h->hp.ny);
-                const size_t slots = (size_t)lbm::kResidentRing * std::max(1, blocks - 1);
+                h->ilf_blocks = lbm::ilfbm_2d_blocks(h->hp.q, h->hp.nx, h->hp.ny);
+                const size_t slots = (size_t)lbm::kResidentRing * (h->ilf_blocks - 1);
                 if (slots > h->res.slots && !h->dilf_slots) {
                     CUDA_TRY(cudaMalloc(&h->dilf_slots, kBarBytes + slots * lbm::resident_slot_bytes()));
                     CUDA_TRY(cudaMemsetAsync(h->dilf_slots, 0, sizeof(lbm::ResidentBar), h->stream));
@@ -841,11 +842,11 @@ extern "C" lbm_status lbm_stefan_step(lbm_stefan* h, int nsteps)
         return LBM_OK;
     }
     if (h->hp.method == LBM_ILFBM) {
-        // 2D: one cooperative launch, a barrier per inner iteration
+        // 2D: cooperative launches, a barrier per inner iteration
         char* own = static_cast<char*>(h->dilf_slots);
-        CUDA_TRY(lbm::launch_ilfbm_2d(h->hp, h->parity, nsteps, h->dilf, h->dstats, own ? own + kBarBytes : h->dslots,
+        CUDA_TRY(lbm::launch_ilfbm_2d(h->hp, &h->parity, &nsteps, &h->ilf_blocks, h->dilf, h->dstats,
+                                      own ? own + kBarBytes : h->dslots,
                                       own ? reinterpret_cast<lbm::ResidentBar*>(own) : h->dbar, h->lim, h->stream));
-        h->parity ^= nsteps & 1;
         return LBM_OK;
     }
     if (h->p.lattice == LBM_D1Q3 && lbm::d1q3_fused_fits(h->precision, h->hp.nx)) {
