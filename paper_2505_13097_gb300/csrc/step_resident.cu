@@ -591,6 +591,10 @@ __global__ void __launch_bounds__(kResidentThreads<P, Q>, 1) resident_kernel(con
                 if (a.tiles) __syncthreads();
                 const unsigned queued = queue.count;
                 const unsigned total = own + (queued + 31u) / 32u;
+                // the first items, the block's own among them, are dealt, the others taken: an FP32
+                // lane adds its nodes' terms in float pairs, whose rounding depends on their order;
+                // the queued nodes' terms are added exactly
+                const unsigned dealt = own > (unsigned)nwb ? (own + nwb - 1u) / nwb * nwb : (unsigned)nwb;
                 unsigned it = (unsigned)warp;
                 while (it < total) {
                     int x = 0, y = 0;
@@ -620,9 +624,10 @@ __global__ void __launch_bounds__(kResidentThreads<P, Q>, 1) resident_kernel(con
                         }
                     }
                     item_update<P, Q, EEBM>(pb, a.stats, src, dst, rec, x, y, valid, lane, sh, acc, w);
-                    // the first items are dealt, the others taken
-                    if (total <= (unsigned)nwb) break;
-                    if (lane == 0) it = (unsigned)nwb + atomicAdd(&next_item, 1u);
+                    it += nwb;
+                    if (it < dealt) continue;
+                    if (total <= dealt) break;
+                    if (lane == 0) it = dealt + atomicAdd(&next_item, 1u);
                     it = __shfl_sync(kFull, it, 0);
                 }
                 own = 0u;
