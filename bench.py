@@ -50,18 +50,10 @@ FLAT_TRAFFIC_NOTE = ("ncu capture of one launch (left half of the strips) on the
                      "still in L2 when the launch ends are written back during the next; scaled by nodes")
 
 
-# DRAM bytes per node and step of the resident D2Q9 FP32 kernel (ncu, a smaller case), None: not captured
-RESIDENT_TRAFFIC_PER_NODE = None
-RESIDENT_TRAFFIC_NOTE = None
-
-
-def resident_launches(nx, ny, steps):
-    """Launches of `steps` FP32 D2Q9 IREBM steps that run resident (up to 2^25
-    nodes; a launch runs up to 2^32 node updates, 32 to 8,192 steps); None for
-    larger lattices, whose steps are separate kernels."""
-    if nx * ny > 1 << 25:
-        return None
-    return -(-steps // max(32, min(8192, (1 << 32) // (nx * ny))))
+# DRAM bytes (read + write) per node and step of the resident D2Q9 FP32 kernel
+RESIDENT_TRAFFIC_PER_NODE = (650978816 + 581882368) / (4 * 2048 * 2048)
+RESIDENT_TRAFFIC_NOTE = ("ncu capture of one launch of four steps on the 2048^2 melting front: 651 MB read + 582 MB "
+                         "written, 73.5 B per node and step; scaled by nodes and steps")
 
 
 def flat_nodes(nx, ny):
@@ -183,13 +175,16 @@ def bench_single(torch, solver, case, steps, warmup, stream, barrier=None, centr
     S.sync()
     if barrier:
         barrier()
+    before = S.resident_launches()
     ms = time_steps(torch, S, steps, stream)
+    launches, resident = (b - a for a, b in zip(before, S.resident_launches()))
     st = S.stats()
     # per-kernel device times of the separate kernels (lbm_stefan_step_timed; resident steps have one kernel)
     if case.lattice == 2 and case.precision == 1:
         k0, k1, kf = S.step_timed(min(steps, 50), flat=True)
         st["kernel_ms"], st["flat_ms"] = (k0, k1), kf
-        st["resident_launches"] = resident_launches(case.nx, case.ny, steps)
+        # None: the timed steps were separate kernels
+        st["resident_launches"] = launches if resident == steps else None
     else:
         st["kernel_ms"] = S.step_timed(min(steps, 50)) if case.lattice in (2, 3) else None
     S.close()

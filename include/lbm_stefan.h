@@ -212,6 +212,12 @@ lbm_status lbm_stefan_set_wait_test(lbm_stefan* h, double wait_limit_s, int with
  * every problem after LBM_ERR_TIMEOUT). */
 lbm_status lbm_stefan_set_launch_test(lbm_stefan* h, double wait_limit_s, int withhold, int max_blocks, int max_steps);
 
+/* How the handle has stepped: D2Q9 / D2Q5 launches of IREBM and EEBM steps that ran
+ * resident since its creation (those of a captured adjoint segment count when it is
+ * captured), and the steps in them; the other steps ran by the separate kernels.
+ * Either pointer may be NULL.  For measurements. */
+lbm_status lbm_stefan_resident_launches(lbm_stefan* h, long long* launches, long long* steps);
+
 /* Advance nsteps steps and write theta(t+1), ..., theta(t+nsteps) to
  * theta_traj (device, nsteps planes of ny*row_stride doubles, row_stride from
  * lbm_stefan_layout).  Used to recompute a checkpoint segment for the adjoint. */

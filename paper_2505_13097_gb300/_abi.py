@@ -54,6 +54,7 @@ class lbm_stefan_problem(ctypes.Structure):
 
 _V = ctypes.c_void_p
 _D = ctypes.POINTER(ctypes.c_double)
+_L = ctypes.POINTER(ctypes.c_longlong)
 _I = ctypes.c_int
 _S = ctypes.c_int   # lbm_status
 
@@ -66,6 +67,7 @@ SIGNATURES = {
     "lbm_stefan_step": (_S, [_V, _I]),
     "lbm_stefan_step_timed": (_S, [_V, _I, _D]),
     "lbm_stefan_set_wait_test": (_S, [_V, ctypes.c_double, _I]),
+    "lbm_stefan_resident_launches": (_S, [_V, _L, _L]),
     "lbm_stefan_set_launch_test": (_S, [_V, ctypes.c_double, _I, _I, _I]),
     "lbm_stefan_step_record": (_S, [_V, _I, _V]),
     "lbm_stefan_sync": (_S, [_V]),

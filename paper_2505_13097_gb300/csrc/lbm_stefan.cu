@@ -92,6 +92,7 @@ struct lbm_stefan {
     lbm::TmaMaps tma;
     int withhold_load = -1;            // test hook of the TMA kernel's row loads (-1: off)
     lbm::ResidentLimits lim;           // bound of the resident launches' waits, their test hook
+    long long res_launches = 0, res_steps = 0;   // resident launches of this handle, and their steps
     cudaStream_t side = nullptr;       // split FP32 D2Q9 step: stream of the left half's Newton solves
     cudaEvent_t ev_fork = nullptr, ev_half = nullptr, ev_join = nullptr;
     cudaEvent_t ev_walls = nullptr;   // split step: the wall kernels are done (list A's wall part is final)
@@ -486,6 +487,8 @@ static cudaError_t run_resident(lbm_stefan* h, int* nsteps, int* parity, double*
             }
             return e;
         }
+        ++h->res_launches;
+        h->res_steps += n;
         *parity ^= n & 1;
         *nsteps -= n;
         if (*rec) *rec += n * plane;
@@ -1049,6 +1052,14 @@ extern "C" lbm_status lbm_stefan_set_wait_test(lbm_stefan* h, double wait_limit_
     h->withhold_load = withhold_load;
     h->graph.reset();   // captured launches carry the old values
     h->reset_seg_graphs();
+    return LBM_OK;
+}
+
+extern "C" lbm_status lbm_stefan_resident_launches(lbm_stefan* h, long long* launches, long long* steps)
+{
+    if (!h) return fail(LBM_ERR_ARG, "NULL handle");
+    if (launches) *launches = h->res_launches;
+    if (steps) *steps = h->res_steps;
     return LBM_OK;
 }
 

@@ -126,6 +126,12 @@ class Stefan:
         of a launch (0: no limit)."""
         check(self.lib.lbm_stefan_set_launch_test(self.h, float(wait_limit_s), int(withhold), int(max_blocks), int(max_steps)))
 
+    def resident_launches(self):
+        """(launches, steps) that ran resident since the handle was made."""
+        a, b = ctypes.c_longlong(), ctypes.c_longlong()
+        check(self.lib.lbm_stefan_resident_launches(self.h, ctypes.byref(a), ctypes.byref(b)))
+        return a.value, b.value
+
     def step_record(self, n, traj):
         """traj: CUDA float64 tensor holding at least n planes of ny x row_stride."""
         if not _is_cuda_tensor(traj) or traj.dtype != torch.float64:

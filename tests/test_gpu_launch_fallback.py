@@ -170,3 +170,22 @@ def test_handles_side_by_side():
         t.join()
     for (th, st), (t2, s2) in zip(alone, got):
         assert np.array_equal(th, t2) and st == s2
+
+
+def test_launch_counts():
+    """What bench.py reports as launches: counted where they are made."""
+    import torch
+    from paper_2505_13097_gb300 import solver
+    S = solver.Stefan(2, 1021, 777, 1.0, 0.01, 0.1, 1, {"W": (1, 1.0)}, stream=torch.cuda.Stream())
+    S.set_ic(_field(1021, 777))
+    assert S.resident_launches() == (0, 0)
+    S.step(6000)   # 2^32 node updates, 5,413 steps, in a launch
+    assert S.resident_launches() == (2, 6000)
+    S.set_launch_test(max_steps=4)
+    S.step(10)
+    assert S.resident_launches() == (5, 6010)
+    S.set_launch_test(max_blocks=1)
+    S.step(40)
+    S.sync()
+    assert S.resident_launches() == (5, 6010) and S.stats()["steps"] == 6050
+    S.close()
