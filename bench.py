@@ -3,8 +3,8 @@
 Headline: D2Q9 MLUPS of the step in the FP32 form (FP32 populations, FP64
 Newton; the steps run in resident cooperative launches of up to 2^32 node
 updates; lattices of more than 2^25 nodes: six launches per step) on the
-4096 x 4096 melting workload, timed with CUDA events on the launching stream over --steps steps after --warmup untimed steps.  The
-timed window sits at the middle of the 10,000-step job (the state is first
+4096 x 4096 melting workload, timed with CUDA events on the launching stream
+over --steps steps after --warmup untimed steps.  The timed window sits at the middle of the 10,000-step job (the state is first
 advanced, untimed, to step 5,000 - (warmup + steps)/2) so the Newton front band
 has its average width.  The state (1.2 GB) is larger than L2 (129 MB), so
 every step reads and writes HBM; no flush is needed.

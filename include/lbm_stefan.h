@@ -10,9 +10,12 @@
  * local Newton solve of Eq. (14), the source of Eq. (13), and the next
  * collision.  D2Q9 and D2Q5 lattices up to 2^25 nodes (FP32 D2Q9; its EEBM
  * 2^24) or 2^31 elements of a state (the other forms) run all the steps of a
- * call in cooperative launches (of up to 2^32 node updates and 8,192 steps) whose
- * blocks stay on the GPU and meet at a barrier after every step; so do FP32
- * batches.  Kernel launches per step otherwise: D2Q9 with FP32 populations, four on
+ * call in cooperative launches (of up to 2^32 node updates, but 32 steps at least
+ * and 8,192 at most) whose blocks stay on the GPU and meet at a barrier after
+ * every step; so do FP32 batches and LBM_ILFBM on D2Q9 / D2Q5.  Steps that the
+ * caller captures into a CUDA graph of its own, and those of a device that the
+ * cooperative grid does not fit, run as separate launches, which read walls and
+ * Stefan number on the device.  Kernel launches per step then: D2Q9 with FP32 populations, four on
  * the legacy default stream (the nodes on or next to a wall in two, rows 1 .. ny-2
  * of every 128-column strip, then the kernel that solves the list of nodes
  * that need the Newton iteration and publishes the step), six on a stream of
@@ -41,7 +44,9 @@
  *  - Kernels run asynchronously on the stream given at creation.  Errors the
  *    device detects (Newton not converged, non-finite values) are sticky and
  *    returned by the next call that synchronizes (lbm_stefan_sync,
- *    lbm_stefan_get_fields, lbm_stefan_get_stats, ...).
+ *    lbm_stefan_get_fields, lbm_stefan_get_stats, ...).  LBM_EEBM and LBM_ILFBM
+ *    solve nothing that would notice a non-finite value: in FP64 (D1Q3: also FP32)
+ *    the energy, flux and imbalance of such a state are NaN.
  */
 #ifndef LBM_STEFAN_H
 #define LBM_STEFAN_H
@@ -91,7 +96,8 @@ typedef struct {
 } lbm_stefan_params;
 
 typedef struct {
-    double energy;         /* E = sum_x theta + phi(theta)/Ste after the last step (FP64) */
+    double energy;         /* E = sum_x theta + phi(theta)/Ste after the last step (FP64); NaN if a
+                              term is not finite or 2^67 or more */
     double energy_prev;    /* E before the last step */
     double flux;           /* boundary flux of the last step: filled q minus Omega leaving */
     double imbalance;      /* E - energy_prev - flux of the last step (energy balance) */
@@ -145,9 +151,9 @@ lbm_status lbm_stefan_set_ste(lbm_stefan* h, double ste);
  * lbm_stefan_set_ic afterwards.  LBM_ERR_ARG for an unknown method.
  * LBM_ILFBM: the implicit liquid fraction based method of Algorithm 1
  * (Sec. 3.3), the paper's other comparison scheme, in FP64 on D1Q3 (up to
- * 2,844 nodes, one block) and on D2Q9 / D2Q5 (one launch per inner
- * iteration; the state buffers grow by one plane, so lbm_stefan_layout's
- * state_bytes changes): theta = M0(f), f_i^eq = w_i theta, and a
+ * 2,844 nodes, one block) and on D2Q9 / D2Q5 (cooperative launches of up to
+ * 256 steps, a grid barrier per inner iteration; the state buffers grow by one
+ * plane, so lbm_stefan_layout's state_bytes changes): theta = M0(f), f_i^eq = w_i theta, and a
  * liquid-fraction field l (the plane after the q populations: the fourth
  * plane of the D1Q3 state, zero for the other methods) updated
  * by an inner loop of collision with the source (w_i/Ste)(l - l^(k-1)),
@@ -171,35 +177,37 @@ lbm_status lbm_stefan_set_ic(lbm_stefan* h, const double* theta0, int on_device)
  * Every step also forms the energy E and the boundary flux on the device. */
 lbm_status lbm_stefan_step(lbm_stefan* h, int nsteps);
 
-/* D2Q9 and D2Q5: advance nsteps >= 1 steps launched one by one (no graph) with a
- * CUDA event before, between and after the kernels of each step, wait for
- * them, and return the mean device time per step of each kernel in ms:
+/* D2Q9 and D2Q5: advance nsteps >= 1 steps by the separate kernels (not the
+ * resident ones that lbm_stefan_step runs where it can), launched one by one (no
+ * graph) with a CUDA event before, between and after the kernels of each step, wait
+ * for them, and return the mean device time per step of each kernel in ms:
  * ms_kernels (3 doubles): [0] the stream/collide kernel (FP32 D2Q9: every
  * launch of the step but the last Newton launch), [1] the (last) Newton job
  * kernel, [2] FP32 D2Q9: the flat kernel's launches alone (events on the
- * handle's stream around each; 0 for the other forms).  Same result as
- * lbm_stefan_step; for measuring each kernel against its roofline.
- * Synchronizes. */
+ * handle's stream around each; 0 for the other forms).  The populations of
+ * lbm_stefan_step, in FP32 bit for bit, in FP64 up to rounding; for measuring
+ * each kernel against its roofline.  Synchronizes. */
 lbm_status lbm_stefan_step_timed(lbm_stefan* h, int nsteps, double* ms_kernels);
 
-/* Test hook of the TMA row-pipeline kernel (the FP32 D2Q9 kernel whose
- * blocks wait for row loads that they issued themselves; FP32 D2Q9 batches
- * run it).  Only FP32 D2Q9 handles use it; other handles ignore it.
+/* Test hook of the TMA row-pipeline kernel (an FP32 D2Q9 kernel whose blocks
+ * wait for row loads that they issued themselves; it runs under this hook
+ * only).  Only FP32 D2Q9 handles use it; other handles ignore it.
  * wait_limit_s > 0 bounds every such wait (default 2 s).  While
  * withhold_load is in {0, 1, 2}, the handle's steps run that kernel in place
- * of the flat interior / wall-row pair, and its first block skips that row
+ * of the resident one, and its first block skips that row
  * load (its rows are a range of the 128-column strip at x = 0; load 0 is the
  * row above the range, load 1 its first row): the waits for it run out, the
  * block stops after the loads it has in flight have landed (each of those
  * waits bounded too), and the next synchronizing call returns
  * LBM_ERR_TIMEOUT (the handle's state is then undefined; create a new one).
- * withhold_load = -1 restores normal steps (the flat pair).  LBM_ERR_ARG for
+ * withhold_load = -1 restores normal steps.  LBM_ERR_ARG for
  * a value outside [-1, 2] or a wait limit outside (0, 60] s. */
 lbm_status lbm_stefan_set_wait_test(lbm_stefan* h, double wait_limit_s, int withhold_load);
 
 /* Test hook of the resident launches, whose blocks wait for one another at
  * barriers in device memory.  wait_limit_s in (0, 60] bounds every such wait
- * (default 5 s).  withhold >= 0: the first block does not arrive at that barrier
+ * (default 5 s): it runs out when no block of the launch has arrived at any barrier
+ * for that long (to twice that long).  withhold >= 0: the first block does not arrive at that barrier
  * of each launch (0: after the launch's first step; LBM_ILFBM: an inner
  * iteration's), so the waits for it run out, the launch ends normally and the next
  * synchronizing call returns LBM_ERR_TIMEOUT; the state is undefined until the
@@ -298,7 +306,7 @@ lbm_status lbm_stefan_adjoint_run(lbm_stefan* h, int nsteps, const double* theta
  * entry; *result_index tells which buffer holds lambda at its start).  On a
  * non-default stream the launches after the checkpoint copy are captured
  * once per (nsteps, theta_traj, adj, adj_other) and replayed as a CUDA graph
- * (at most 8 kept; set_bc, set_ste and set_method drop them).  Afterwards
+ * (at most 8 kept; set_bc, set_ste, set_method and the test hooks drop them).  Afterwards
  * the current state is the segment's end.  Asynchronous on the handle's
  * stream.  LBM_ERR_ARG for NULL pointers, nsteps < 1, adj == adj_other or
  * another lattice; LBM_ERR_STATE for another method. */
@@ -314,15 +322,17 @@ lbm_status lbm_stefan_adjoint_finish(lbm_stefan* h, const void* adj0, double* g_
 void lbm_stefan_destroy(lbm_stefan* h);
 
 /* ---------------------------------------------------------------- batches
- * Many independent D2Q9 problems of uneven sizes advanced by kernel launches
- * over all problems at once, then the Newton job kernel; the launches of a
- * call are captured in a CUDA graph.  FP32: the kernels of the single-problem
- * FP32 step over tables (the S and N wall rows and the W and E wall groups of
- * every problem, one block per 128-column x 8-row tile of every problem); on
- * a stream of the batch's own, the single problem's split step (the left
- * halves' Newton solves beside the right halves' streaming on a second
- * stream); FP64: the persistent warp-tile kernel over a schedule of warp
- * tiles.  The order of the problems (and, in FP64, the tile height) come from
+ * Many independent D2Q9 problems of uneven sizes advanced together.  FP32: all
+ * the steps of a call in cooperative launches over units of every problem
+ * (128-column x 8-row tiles, wall rows, W and E wall groups), as
+ * lbm_stefan_step's.  Where that grid does not fit, or a problem has 65,536
+ * columns or rows or 2^31 elements: the separate kernels of the FP32 step over
+ * tables of tiles, wall rows and wall groups, then the Newton job kernel, on a
+ * stream of the batch's own as the split step (the left halves' Newton solves
+ * beside the right halves' streaming on a second stream).  FP64: the persistent
+ * warp-tile kernel over a schedule of warp tiles and the job kernel.  Separate
+ * kernels are replayed from a CUDA graph on a stream of the batch's own.  The
+ * order of the problems (and, in FP64, the tile height) come from
  * lbm_stefan_batch_autotune (or defaults). */
 
 typedef struct {

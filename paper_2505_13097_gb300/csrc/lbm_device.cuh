@@ -494,7 +494,9 @@ __device__ __forceinline__ NewtonNode newton_mixed(double mm, double tt, double 
 }
 
 // ---------------------------------------------------------------- exact sums
-// sum of Q doubles, to within 2^-6 ulp of the largest per term, rounded once:
+// sum of Q doubles, to within 2^-6 ulp of the largest per term, rounded once
+// (error against 113-bit sums of populations, units of 2^-53 of the largest: at most
+// 3.8, 0.95 rms for nine; added one after the other 8.0 and 1.4):
 // the mantissas are aligned to the largest exponent with six guard bits (59
 // bits; nine of them stay below 2^63) and added as integers, 15 integer
 // instructions per term against 64 cycles of FP64 pipe per addition.  Terms

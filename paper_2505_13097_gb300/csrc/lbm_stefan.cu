@@ -461,8 +461,9 @@ static cudaError_t launch_one(lbm_stefan* h, int parity, double* rec)
 // What a barrier takes before the sums of its launch.
 constexpr size_t kBarBytes = (sizeof(lbm::ResidentBar) + 255) / 256 * 256;
 
-// Steps of one resident launch: 2^32 node updates (some 60 ms), so that other streams
-// get the GPU in between; at most 8,192.
+// Steps of one resident launch: 2^32 node updates (55 ms of FP32 D2Q9 steps at 4096^2, 146 ms
+// in FP64), so that other streams get the GPU in between; at least 32 (the most updates beyond
+// 2^27 nodes) and at most 8,192.
 static int resident_steps(long long nodes, const lbm::ResidentLimits& lim)
 {
     const int n = (int)std::max(32ll, std::min(8192ll, (1ll << 32) / std::max(1ll, nodes)));
@@ -500,10 +501,12 @@ static cudaError_t run_resident(lbm_stefan* h, int* nsteps, int* parity, double*
 #define LBM_RESIDENT 1
 #endif
 // The largest lattice that steps in resident launches (measured us per step, separate
-// kernels / resident).  FP32 D2Q9 IREBM: 235 / 221 at 4096^2, 473 / 443 at 8192 x 4096,
-// 849 / 855 at 8192^2; EEBM, which has no Newton work to hide: 69 / 56 at 2048^2, 203 / 199
-// at 4096^2.  FP64 and D2Q5 gain at every size (D2Q9 FP64 966 / 547 and D2Q5 FP32 183 / 124
-// at 4096^2): the bound is that of the 32-bit indices, 2^31 elements of a state.
+// kernels / resident).  FP32 D2Q9 IREBM: 235 / 216 at 4096^2, 306 / 282 at 5000 x 4400, 447 /
+// 435 at 5792^2, 433 / 438 at 8192 x 4096 (2^25 nodes: even), 843 / 873 at 8192^2; EEBM, which
+// has no Newton work to hide: 68 / 55 at 2048^2, 202 / 199 at 4096^2, 262 / 266 at 5000 x 4400,
+// 400 / 426 at 8192 x 4096.  FP64 and D2Q5 gain at every size (D2Q9 FP64 880 / 570, D2Q5 FP32
+// 179 / 123 and FP64 509 / 465 at 4096^2): the bound is that of the 32-bit indices, 2^31
+// elements of a state.
 static long long resident_max_nodes(int lattice, int precision, int method)
 {
     if (!LBM_RESIDENT) return 0;

@@ -1,16 +1,16 @@
 // D2Q9 and D2Q5 steps in one resident launch: a cooperative grid keeps its
-// blocks on the SMs for all the steps of a call, one node per thread, the
-// Newton solve of Eq. (14) in place, one grid barrier per step.
+// blocks on the SMs for all the steps of a call, four nodes per thread (FP64:
+// one), the Newton solve of Eq. (14) in place, one grid barrier per step.
 //
 // What bounds it.  A step of a small lattice launched kernel by kernel is a
 // chain of latencies: the wall kernels, the stencil, the side and the last
 // Newton launch and the publication of the statistics, 45 us whatever the size
 // (130 x 64 nodes, FP32).  Here a step ends at one barrier (load, arrival, poll
 // and fence: 4 to 5 us on a lattice of a few hundred nodes), and its sums are
-// added up by a block of their own while the next step runs.  Measured, us per
-// step before and now: D2Q9 FP32 130 x 64 45 / 9, 1021 x 777 61 / 16.5, 4096^2
-// 232 / 214; D2Q9 FP64 2048^2 387 / 150; D2Q5 FP32 4096^2 205 / 123, FP64 401^2
-// 116 / 17.
+// added up by a block of their own while the next step runs.  Measured on the same
+// states, us per step by the separate kernels / here: D2Q9 FP32 130 x 64 33 / 9.2,
+// 1021 x 777 39 / 15.8, 4096^2 235 / 216; D2Q9 FP64 2048^2 310 / 154; D2Q5 FP32
+// 4096^2 179 / 123, FP64 401^2 117 / 17.
 //
 // A step has two passes over what a block owns, between barriers of the block:
 //  1. plain nodes.  A warp takes a group of 32 N consecutive columns of one of
@@ -18,7 +18,7 @@
 //     flat kernel; 1 in FP64).  Saturated nodes are updated, the nodes that
 //     need the Newton solve go to a queue in shared memory.
 //  2. items of 32 nodes, one per lane: the queued nodes, gathered densely so
-//     that a solve (a chain of 43 FP64 instructions of 64 cycles) serves full
+//     that a solve (a chain of 43 or 44 FP64 instructions of 64 cycles) serves full
 //     warps, the rows 0 and ny-1, and the column groups at the W and E walls.
 // Groups of a wave lie side by side (their halo rows and columns meet in L1 and
 // L2), and a block's place in the wave rotates from wave to wave, so that the
@@ -33,14 +33,21 @@
 // Arithmetic: that of the kernels in step_d2q9.cu / step_d2q5.cu node by node.
 // FP64 form: the zeroth moment is summed in block floating point with integer
 // instructions (sum_q) and w_i c takes two multiplications, 11 FP64
-// instructions per D2Q9 node instead of 28: the FP64 pipe, one warp
-// instruction per 64 cycles of an SM quarter, bounds the FP64 form.
+// instructions per D2Q9 node instead of 28, on a pipe that takes one warp
+// instruction per 64 cycles of an SM quarter.  That pipe is 63 % busy at 2048^2
+// and DRAM 46 % of its peak; the rest is latency at 24 warps per SM (stalls per
+// issue: loads 3.6, fixed latencies 2.6, barrier 2.1, shared memory 1.9).
 #include <algorithm>
 
 #include "d2q5_row.cuh"
 #include "d2q9_row.cuh"
 #include "resident.cuh"
 
+// Lattices of up to this many units (32 columns of a row) per computing block take no
+// first pass.  us per step with items alone / with two passes: D2Q9 FP32 128^2 9.0 /
+// 14.5, 160^2 10.1 / 10.9, 256^2 14.2 / 10.6, FP64 128^2 13.3 / 16.9, 256^2 28.9 / 17.1,
+// D2Q5 FP32 128^2 8.1 / 20.8, 160^2 9.1 / 11.5, 256^2 12.7 / 11.6 (8 units per block lie
+// near 195^2).
 #ifndef LBM_RES_SCALAR
 #define LBM_RES_SCALAR 8
 #endif
@@ -320,8 +327,8 @@ __device__ __forceinline__ void ld4(const float* p, float (&v)[4])
 
 // The queue (dynamic shared memory) has room for every node of kResidentWaves
 // waves of the first pass; the second pass follows that many waves.  FP32: 64 and
-// 96 KB; more costs L1 (4096^2 with 16 waves 232 us instead of 220), FP64 48 KB
-// (2048^2 with 8 / 16 waves: 161 / 154 us).
+// 96 KB; more costs L1 (8 / 16 waves, us per step: D2Q9 4096^2 218 / 222, EEBM 201 / 210,
+// D2Q5 124 / 156).  FP64: 48 KB (8 / 16 waves: D2Q9 2048^2 177 / 166, 4096^2 608 / 571).
 template <typename P> constexpr int kResidentWaves = sizeof(P) == 4 ? 8 : 16;
 
 struct ResidentQueue {
@@ -531,9 +538,9 @@ __device__ __forceinline__ void plain_update(const Problem& pb, const double* sr
 
 // One block per SM.  D2Q9 in FP32: 512 threads leave 128 registers, without spills,
 // and 16 warps take two 8-row tiles at a time (us per step with 768 / 512 threads:
-// 4096^2 227 / 221, EEBM 2048^2 60 / 56); D2Q5 in FP32 streams less per node and wants
-// the warps (4096^2, 768 / 640: 127 / 141), and so does FP64, whose sums are integer
-// work beside the FP64 pipe (2048^2, 768 / 640: 161 / 180).
+// 4096^2 221 / 218, EEBM 212 / 201); D2Q5 in FP32 streams less per node and wants
+// the warps (4096^2, 640 / 768: 140 / 124), and so does FP64, whose sums are integer
+// work beside the FP64 pipe (2048^2, 640 / 768: D2Q9 183 / 166, D2Q5 145 / 130).
 template <typename P, int Q> constexpr int kResidentThreads = sizeof(P) == 4 && Q == 9 ? 512 : 768;
 
 template <typename P, int Q, bool EEBM>
@@ -947,7 +954,13 @@ static ResidentPlan resident_plan_t(int nx, int ny)
         r.threads = wpb * 32;
     } else {
         r.strips = (nx + 32 * N - 1) / (32 * N);
-        // tall tiles share their halo rows; short ones spread a front band over the blocks
+        // tall tiles share their halo rows; short ones spread a front band over the blocks and leave
+        // fewer warps idle in the last wave.  us per step with 8 / 2 rows, the line (16 units per
+        // warp) at 2232^2 in FP32 D2Q9, 1367^2 in FP64, 2733^2 in FP32 D2Q5: D2Q9 FP32 512^2
+        // 13.3 / 11.9, 1400^2 36.6 / 33.5, 3000^2 123.7 / 125.3, 4096^2 214.3 / 215.5; D2Q9 FP64
+        // 1200^2 72.1 / 67.8, 1600^2 111.0 / 108.3, 2048^2 166.6 / 170.8; D2Q5 FP32 1800^2 36.7 /
+        // 29.9, 3200^2 84.7 / 77.8, 4096^2 122.6 / 122.3; D2Q5 FP64 1600^2 85.4 / 82.9, 2048^2
+        // 130.3 / 132.7.  (In FP64 and D2Q5 2 rows still gain up to a tenth just beyond the line.)
         r.th = vec >= 16ll * most * cap ? 8 : 2;
         r.tiles = r.strips * ((ny - 2 + r.th - 1) / r.th);
         r.items = 2 * r.nseg + (ny - 2 + 32 / (2 * N) - 1) / (32 / (2 * N));
